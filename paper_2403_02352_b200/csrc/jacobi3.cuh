@@ -95,126 +95,293 @@ __device__ __forceinline__ bool group_barrier(unsigned *sync, unsigned gen, unsi
     return ok_s != 0;
 }
 
-// Rotation (c, s) that annihilates the (p, q) entry of a symmetric matrix; identity when the entry is
-// already small against its diagonal. With a = g_qq - g_pp, b = 2 g_pq, r = sqrt(a^2 + b^2):
-//   cos 2t = |a| / r,  c = sqrt((1 + cos 2t) / 2),  s = sign(a) b / (2 r c)      (|t| <= pi/4).
-__device__ __forceinline__ float2 rotation(float gpp, float gqq, float gpq, float tol_rot)
-{
-    float c = 1.f, s = 0.f;
-    if (gpq != 0.f && gpq * gpq > tol_rot * tol_rot * fmaxf(gpp, 0.f) * fmaxf(gqq, 0.f)) {
-        float a = gqq - gpp, b = 2.f * gpq;
-        const float m = fmaxf(fabsf(a), fabsf(b));
-        const float sc = m < 1e-18f ? 0x1p60f : (m > 1e18f ? 0x1p-60f : 1.f);
-        a *= sc; b *= sc;
-        const float rh = rsqrtf(fmaf(a, a, b * b));
-        const float c2 = fmaf(0.5f * fabsf(a), rh, 0.5f);
-        const float rc = rsqrtf(c2);
-        c = c2 * rc;
-        s = copysignf(0.5f, a) * b * rh * rc;
+// ---- pivot phase -------------------------------------------------------------------------------
+// The 64 rows of a pivot block sit in 32 "even" and 32 "odd" slots. A phase of width M rotates, in M rounds, every
+// even slot k with the odd slots of its own group of M: in round rd with slot base(k) + ((k - rd) mod M). Width 32
+// pairs every row of the first block with every row of the second; widths 16, 8, 4, 2, 1 pair the rows inside the
+// blocks; together the 63 rounds rotate each of the 2016 pairs exactly once. Slot -> logical row (0..31 first block,
+// 32..63 second block): the logical rows are cut in groups of 2M; the first M of a group are even slots, the last M odd.
+//
+// What bounds a round is the chain rotation -> entry of the next pair -> next rotation, so the layout makes that
+// chain live in one warp. Lane k of a warp holds, for offsets d = 0 .. M/2, the 2 x 2 blocks between the pairs k and
+// k + d (mod M; the matrix is symmetric, so half of the offsets suffice):
+//     ee[d] = A[E(k)][E(k+d)]   eo[d] = A[E(k)][O(k+d)]   oe[d] = A[O(k)][E(k+d)]   oo[d] = A[O(k)][O(k+d)]
+// with O(k) the odd row now paired with E(k). Moving to the next pairing, O(k) <- O(k-1), is then
+//     oo[d] <- oo[d] of lane k-1,   oe[d] <- oe[d+1] of lane k-1,   eo[d] <- eo[d-1] of the same lane,
+//     eo[0] <- oe[1] of lane k-1,   oe[M/2] <- eo[M/2-1] of lane k+M/2,
+// and the 2 x 2 problem of the next round needs the offsets 0 and 1 only: warp 0 owns them, derives the next 32
+// rotations from two shuffles and publishes them. Width 32: offsets 0-2, 3-7, 8-12, 13-16 live in warps 0-3, and the
+// entries that cross a warp boundary go through shared memory; one block barrier a round. Widths <= 16 only need the
+// diagonal sub-blocks (the block itself is discarded afterwards, only the transform is kept): warp 0 holds them all.
+// Warps 4-7 apply the published rotations to the transform: lane = two columns, warp = a quarter of the row pairs.
+// Second bound: issue slots, FMA and shared-memory cycles of those updates. The rotations are therefore applied without
+// their common factor c (Gentleman's fast Givens form): row = d * stored row, and with t = s / c
+//     x~ <- x~ - beta y~,  y~ <- y~ + gamma x~,   beta = t d_y / d_x,  gamma = t d_x / d_y,   d_x, d_y <- c d_x, c d_y,
+// two multiply-adds instead of four operations; |t| <= 1, so d loses at most a factor 2^-16 in 32 rounds. The factors
+// live in warp 0 and are multiplied back at the end of a phase.
+// Cross phase of 32 rounds, one CTA alone on an SM: 31500 -> 9600 cycles; all 63 rounds: 68000 -> 23600 (the layout
+// before put a quarter of the rows in each thread: every round moved a row between warps behind a second barrier, and
+// the next rotation waited for all of it). Packed fp32x2 arithmetic was slower: 13900 cycles, it adds register moves.
+constexpr int LDP = 65;           // row stride of the logical pivot block and transform in shared memory
+
+struct PivotShared {
+    float2 bg[2][32];             // (beta, gamma) of the current round, by round parity
+    float2 vx[2][4][32];          // last odd row of each quarter of the transform
+    float up[2][3][32];           // eo of the last offset of warp w, for warp w + 1
+    float dn[2][3][32];           // oe of the first offset of warp w + 1, for warp w
+    float sd[2][64];              // row factors d at the end of a phase (even slots, odd slots), by phase parity
+    float red[4];
+};
+
+__device__ __forceinline__ float rsqrt_ftz(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+
+// The rotations of the pairs of warp 0, one per lane, with the row factors of the pair (and their reciprocals) and the
+// two diagonal entries.
+struct Rotor {
+    float de, ie, dod, io, gpp, gqq;
+    __device__ __forceinline__ void reset(float ee, float oo) { de = ie = dod = io = 1.f; gpp = ee; gqq = oo; }
+    // Rotation that annihilates the entry between the rows p (even) and q (odd) of a symmetric matrix, stored as eo;
+    // identity when the entry is already small against its diagonal. With a = g_qq - g_pp, b = 2 g_pq,
+    // r = sqrt(a^2 + b^2):
+    //   cos 2t = |a| / r,  c = sqrt((1 + cos 2t) / 2),  tan t = sign(a) b / (2 r c^2)      (|t| <= pi/4).
+    // What does not depend on eo (it arrives last) comes first; the squares are kept in range by a power of two chosen
+    // from the diagonal. Returns (beta, gamma) and advances the factors and the diagonal.
+    __device__ __forceinline__ float2 next(float eo, float tol2)
+    {
+        const float w = de * dod, dp = fmaxf(gpp, 0.f), dq = fmaxf(gqq, 0.f), md = fmaxf(dp, dq);
+        const float sc = md < 1e-18f ? 0x1p60f : (md > 1e18f ? 0x1p-60f : 1.f);
+        const float a = (gqq - gpp) * sc, a2 = a * a, ah = 0.5f * fabsf(a), sgw = copysignf(sc, a) * w;
+        const float thr = tol2 * dp * dq, scw = 2.f * sc * w, kb = dod * ie, kg = de * io;
+        const float b = eo * scw;
+        const float r2 = fmaf(b, b, a2);
+        const float rh = rsqrt_ftz(r2);
+        const float c2 = fmaf(ah, rh, 0.5f);
+        const float rc = rsqrt_ftz(c2);
+        const float gpq = eo * w;
+        const bool on = gpq * gpq > thr && r2 > 0.f;
+        const float t = on ? (eo * sgw) * rh * (rc * rc) : 0.f;
+        const float2 out = make_float2(t * kb, t * kg);
+        gpp = fmaf(-t, gpq, gpp); gqq = fmaf(t, gpq, gqq);
+        const float c = on ? c2 * rc : 1.f, ic = on ? rc : 1.f;
+        de *= c; dod *= c; ie *= ic; io *= ic;
+        ie = ie * fmaf(-de, ie, 2.f); io = io * fmaf(-dod, io, 2.f);      // keeps d * (1 / d) = 1 to the last bit or so
+        return out;
     }
-    return make_float2(c, s);
+    __device__ __forceinline__ void shift(int km)
+    {
+        dod = __shfl_sync(0xffffffffu, dod, km); io = __shfl_sync(0xffffffffu, io, km); gqq = __shfl_sync(0xffffffffu, gqq, km);
+    }
+};
+
+// [ee eo; oe oo] <- R(ra) [ee eo; oe oo] R(rb)^T with R(r) = [1 -beta; gamma 1]
+__device__ __forceinline__ void rotate_block(float2 ra, float2 rb, float &ee, float &eo, float &oe, float &oo)
+{
+    const float r0 = fmaf(-ra.x, oe, ee), r1 = fmaf(-ra.x, oo, eo);
+    const float r2 = fmaf(ra.y, ee, oe), r3 = fmaf(ra.y, eo, oo);
+    ee = fmaf(-rb.x, r1, r0); eo = fmaf(rb.y, r0, r1);
+    oe = fmaf(-rb.x, r3, r2); oo = fmaf(rb.y, r2, r3);
 }
 
-// ---- pivot phase -------------------------------------------------------------------------------
-// The 64 rows of a pivot block sit in 32 "even" and 32 "odd" slots. A phase of width m rotates, in m
-// rounds, every even slot k with the odd slots of its own group of m: in round rd with slot
-// base(k) + ((k - rd) mod m). The data never moves between rounds, only the pairing shifts, so every
-// thread keeps its elements in registers:
-//   thread (warp w, lane l) owns the even rows 4w..4w+3 and column slot l of the four quadrants
-//     ee[a] = A[E(4w+a)][E(l)]   eo[a] = A[E(4w+a)][O(s(l))]
-//     oe[a] = A[O(s(4w+a))][E(l)]   oo[a] = A[O(s(4w+a))][O(s(l))]         s = current pairing
-//   and the same rows of the accumulated transform Vt (two logical columns l, l + 32).
-// The 2 x 2 problem of pair k is complete in the thread with 4w+a = l, which derives the rotation and
-// publishes it; everybody applies the rotations of its four row pairs and of its column pair. Moving
-// to the next pairing shifts the odd quadrants by one slot: along the columns by a lane shuffle,
-// along the rows inside the thread, except the last of its four rows, which goes to the next warp
-// through shared memory (4 floats per thread and round).
-// Slot -> logical row (0..31 first block, 32..63 second block) for a phase of width m: the logical
-// rows are cut in groups of 2m; the first m of a group are even slots, the last m odd slots. Width 32
-// pairs every row of the first block with every row of the second; widths 16, 8, 4, 2, 1 pair the rows
-// inside the blocks; together the 63 rounds rotate each of the 2016 pairs exactly once.
-constexpr int LDP = 65;           // row stride of the logical A and Vt copies in shared memory
-__device__ __forceinline__ int slot_even(int i, int m) { return 2 * m * (i / m) + (i % m); }
-
-__device__ void cross_phase(float *As, float *Vs, float2 *rot, float4 *xch, int m, float tol_rot)
-{
-    const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
-    float ee[4], eo[4], oe[4], oo[4], ve[4][2], vo[4][2];
-    const int cE = slot_even(l, m), cO = cE + m;
+// Offsets of a width-32 phase in warp W of 0..3: 0-2, 3-7, 8-12, 13-16 (warp 0 has the rotations to do as well).
+template <int W> struct Band {
+    static constexpr int D0 = W == 0 ? 0 : 5 * W - 2, ND = W == 0 ? 3 : (W == 3 ? 4 : 5);
+    float ee[ND], eo[ND], oe[ND], oo[ND];
+    // loads the offsets from As, returns the largest scaled off-diagonal entry among them
+    __device__ __forceinline__ float load(const float *As)
+    {
+        const int k = threadIdx.x & 31;
+        const float de = fmaxf(As[k * (LDP + 1)], 0.f), dd = fmaxf(As[(32 + k) * (LDP + 1)], 0.f);
+        float mo = 0.f;
+        auto see = [&](float g, float d0, float d1) {
+            const float d2 = d0 * d1;
+            if (d2 > 0.f) mo = fmaxf(mo, fabsf(g) * rsqrtf(d2));
+        };
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int rE = slot_even(4 * w + a, m) * LDP, rO = rE + m * LDP;
-        ee[a] = As[rE + cE]; eo[a] = As[rE + cO]; oe[a] = As[rO + cE]; oo[a] = As[rO + cO];
-        ve[a][0] = Vs[rE + l]; ve[a][1] = Vs[rE + l + 32];
-        vo[a][0] = Vs[rO + l]; vo[a][1] = Vs[rO + l + 32];
-    }
-    const int ad = l - 4 * w;                                   // 0..3: this thread completes pair 4w + ad
-    const int src_lane = (l & ~(m - 1)) | ((l - 1) & (m - 1));  // previous column slot of the group
-    const int wg = m >= 8 ? m / 4 : 1;                          // warps per row group
-    const int wprev = (w & ~(wg - 1)) | ((w - 1) & (wg - 1));
-    for (int rd = 0; rd < m; ++rd) {
-        float2 *rt = rot + (rd & 1) * 32;
-        if ((unsigned)ad < 4u) {
-            const float x = ad == 0 ? ee[0] : ad == 1 ? ee[1] : ad == 2 ? ee[2] : ee[3];
-            const float y = ad == 0 ? oo[0] : ad == 1 ? oo[1] : ad == 2 ? oo[2] : oo[3];
-            const float z = ad == 0 ? eo[0] : ad == 1 ? eo[1] : ad == 2 ? eo[2] : eo[3];
-            rt[l] = rotation(x, y, z, tol_rot);
+        for (int i = 0; i < ND; ++i) {
+            const int l = (k + D0 + i) & 31;
+            ee[i] = As[k * LDP + l]; eo[i] = As[k * LDP + 32 + l];
+            oe[i] = As[(32 + k) * LDP + l]; oo[i] = As[(32 + k) * LDP + 32 + l];
+            const float le = fmaxf(As[l * (LDP + 1)], 0.f), lo = fmaxf(As[(32 + l) * (LDP + 1)], 0.f);
+            if (D0 + i > 0) { see(ee[i], de, le); see(oo[i], dd, lo); }
+            see(eo[i], de, lo); see(oe[i], dd, le);
         }
+        return mo;
+    }
+    // the 32 rounds; with `store` the diagonal quadrants (both blocks after the cross rotations) go back to As
+    __device__ __forceinline__ void rounds(float *As, PivotShared &sh, float tol2, bool store)
+    {
+        const int k = threadIdx.x & 31, km = (k - 1) & 31;
+        float2 own = make_float2(0.f, 0.f), nxt = own;           // warp 0: rotations of the pairs k and k + 1
+        Rotor rot;
+        auto publish = [&](int par, bool last) {
+            own = rot.next(eo[0], tol2);
+            sh.bg[par][k] = own;
+            if (last) { sh.sd[0][k] = rot.de; sh.sd[0][32 + ((k + 1) & 31)] = rot.dod; }
+            rot.shift(km);
+            nxt.x = __shfl_sync(0xffffffffu, own.x, (k + 1) & 31);
+            nxt.y = __shfl_sync(0xffffffffu, own.y, (k + 1) & 31);
+        };
+        if (W == 0) { rot.reset(ee[0], oo[0]); publish(0, false); }
         __syncthreads();
-        const float2 cb = rt[l];
+#pragma unroll 2
+        for (int rd = 0; rd < 32; ++rd) {
+            const int par = rd & 1;
+            const float2 ra = W == 0 ? own : sh.bg[par][k];
+            float2 rb[ND];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const float2 ca = rt[4 * w + a];
-            const float r0 = ca.x * ee[a] - ca.y * oe[a], r1 = ca.x * eo[a] - ca.y * oo[a];
-            const float r2 = ca.y * ee[a] + ca.x * oe[a], r3 = ca.y * eo[a] + ca.x * oo[a];
-            ee[a] = cb.x * r0 - cb.y * r1; eo[a] = cb.y * r0 + cb.x * r1;
-            oe[a] = cb.x * r2 - cb.y * r3; oo[a] = cb.y * r2 + cb.x * r3;
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const float x = ve[a][c], y = vo[a][c];
-                ve[a][c] = ca.x * x - ca.y * y; vo[a][c] = ca.y * x + ca.x * y;
+            for (int i = 0; i < ND; ++i) rb[i] = W == 0 && i == 0 ? own : W == 0 && i == 1 ? nxt : sh.bg[par][(k + D0 + i) & 31];
+            if (rd > 0) {                                        // entries that crossed a warp boundary in the last shift
+                if (W > 0) eo[0] = sh.up[par ^ 1][W > 0 ? W - 1 : 0][k];
+                if (W < 3) oe[ND - 1] = sh.dn[par ^ 1][W < 3 ? W : 0][km];
             }
-        }
-        if (m == 1) break;
-        // next pairing: odd rows shift by one slot inside their group ...
-        float4 in;
-        if (m >= 8) {
-            xch[tid] = make_float4(oe[3], oo[3], vo[3][0], vo[3][1]);
+#pragma unroll
+            for (int i = 0; i < ND; ++i) rotate_block(ra, rb[i], ee[i], eo[i], oe[i], oo[i]);
+            // next pairing
+            if (W < 3) sh.up[par][W < 3 ? W : 0][k] = eo[ND - 1];
+            if (W > 0) sh.dn[par][W > 0 ? W - 1 : 0][k] = oe[0];
+            float wrap = 0.f, in0 = 0.f;
+            if (W == 0) in0 = __shfl_sync(0xffffffffu, oe[1], km);
+            if (W == 3) wrap = __shfl_sync(0xffffffffu, eo[ND - 2], k ^ 16);
+#pragma unroll
+            for (int i = 0; i < ND; ++i) oo[i] = __shfl_sync(0xffffffffu, oo[i], km);
+#pragma unroll
+            for (int i = ND - 1; i > 0; --i) eo[i] = eo[i - 1];
+            if (W == 0) eo[0] = in0;
+            if (W == 0 && rd < 31) publish(par ^ 1, rd == 30);
+#pragma unroll
+            for (int i = 0; i + 1 < ND; ++i) oe[i] = __shfl_sync(0xffffffffu, oe[i + 1], km);
+            if (W == 3) oe[ND - 1] = wrap;
             __syncthreads();
-            in = xch[wprev * 32 + l];
-        } else if (m == 4) {
-            in = make_float4(oe[3], oo[3], vo[3][0], vo[3][1]);
         }
-        if (m >= 4) {
+        if (store) {
+            const float de = sh.sd[0][k], dd = sh.sd[0][32 + k];
 #pragma unroll
-            for (int a = 3; a > 0; --a) { oe[a] = oe[a - 1]; oo[a] = oo[a - 1]; vo[a][0] = vo[a - 1][0]; vo[a][1] = vo[a - 1][1]; }
-            oe[0] = in.x; oo[0] = in.y; vo[0][0] = in.z; vo[0][1] = in.w;
-        } else {                                                // m == 2: rows (0,1) and (2,3) swap
-#pragma unroll
-            for (int a = 0; a < 4; a += 2) {
-                float t;
-                t = oe[a]; oe[a] = oe[a + 1]; oe[a + 1] = t;
-                t = oo[a]; oo[a] = oo[a + 1]; oo[a + 1] = t;
-                t = vo[a][0]; vo[a][0] = vo[a + 1][0]; vo[a + 1][0] = t;
-                t = vo[a][1]; vo[a][1] = vo[a + 1][1]; vo[a + 1][1] = t;
+            for (int i = 0; i < ND; ++i) {
+                const int l = (k + D0 + i) & 31;
+                const float e = ee[i] * de * sh.sd[0][l], o = oo[i] * dd * sh.sd[0][32 + l];
+                As[k * LDP + l] = e; As[l * LDP + k] = e;
+                As[(32 + k) * LDP + 32 + l] = o; As[(32 + l) * LDP + 32 + k] = o;
             }
         }
-        // ... and so do the odd columns
+    }
+};
+
+// A phase of width M <= 16 on the diagonal sub-blocks of 2M rows, in warp 0; one block barrier per round. ph: phase parity.
+template <int M> __device__ __forceinline__ void inner_phase(float *As, PivotShared &sh, float tol2, int ph)
+{
+    constexpr int ND = M / 2 + 1;
+    const int k = threadIdx.x & 31, g = k & ~(M - 1), q = k & (M - 1);
+    const int E = 2 * g + q, km = g | ((q - 1) & (M - 1)), kp = g | ((q + 1) & (M - 1)), kh = g | ((q + M / 2) & (M - 1));
+    float ee[ND], eo[ND], oe[ND], oo[ND];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            eo[a] = __shfl_sync(0xffffffffu, eo[a], src_lane);
-            oo[a] = __shfl_sync(0xffffffffu, oo[a], src_lane);
+    for (int i = 0; i < ND; ++i) {
+        const int F = 2 * g + ((q + i) & (M - 1));
+        ee[i] = As[E * LDP + F]; eo[i] = As[E * LDP + F + M];
+        oe[i] = As[(E + M) * LDP + F]; oo[i] = As[(E + M) * LDP + F + M];
+    }
+    Rotor rot;
+    rot.reset(ee[0], oo[0]);
+    float2 own = rot.next(eo[0], tol2);
+    sh.bg[0][k] = own;
+    if (M == 1) { sh.sd[ph][k] = rot.de; sh.sd[ph][32 + k] = rot.dod; }
+    rot.shift(km);
+#pragma unroll 1
+    for (int rd = 0; rd < M; ++rd) {
+        const int par = rd & 1;
+        __syncthreads();
+        float2 rb[ND];
+#pragma unroll
+        for (int i = 0; i < ND; ++i) rb[i] = i == 0 ? own : sh.bg[par][g | ((q + i) & (M - 1))];
+#pragma unroll
+        for (int i = 0; i < ND; ++i) rotate_block(own, rb[i], ee[i], eo[i], oe[i], oo[i]);
+        if (M > 1) {
+            const float in0 = __shfl_sync(0xffffffffu, oe[ND > 1 ? 1 : 0], km);
+            const float wrap = __shfl_sync(0xffffffffu, eo[ND > 1 ? ND - 2 : 0], kh);
+#pragma unroll
+            for (int i = 0; i < ND; ++i) oo[i] = __shfl_sync(0xffffffffu, oo[i], km);
+#pragma unroll
+            for (int i = ND - 1; i > 0; --i) eo[i] = eo[i - 1];
+            eo[0] = in0;
+            if (rd + 1 < M) {
+                own = rot.next(eo[0], tol2);
+                sh.bg[par ^ 1][k] = own;
+                if (rd + 2 == M) { sh.sd[ph][k] = rot.de; sh.sd[ph][32 + kp] = rot.dod; }
+                rot.shift(km);
+            }
+#pragma unroll
+            for (int i = 0; i + 1 < ND; ++i) oe[i] = __shfl_sync(0xffffffffu, oe[i + 1], km);
+            oe[ND - 1] = wrap;
         }
     }
-    // after m shifts (none for m = 1) every element is back where it was loaded from
+    if (M > 1) {
+        const float de = sh.sd[ph][k], dd = sh.sd[ph][32 + k];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int rE = slot_even(4 * w + a, m) * LDP, rO = rE + m * LDP;
-        As[rE + cE] = ee[a]; As[rE + cO] = eo[a]; As[rO + cE] = oe[a]; As[rO + cO] = oo[a];
-        Vs[rE + l] = ve[a][0]; Vs[rE + l + 32] = ve[a][1];
-        Vs[rO + l] = vo[a][0]; Vs[rO + l + 32] = vo[a][1];
+        for (int i = 0; i < ND; ++i) {
+            const int l = (q + i) & (M - 1), F = 2 * g + l;
+            const float e = ee[i] * de * sh.sd[ph][g + l], o = oo[i] * dd * sh.sd[ph][32 + g + l];
+            As[E * LDP + F] = e; As[F * LDP + E] = e;
+            As[(E + M) * LDP + F + M] = o; As[(F + M) * LDP + E + M] = o;
+        }
+        __syncwarp();
     }
-    __syncthreads();
+}
+
+// The transform's share of a phase (warps 4..7): lane = columns l and l + 32, warp 4 + h = the rows of the pairs
+// 8 h .. 8 h + 7. Widths 32 and 16: ve / vo = even and odd rows in slot order; the odd row that leaves the quarter goes to
+// the next quarter of its group through shared memory. Widths <= 8: the 16 rows 16 h .. 16 h + 15 in v.
+__device__ __forceinline__ void rotate_rows(float b, float g, float2 &x, float2 &y)
+{
+    const float2 t = x;
+    x = make_float2(fmaf(-b, y.x, t.x), fmaf(-b, y.y, t.y));
+    y = make_float2(fmaf(g, t.x, y.x), fmaf(g, t.y, y.y));
+}
+__device__ __forceinline__ void scale_row(float2 &x, float d) { x.x *= d; x.y *= d; }
+__device__ __forceinline__ void transform_wide(float2 (&ve)[8], float2 (&vo)[8], PivotShared &sh, int rounds, int h, int from)
+{
+    const int l = threadIdx.x & 31;
+#pragma unroll 2
+    for (int rd = 0; rd < rounds; ++rd) {
+        const int par = rd & 1;
+        __syncthreads();
+        if (rd > 0) vo[0] = sh.vx[par ^ 1][from][l];
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+            const float4 r = *(const float4 *)&sh.bg[par][8 * h + i];
+            rotate_rows(r.x, r.y, ve[i], vo[i]);
+            rotate_rows(r.z, r.w, ve[i + 1], vo[i + 1]);
+        }
+        sh.vx[par][h][l] = vo[7];
+#pragma unroll
+        for (int i = 7; i > 0; --i) vo[i] = vo[i - 1];
+    }
+}
+template <int M> __device__ __forceinline__ void transform_inner(float2 (&v)[16], PivotShared &sh, int h, int ph)
+{
+#pragma unroll 1
+    for (int rd = 0; rd < M; ++rd) {
+        const int par = rd & 1;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+            const float4 r = *(const float4 *)&sh.bg[par][8 * h + i];
+            const int e0 = 2 * M * (i / M) + i % M, e1 = 2 * M * ((i + 1) / M) + (i + 1) % M;
+            rotate_rows(r.x, r.y, v[e0], v[e0 + M]);
+            rotate_rows(r.z, r.w, v[e1], v[e1 + M]);
+        }
+#pragma unroll
+        for (int g = 0; g < 8 / M; ++g) {                        // odd rows of a group move on by one slot
+            const int o = 2 * M * g + M;
+            const float2 last = v[o + M - 1];
+#pragma unroll
+            for (int i = M - 1; i > 0; --i) v[o + i] = v[o + i - 1];
+            v[o] = last;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int e = 2 * M * (i / M) + i % M;
+        scale_row(v[e], sh.sd[ph][8 * h + i]); scale_row(v[e + M], sh.sd[ph][32 + 8 * h + i]);
+    }
 }
 
 // global row / column of local index l of the pair (I, J)
@@ -237,36 +404,91 @@ __device__ void pivot_load(float *sm, const float *G, int np, int I, int J)
 // vout. cross_only: the 32 rounds that pair the two blocks' rows; otherwise all 63 rounds. Returns the largest
 // scaled off-diagonal entry found in the block before rotating (block-uniform); when it is <= tol_rot nothing is
 // rotated or published.
-__device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *vout, bool &rotated)
+template <int W> __device__ __forceinline__ float pivot_warp(float *As, PivotShared &sh, bool cross_only, float tol_rot)
 {
-    __shared__ float red[NT / 32];
-    __shared__ float2 rot[64];
-    __shared__ float4 xch[NT];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float *As = sm, *Vs = sm + BLK * LDP;
-    for (int e = tid; e < BLK * BLK; e += NT) Vs[(e >> 6) * LDP + (e & 63)] = ((e >> 6) == (e & 63)) ? 1.f : 0.f;
-    __syncthreads();
-    float mo = 0.f;
-    for (int e = tid; e < BLK * BLK; e += NT) {
-        const int i = e >> 6, j = e & 63;
-        if (i != j) {
-            const float dd = fmaxf(As[i * LDP + i], 0.f) * fmaxf(As[j * LDP + j], 0.f);
-            if (dd > 0.f) mo = fmaxf(mo, fabsf(As[i * LDP + j]) * rsqrtf(dd));
-        }
-    }
+    const float tol2 = tol_rot * tol_rot;
+    Band<W> band;
+    float mo = band.load(As);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mo = fmaxf(mo, __shfl_xor_sync(0xffffffffu, mo, o));
-    if (lane == 0) red[warp] = mo;
+    if ((threadIdx.x & 31) == 0) sh.red[W] = mo;
     __syncthreads();
-    mo = red[0];
+    mo = fmaxf(fmaxf(sh.red[0], sh.red[1]), fmaxf(sh.red[2], sh.red[3]));
+    if (!(mo > tol_rot)) return mo;
+    band.rounds(As, sh, tol2, !cross_only);
+    if (!cross_only) {
+        __syncthreads();
+        if (W == 0) {
+            inner_phase<16>(As, sh, tol2, 1); inner_phase<8>(As, sh, tol2, 0); inner_phase<4>(As, sh, tol2, 1);
+            inner_phase<2>(As, sh, tol2, 0); inner_phase<1>(As, sh, tol2, 1);
+        } else {
+#pragma unroll 1
+            for (int rd = 0; rd < 31; ++rd) __syncthreads();
+        }
+    }
+    return mo;
+}
+__device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *vout, bool &rotated)
+{
+    __shared__ __align__(16) PivotShared sh;
+    const int tid = threadIdx.x, warp = tid >> 5, l = tid & 31;
+    float *As = sm, *Vs = sm + BLK * LDP;
+    float mo;
+    __syncthreads();
+    if (warp == 0) mo = pivot_warp<0>(As, sh, cross_only, tol_rot);
+    else if (warp == 1) mo = pivot_warp<1>(As, sh, cross_only, tol_rot);
+    else if (warp == 2) mo = pivot_warp<2>(As, sh, cross_only, tol_rot);
+    else if (warp == 3) mo = pivot_warp<3>(As, sh, cross_only, tol_rot);
+    else {
+        const int h = warp - 4;
+        __syncthreads();
+        mo = fmaxf(fmaxf(sh.red[0], sh.red[1]), fmaxf(sh.red[2], sh.red[3]));
+        if (mo > tol_rot) {
+            float2 ve[8], vo[8];
 #pragma unroll
-    for (int w = 1; w < NT / 32; ++w) mo = fmaxf(mo, red[w]);
+            for (int i = 0; i < 8; ++i) {
+                const int e = 8 * h + i, o = 32 + e;
+                ve[i] = make_float2(e == l ? 1.f : 0.f, e == l + 32 ? 1.f : 0.f);
+                vo[i] = make_float2(o == l ? 1.f : 0.f, o == l + 32 ? 1.f : 0.f);
+            }
+            transform_wide(ve, vo, sh, 32, h, (h - 1) & 3);
+            __syncthreads();
+            vo[0] = sh.vx[1][(h - 1) & 3][l];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) { scale_row(ve[i], sh.sd[0][8 * h + i]); scale_row(vo[i], sh.sd[0][32 + 8 * h + i]); }
+            auto put = [&](float *dst, int ld, int row, float2 v) { dst[row * ld + l] = v.x; dst[row * ld + l + 32] = v.y; };
+            auto get = [&](int row) { return make_float2(Vs[row * LDP + l], Vs[row * LDP + l + 32]); };
+            auto vbar = [] { asm volatile("bar.sync 1, 128;" ::: "memory"); };          // the warps of the transform
+            if (cross_only) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { put(vout, BLK, 8 * h + i, ve[i]); put(vout, BLK, 32 + 8 * h + i, vo[i]); }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { put(Vs, LDP, 8 * h + i, ve[i]); put(Vs, LDP, 32 + 8 * h + i, vo[i]); }
+                vbar();
+                const int e16 = 32 * (h >> 1) + 8 * (h & 1);     // width 16: even rows e16 + i, odd rows 16 further on
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { ve[i] = get(e16 + i); vo[i] = get(e16 + 16 + i); }
+                __syncthreads();
+                transform_wide(ve, vo, sh, 16, h, h ^ 1);
+                vbar();
+                vo[0] = sh.vx[1][h ^ 1][l];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { scale_row(ve[i], sh.sd[1][8 * h + i]); scale_row(vo[i], sh.sd[1][32 + 8 * h + i]); }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { put(Vs, LDP, e16 + i, ve[i]); put(Vs, LDP, e16 + 16 + i, vo[i]); }
+                vbar();
+                float2 v[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[i] = get(16 * h + i);
+                transform_inner<8>(v, sh, h, 0); transform_inner<4>(v, sh, h, 1); transform_inner<2>(v, sh, h, 0);
+                transform_inner<1>(v, sh, h, 1);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) put(vout, BLK, 16 * h + i, v[i]);
+            }
+        }
+    }
     rotated = mo > tol_rot;
-    if (!rotated) return mo;
-    cross_phase(As, Vs, rot, xch, 32, tol_rot);
-    if (!cross_only)
-        for (int m = 16; m >= 1; m >>= 1) cross_phase(As, Vs, rot, xch, m, tol_rot);
-    for (int e = tid; e < BLK * BLK; e += NT) vout[e] = Vs[(e >> 6) * LDP + (e & 63)];
     return mo;
 }
 
