@@ -342,27 +342,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                             }
                         __syncthreads();
                     }
-                    const int tx = tid & 15, ty = tid >> 4;
-                    double acc[4][4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-#pragma unroll 4
-                    for (int k = 0; k < 64; ++k) {
-                        const float4 a = *(const float4 *)&sA[k * LDA + ty * 4];
-                        const float4 b = *(const float4 *)&sA[k * LDA + tx * 4];
-                        const double av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
-                    }
-                    double *dst = sq.gpart + (size_t)t * 4096;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) dst[(ty * 4 + i) * 64 + tx * 4 + j] = acc[i][j];
+                    gram_tile_64(sA, LDA, Gs, sq.gpart + (size_t)t * 4096);
                     __syncthreads();
                 }
                 barrier();
@@ -378,6 +358,9 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             default: {                                                   // OP_APPLY
                 const uint64_t nseed = seed + 7919ull * (uint64_t)(pj * 2 + arep);
                 const float rscale = rsqrtf((float)n * (1.f / 3.f));     // replacement columns of about unit norm
+                int fl[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) fl[k] = __ldcg(sq.flags + (tid & 15) * 4 + k);
                 for (int t = rank; t < ntile; t += ncta) {
                     const int rv = min(64, n - t * 64);
                     load_tile(sA, LDA, sq.M + (size_t)t * 64 * ld + j0, ld, rv, w, vec);
@@ -385,24 +368,34 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                     __syncthreads();
                     float acc[4][4] = {};
                     tile_mac<P_FINE, false>(sA, LDA, sB, LDB, m0, n0, acc);
-                    const int lane = tid & 31, g = lane >> 2, tq = lane & 3;
+                    __syncthreads();
+                    store_acc(sA, LDA, m0, n0, acc);
+                    __syncthreads();
+                    // out row by row, four columns a thread (the flags are read once, before any store)
 #pragma unroll
-                    for (int nt = 0; nt < 4; ++nt)
+                    for (int i = 0; i < 4; ++i) {
+                        const int r = (tid >> 4) + 16 * i, c = (tid & 15) * 4, grow = t * 64 + r;
+                        if (r >= rv || c >= w) continue;
+                        const float4 q = *(const float4 *)(sA + r * LDA + c);
+                        float v[4] = {q.x, q.y, q.z, q.w};
+                        __nv_bfloat162 h[2], l[2];
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int r = m0 + g + (i >= 2 ? 8 : 0), c = n0 + nt * 8 + 2 * tq + (i & 1);
-                            if (r >= rv || c >= w) continue;
-                            const int grow = t * 64 + r;
-                            float v = acc[nt][i];
-                            if (__ldcg(sq.flags + c))
-                                v = rscale * hash_uniform(nseed, ((uint64_t)sq.index << 40) ^ ((uint64_t)grow << 8) ^ (uint64_t)c);
-                            sq.M[(size_t)grow * ld + j0 + c] = v;
-                            if (last && sq.hi) {
-                                const __nv_bfloat16 h = __float2bfloat16_rn(v);
-                                sq.hi[(size_t)grow * sq.ldh + j0 + c] = h;
-                                sq.lo[(size_t)grow * sq.ldh + j0 + c] = __float2bfloat16_rn(v - __bfloat162float(h));
-                            }
+                        for (int k = 0; k < 4; ++k)
+                            if (fl[k]) v[k] = rscale * hash_uniform(nseed, ((uint64_t)sq.index << 40) ^ ((uint64_t)grow << 8) ^ (uint64_t)(c + k));
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            h[k] = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+                            l[k] = __floats2bfloat162_rn(v[2 * k] - __low2float(h[k]), v[2 * k + 1] - __high2float(h[k]));
                         }
+                        float *dm = sq.M + (size_t)grow * ld + j0 + c;
+                        if (vec && c + 3 < w) *(float4 *)dm = make_float4(v[0], v[1], v[2], v[3]);
+                        else for (int k = 0; k < 4 && c + k < w; ++k) dm[k] = v[k];
+                        if (last && sq.hi) {
+                            // the pair's rows are padded to multiples of 8 columns; what lies beyond rt is never read
+                            *(uint2 *)(sq.hi + (size_t)grow * sq.ldh + j0 + c) = *(const uint2 *)h;
+                            *(uint2 *)(sq.lo + (size_t)grow * sq.ldh + j0 + c) = *(const uint2 *)l;
+                        }
+                    }
                     __syncthreads();
                 }
                 barrier();

@@ -12,16 +12,21 @@
 //   3. everybody below subtracts L_i L_k^T from G (columns right of jb) or L_i X_b from X (columns up
 //      to jb): 64 independent multiply-adds per thread.
 // Two barriers per four columns (named barrier 1, 256 threads: exactly the threads 0..255 must call).
+// Bound by the chain of 64 pivots (reciprocal root, scaling, next pivot) and the two barriers of a block step. The
+// published rows are stored column-wise (lc[c][row]), so that step 3 reads them in 16-byte pieces with at most two
+// lanes on a bank; row-wise they collided 16-fold, and the reciprocal root went through two fp32 conversions:
+// 40300 -> 34600 cycles.
 #pragma once
 #include "common.cuh"
+#include "jacobi3.cuh"
 
 constexpr int PB = 64;            // orthonormalisation panel width
 
 __device__ __noinline__ void chol_invert_64(const double *Gs, int n, float *rinv, int *flags)
 {
     __shared__ double rs[PB];          // 1 / sqrt(diagonal of the Gram matrix)
-    __shared__ double lcol4[PB][4];    // block column jb of L (rows below the diagonal block)
-    __shared__ double xrow4[4][PB];    // block row jb of L^-1
+    __shared__ __align__(16) double lc[4][PB];    // block column jb of L (rows below the diagonal block), by column
+    __shared__ __align__(16) double xrow4[4][PB]; // block row jb of L^-1
     __shared__ double Lbb[4][4];       // the factored diagonal block (strictly lower part)
     __shared__ double rinv4[4];        // 1 / L_jj, 0 for a dependent column
     __shared__ int dep[PB];
@@ -69,10 +74,11 @@ __device__ __noinline__ void chol_invert_64(const double *Gs, int n, float *rinv
 #pragma unroll
                 for (int k = 0; k < c; ++k) piv = fma(-blk[c][k], blk[c][k], piv);
                 const bool bad = !(piv > 1e-10);
-                // 1/sqrt from the fp32 approximation and one Newton step (piv is in (1e-10, ~1]): ~2^-44 relative,
-                // far below the fp32 precision the result is stored in
-                double y = (double)rsqrtf((float)piv);
-                y = y * (1.5 - 0.5 * piv * y * y);
+                // 1/sqrt from the hardware's 20-bit approximation and one Newton step: ~2^-40 relative, far below the
+                // fp32 precision the result is stored in
+                double y;
+                asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(piv));
+                y = fma(0.5 * y, fma(-piv * y, y, 1.0), y);
                 ri[c] = bad ? 0.0 : y;
                 if (bad && 4 * jb + c < n) dep[4 * jb + c] = 1;
 #pragma unroll
@@ -103,7 +109,7 @@ __device__ __noinline__ void chol_invert_64(const double *Gs, int n, float *rinv
 #pragma unroll
                     for (int k = 0; k < c; ++k) v = fma(-l[k], Lbb[c][k], v);
                     l[c] = v * rinv4[c];
-                    lcol4[4 * br + a][c] = l[c];
+                    lc[c][4 * br + a] = l[c];
                 }
             }
             to_x();
@@ -125,20 +131,17 @@ __device__ __noinline__ void chol_invert_64(const double *Gs, int n, float *rinv
         }
         bar256();
         if (br > jb && bc <= br) {
-            // 3. trailing update (operands re-read from shared memory per row: registers are scarce here)
-            const bool gpart = bc > jb;
+            // 3. trailing update, one column of L (and its row of X) at a time
+            const double *rsrc = bc > jb ? &lc[0][4 * bc] : &xrow4[0][4 * bc];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                double rb[4];
+            for (int c = 0; c < 4; ++c) {
+                const double2 a0 = *(const double2 *)&lc[c][4 * br], a1 = *(const double2 *)&lc[c][4 * br + 2];
+                const double2 b0 = *(const double2 *)(rsrc + c * PB), b1 = *(const double2 *)(rsrc + c * PB + 2);
+                const double la[4] = {a0.x, a0.y, a1.x, a1.y}, rb[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
-                for (int c = 0; c < 4; ++c) rb[c] = gpart ? lcol4[4 * bc + b][c] : xrow4[c][4 * bc + b];
+                for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    double acc = blk[a][b];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc = fma(-lcol4[4 * br + a][c], rb[c], acc);
-                    blk[a][b] = acc;
-                }
+                    for (int b = 0; b < 4; ++b) blk[a][b] = fma(-la[a], rb[b], blk[a][b]);
             }
         }
     }
@@ -164,57 +167,109 @@ __device__ __noinline__ void chol_invert_64(const double *Gs, int n, float *rinv
 // diagonal entry is positive and the largest absolute row sum of E is at most LOWDIN_LIMIT (then the neglected
 // term is below 4e-8); otherwise nothing is written and the caller factors the matrix. Returns the decision
 // (block-uniform). Es: a 64 x LDE fp32 tile of shared memory; 256 threads.
+// E^2 is at most 2.5e-5, so plain TF32 products (2^-10 relative) leave an error near 1e-8. Thread = 4 x 4 block: a row sum
+// is complete within half a warp. 11600 -> 3300 cycles (per-element reductions, atomics and an fp32 product before).
 constexpr float LOWDIN_LIMIT = 5e-3f;
 constexpr int LDE = 72;
 __device__ __noinline__ bool lowdin_64(const double *Gs, int n, float *Es, float *rinv, int *flags)
 {
     __shared__ double rsq[PB];
-    __shared__ float rowsum[PB];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     bool bad = false;
     if (tid < PB) {
         const double d = Gs[tid * PB + tid];
         const bool pos = tid < n && d > 0.0;
         rsq[tid] = pos ? rsqrt(d) : 0.0;
-        rowsum[tid] = 0.f;
         bad = tid < n && !pos;
     }
     __syncthreads();
-    for (int e = tid; e < PB * PB; e += 256) {
-        const int i = e >> 6, j = e & 63;
-        float v = 0.f;
-        if (i < n && j < n && i != j) v = (float)(Gs[e] * rsq[i] * rsq[j]);
-        Es[i * LDE + j] = v;
-        float a = fabsf(v);                                      // row i lies in two warps: 32 columns each
+    float sum[4];
+    const double sc[4] = {rsq[tx * 4], rsq[tx * 4 + 1], rsq[tx * 4 + 2], rsq[tx * 4 + 3]};
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if ((tid & 31) == 0) atomicAdd(&rowsum[i], a);
-    }
-    __syncthreads();
-    if (tid < PB && !(rowsum[tid] <= LOWDIN_LIMIT)) bad = true;
-    if (__syncthreads_or(bad)) return false;
-    // E^2 (E is symmetric): thread (ty, tx) owns the 4 x 4 block at rows 4 ty, columns 4 tx
-    const int tx = tid & 15, ty = tid >> 4;
-    float acc[4][4] = {};
-#pragma unroll 4
-    for (int k = 0; k < PB; ++k) {
-        const float4 a = *(const float4 *)&Es[k * LDE + ty * 4];
-        const float4 b = *(const float4 *)&Es[k * LDE + tx * 4];
-        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i) {
+        const int r = ty * 4 + i;
+        const double sr = rsq[r];
+        const double2 g0 = *(const double2 *)&Gs[r * PB + tx * 4], g1 = *(const double2 *)&Gs[r * PB + tx * 4 + 2];
+        const double g[4] = {g0.x, g0.y, g1.x, g1.y};
+        float e[4];
+        sum[i] = 0.f;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int r = ty * 4 + i, c = tx * 4 + j;
-            float w = 0.f;
-            if (r < n && c < n) w = (float)rsq[r] * ((r == c ? 1.f : 0.f) - 0.5f * Es[r * LDE + c] + 0.375f * acc[i][j]);
-            rinv[r * PB + c] = w;
+            const int c = tx * 4 + j;
+            e[j] = r < n && c < n && r != c ? (float)(g[j] * sr * sc[j]) : 0.f;
+            sum[i] += fabsf(e[j]);
         }
+        *(float4 *)&Es[r * LDE + tx * 4] = make_float4(e[0], e[1], e[2], e[3]);
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sum[i] += __shfl_xor_sync(0xffffffffu, sum[i], o);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) bad |= !(sum[i] <= LOWDIN_LIMIT);
+    if (__syncthreads_or(bad)) return false;
+    // E^2 (E is symmetric); this warp: rows m0 .. + 15, columns n0 .. + 31
+    const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32;
+    float acc[4][4] = {};
+    j3::product64_acc<true, false, 1>(Es, LDE, Es, LDE, m0, n0, acc);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int r = m0 + g + 8 * h;
+        const float sr = (float)rsq[r];
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt) {
+            const int c = n0 + nt * 8 + 2 * t;
+            float w[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                w[k] = r < n && c + k < n ? sr * ((r == c + k ? 1.f : 0.f) - 0.5f * Es[r * LDE + c + k] + 0.375f * acc[nt][2 * h + k]) : 0.f;
+            *(float2 *)(rinv + r * PB + c) = make_float2(w[0], w[1]);
+        }
+    }
     if (tid < PB) flags[tid] = 0;
     return true;
+}
+
+// Partial Gram matrix of a 64 x 64 fp32 tile T (64 rows of a panel, row stride lds): dst[i][j] = sum_k T[k][i] T[k][j] in
+// fp64, on the fp64 matrix units (mma.m8n8k4; 36 tiles of 8 x 8 by symmetry, four or five per warp). Td: 4096 doubles of
+// shared memory for the converted tile, columns swizzled so that the fragment loads are conflict-free. Converting once
+// instead of per product matters: 9500 -> 5100 cycles (fp64 FMA with conversions in the inner loop before: conversions
+// run at 16 a cycle). 256 threads, T complete before the call; the caller synchronises before T or Td is reused.
+__device__ __forceinline__ void gram_tile_64(const float *T, int lds, double *Td, double *dst)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = lane & 3, p = lane >> 2;
+    for (int f = tid; f < PB * PB / 4; f += 256) {
+        const int r = f >> 4, c = (f & 15) * 4, cs = c ^ ((r & 3) << 2);
+        const float4 v = *(const float4 *)(T + r * lds + c);
+        *(double2 *)&Td[r * PB + cs] = make_double2(v.x, v.y);
+        *(double2 *)&Td[r * PB + cs + 2] = make_double2(v.z, v.w);
+    }
+    __syncthreads();
+    // tiles (i, j), i <= j, numbered row by row: warp w takes w, w + 8, ...
+    int ti[5], tj[5];
+#pragma unroll
+    for (int s = 0; s < 5; ++s) {
+        int t = warp + 8 * s, i = 0;
+        while (i < 7 && t >= 8 - i) { t -= 8 - i; ++i; }
+        ti[s] = i; tj[s] = min(i + t, 7);
+    }
+    double acc[5][2] = {};
+#pragma unroll 2
+    for (int k0 = 0; k0 < PB; k0 += 4) {
+        const double *row = Td + (k0 + q) * PB;
+#pragma unroll
+        for (int s = 0; s < 5; ++s) {
+            if (s == 4 && warp >= 4) break;
+            const double a = row[(8 * ti[s] + p) ^ (q << 2)], b = row[(8 * tj[s] + p) ^ (q << 2)];
+            asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+                : "+d"(acc[s][0]), "+d"(acc[s][1]) : "d"(a), "d"(b));
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < 5; ++s) {
+        if (s == 4 && warp >= 4) break;
+        const int r = 8 * ti[s] + p, c = 8 * tj[s] + 2 * q;
+        *(double2 *)&dst[r * PB + c] = make_double2(acc[s][0], acc[s][1]);
+        if (ti[s] != tj[s]) { dst[c * PB + r] = acc[s][0]; dst[(c + 1) * PB + r] = acc[s][1]; }
+    }
 }
