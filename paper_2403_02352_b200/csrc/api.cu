@@ -178,9 +178,98 @@ const char *atp_status_string(atp_status s)
 }  // extern "C"
 
 // ----------------------------------------------------------------------------------------------
-// Norm box of Fig. 3: one warp per row, row statistics in fp32, two passes over the row (the
-// second one hits L1/L2). HBM-bound: one read and one write of X.
+// Norm box of Fig. 3, rows kept in registers: G threads per row (a warp or 2, 4, 8 of them), each with up to NV pieces of
+// 16 bytes, so X and the residual are read once, in 16-byte loads that are all in flight together, and the statistics
+// (fp32; LayerNorm's second moment about the mean) are taken from registers. HBM-bound: 2 or 3 times rows * cols * size.
+// 4096 x 4096 bf16 with residual: 73 -> 22.5 us (4470 GB/s; the row-in-memory kernel below read two bytes a lane, and
+// everything two or three times).
 // ----------------------------------------------------------------------------------------------
+template <typename T> struct Vec16 { static constexpr int N = 16 / sizeof(T); };
+template <typename T, int NV>
+__global__ void __launch_bounds__(256)
+norm_rows_kernel(const T *X, const T *R, T *Y, int rows, int cols, int ldx, int ldr, int ldy, int kind, float eps, int G)
+{
+    constexpr int N = Vec16<T>::N;
+    __shared__ float part[2][8];
+    const int tid = threadIdx.x, wpr = G >> 5, warp = tid >> 5, lane = tid & 31;
+    const int row = blockIdx.x * (256 / G) + tid / G, gt = tid & (G - 1);
+    const bool on = row < rows;
+    const T *x = X + (size_t)row * ldx, *r = R ? R + (size_t)row * ldr : nullptr;
+    // all loads of the row first, whole pieces only; the partly filled last piece of a row is rare and comes after
+    // (plain loads: Y may alias X)
+    uint4 qx[NV], qr[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        const int c = (gt + k * G) * N;
+        qx[k] = make_uint4(0u, 0u, 0u, 0u);
+        qr[k] = make_uint4(0u, 0u, 0u, 0u);
+        if (on && c + N <= cols) {
+            qx[k] = *(const uint4 *)(x + c);
+            if (R) qr[k] = *(const uint4 *)(r + c);
+        }
+    }
+    float v[NV][N];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        const int c = (gt + k * G) * N;
+        if (on && c < cols && c + N > cols) {
+            T *ex = (T *)&qx[k], *er = (T *)&qr[k];
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+                if (c + i < cols) { ex[i] = x[c + i]; if (R) er[i] = r[c + i]; }
+        }
+        const T *ex = (const T *)&qx[k], *er = (const T *)&qr[k];
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[k][i] = to_f32(ex[i]) + to_f32(er[i]);
+    }
+    auto row_sum = [&](float s, int slot) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (wpr == 1) return s;                                  // G is uniform
+        if (lane == 0) part[slot][warp] = s;
+        __syncthreads();
+        const int w0 = warp & ~(wpr - 1);
+        s = part[slot][w0];
+        for (int i = 1; i < wpr; ++i) s += part[slot][w0 + i];
+        return s;
+    };
+    float mean = 0.f;
+    if (kind == ATP_NORM_LAYER) {
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+#pragma unroll
+            for (int i = 0; i < N; ++i) s += v[k][i];
+        mean = row_sum(s, 0) / cols;
+    }
+    float s2 = 0.f;
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const float dv = (gt + k * G) * N + i < cols ? v[k][i] - mean : 0.f;
+            v[k][i] = dv;
+            s2 = fmaf(dv, dv, s2);
+        }
+    const float inv = rsqrtf(row_sum(s2, 1) / cols + eps);
+    if (!on) return;
+    T *y = Y + (size_t)row * ldy;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        const int c = (gt + k * G) * N;
+        if (c >= cols) continue;
+        uint4 q;
+        T *e = (T *)&q;
+#pragma unroll
+        for (int i = 0; i < N; ++i) e[i] = from_f32<T>(v[k][i] * inv);
+        if (c + N <= cols) *(uint4 *)(y + c) = q;
+        else
+            for (int i = 0; c + i < cols; ++i) y[c + i] = e[i];
+    }
+}
+
+// The same for rows longer than 8 pieces of 16 bytes for each of 256 threads, or fp32 rows that are not 16-byte aligned:
+// one warp per row, statistics in fp32, the row read again from L1/L2 for each pass.
 template <typename T>
 __global__ void __launch_bounds__(256)
 norm_kernel(const T *X, const T *R, T *Y, int rows, int cols, int ldx, int ldr, int ldy, int kind, float eps)
@@ -240,6 +329,26 @@ extern "C" atp_status atp_input_norm(atp_ctx *ctx, const atp_mat *X, const atp_m
     int rows = (int)X->rows, cols = (int)X->cols;
     dim3 grid(ceil_div(rows, 8));
     ATP_KERNEL(ctx, "norm", 0, (double)rows * cols * dtype_size(X->dtype) * (residual ? 3 : 2));
+    auto vec_ok = [](const atp_mat *m) { return ((uintptr_t)m->data & 15) == 0 && (m->ld * dtype_size(m->dtype)) % 16 == 0; };
+    const int pieces = ceil_div(cols, 16 / (int)dtype_size(X->dtype));
+    if (vec_ok(X) && vec_ok(Y) && (!residual || vec_ok(residual)) && pieces <= 8 * 256) {
+        // threads per row: the fewest for which a thread holds at most four pieces (eight only at the longest rows; two: 23.3 us), so that
+        // narrow rows still fill a CTA and wide ones have all their loads in flight
+        int G = 32;
+        while (G < 256 && pieces > 4 * G) G *= 2;
+        const int nv = ceil_div(pieces, G);
+        const dim3 rgrid(ceil_div(rows, 256 / G));
+        auto go = [&](auto t) {
+            using T = decltype(t);
+            auto kern = nv <= 1 ? norm_rows_kernel<T, 1> : nv <= 2 ? norm_rows_kernel<T, 2> : nv <= 4 ? norm_rows_kernel<T, 4> : norm_rows_kernel<T, 8>;
+            kern<<<rgrid, 256, 0, ctx->stream>>>((const T *)X->data, residual ? (const T *)residual->data : nullptr, (T *)Y->data, rows, cols,
+                                                 (int)X->ld, residual ? (int)residual->ld : 0, (int)Y->ld, kind, eps, G);
+        };
+        if (X->dtype == ATP_F32) go(float{});
+        else go(__nv_bfloat16{});
+        ATP_LAUNCHED(ctx);
+        return ATP_OK;
+    }
     if (X->dtype == ATP_F32)
         norm_kernel<float><<<grid, 256, 0, ctx->stream>>>((const float *)X->data, residual ? (const float *)residual->data : nullptr,
                                                           (float *)Y->data, rows, cols, (int)X->ld, residual ? (int)residual->ld : 0,
