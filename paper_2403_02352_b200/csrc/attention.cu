@@ -203,9 +203,9 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
                 g1.push_back(tc::HostProblem{X_r->data, WQ->data, nullptr, pl.Qph, pl.Qpl, nullptr, (int)tr, dp, d, (int)X_r->ld, (int)WQ->ld, ldq, 0});
             else
                 g1.push_back(tc::HostProblem{X->data, WQ->data, nullptr, pl.Qh, pl.Ql, nullptr, (int)tl, dp, d, (int)X->ld, (int)WQ->ld, ldq, 0});
-            if ((st = tc::launch<false, false, tc::OUT_BF16_SPLIT>(ctx, g1, store)) != ATP_OK) return st;
+            if ((st = tc::launch<false, 1, tc::OUT_BF16_SPLIT>(ctx, g1, store)) != ATP_OK) return st;
             g2.push_back(tc::HostProblem{X_r->data, WV->data, nullptr, pl.Vb, nullptr, nullptr, (int)tr, dp, d, (int)X_r->ld, (int)WV->ld, ldq, 0});
-            if ((st = tc::launch<false, false, tc::OUT_BF16>(ctx, g2, store)) != ATP_OK) return st;
+            if ((st = tc::launch<false, 1, tc::OUT_BF16>(ctx, g2, store)) != ATP_OK) return st;
             if (q_mode == ATP_Q_LOWRANK) {
                 std::vector<tc::HostProblem> qe;
                 for (auto &s : seqs)
@@ -213,7 +213,7 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
                         qe.push_back(tc::HostProblem{(const T *)U_r->data + (size_t)s.row0 * U_r->ld, pl.Qph + (size_t)s.rank0 * ldq,
                                                      pl.Qpl + (size_t)s.rank0 * ldq, pl.Qh + (size_t)s.row0 * ldq, pl.Ql + (size_t)s.row0 * ldq,
                                                      nullptr, s.L, dp, s.r, (int)U_r->ld, ldq, ldq, 0});
-                if ((st = tc::launch<false, true, tc::OUT_BF16_SPLIT>(ctx, qe, store)) != ATP_OK) return st;
+                if ((st = tc::launch<false, 2, tc::OUT_BF16_SPLIT>(ctx, qe, store)) != ATP_OK) return st;
             }
             std::vector<atc::HostSeq> hs;
             float *nrm = pl.nrm;
@@ -236,18 +236,18 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
         kv.push_back(tc::HostProblem{X_r->data, WV->data, nullptr, pl.Vp, nullptr, nullptr, (int)tr, dp, d, (int)X_r->ld, (int)WV->ld, dp, 0});
         if (q_mode == ATP_Q_FULL)
             kv.push_back(tc::HostProblem{X->data, WQ->data, nullptr, pl.Q, nullptr, nullptr, (int)tl, dp, d, (int)X->ld, (int)WQ->ld, dp, 0});
-        if ((st = tc::launch<false, false, tc::OUT_F32>(ctx, kv, store)) != ATP_OK) return st;
+        if ((st = tc::launch<false, 1, tc::OUT_F32>(ctx, kv, store)) != ATP_OK) return st;
         if (q_mode == ATP_Q_LOWRANK) {
             std::vector<tc::HostProblem> qp;
             qp.push_back(tc::HostProblem{X_r->data, WQ->data, nullptr, pl.Qph, pl.Qpl, nullptr, (int)tr, dp, d, (int)X_r->ld, (int)WQ->ld, ldq, 0});
-            if ((st = tc::launch<false, false, tc::OUT_BF16_SPLIT>(ctx, qp, store)) != ATP_OK) return st;
+            if ((st = tc::launch<false, 1, tc::OUT_BF16_SPLIT>(ctx, qp, store)) != ATP_OK) return st;
             std::vector<tc::HostProblem> qe;
             for (auto &s : seqs)
                 if (s.L > 0)
                     qe.push_back(tc::HostProblem{(const T *)U_r->data + (size_t)s.row0 * U_r->ld, pl.Qph + (size_t)s.rank0 * ldq,
                                                  pl.Qpl + (size_t)s.rank0 * ldq, pl.Q + (size_t)s.row0 * dp, nullptr, nullptr,
                                                  s.L, dp, s.r, (int)U_r->ld, ldq, dp, 0});
-            if ((st = tc::launch<false, true, tc::OUT_F32>(ctx, qe, store)) != ATP_OK) return st;
+            if ((st = tc::launch<false, 2, tc::OUT_F32>(ctx, qe, store)) != ATP_OK) return st;
         }
     } else {
     {   // Q', K', V' = X_r W (Eq. 6), all sequences at once

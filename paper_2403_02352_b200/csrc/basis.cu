@@ -698,7 +698,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 SeqPlan &p = bp.seqs[i];
                 hp.push_back(tc::HostProblem{Xb(p), bp.omega_b, nullptr, p.Y, nullptr, nullptr, p.dims.L, p.rt, d, (int)X->ld, ldo, p.rt, 0});
             }
-            if ((st = tc::launch<false, false, tc::OUT_F32>(ctx, hp, store)) != ATP_OK) return st;
+            if ((st = tc::launch<false, 1, tc::OUT_F32>(ctx, hp, store)) != ATP_OK) return st;
             if ((st = orthonormalise<std::is_same<T, __nv_bfloat16>::value>(ctx, bp, i0, i1, seed, 2)) != ATP_OK) return st;
             for (int it = 0; it < power_iters; ++it) {
                 hp.clear();
@@ -707,14 +707,14 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                     int ldb = (int)align_up((size_t)p.rt, 8);
                     hp.push_back(tc::HostProblem{Xb(p), p.Yb, p.Yl, p.Zb, p.Zl, nullptr, d, p.rt, p.dims.L, (int)X->ld, ldb, ldb, 0});
                 }
-                if ((st = tc::launch<true, true, tc::OUT_BF16_SPLIT>(ctx, hp, store)) != ATP_OK) return st;
+                if ((st = tc::launch<true, 2, tc::OUT_BF16_SPLIT>(ctx, hp, store)) != ATP_OK) return st;
                 hp.clear();
                 for (size_t i = i0; i < i1; ++i) {      // Y = X Z
                     SeqPlan &p = bp.seqs[i];
                     int ldb = (int)align_up((size_t)p.rt, 8);
                     hp.push_back(tc::HostProblem{Xb(p), p.Zb, p.Zl, p.Y, nullptr, nullptr, p.dims.L, p.rt, d, (int)X->ld, ldb, p.rt, 0});
                 }
-                if ((st = tc::launch<false, true, tc::OUT_F32>(ctx, hp, store)) != ATP_OK) return st;
+                if ((st = tc::launch<false, 2, tc::OUT_F32>(ctx, hp, store)) != ATP_OK) return st;
                 if ((st = orthonormalise<std::is_same<T, __nv_bfloat16>::value>(ctx, bp, i0, i1, seed + 2000003ull * (it + 1), 2)) != ATP_OK) return st;
                 }
         } else {
@@ -835,7 +835,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                     int ldb = (int)align_up((size_t)p.rt, 8);
                     hp.push_back(tc::HostProblem{Xb(p), p.Yb, p.Yl, p.Bth, p.Btl, nullptr, d, p.rt, p.dims.L, (int)X->ld, ldb, ldb, 0});
                 }
-                if ((st = tc::launch<true, true, tc::OUT_BF16_SPLIT>(ctx, hp, store)) != ATP_OK) return st;
+                if ((st = tc::launch<true, 2, tc::OUT_BF16_SPLIT>(ctx, hp, store)) != ATP_OK) return st;
             } else {
                 if ((st = launch_gemm_simt<T, float, float, true>(ctx, g, store)) != ATP_OK) return st;
             }
@@ -857,7 +857,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                         h.A2 = bl;
                         hp.push_back(h);
                     }
-                    if ((st = tc::launch<true, true, tc::OUT_F32, false, true>(ctx, hp, store, "gemm_tc_gram")) != ATP_OK) return st;
+                    if ((st = tc::launch<true, 2, tc::OUT_F32, false, true>(ctx, hp, store, "gemm_tc_gram")) != ATP_OK) return st;
                 } else {
                     if ((st = launch_gemm_simt<float, float, float, true, false>(ctx, gg, store, 1, nullptr, 0, "gemm_simt_gram")) != ATP_OK) return st;
                 }
@@ -894,8 +894,8 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                             h2.push_back(c);
                             fb.s[i - i0].Yh = p.Y2h; fb.s[i - i0].Yl = p.Y2l;
                         }
-                        if ((st = tc::launch<false, true, tc::OUT_BF16_SPLIT, true, true>(ctx, h1, store, "gemm_tc_rot")) != ATP_OK) return st;
-                        if ((st = tc::launch<false, true, tc::OUT_BF16_SPLIT, true, true>(ctx, h2, store, "gemm_tc_rot")) != ATP_OK) return st;
+                        if ((st = tc::launch<false, 2, tc::OUT_BF16_SPLIT, true, true>(ctx, h1, store, "gemm_tc_rot")) != ATP_OK) return st;
+                        if ((st = tc::launch<false, 2, tc::OUT_BF16_SPLIT, true, true>(ctx, h2, store, "gemm_tc_rot")) != ATP_OK) return st;
                     } else {
                         GemmBatch r1, r2; r1.count = r2.count = cnt;
                         for (size_t i = i0; i < i1; ++i) {
@@ -936,8 +936,8 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                     c.A2 = p.Y2l;
                     h2.push_back(c);
                 }
-                if ((st = tc::launch<true, true, tc::OUT_BF16, true, true>(ctx, h1, store, "gemm_tc_out")) != ATP_OK) return st;
-                if ((st = tc::launch<false, true, tc::OUT_BF16, false, true>(ctx, h2, store, "gemm_tc_out")) != ATP_OK) return st;
+                if ((st = tc::launch<true, 2, tc::OUT_BF16, true, true>(ctx, h1, store, "gemm_tc_out")) != ATP_OK) return st;
+                if ((st = tc::launch<false, 2, tc::OUT_BF16, false, true>(ctx, h2, store, "gemm_tc_out")) != ATP_OK) return st;
             } else {
                 for (size_t i = i0; i < i1; ++i) {
                     SeqPlan &p = bp.seqs[i];

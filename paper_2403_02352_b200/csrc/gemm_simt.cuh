@@ -23,7 +23,8 @@ enum GemmEpiKind {
     EPI_D_MINUS = 1,      // C = D - A B
     EPI_BIAS = 2,         // C = A B + bias
     EPI_BIAS_GELU = 3,    // C = gelu_erf(A B + bias)
-    EPI_SILU_D_MUL = 4    // C = silu(D) * (A B)
+    EPI_SILU_D_MUL = 4,   // C = silu(D) * (A B)
+    EPI_ROPE = 5          // pairs of columns of A B turned by (cos, sin) from D (tensor-core GEMM only)
 };
 struct GemmEpi {
     int kind;

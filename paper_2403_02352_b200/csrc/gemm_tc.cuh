@@ -1,13 +1,19 @@
 // Batched bf16 GEMM on the 5th-generation tensor cores (tcgen05.mma, accumulator in TMEM, operands
 // staged in shared memory by TMA with the 128-byte swizzle): C = epilogue(op(A) * B).
 //   A: M x K row-major (K-major operand) or K x M row-major (M-major operand), bf16
-//   B: K x N row-major (N-major operand) or N x K row-major (K-major operand), bf16; optionally a
-//      second matrix B_lo of the same shape whose product is accumulated on top (split precision:
-//      B = B_hi + B_lo), and a second matrix A_lo as well: A_hi B_hi + A_hi B_lo + A_lo B_hi carries
+//   B: K x N row-major (N-major operand) or N x K row-major (K-major operand), bf16; optionally more
+//      matrices of the same shape whose products are accumulated on top (split precision: B = B_hi + B_lo [+ B_lo2],
+//      16 [24] mantissa bits), and a second matrix A_lo as well: A_hi B_hi + A_hi B_lo + A_lo B_hi carries
 //      about 16 mantissa bits of both operands, for fp32 data cut into bf16 hi/lo pairs
-//   C: M x N row-major, fp32 or bf16, or a bf16 hi/lo pair; D (optional): M x N fp32
-// One CTA computes one 128 x 128 tile: warp 4 issues the TMA loads, warp 5 allocates TMEM and issues
-// the MMAs, warps 0-3 read the accumulator back (tcgen05.ld) and run the epilogue. Extents come
+//   C: M x N row-major, fp32 or bf16, or a bf16 hi/lo pair or hi/lo/lo2 triple; D (optional): M x N fp32
+//   DUAL: two matrices B and B_gate side by side in one tile, C = silu(A B_gate) * (A B)
+// Persistent: a CTA (or a pair of CTAs) walks over its tiles with two accumulators in TMEM, so that the epilogue of a tile
+// runs beside the products of the next. Two forms (see choose_pairs for the rule):
+//   CG = 2: a cluster of two CTAs makes 256 x 256 tiles (tcgen05.mma.cta_group::2): each CTA stages 128 rows of A and 128
+//           columns of B. What bounds a bf16 GEMM here is the L2 -> shared-memory path, about 64 bytes a clock and SM: a
+//           128 x 128 tile needs 128 bytes a clock at the full tensor rate, the pair's tile 64.
+//   CG = 1: 128 x 128 tiles, for problems with too few 256 x 256 tiles to fill the GPU.
+// Warp roles: EW epilogue warps (tcgen05.ld), one TMA warp, one warp that allocates TMEM and issues the MMAs. Extents come
 // from per-problem tensor maps, so ragged M, N, K are zero-filled by TMA and masked at the store.
 // Every mbarrier wait is bounded; on expiry the kernel records ATP_ERR_TIMEOUT and winds down.
 #pragma once
@@ -17,22 +23,22 @@
 
 namespace tc {
 
-constexpr int BM = 128, BN = 128, BK = 64;
+constexpr int BM = 128, BN = 128, BK = 64;      // rows of A and columns of B staged by one CTA; K per stage
 constexpr int MAX_PROB = 16;
 constexpr uint32_t WAIT_LIMIT = 1u << 22;
 
 struct Problem {
-    CUtensorMap ta, ta2, tb, tb2; // ta2 / tb2 only with a split A / B
-    void *C; void *C2; const float *D;
+    CUtensorMap ta, ta2, tb, tb2, tb3; // ta2: low part of a split A; tb2, tb3: low parts of a split B, or (tb2) the gate matrix
+    void *C; void *C2; void *C3; const float *D;
     int M, N, K, ldc, ldd;
     int tile0, tiles_n, tiles_m; // first linear tile index of this problem, tiles along N and along M
 };
-struct Batch {
-    Problem p[MAX_PROB];
+template <int P> struct Batch {         // (small launches carry a small parameter block)
+    Problem p[P];
     int count, total_tiles;
 };
 
-enum OutKind { OUT_F32 = 0, OUT_BF16 = 1, OUT_BF16_SPLIT = 2 };
+enum OutKind { OUT_F32 = 0, OUT_BF16 = 1, OUT_BF16_SPLIT = 2, OUT_BF16_SPLIT3 = 3 };
 
 // ---- PTX wrappers -----------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -143,187 +149,318 @@ __host__ __device__ constexpr uint32_t instr_desc(int M, int N, bool a_mn_major,
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-template <bool SPLIT_B, bool SPLIT_A = false> struct Cfg {
-    static constexpr int STAGES = SPLIT_A ? 3 : (SPLIT_B ? 4 : 3);
+// ---- cluster forms (CG = 2: a pair of CTAs, rank 0 leads) --------------------------------------------
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync_all()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+template <int CG> __device__ __forceinline__ void tma_load_cg(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar)
+{
+    if (CG == 1) tma_load_2d(dst, map, c0, c1, bar);
+    else asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
+                      ::"r"(dst), "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1) : "memory");
+}
+template <int CG> __device__ __forceinline__ void tmem_alloc_cg(uint32_t dst_smem, uint32_t ncols)
+{
+    if (CG == 1) tmem_alloc(dst_smem, ncols);
+    else {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+}
+template <int CG> __device__ __forceinline__ void tmem_dealloc_cg(uint32_t taddr, uint32_t ncols)
+{
+    if (CG == 1) tmem_dealloc(taddr, ncols);
+    else asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+template <int CG> __device__ __forceinline__ void umma_cg(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc)
+{
+    if (CG == 1) umma_bf16(d, ad, bd, idesc, acc);
+    else asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                      ::"r"(d), "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
+}
+// completion of the MMAs issued so far arrives at the barrier of both CTAs of the pair
+template <int CG> __device__ __forceinline__ void umma_commit_cg(uint32_t bar)
+{
+    if (CG == 1) umma_commit(bar);
+    else asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                      ::"r"(bar), "h"((uint16_t)3) : "memory");
+}
+template <int CG> __device__ __forceinline__ void arrive_at(uint32_t bar)      // bar: an address of the leader (map_to_rank) for CG = 2
+{
+    if (CG == 1) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+    else asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+template <int CG, int NB, bool SPLIT_A> struct Cfg {
     static constexpr int A_BYTES = BM * BK * 2;                 // 16 KB
     static constexpr int B_BYTES = BK * BN * 2;                 // 16 KB
     static constexpr int B_OFF = A_BYTES * (SPLIT_A ? 2 : 1);
-    static constexpr int STAGE_BYTES = B_OFF + B_BYTES * (SPLIT_B ? 2 : 1);
+    static constexpr int STAGE_BYTES = B_OFF + B_BYTES * NB;
+    // one CTA per SM and as many stages as fit; only the plain 128 x 128 form stays small enough for two
+    static constexpr bool TWO_PER_SM = CG == 1 && NB == 1 && !SPLIT_A;
+    static constexpr int STAGES = TWO_PER_SM ? 3 : 200 * 1024 / STAGE_BYTES;
+    static constexpr int NACC = CG * BN;                        // accumulator columns of a tile
+    static constexpr int EW = CG == 2 ? 8 : 4;                  // epilogue warps
     static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
 };
 
-template <bool A_MN, bool SPLIT_B, int OUT, bool B_KMAJ = false, bool SPLIT_A = false>
-__global__ void __launch_bounds__(192)
-gemm_tc_kernel(const __grid_constant__ Batch batch, GemmEpi epi, int *dev_status)
+__device__ __forceinline__ void store_32b(void *dst, const uint32_t (&v)[8])
 {
-    using C_ = Cfg<SPLIT_B, SPLIT_A>;
-    static_assert(!SPLIT_A || SPLIT_B, "a split A comes with a split B");
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+// 32 consecutive values of a row as bf16; part k = 0, 1, 2 of the hi / lo / lo2 cut leaves the remainder in v
+__device__ __forceinline__ void store_row32_bf16(__nv_bfloat16 *dst, float (&v)[32], int valid, bool v32, bool v16, bool more)
+{
+    uint32_t h[16];
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * t], v[2 * t + 1]);
+        h[t] = *(const uint32_t *)&b;
+        if (more) { v[2 * t] -= __low2float(b); v[2 * t + 1] -= __high2float(b); }
+    }
+    if (v32) {
+#pragma unroll
+        for (int t = 0; t < 16; t += 8) {
+            const uint32_t q[8] = {h[t], h[t + 1], h[t + 2], h[t + 3], h[t + 4], h[t + 5], h[t + 6], h[t + 7]};
+            store_32b(dst + 2 * t, q);
+        }
+    } else if (v16) {
+#pragma unroll
+        for (int t = 0; t < 16; t += 4) *(uint4 *)(dst + 2 * t) = make_uint4(h[t], h[t + 1], h[t + 2], h[t + 3]);
+    } else {
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+            const __nv_bfloat162 b = *(const __nv_bfloat162 *)&h[t];
+            if (2 * t < valid) dst[2 * t] = __low2bfloat16(b);
+            if (2 * t + 1 < valid) dst[2 * t + 1] = __high2bfloat16(b);
+        }
+    }
+}
+
+template <int CG, bool A_MN, int NB, int OUT, bool B_KMAJ, bool SPLIT_A, bool DUAL, int P>
+__global__ void __launch_bounds__(Cfg<CG, NB, SPLIT_A>::EW * 32 + 64)
+gemm_tc_kernel(const __grid_constant__ Batch<P> batch, GemmEpi epi, int *dev_status)
+{
+    using C_ = Cfg<CG, NB, SPLIT_A>;
+    static_assert(!SPLIT_A || NB == 2, "a split A comes with a split B");
+    static_assert(!DUAL || (NB == 1 && !SPLIT_A && !B_KMAJ), "the gated form takes plain row-major weights");
+    constexpr int S = C_::STAGES, EW = C_::EW, TN = DUAL ? C_::NACC / 2 : C_::NACC;   // output columns of a tile
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;                // swizzled tiles need 1024-byte alignment
     uint8_t *gbase = smem_raw + (base - raw);
-    const uint32_t bars = base + C_::STAGES * C_::STAGE_BYTES;   // full[S], empty[S], tmem_full, then tmem slot
-    uint32_t *tmem_slot = (uint32_t *)(gbase + C_::STAGES * C_::STAGE_BYTES + 8 * (2 * C_::STAGES + 1));
+    const uint32_t bars = base + S * C_::STAGE_BYTES;            // full[S], empty[S], acc full[2], acc free[2], then tmem slot
+    const uint32_t b_full = bars, b_empty = bars + 8 * S, b_afull = b_empty + 8 * S, b_afree = b_afull + 16;
+    uint32_t *tmem_slot = (uint32_t *)(gbase + S * C_::STAGE_BYTES + 8 * (2 * S + 4));
     __shared__ int abort_flag;
 
-    // which tile
-    const int tile = blockIdx.x;
-    int pi = 0;
-#pragma unroll 1
-    for (int i = 1; i < batch.count; ++i) if (tile >= batch.p[i].tile0) pi = i;
-    const Problem &pr = batch.p[pi];
-    const int lt = tile - pr.tile0;
-    // Where N is much larger than M, consecutive CTAs walk along M: they share a tile of the large operand B, and
-    // the operand that is re-read from L2 is the small one, A (a 4096 x 2048 x 11008 product read 1 GB
-    // from DRAM in row-major tile order: its 45 MB B operand was evicted by the streamed epilogue operand).
-    const bool along_m = pr.tiles_n > 2 * pr.tiles_m;
-    const int m0 = (along_m ? lt % pr.tiles_m : lt / pr.tiles_n) * BM, n0 = (along_m ? lt / pr.tiles_m : lt % pr.tiles_n) * BN;
-    const int num_kt = (pr.K + BK - 1) / BK;
-
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = CG == 2 ? cluster_rank() : 0u;
+    const int first = (int)blockIdx.x / CG, step = (int)gridDim.x / CG, total = batch.total_tiles;
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        for (int s = 0; s < C_::STAGES; ++s) { mbar_init(bars + 8 * s, 1); mbar_init(bars + 8 * (C_::STAGES + s), 1); }
-        mbar_init(bars + 8 * (2 * C_::STAGES), 1);
+        for (int s = 0; s < S; ++s) { mbar_init(b_full + 8 * s, 1); mbar_init(b_empty + 8 * s, 1); }
+        for (int a = 0; a < 2; ++a) { mbar_init(b_afull + 8 * a, 1); mbar_init(b_afree + 8 * a, CG * EW); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 5) tmem_alloc(smem_u32(tmem_slot), BN);
+    if (warp == EW + 1) tmem_alloc_cg<CG>(smem_u32(tmem_slot), 2 * C_::NACC);
     tc_fence_before();
     __syncthreads();
+    if (CG == 2) cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();                                                  // set-up done; from here on memory of the launch before is touched
+    pdl_trigger();
 
-    if (warp == 4) {
+    // Tile t: problem, first row and column of the whole tile (both CTAs of a pair). Where N is much larger than M,
+    // consecutive tiles walk along M: they share a tile of the large operand B, and the operand that is re-read from L2 is
+    // the small one, A (a 4096 x 2048 x 11008 product read 1 GB from DRAM in row-major tile order).
+    auto locate = [&](int t, int &m0, int &n0) -> const Problem & {
+        int pi = 0;
+#pragma unroll 1
+        for (int i = 1; i < batch.count; ++i) if (t >= batch.p[i].tile0) pi = i;
+        const Problem &pr = batch.p[pi];
+        const int lt = t - pr.tile0;
+        const bool along_m = pr.tiles_n > 2 * pr.tiles_m;
+        m0 = (along_m ? lt % pr.tiles_m : lt / pr.tiles_n) * (CG * BM);
+        n0 = (along_m ? lt / pr.tiles_m : lt % pr.tiles_n) * TN;
+        return pr;
+    };
+
+    if (warp == EW) {
         if (lane == 0) {
-            for (int kt = 0; kt < num_kt; ++kt) {
-                const int s = kt % C_::STAGES;
-                if (kt >= C_::STAGES && !mbar_wait(bars + 8 * (C_::STAGES + s), ((kt / C_::STAGES) - 1) & 1, &abort_flag)) break;
-                const uint32_t full = bars + 8 * s;
-                const uint32_t sa = base + s * C_::STAGE_BYTES, sb = sa + C_::B_OFF;
-                mbar_expect_tx(full, C_::STAGE_BYTES);
-                const int k0 = kt * BK;
-                if (!A_MN) {
-                    tma_load_2d(sa, &pr.ta, k0, m0, full);                       // box {64 k, 128 m}
-                    if (SPLIT_A) tma_load_2d(sa + C_::A_BYTES, &pr.ta2, k0, m0, full);
-                } else {
-                    tma_load_2d(sa, &pr.ta, m0, k0, full);                       // box {64 m, 64 k} x 2
-                    tma_load_2d(sa + 8192, &pr.ta, m0 + 64, k0, full);
-                    if (SPLIT_A) {
-                        tma_load_2d(sa + C_::A_BYTES, &pr.ta2, m0, k0, full);
-                        tma_load_2d(sa + C_::A_BYTES + 8192, &pr.ta2, m0 + 64, k0, full);
-                    }
-                }
-                if (B_KMAJ) {
-                    tma_load_2d(sb, &pr.tb, k0, n0, full);                       // box {64 k, 128 n}
-                    if (SPLIT_B) tma_load_2d(sb + C_::B_BYTES, &pr.tb2, k0, n0, full);
-                } else {
-                    tma_load_2d(sb, &pr.tb, n0, k0, full);                       // box {64 n, 64 k} x 2
-                    tma_load_2d(sb + 8192, &pr.tb, n0 + 64, k0, full);
-                    if (SPLIT_B) {
-                        tma_load_2d(sb + C_::B_BYTES, &pr.tb2, n0, k0, full);
-                        tma_load_2d(sb + C_::B_BYTES + 8192, &pr.tb2, n0 + 64, k0, full);
+            int ks = 0;                                          // stages filled so far
+            bool ok = true;
+            for (int t = first; t < total && ok; t += step) {
+                int m0, n0;
+                const Problem &pr = locate(t, m0, n0);
+                m0 += rank * BM;
+                const int num_kt = (pr.K + BK - 1) / BK;
+                for (int kt = 0; kt < num_kt; ++kt, ++ks) {
+                    const int s = ks % S;
+                    if (ks >= S && !mbar_wait(b_empty + 8 * s, ((ks / S) - 1) & 1, &abort_flag)) { ok = false; break; }
+                    const uint32_t full = CG == 2 ? map_to_rank(b_full + 8 * s, 0) : b_full + 8 * s;
+                    const uint32_t sa = base + s * C_::STAGE_BYTES, sb = sa + C_::B_OFF;
+                    if (rank == 0) mbar_expect_tx(b_full + 8 * s, CG * C_::STAGE_BYTES);
+                    const int k0 = kt * BK;
+                    auto load_a = [&](uint32_t dst, const CUtensorMap *m) {
+                        if (!A_MN) tma_load_cg<CG>(dst, m, k0, m0, full);                    // box {64 k, 128 m}
+                        else {
+                            tma_load_cg<CG>(dst, m, m0, k0, full);                           // box {64 m, 64 k} x 2
+                            tma_load_cg<CG>(dst + 8192, m, m0 + 64, k0, full);
+                        }
+                    };
+                    load_a(sa, &pr.ta);
+                    if (SPLIT_A) load_a(sa + C_::A_BYTES, &pr.ta2);
+                    if (DUAL) {
+                        // pair: CTA 0 stages 128 columns of B, CTA 1 the same columns of the gate; alone: 64 of each
+                        const CUtensorMap *m0p = CG == 2 && rank == 1 ? &pr.tb2 : &pr.tb, *m1p = CG == 2 ? m0p : &pr.tb2;
+                        tma_load_cg<CG>(sb, m0p, n0, k0, full);
+                        tma_load_cg<CG>(sb + 8192, m1p, CG == 2 ? n0 + 64 : n0, k0, full);
+                    } else {
+                        const int nn = n0 + (int)rank * BN;
+                        auto load_b = [&](uint32_t dst, const CUtensorMap *m) {
+                            if (B_KMAJ) tma_load_cg<CG>(dst, m, k0, nn, full);               // box {64 k, 128 n}
+                            else {
+                                tma_load_cg<CG>(dst, m, nn, k0, full);                       // box {64 n, 64 k} x 2
+                                tma_load_cg<CG>(dst + 8192, m, nn + 64, k0, full);
+                            }
+                        };
+                        load_b(sb, &pr.tb);
+                        if (NB > 1) load_b(sb + C_::B_BYTES, &pr.tb2);
+                        if (NB > 2) load_b(sb + 2 * C_::B_BYTES, &pr.tb3);
                     }
                 }
             }
         }
-    } else if (warp == 5) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc(BM, BN, A_MN, !B_KMAJ);
+    } else if (warp == EW + 1) {
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc = instr_desc(CG * BM, C_::NACC, A_MN, !B_KMAJ);
             bool ok = true;
-            for (int kt = 0; kt < num_kt && ok; ++kt) {
-                const int s = kt % C_::STAGES;
-                ok = mbar_wait(bars + 8 * s, (kt / C_::STAGES) & 1, &abort_flag);
+            int ks = 0, it = 0;
+            for (int t = first; t < total && ok; t += step, ++it) {
+                int m0, n0;
+                const Problem &pr = locate(t, m0, n0);
+                const int num_kt = (pr.K + BK - 1) / BK, ab = it & 1;
+                if (it >= 2) ok = mbar_wait(b_afree + 8 * ab, ((it >> 1) - 1) & 1, &abort_flag);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t sa = base + s * C_::STAGE_BYTES, sb = sa + C_::B_OFF;
+                const uint32_t d = tmem_base + ab * C_::NACC;
+                for (int kt = 0; kt < num_kt; ++kt, ++ks) {
+                    const int s = ks % S;
+                    ok = mbar_wait(b_full + 8 * s, (ks / S) & 1, &abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t sa = base + s * C_::STAGE_BYTES, sb = sa + C_::B_OFF;
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk) {
-                    auto adesc = [&](uint32_t a0) { return A_MN ? smem_desc(a0 + kk * 2048, 8192, 1024) : smem_desc(a0 + kk * 32, 16, 1024); };
-                    auto bdesc = [&](uint32_t b0) { return B_KMAJ ? smem_desc(b0 + kk * 32, 16, 1024) : smem_desc(b0 + kk * 2048, 8192, 1024); };
-                    const uint64_t ad = adesc(sa), bd = bdesc(sb);
-                    // small terms first, the hi * hi product last
-                    if (SPLIT_A) umma_bf16(tmem_base, adesc(sa + C_::A_BYTES), bd, idesc, (kt > 0 || kk > 0) ? 1u : 0u);
-                    if (SPLIT_B) umma_bf16(tmem_base, ad, bdesc(sb + C_::B_BYTES), idesc, (SPLIT_A || kt > 0 || kk > 0) ? 1u : 0u);
-                    umma_bf16(tmem_base, ad, bd, idesc, (SPLIT_B || kt > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 0; kk < BK / 16; ++kk) {
+                        auto adesc = [&](uint32_t a0) { return A_MN ? smem_desc(a0 + kk * 2048, 8192, 1024) : smem_desc(a0 + kk * 32, 16, 1024); };
+                        auto bdesc = [&](uint32_t b0) { return B_KMAJ ? smem_desc(b0 + kk * 32, 16, 1024) : smem_desc(b0 + kk * 2048, 8192, 1024); };
+                        const uint64_t ad = adesc(sa), bd = bdesc(sb);
+                        uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
+                        // small terms first, the hi * hi product last
+                        if (NB > 2) { umma_cg<CG>(d, ad, bdesc(sb + 2 * C_::B_BYTES), idesc, acc); acc = 1u; }
+                        if (SPLIT_A) { umma_cg<CG>(d, adesc(sa + C_::A_BYTES), bd, idesc, acc); acc = 1u; }
+                        if (NB > 1) { umma_cg<CG>(d, ad, bdesc(sb + C_::B_BYTES), idesc, acc); acc = 1u; }
+                        umma_cg<CG>(d, ad, bd, idesc, acc);
+                    }
+                    umma_commit_cg<CG>(b_empty + 8 * s);         // frees the stage once these MMAs have read it
                 }
-                umma_commit(bars + 8 * (C_::STAGES + s));        // frees the stage once these MMAs have read it
+                if (ok) umma_commit_cg<CG>(b_afull + 8 * ab);    // accumulator complete
             }
-            umma_commit(bars + 8 * (2 * C_::STAGES));            // accumulator complete
         }
     } else {
-        // epilogue warps 0..3: TMEM lane = row of the tile
-        int ok_i = 0;
-        if (lane == 0) ok_i = mbar_wait(bars + 8 * (2 * C_::STAGES), 0, &abort_flag) ? 1 : 0;
-        const bool ok = __shfl_sync(0xffffffffu, ok_i, 0) != 0;      // warp-uniform: tcgen05.ld is warp-collective
-        tc_fence_after();
-        const int row = m0 + warp * 32 + lane;
-        if (ok) {
+        // epilogue: TMEM lane = row of the tile; EW = 8: warps 4..7 take the second half of the columns
+        const int quad = warp & 3, half = warp >> 2;
+        constexpr int CW = TN / (EW / 4);                        // output columns of this warp
+        const uint32_t afree = CG == 2 ? map_to_rank(b_afree, 0) : b_afree;
+        int it = 0;
+        for (int t = first; t < total; t += step, ++it) {
+            int m0, n0;
+            const Problem &pr = locate(t, m0, n0);
+            const int ab = it & 1;
+            int ok_i = 0;
+            if (lane == 0) ok_i = mbar_wait(b_afull + 8 * ab, (it >> 1) & 1, &abort_flag) ? 1 : 0;
+            if (__shfl_sync(0xffffffffu, ok_i, 0) == 0) break;           // warp-uniform: tcgen05.ld is warp-collective
+            tc_fence_after();
+            const int row = m0 + (int)rank * BM + quad * 32 + lane;
+            const uint32_t tacc = tmem_base + ab * C_::NACC + ((uint32_t)(quad * 32) << 16);
 #pragma unroll 1
-            for (int c = 0; c < BN; c += 32) {
-                uint32_t r[32];
-                tmem_ld32(tmem_base + ((uint32_t)(warp * 32) << 16) + c, r);
-                const int col0 = n0 + c;
-                if (row < pr.M && col0 < pr.N) {
+            for (int c = half * CW; c < half * CW + CW; c += 32) {
+                uint32_t r[32], gte[32];
+                tmem_ld32_nowait(tacc + c, r);
+                if (DUAL) tmem_ld32_nowait(tacc + TN + c, gte);
+                tmem_ld_wait();
+                if (c + 32 == half * CW + CW) {                  // last read of this accumulator by this warp
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) arrive_at<CG>(afree + 8 * ab);
+                }
+                const int col0 = n0 + c, valid = pr.N - col0;
+                if (row < pr.M && valid > 0) {
                     float v[32];
-                    const bool full_chunk = (col0 + 32 <= pr.N);
-                    // the D operand of this thread's 32 columns: eight 16-byte loads in flight instead of 32 scalar ones
-                    const bool d_vec = (epi.kind == EPI_D_MINUS || epi.kind == EPI_SILU_D_MUL) && full_chunk &&
-                                       ((pr.ldd & 3) == 0) && (((size_t)pr.D & 15) == 0);
-                    float dv[32];
-                    if (d_vec) {
-                        const float4 *dp = (const float4 *)(pr.D + (size_t)row * pr.ldd + col0);
+                    const bool full_chunk = valid >= 32;
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const float4 q = __ldg(dp + j);
-                            dv[4 * j] = q.x; dv[4 * j + 1] = q.y; dv[4 * j + 2] = q.z; dv[4 * j + 3] = q.w;
-                        }
-                    }
+                    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+                    if (DUAL) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        float x = __uint_as_float(r[j]);
-                        const int col = col0 + j;
-                        if (col < pr.N) {
-                            switch (epi.kind) {
-                                case EPI_D_MINUS: x = (d_vec ? dv[j] : pr.D[(size_t)row * pr.ldd + col]) - x; break;
-                                case EPI_BIAS: if (epi.bias) x += epi.bias[col]; break;
-                                case EPI_BIAS_GELU: if (epi.bias) x += epi.bias[col]; x = gelu_erf_f(x); break;
-                                case EPI_SILU_D_MUL: x = silu_f(d_vec ? dv[j] : pr.D[(size_t)row * pr.ldd + col]) * x; break;
-                                default: break;
-                            }
+                        for (int j = 0; j < 32; ++j) v[j] *= silu_f(__uint_as_float(gte[j]));
+                    } else if (epi.kind == EPI_BIAS || epi.kind == EPI_BIAS_GELU) {
+                        if (epi.bias)
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) if (j < valid) v[j] += __ldg(epi.bias + col0 + j);
+                        if (epi.kind == EPI_BIAS_GELU)
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) v[j] = gelu_erf_f(v[j]);
+                    } else if (epi.kind == EPI_ROPE) {
+                        // pairs of columns turn by the angle of (row, pair of the head): D holds (cos, sin) per row and pair
+                        const float *cs = pr.D + (size_t)row * pr.ldd;
+#pragma unroll
+                        for (int j = 0; j < 32; j += 2) {
+                            const float2 t2 = __ldg((const float2 *)(cs + (col0 + j) % pr.ldd));
+                            const float x = v[j], y = v[j + 1];
+                            v[j] = x * t2.x - y * t2.y; v[j + 1] = x * t2.y + y * t2.x;
                         }
-                        v[j] = x;
                     }
                     if (OUT == OUT_F32) {
                         float *dst = (float *)pr.C + (size_t)row * pr.ldc + col0;
-                        if (full_chunk && ((pr.ldc & 3) == 0)) {
+                        if (full_chunk && ((uintptr_t)dst & 31) == 0) {
+#pragma unroll
+                            for (int j = 0; j < 32; j += 8) {
+                                const uint32_t q[8] = {__float_as_uint(v[j]), __float_as_uint(v[j + 1]), __float_as_uint(v[j + 2]), __float_as_uint(v[j + 3]),
+                                                       __float_as_uint(v[j + 4]), __float_as_uint(v[j + 5]), __float_as_uint(v[j + 6]), __float_as_uint(v[j + 7])};
+                                store_32b(dst + j, q);
+                            }
+                        } else if (full_chunk && ((uintptr_t)dst & 15) == 0) {
 #pragma unroll
                             for (int j = 0; j < 32; j += 4) *(float4 *)(dst + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
                         } else {
-                            for (int j = 0; j < 32 && col0 + j < pr.N; ++j) dst[j] = v[j];
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) if (j < valid) dst[j] = v[j];
                         }
                     } else {
-                        __nv_bfloat16 *dst = (__nv_bfloat16 *)pr.C + (size_t)row * pr.ldc + col0;
-                        __nv_bfloat16 *dst2 = (OUT == OUT_BF16_SPLIT) ? (__nv_bfloat16 *)pr.C2 + (size_t)row * pr.ldc + col0 : nullptr;
-                        if (full_chunk && ((pr.ldc & 7) == 0)) {
-#pragma unroll
-                            for (int j = 0; j < 32; j += 8) {
-                                __nv_bfloat162 h[4], l[4];
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) {
-                                    h[t] = __floats2bfloat162_rn(v[j + 2 * t], v[j + 2 * t + 1]);
-                                    if (OUT == OUT_BF16_SPLIT)
-                                        l[t] = __floats2bfloat162_rn(v[j + 2 * t] - __low2float(h[t]), v[j + 2 * t + 1] - __high2float(h[t]));
-                                }
-                                *(uint4 *)(dst + j) = *(uint4 *)h;
-                                if (OUT == OUT_BF16_SPLIT) *(uint4 *)(dst2 + j) = *(uint4 *)l;
-                            }
-                        } else {
-                            for (int j = 0; j < 32 && col0 + j < pr.N; ++j) {
-                                __nv_bfloat16 h = __float2bfloat16_rn(v[j]);
-                                dst[j] = h;
-                                if (OUT == OUT_BF16_SPLIT) dst2[j] = __float2bfloat16_rn(v[j] - __bfloat162float(h));
-                            }
-                        }
+                        const size_t at = (size_t)row * pr.ldc + col0;
+                        __nv_bfloat16 *dst = (__nv_bfloat16 *)pr.C + at;
+                        const bool v32 = full_chunk && (((uintptr_t)dst | (OUT >= OUT_BF16_SPLIT ? (uintptr_t)pr.C2 : 0) | (OUT == OUT_BF16_SPLIT3 ? (uintptr_t)pr.C3 : 0)) & 31) == 0 && ((pr.ldc & 15) == 0);
+                        const bool v16 = full_chunk && ((pr.ldc & 7) == 0);
+                        store_row32_bf16(dst, v, valid, v32, v16, OUT >= OUT_BF16_SPLIT);
+                        if (OUT >= OUT_BF16_SPLIT) store_row32_bf16((__nv_bfloat16 *)pr.C2 + at, v, valid, v32, v16, OUT == OUT_BF16_SPLIT3);
+                        if (OUT == OUT_BF16_SPLIT3) store_row32_bf16((__nv_bfloat16 *)pr.C3 + at, v, valid, v32, v16, false);
                     }
                 }
             }
@@ -332,9 +469,10 @@ gemm_tc_kernel(const __grid_constant__ Batch batch, GemmEpi epi, int *dev_status
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0 && abort_flag && dev_status) raise_status(dev_status, ATP_ERR_TIMEOUT);
-    if (warp == 5) {
+    if (CG == 2) cluster_sync_all();                             // nobody leaves while the other CTA may still signal it
+    if (warp == EW + 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, BN);
+        tmem_dealloc_cg<CG>(tmem_base, 2 * C_::NACC);
     }
 }
 
@@ -373,6 +511,8 @@ struct HostProblem {
     const void *A; const void *B; const void *B2; void *C; void *C2; const float *D;
     int M, N, K, lda, ldb, ldc, ldd;
     const void *A2 = nullptr;     // low part of a split A
+    const void *B3 = nullptr;     // third part of B
+    void *C3 = nullptr;           // third part of C
 };
 
 static inline bool operands_ok(const HostProblem &h)
@@ -381,53 +521,86 @@ static inline bool operands_ok(const HostProblem &h)
     return al(h.A) && al(h.B) && (!h.B2 || al(h.B2)) && (h.lda % 8 == 0) && (h.ldb % 8 == 0) && h.M > 0 && h.N > 0 && h.K > 0;
 }
 
-template <bool A_MN, bool SPLIT_B, int OUT, bool B_KMAJ = false, bool SPLIT_A = false>
-static atp_status launch(atp_ctx *ctx, const std::vector<HostProblem> &probs, GemmEpi epi, const char *tag = nullptr)
+template <int CG, bool A_MN, int NB, int OUT, bool B_KMAJ, bool SPLIT_A, bool DUAL, int P>
+static atp_status launch_form(atp_ctx *ctx, const HostProblem *probs, int count, GemmEpi epi, const char *tag)
 {
-    using C_ = Cfg<SPLIT_B, SPLIT_A>;
+    using C_ = Cfg<CG, NB, SPLIT_A>;
+    auto kern = gemm_tc_kernel<CG, A_MN, NB, OUT, B_KMAJ, SPLIT_A, DUAL, P>;
     static PerDeviceOnce attr_once;        // the shared-memory opt-in is a per-device attribute
-    ATP_CUDA_OK(ctx, attr_once.run(ctx->device, [] {
-        return cudaFuncSetAttribute(gemm_tc_kernel<A_MN, SPLIT_B, OUT, B_KMAJ, SPLIT_A>, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM);
-    }));
-    size_t i = 0;
-    while (i < probs.size()) {
-        Batch b; b.count = 0; b.total_tiles = 0;
-        double flops = 0, bytes = 0;
-        for (; i < probs.size() && b.count < MAX_PROB; ++i) {
-            const HostProblem &h = probs[i];
-            if (h.M <= 0 || h.N <= 0 || h.K <= 0) continue;
-            Problem &p = b.p[b.count];
-            bool ok = A_MN ? make_map(&p.ta, h.A, h.K, h.M, h.lda, 64) : make_map(&p.ta, h.A, h.M, h.K, h.lda, BM);
-            if (SPLIT_A) ok = ok && h.A2 && (A_MN ? make_map(&p.ta2, h.A2, h.K, h.M, h.lda, 64) : make_map(&p.ta2, h.A2, h.M, h.K, h.lda, BM));
-            auto bmap = [&](CUtensorMap *m, const void *ptr) { return B_KMAJ ? make_map(m, ptr, h.N, h.K, h.ldb, BN) : make_map(m, ptr, h.K, h.N, h.ldb, 64); };
-            ok = ok && bmap(&p.tb, h.B);
-            if (SPLIT_B) ok = ok && h.B2 && bmap(&p.tb2, h.B2);
-            if (!ok) return ATP_ERR_INVALID_ARG;
-            p.C = h.C; p.C2 = h.C2; p.D = h.D; p.M = h.M; p.N = h.N; p.K = h.K; p.ldc = h.ldc; p.ldd = h.ldd;
-            p.tiles_n = ceil_div(h.N, BN);
-            p.tiles_m = ceil_div(h.M, BM);
-            p.tile0 = b.total_tiles;
-            b.total_tiles += ceil_div(h.M, BM) * p.tiles_n;
-            b.count++;
-            flops += 2.0 * h.M * h.N * h.K * (SPLIT_A ? 3 : (SPLIT_B ? 2 : 1));
-            bytes += 2.0 * ((double)h.M * h.K + (double)h.K * h.N * (SPLIT_B ? 2 : 1)) + (double)h.M * h.N * (OUT == OUT_F32 ? 4 : (OUT == OUT_BF16 ? 2 : 4));
-        }
-        if (b.count == 0) continue;
-        ATP_KERNEL(ctx, tag ? tag : (SPLIT_A ? "gemm_tc_split3" : (SPLIT_B ? "gemm_tc_split" : "gemm_tc")), flops, bytes);
-        gemm_tc_kernel<A_MN, SPLIT_B, OUT, B_KMAJ, SPLIT_A><<<b.total_tiles, 192, C_::SMEM, ctx->stream>>>(b, epi, ctx->dev_status);
-        ATP_LAUNCHED(ctx);
+    ATP_CUDA_OK(ctx, attr_once.run(ctx->device, [&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM); }));
+    constexpr int TN = DUAL ? C_::NACC / 2 : C_::NACC;
+    Batch<P> b; b.count = 0; b.total_tiles = 0;
+    double flops = 0, bytes = 0;
+    for (int i = 0; i < count; ++i) {
+        const HostProblem &h = probs[i];
+        Problem &p = b.p[b.count];
+        auto amap = [&](CUtensorMap *m, const void *ptr) { return A_MN ? make_map(m, ptr, h.K, h.M, h.lda, 64) : make_map(m, ptr, h.M, h.K, h.lda, BM); };
+        auto bmap = [&](CUtensorMap *m, const void *ptr) { return B_KMAJ ? make_map(m, ptr, h.N, h.K, h.ldb, BN) : make_map(m, ptr, h.K, h.N, h.ldb, 64); };
+        bool ok = amap(&p.ta, h.A) && bmap(&p.tb, h.B);
+        if (SPLIT_A) ok = ok && h.A2 && amap(&p.ta2, h.A2);
+        if (NB > 1 || DUAL) ok = ok && h.B2 && bmap(&p.tb2, h.B2);
+        if (NB > 2) ok = ok && h.B3 && bmap(&p.tb3, h.B3);
+        if (!ok) return ATP_ERR_INVALID_ARG;
+        p.C = h.C; p.C2 = h.C2; p.C3 = h.C3; p.D = h.D; p.M = h.M; p.N = h.N; p.K = h.K; p.ldc = h.ldc; p.ldd = h.ldd;
+        p.tiles_n = ceil_div(h.N, TN);
+        p.tiles_m = ceil_div(h.M, CG * BM);
+        p.tile0 = b.total_tiles;
+        b.total_tiles += p.tiles_m * p.tiles_n;
+        b.count++;
+        flops += 2.0 * h.M * h.N * h.K * (SPLIT_A || NB == 3 ? 3 : (NB == 2 || DUAL ? 2 : 1));
+        bytes += 2.0 * ((double)h.M * h.K + (double)h.K * h.N * (DUAL ? 2 : NB)) + (double)h.M * h.N * (OUT == OUT_F32 ? 4 : 2 * (OUT == OUT_BF16 ? 1 : OUT));
     }
+    const int slots = CG == 2 ? ctx->sm_count / 2 : ctx->sm_count * (C_::TWO_PER_SM ? 2 : 1);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(std::min(slots, b.total_tiles) * CG); cfg.blockDim = dim3(C_::EW * 32 + 64);
+    cfg.dynamicSmemBytes = C_::SMEM; cfg.stream = ctx->stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = CG; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = CG == 2 ? 2 : 1;
+    ATP_KERNEL(ctx, tag ? tag : (SPLIT_A || NB == 3 ? "gemm_tc_split3" : (NB == 2 ? "gemm_tc_split" : "gemm_tc")), flops, bytes);
+    ATP_CUDA_OK(ctx, cudaLaunchKernelEx(&cfg, kern, b, epi, ctx->dev_status));
+    ATP_LAUNCHED(ctx);
     return ATP_OK;
 }
 
-// fp32 -> bf16 copy (rows x cols), destination leading dimension ldd (multiple of 8 for TMA).
-static __global__ void f32_to_bf16_kernel(const float *src, int lds, __nv_bfloat16 *dst, int ldd, int rows, int cols)
+// Pairs of CTAs (256 x 256 tiles) or single ones (128 x 128 tiles, 128 x 64 gated): the form with the smaller number of
+// waves times the time of a stage of one tile. A stage takes a pair about 560 cycles whatever runs beside it; a single CTA
+// about 330 when it has the L2 path to itself (all tiles in one wave), 500 when every SM loads at the full rate.
+template <bool DUAL>
+static inline bool choose_pairs(const HostProblem *probs, int count, int sm_count)
 {
-    size_t n = (size_t)rows * cols;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        int r = (int)(e / cols), c = (int)(e - (size_t)r * cols);
-        dst[(size_t)r * ldd + c] = __float2bfloat16_rn(src[(size_t)r * lds + c]);
+    int t1 = 0, t2 = 0;
+    for (int i = 0; i < count; ++i) {
+        const int n2 = DUAL ? 128 : 256, n1 = n2 / 2;
+        t2 += ceil_div(probs[i].M, 256) * ceil_div(probs[i].N, n2);
+        t1 += ceil_div(probs[i].M, 128) * ceil_div(probs[i].N, n1);
     }
+    return ceil_div(t2, sm_count / 2) * 560 <= ceil_div(t1, sm_count) * (t1 <= sm_count ? 330 : 500);
+}
+
+template <bool A_MN, int NB, int OUT, bool B_KMAJ = false, bool SPLIT_A = false, bool DUAL = false>
+static atp_status launch(atp_ctx *ctx, const std::vector<HostProblem> &all, GemmEpi epi, const char *tag = nullptr)
+{
+    HostProblem probs[MAX_PROB];
+    size_t i = 0;
+    while (i < all.size()) {
+        int n = 0;
+        for (; i < all.size() && n < MAX_PROB; ++i)
+            if (all[i].M > 0 && all[i].N > 0 && all[i].K > 0) probs[n++] = all[i];
+        if (n == 0) continue;
+        atp_status st;
+        if (choose_pairs<DUAL>(probs, n, ctx->sm_count))
+            st = n <= 2 ? launch_form<2, A_MN, NB, OUT, B_KMAJ, SPLIT_A, DUAL, 2>(ctx, probs, n, epi, tag)
+                        : launch_form<2, A_MN, NB, OUT, B_KMAJ, SPLIT_A, DUAL, MAX_PROB>(ctx, probs, n, epi, tag);
+        else
+            st = n <= 2 ? launch_form<1, A_MN, NB, OUT, B_KMAJ, SPLIT_A, DUAL, 2>(ctx, probs, n, epi, tag)
+                        : launch_form<1, A_MN, NB, OUT, B_KMAJ, SPLIT_A, DUAL, MAX_PROB>(ctx, probs, n, epi, tag);
+        if (st != ATP_OK) return st;
+    }
+    return ATP_OK;
 }
 
 // fp32 -> bf16 hi/lo pair: hi = bf16(x), lo = bf16(x - hi).

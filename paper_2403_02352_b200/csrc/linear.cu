@@ -55,22 +55,18 @@ static atp_status linear_impl(atp_ctx *ctx, const atp_mat *U_r, const atp_mat *X
         if (swiglu)
             p1.push_back(tc::HostProblem{X_r->data, Wg->data, nullptr, pl.Tgb, nullptr, nullptr, (int)tr, d_out, d_in,
                                          (int)X_r->ld, (int)Wg->ld, ldt, 0});
-        if ((st = tc::launch<false, false, tc::OUT_BF16>(ctx, p1, GemmEpi{EPI_STORE, nullptr})) != ATP_OK) return st;
-        std::vector<tc::HostProblem> pg, pm;
+        if ((st = tc::launch<false, 1, tc::OUT_BF16>(ctx, p1, GemmEpi{EPI_STORE, nullptr})) != ATP_OK) return st;
+        std::vector<tc::HostProblem> pm;
         for (auto &s : seqs) {
             if (s.L == 0) continue;
-            const T *u = (const T *)U_r->data + (size_t)s.row0 * U_r->ld;
-            T *y = (T *)Y->data + (size_t)s.row0 * Y->ld;
-            float *yg = swiglu ? pl.Yg + (size_t)s.row0 * d_out : nullptr;
-            if (swiglu)
-                pg.push_back(tc::HostProblem{u, pl.Tgb + (size_t)s.rank0 * ldt, nullptr, yg, nullptr, nullptr, s.L, d_out, s.r,
-                                             (int)U_r->ld, ldt, d_out, 0});
-            pm.push_back(tc::HostProblem{u, pl.Tb + (size_t)s.rank0 * ldt, nullptr, y, nullptr, yg, s.L, d_out, s.r,
-                                         (int)U_r->ld, ldt, (int)Y->ld, d_out});
+            pm.push_back(tc::HostProblem{(const T *)U_r->data + (size_t)s.row0 * U_r->ld, pl.Tb + (size_t)s.rank0 * ldt,
+                                         swiglu ? pl.Tgb + (size_t)s.rank0 * ldt : nullptr, (T *)Y->data + (size_t)s.row0 * Y->ld,
+                                         nullptr, nullptr, s.L, d_out, s.r, (int)U_r->ld, ldt, (int)Y->ld, 0});
         }
-        if (swiglu && (st = tc::launch<false, false, tc::OUT_F32>(ctx, pg, GemmEpi{EPI_STORE, nullptr})) != ATP_OK) return st;
-        GemmEpi epi{swiglu ? EPI_SILU_D_MUL : (act == ATP_ACT_GELU ? EPI_BIAS_GELU : EPI_BIAS), bias};
-        return tc::launch<false, false, tc::OUT_BF16>(ctx, pm, epi);
+        // gated: U_r T and U_r T_gate in the two halves of one tile, combined in the epilogue (the fp32 gate product made a
+        // round trip through memory before: 360 MB at 4096 x 11008)
+        if (swiglu) return tc::launch<false, 1, tc::OUT_BF16, false, false, true>(ctx, pm, GemmEpi{EPI_STORE, nullptr});
+        return tc::launch<false, 1, tc::OUT_BF16>(ctx, pm, GemmEpi{act == ATP_ACT_GELU ? EPI_BIAS_GELU : EPI_BIAS, bias});
     }
     // T = X_r W for all sequences at once (rows of X_r are packed)
     {
