@@ -123,33 +123,43 @@ attn_simt_kernel(const __grid_constant__ AttnBatch batch, int dh, int ldq, int l
     }
 }
 
-// Rotary positions (Sec. 4.2, position-encoding paragraph): every row of M (fp32, rows x dp) is rotated
-// by its position: the pair of coordinates (2j, 2j+1) of each head turns by pos * base^(-2j/d_h).
-// pos: per-row positions or nullptr (row index inside its sequence, given by seq_row0). The angle is
-// formed in fp64: at position 3e4 an fp32 angle would already be off by 2e-3 rad.
+// Rotary positions (Sec. 4.2, position-encoding paragraph): the pair of coordinates (2j, 2j+1) of each head of a row turns
+// by pos * base^(-2j/d_h). pos: per-row positions or nullptr (row index inside its sequence, given by seq_row0).
+// rope_table_kernel writes (cos, sin) per row and pair, once for all heads, keys and queries; the angle is formed in fp64: at
+// position 3e4 an fp32 angle would already be off by 2e-3 rad.
 struct RopeSeq { float *K, *Q; int L, row0; };
 struct RopeBatch { RopeSeq s[32]; int count; };
-__global__ void __launch_bounds__(256) rope_kernel(const __grid_constant__ RopeBatch batch, int dp, int dh, double log2_base,
-                                                   const int *pos)
+__global__ void __launch_bounds__(256) rope_table_kernel(const __grid_constant__ RopeBatch batch, int dh, double log2_base, const int *pos,
+                                                         float2 *table)
+{
+    const RopeSeq &q = batch.s[blockIdx.y];
+    const int half = dh / 2;
+    const size_t n = (size_t)q.L * half;
+    for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (size_t)gridDim.x * 256) {
+        const int l = (int)(e / half), j = (int)(e - (size_t)l * half);
+        const double p = pos ? (double)pos[q.row0 + l] : (double)l;
+        double sn, c;
+        sincos(p * exp2(-2.0 * j / dh * log2_base), &sn, &c);
+        table[(size_t)(q.row0 + l) * half + j] = make_float2((float)c, (float)sn);
+    }
+}
+// Rows of K and Q (fp32, rows x dp) turned in place (head widths and data types the tensor-core kernel does not take).
+__global__ void __launch_bounds__(256) rope_kernel(const __grid_constant__ RopeBatch batch, int dp, int dh, const float2 *table)
 {
     const RopeSeq &q = batch.s[blockIdx.y];
     const int half = dp / 2;
     const size_t n = (size_t)q.L * half;
     for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (size_t)gridDim.x * 256) {
         const int l = (int)(e / half), pr = (int)(e - (size_t)l * half);
-        const int j = pr % (dh / 2);
-        const double p = pos ? (double)pos[q.row0 + l] : (double)l;
-        double sn, c;
-        sincos(p * exp2(-2.0 * j / dh * log2_base), &sn, &c);
-        const float cf = (float)c, sf = (float)sn;
+        const float2 cs = table[(size_t)(q.row0 + l) * (dh / 2) + pr % (dh / 2)];
         float *k = q.K + (size_t)l * dp + 2 * pr, *x = q.Q + (size_t)l * dp + 2 * pr;
         const float ka = k[0], kb = k[1], xa = x[0], xb = x[1];
-        k[0] = ka * cf - kb * sf; k[1] = ka * sf + kb * cf;
-        x[0] = xa * cf - xb * sf; x[1] = xa * sf + xb * cf;
+        k[0] = ka * cs.x - kb * cs.y; k[1] = ka * cs.y + kb * cs.x;
+        x[0] = xa * cs.x - xb * cs.y; x[1] = xa * cs.y + xb * cs.x;
     }
 }
 
-struct AttnPlan { float *Qp, *Kp, *Vp, *Q, *Kf; __nv_bfloat16 *Qph, *Qpl, *Kh, *Kl, *Vb, *Qh, *Ql; float *nrm; };
+struct AttnPlan { float *Qp, *Kp, *Vp, *Q, *Kf; __nv_bfloat16 *Qph, *Qpl, *Kh, *Kl, *Vb, *Qh, *Ql; float *nrm; float2 *tab; };
 static void plan_attn(Arena &ar, int64_t tr, int64_t tl, int64_t dp, int64_t nseq, AttnPlan &p)
 {
     p.Qp = ar.take<float>((size_t)tr * dp);
@@ -165,6 +175,7 @@ static void plan_attn(Arena &ar, int64_t tr, int64_t tl, int64_t dp, int64_t nse
     p.Qh = ar.take<__nv_bfloat16>((size_t)tl * align_up((size_t)dp, 8));
     p.Ql = ar.take<__nv_bfloat16>((size_t)tl * align_up((size_t)dp, 8));
     p.nrm = ar.take<float>((size_t)(tl / 128 + nseq) * dp + (size_t)(tr / 128 + nseq) * dp);    // per head norms: query tiles, key blocks
+    p.tab = ar.take<float2>((size_t)tl * 64);                                  // rotary (cos, sin) per row and pair (d_h <= 128)
 }
 size_t attention_workspace_bytes(const std::vector<SeqDims> &seqs, int64_t dp)
 {
@@ -192,18 +203,56 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
     if (ar.overflow || !ctx->workspace) return ATP_ERR_WORKSPACE_TOO_SMALL;
     atp_status st;
     GemmEpi store{EPI_STORE, nullptr};
+    auto make_rope_table = [&]() -> atp_status {
+        RopeBatch rb; rb.count = 0;
+        int maxL = 0;
+        auto flush = [&]() -> atp_status {
+            if (rb.count == 0) return ATP_OK;
+            ATP_KERNEL(ctx, "rope_table", 0, 0);
+            rope_table_kernel<<<dim3(std::min(512, ceil_div(maxL * (dh / 2), 256)), rb.count), 256, 0, ctx->stream>>>(
+                rb, dh, log2((double)rope_base), positions, pl.tab);
+            ATP_LAUNCHED(ctx);
+            rb.count = 0; maxL = 0;
+            return ATP_OK;
+        };
+        for (auto &sq : seqs)
+            if (sq.L > 0) {
+                rb.s[rb.count++] = RopeSeq{nullptr, nullptr, sq.L, sq.row0};
+                maxL = std::max(maxL, sq.L);
+                atp_status r;
+                if (rb.count == 32 && (r = flush()) != ATP_OK) return r;
+            }
+        return flush();
+    };
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-        if ((dh == 64 || dh == 128) && !rope) {
+        if (dh == 64 || dh == 128) {
             // bf16, head width 64 or 128: everything on the tensor cores. K' and Q are produced as
             // bf16 hi/lo pairs by the GEMM epilogues, V' as bf16; the fused kernel does the rest.
             const int ldq = (int)align_up((size_t)dp, 8);
+            // rotary positions: K = U_r K' is rotated in the epilogue of its GEMM and goes back as K'_rot = U_r^T K. K' and K
+            // travel as bf16 triples (24 mantissa bits, so nothing is lost against fp32); the scratch of the fp32 path holds them.
+            // Q is rotated in the epilogue of the GEMM that makes it. (8 x 1024 ragged, 32 heads of 128: 1749 -> 543 us; the
+            // two extra contractions ran on the fp32 units, the angles were formed again for every head.)
+            __nv_bfloat16 *K1[3] = {(__nv_bfloat16 *)pl.Kp, (__nv_bfloat16 *)pl.Qp, (__nv_bfloat16 *)pl.Vp};
+            __nv_bfloat16 *Kr[3] = {(__nv_bfloat16 *)pl.Q, (__nv_bfloat16 *)pl.Q + (size_t)tl * ldq, (__nv_bfloat16 *)pl.Kf};
+            const GemmEpi turn{EPI_ROPE, nullptr};
+            const float *tab = (const float *)pl.tab;
+            if (rope && (st = make_rope_table()) != ATP_OK) return st;
             std::vector<tc::HostProblem> g1, g2;
-            g1.push_back(tc::HostProblem{X_r->data, WK->data, nullptr, pl.Kh, pl.Kl, nullptr, (int)tr, dp, d, (int)X_r->ld, (int)WK->ld, ldq, 0});
+            if (!rope)
+                g1.push_back(tc::HostProblem{X_r->data, WK->data, nullptr, pl.Kh, pl.Kl, nullptr, (int)tr, dp, d, (int)X_r->ld, (int)WK->ld, ldq, 0});
+            else {
+                tc::HostProblem h{X_r->data, WK->data, nullptr, K1[0], K1[1], nullptr, (int)tr, dp, d, (int)X_r->ld, (int)WK->ld, ldq, 0};
+                h.C3 = K1[2];
+                g2.push_back(h);
+                if ((st = tc::launch<false, 1, tc::OUT_BF16_SPLIT3>(ctx, g2, store)) != ATP_OK) return st;
+                g2.clear();
+            }
             if (q_mode == ATP_Q_LOWRANK)
                 g1.push_back(tc::HostProblem{X_r->data, WQ->data, nullptr, pl.Qph, pl.Qpl, nullptr, (int)tr, dp, d, (int)X_r->ld, (int)WQ->ld, ldq, 0});
             else
-                g1.push_back(tc::HostProblem{X->data, WQ->data, nullptr, pl.Qh, pl.Ql, nullptr, (int)tl, dp, d, (int)X->ld, (int)WQ->ld, ldq, 0});
-            if ((st = tc::launch<false, 1, tc::OUT_BF16_SPLIT>(ctx, g1, store)) != ATP_OK) return st;
+                g1.push_back(tc::HostProblem{X->data, WQ->data, nullptr, pl.Qh, pl.Ql, tab, (int)tl, dp, d, (int)X->ld, (int)WQ->ld, ldq, dh});
+            if ((st = tc::launch<false, 1, tc::OUT_BF16_SPLIT>(ctx, g1, rope && q_mode == ATP_Q_FULL ? turn : store)) != ATP_OK) return st;
             g2.push_back(tc::HostProblem{X_r->data, WV->data, nullptr, pl.Vb, nullptr, nullptr, (int)tr, dp, d, (int)X_r->ld, (int)WV->ld, ldq, 0});
             if ((st = tc::launch<false, 1, tc::OUT_BF16>(ctx, g2, store)) != ATP_OK) return st;
             if (q_mode == ATP_Q_LOWRANK) {
@@ -212,8 +261,25 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
                     if (s.L > 0)
                         qe.push_back(tc::HostProblem{(const T *)U_r->data + (size_t)s.row0 * U_r->ld, pl.Qph + (size_t)s.rank0 * ldq,
                                                      pl.Qpl + (size_t)s.rank0 * ldq, pl.Qh + (size_t)s.row0 * ldq, pl.Ql + (size_t)s.row0 * ldq,
-                                                     nullptr, s.L, dp, s.r, (int)U_r->ld, ldq, ldq, 0});
-                if ((st = tc::launch<false, 2, tc::OUT_BF16_SPLIT>(ctx, qe, store)) != ATP_OK) return st;
+                                                     tab + (size_t)s.row0 * dh, s.L, dp, s.r, (int)U_r->ld, ldq, ldq, dh});
+                if ((st = tc::launch<false, 2, tc::OUT_BF16_SPLIT>(ctx, qe, rope ? turn : store)) != ATP_OK) return st;
+            }
+            if (rope) {
+                std::vector<tc::HostProblem> up, down;
+                for (auto &s : seqs)
+                    if (s.L > 0) {
+                        const T *u = (const T *)U_r->data + (size_t)s.row0 * U_r->ld;
+                        const size_t k1 = (size_t)s.rank0 * ldq, kr = (size_t)s.row0 * ldq;
+                        tc::HostProblem a{u, K1[0] + k1, K1[1] + k1, Kr[0] + kr, Kr[1] + kr, tab + (size_t)s.row0 * dh, s.L, dp, s.r,
+                                          (int)U_r->ld, ldq, ldq, dh};
+                        a.B3 = K1[2] + k1; a.C3 = Kr[2] + kr;
+                        up.push_back(a);
+                        tc::HostProblem b{u, Kr[0] + kr, Kr[1] + kr, pl.Kh + k1, pl.Kl + k1, nullptr, s.r, dp, s.L, (int)U_r->ld, ldq, ldq, 0};
+                        b.B3 = Kr[2] + kr;
+                        down.push_back(b);
+                    }
+                if ((st = tc::launch<false, 3, tc::OUT_BF16_SPLIT3>(ctx, up, turn, "gemm_tc_rope")) != ATP_OK) return st;
+                if ((st = tc::launch<true, 3, tc::OUT_BF16_SPLIT>(ctx, down, store, "gemm_tc_rope")) != ATP_OK) return st;
             }
             std::vector<atc::HostSeq> hs;
             float *nrm = pl.nrm;
@@ -274,6 +340,7 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
     }
     if (rope) {
         // K = U_r K' (Eq. 6), rows of K and Q rotated by their positions, principal keys K'_rot = U_r^T K_rot
+        if ((st = make_rope_table()) != ATP_OK) return st;
         std::vector<GemmProblem> up, down;
         RopeBatch rb; rb.count = 0;
         auto flush_rope = [&]() -> atp_status {
@@ -282,7 +349,7 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
             for (int i = 0; i < rb.count; ++i) maxL = std::max(maxL, rb.s[i].L);
             ATP_KERNEL(ctx, "rope", 0, 0);
             rope_kernel<<<dim3(std::min(512, ceil_div(maxL * (dp / 2), 256)), rb.count), 256, 0, ctx->stream>>>(
-                rb, dp, dh, log2((double)rope_base), positions);
+                rb, dp, dh, pl.tab);
             ATP_LAUNCHED(ctx);
             rb.count = 0;
             return ATP_OK;
@@ -305,31 +372,6 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
                                            pl.Kp + (size_t)sq.rank0 * dp, nullptr, sq.r, dp, sq.L, (int)U_r->ld, dp, dp, 0});
         st = for_each_chunk(down, [&](const GemmBatch &b) { return launch_gemm_simt<T, float, float, true>(ctx, b, store, 1, nullptr, 0, "gemm_simt_rope"); });
         if (st != ATP_OK) return st;
-    }
-    if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-        if (dh == 64 || dh == 128) {
-            // rotary positions with a tensor-core head width: the fp32 K'_rot, Q_rot and V' are cut into the
-            // bf16 (hi/lo) operands of the fused kernel
-            const int ldq = (int)align_up((size_t)dp, 8);
-            ATP_KERNEL(ctx, "f32_to_bf16", 0, (double)(2 * tr + tl) * dp * 8);
-            tc::f32_to_bf16_split_kernel<<<1024, 256, 0, ctx->stream>>>(pl.Kp, dp, pl.Kh, pl.Kl, ldq, (int)tr, dp);
-            ATP_LAUNCHED(ctx);
-            tc::f32_to_bf16_split_kernel<<<1024, 256, 0, ctx->stream>>>(pl.Q, dp, pl.Qh, pl.Ql, ldq, (int)tl, dp);
-            ATP_LAUNCHED(ctx);
-            tc::f32_to_bf16_split_kernel<<<1024, 256, 0, ctx->stream>>>(pl.Vp, dp, pl.Vb, pl.Qpl, ldq, (int)tr, dp);   // lo part unused
-            ATP_LAUNCHED(ctx);
-            std::vector<atc::HostSeq> hs;
-            float *nrm = pl.nrm;
-            for (auto &sq : seqs)
-                if (sq.L > 0) {
-                    float *qmax = nrm, *kmax = nrm + (size_t)heads * ceil_div(sq.L, 128);
-                    nrm += (size_t)heads * (ceil_div(sq.L, 128) + ceil_div(sq.r, 128));
-                    hs.push_back(atc::HostSeq{pl.Qh + (size_t)sq.row0 * ldq, pl.Ql + (size_t)sq.row0 * ldq, pl.Kh + (size_t)sq.rank0 * ldq,
-                                              pl.Kl + (size_t)sq.rank0 * ldq, pl.Vb + (size_t)sq.rank0 * ldq,
-                                              (T *)O->data + (size_t)sq.row0 * O->ld, sq.L, sq.r, ldq, ldq, (int)O->ld, dp, qmax, kmax});
-                }
-            return dh == 64 ? atc::launch<64>(ctx, hs, heads, scale) : atc::launch<128>(ctx, hs, heads, scale);
-        }
     }
     size_t smem = ((size_t)dh * 68 * 2 + (size_t)64 * dh + 64 * 65) * sizeof(float);
     ATP_CUDA_OK(ctx, cudaFuncSetAttribute(attn_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

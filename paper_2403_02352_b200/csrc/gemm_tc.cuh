@@ -428,13 +428,15 @@ gemm_tc_kernel(const __grid_constant__ Batch<P> batch, GemmEpi epi, int *dev_sta
 #pragma unroll
                             for (int j = 0; j < 32; ++j) v[j] = gelu_erf_f(v[j]);
                     } else if (epi.kind == EPI_ROPE) {
-                        // pairs of columns turn by the angle of (row, pair of the head): D holds (cos, sin) per row and pair
-                        const float *cs = pr.D + (size_t)row * pr.ldd;
+                        // pairs of columns turn by the angle of (row, pair of the head): D holds (cos, sin) per row and pair;
+                        // the head width ldd is a multiple of 32, so the chunk lies inside one head
+                        const float4 *cs = (const float4 *)(pr.D + (size_t)row * pr.ldd + col0 % pr.ldd);
 #pragma unroll
-                        for (int j = 0; j < 32; j += 2) {
-                            const float2 t2 = __ldg((const float2 *)(cs + (col0 + j) % pr.ldd));
-                            const float x = v[j], y = v[j + 1];
-                            v[j] = x * t2.x - y * t2.y; v[j + 1] = x * t2.y + y * t2.x;
+                        for (int j = 0; j < 32; j += 4) {
+                            const float4 t4 = __ldg(cs + j / 4);
+                            const float x0 = v[j], y0 = v[j + 1], x1 = v[j + 2], y1 = v[j + 3];
+                            v[j] = x0 * t4.x - y0 * t4.y; v[j + 1] = x0 * t4.y + y0 * t4.x;
+                            v[j + 2] = x1 * t4.z - y1 * t4.w; v[j + 3] = x1 * t4.w + y1 * t4.z;
                         }
                     }
                     if (OUT == OUT_F32) {
@@ -601,19 +603,6 @@ static atp_status launch(atp_ctx *ctx, const std::vector<HostProblem> &all, Gemm
         if (st != ATP_OK) return st;
     }
     return ATP_OK;
-}
-
-// fp32 -> bf16 hi/lo pair: hi = bf16(x), lo = bf16(x - hi).
-static __global__ void f32_to_bf16_split_kernel(const float *src, int lds, __nv_bfloat16 *hi, __nv_bfloat16 *lo, int ldd, int rows, int cols)
-{
-    size_t n = (size_t)rows * cols;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        int r = (int)(e / cols), c = (int)(e - (size_t)r * cols);
-        float x = src[(size_t)r * lds + c];
-        __nv_bfloat16 h = __float2bfloat16_rn(x);
-        hi[(size_t)r * ldd + c] = h;
-        lo[(size_t)r * ldd + c] = __float2bfloat16_rn(x - __bfloat162float(h));
-    }
 }
 
 }  // namespace tc
