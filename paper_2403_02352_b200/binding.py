@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from itertools import accumulate
 from typing import Optional, Sequence
 
 import numpy as np
@@ -40,8 +41,7 @@ class Mat(C.Structure):
 
 
 class Seqs(C.Structure):
-    _fields_ = [("batch", C.c_int32), ("row_off", C.POINTER(C.c_int32)), ("rank", C.POINTER(C.c_int32)),
-                ("rank_off", C.POINTER(C.c_int32))]
+    _fields_ = [("batch", C.c_int32), ("row_off", C.c_void_p), ("rank", C.c_void_p), ("rank_off", C.c_void_p)]
 
 
 class BasisOpts(C.Structure):
@@ -112,47 +112,42 @@ def _check(code: int, where: str):
         raise AtpError(code, where)
 
 
+_DTYPE = {torch.float32: F32, torch.bfloat16: BF16}
+
+
 def mat(t: Optional[torch.Tensor]) -> Optional[Mat]:
     """Describe a 2-D row-major torch tensor (device memory stays owned by the tensor)."""
     if t is None:
         return None
-    if t.dim() != 2 or t.stride(1) != 1 and t.shape[1] > 1:
+    if t.dim() != 2:
         raise ValueError("expected a 2-D tensor with unit stride along columns")
-    if t.dtype == torch.float32:
-        dt = F32
-    elif t.dtype == torch.bfloat16:
-        dt = BF16
-    else:
+    rows, cols = t.shape
+    ld, sc = t.stride()
+    if sc != 1 and cols > 1:
+        raise ValueError("expected a 2-D tensor with unit stride along columns")
+    dt = _DTYPE.get(t.dtype)
+    if dt is None:
         raise AtpError(ERR_UNSUPPORTED_DTYPE, "mat")
-    ld = t.stride(0) if t.shape[0] > 1 else max(t.shape[1], t.stride(0))
-    return Mat(t.data_ptr(), dt, t.shape[0], t.shape[1], ld)
+    return Mat(t.data_ptr(), dt, rows, cols, ld if rows > 1 else max(cols, ld))
 
 
 class SeqDesc:
-    """Host arrays of a packed batch (kept alive for the duration of a call)."""
+    """Host arrays of a packed batch (kept alive for the duration of a call). One ctypes buffer holds the three arrays:
+    row offsets, ranks, rank offsets."""
 
     def __init__(self, lengths: Sequence[int], ranks: Sequence[int]):
         self.lengths = [int(x) for x in lengths]
         self.ranks = [int(x) for x in ranks]
-        if len(self.lengths) != len(self.ranks):
-            raise ValueError("lengths and ranks differ in size")
         n = len(self.lengths)
-        self.row_off = np.zeros(n + 1, dtype=np.int32)
-        self.rank_off = np.zeros(n + 1, dtype=np.int32)
-        self.row_off[1:] = np.cumsum(self.lengths)
-        self.rank_off[1:] = np.cumsum(self.ranks)
-        self.rank = np.asarray(self.ranks, dtype=np.int32)
-        p32 = C.POINTER(C.c_int32)
-        self.c = Seqs(n, self.row_off.ctypes.data_as(p32), self.rank.ctypes.data_as(p32),
-                      self.rank_off.ctypes.data_as(p32))
-
-    @property
-    def total_rows(self):
-        return int(self.row_off[-1])
-
-    @property
-    def total_rank(self):
-        return int(self.rank_off[-1])
+        if n != len(self.ranks):
+            raise ValueError("lengths and ranks differ in size")
+        rows, offs = [0], [0]
+        rows.extend(accumulate(self.lengths))
+        offs.extend(accumulate(self.ranks))
+        self.total_rows, self.total_rank = rows[-1], offs[-1]
+        self._buf = (C.c_int32 * (3 * n + 2))(*rows, *self.ranks, *offs)
+        at = C.addressof(self._buf)
+        self.c = Seqs(n, at, at + 4 * (n + 1), at + 4 * (2 * n + 1))
 
 
 class Context:
@@ -230,6 +225,8 @@ class Context:
 def _padded(shape, like: torch.Tensor) -> torch.Tensor:
     """Uninitialised (rows x cols) tensor whose leading dimension is a multiple of 8 elements."""
     rows, cols = shape
+    if cols % 8 == 0:
+        return torch.empty((rows, cols), dtype=like.dtype, device=like.device)
     return torch.empty((rows, (cols + 7) // 8 * 8), dtype=like.dtype, device=like.device)[:, :cols]
 
 
