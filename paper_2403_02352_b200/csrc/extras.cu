@@ -1,25 +1,39 @@
 // atp_alternating_basis: the paper's own approximate extraction (Algorithm 1, appendix B) - rank-1
 // alternating fits with deflation - and atp_svd_entropy: Eq. 4 with the rank rule of Sec. 3.
 //
-// Algorithm 1 on the GPU. The method is a chain of matrix-vector products over the deflated matrix
-// R (L x d, fp32, resident in the workspace): for every component, `inner` rounds of
+// Algorithm 1 on the GPU. The method is a chain of matrix-vector products over the deflated matrix R (L x d, fp32): for
+// every component, `inner` rounds of
 //   u = R v / |v|^2,   v = R^T u / |u|^2,
-// then R <- R - u v^T. Every product reads R once, so the path is bound by memory traffic
-// ((2 inner + 2) L d 4 bytes per component; R stays in L2 when it fits). Dot products accumulate in
-// fp64 so that the only rounding of a step is the fp32 storage of u, v and R.
+// then R <- R - u v^T. One persistent cooperative launch runs the whole chain for all sequences of a batch: a group of CTAs
+// per sequence, each with a share of the rows of R in shared memory (rows that do not fit stay in the workspace, L2). A
+// round is one visit of the rows: phase A takes the dot products of the rows with v (four rows per warp; in the first
+// round of a component it applies the deflation of the component before on the way), phase B multiplies the same rows by u
+// column by column. The partial columns of the group's CTAs are summed in a fixed order around a group barrier. Dot
+// products accumulate in fp64, so that the only rounding of a step is the fp32 storage of u, v and R.
+// Bound by widening the elements to fp64 (three integer operations, about 32 elements a clock and SM, once per phase; the
+// conversion instruction runs at 16) and by the barrier and the partial sums of a round.
+// 16 sequences of 512 x 1024, r = 64, inner = 2: 5092 -> 1660 us (a chain of 320 launches that read R six times per
+// component from L2 before).
 #include "common.cuh"
+#include "group_barrier.cuh"
 
 constexpr int ALT_MAX = 32;        // sequences per launch
+constexpr int ALT_NT = 512;        // threads per CTA
+constexpr int ALT_DIRECT = 16;     // up to this many CTAs in a group every CTA sums the partial columns itself
 struct AltSeq {
-    float *R, *u, *v;              // deflated copy (L x d), current u (L), current v (d)
+    const void *X;                 // first row of the sequence in the packed input
+    float *R;                      // rows of the deflated matrix that do not fit in shared memory (L x dp)
+    double *part;                  // partial columns: 2 (by round parity) x ncta x (dp + 4)
+    float *vbuf;                   // v of a round, where it is summed in slices
+    unsigned *sync;                // words of the group barrier
     const float *v0;               // start vectors of this sequence (r x d, row stride ldv)
     void *U, *Xp;                  // outputs: U (L x r), X' (r x d)
-    int L, r, ldu, ldx, ldv;
-    int row0;                      // first row of the sequence in the packed input
+    int L, r, ldx_in, ldu, ldx, ldv;
+    int cta0, ncta, rows;          // CTA group, rows per CTA
 };
 struct AltBatch { AltSeq s[ALT_MAX]; int count; };
 
-__device__ __forceinline__ double block_sum_256(double x, double *red)
+template <int W> __device__ __forceinline__ double block_sum(double x, double *red)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -29,105 +43,244 @@ __device__ __forceinline__ double block_sum_256(double x, double *red)
     __syncthreads();
     double s = 0.0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) s += red[i];       // fixed order
+    for (int i = 0; i < W; ++i) s += red[i];       // fixed order
     return s;
 }
 
+// x * 2^-896 in fp64, exactly, by shifting the bits of x into place (the exponent field keeps its value, fp32 denormals
+// become fp64 denormals, zero stays zero). The other factor of a product carries 2^896.
+__device__ __forceinline__ double widen(float x)
+{
+    const int b = __float_as_int(x);
+    return __hiloint2double((b >> 3) & (int)0x8fffffff, b << 29);
+}
+constexpr double WIDEN_SCALE = 0x1p896;
+
+// dp: d rounded up to 4 (row stride of R; columns d .. dp - 1 are zero); srows: rows of a CTA kept in shared memory
 template <typename T>
-__global__ void __launch_bounds__(256) alt_copy_kernel(const __grid_constant__ AltBatch batch, const T *X, int ldx_in, int d)
+__global__ void __launch_bounds__(ALT_NT, 1)
+alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int srows, int maxrows, int inner, int *status)
 {
-    const AltSeq &q = batch.s[blockIdx.y];
-    const size_t n = (size_t)q.L * d;
-    const T *src = X + (size_t)q.row0 * ldx_in;
-    for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (size_t)gridDim.x * 256) {
-        const int l = (int)(e / d), k = (int)(e - (size_t)l * d);
-        q.R[e] = to_f32(src[(size_t)l * ldx_in + k]);
-    }
-}
+    extern __shared__ __align__(16) unsigned char altsm[];
+    constexpr int NW = ALT_NT / 32;
+    __shared__ double red[NW], redu[NW];
+    int si = 0;
+#pragma unroll 1
+    for (int i = 1; i < batch.count; ++i) if ((int)blockIdx.x >= batch.s[i].cta0) si = i;
+    const AltSeq &q = batch.s[si];
+    const int rank = (int)blockIdx.x - q.cta0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (rank >= q.ncta || q.L <= 0) return;
+    double *vd = (double *)altsm, *ud = vd + dp;               // v and u of the current round, times WIDEN_SCALE
+    float *vp = (float *)(ud + maxrows), *uf = vp + dp;        // v of the last round, u in fp32
+    float *sR = (float *)(((uintptr_t)(uf + maxrows) + 15) & ~(uintptr_t)15);   // rows of R
+    const int row0 = rank * q.rows, nrow = max(0, min(q.rows, q.L - row0)), ns = min(srows, nrow);
+    float *gR = q.R + (size_t)row0 * dp;                       // rows ns .. nrow - 1 of this CTA
+    int *abort_flag = status + 1;
+    unsigned gen = 0, round = 0;
+    bool alive = true;
 
-// u = R v / |v|^2; one warp per row. `first`: v is row `comp` of the start vectors.
-__global__ void __launch_bounds__(256) alt_u_kernel(const __grid_constant__ AltBatch batch, int d, int comp, int first)
-{
-    pdl_trigger();
-    pdl_wait();
-    const AltSeq &q = batch.s[blockIdx.y];
-    if (comp >= q.r) return;
-    __shared__ double red[8];
-    const float *v = first ? q.v0 + (size_t)comp * q.ldv : q.v;
-    double part = 0.0;
-    for (int k = threadIdx.x; k < d; k += 256) { const double x = v[k]; part += x * x; }
-    const double vv = block_sum_256(part, red);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int l = blockIdx.x * 8 + warp;
-    if (l >= q.L) return;
-    const float *row = q.R + (size_t)l * d;
-    double acc = 0.0;
-    for (int k = lane; k < d; k += 32) acc = fma((double)row[k], (double)v[k], acc);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) q.u[l] = vv > 0.0 ? (float)(acc / vv) : 0.f;
-}
-
-// v = R^T u / |u|^2; a CTA owns 64 columns, its four quarters split the rows.
-__global__ void __launch_bounds__(256) alt_v_kernel(const __grid_constant__ AltBatch batch, int d, int comp)
-{
-    pdl_trigger();
-    pdl_wait();
-    const AltSeq &q = batch.s[blockIdx.y];
-    if (comp >= q.r) return;
-    __shared__ double red[8];
-    __shared__ double quarter[3][64];
-    double part = 0.0;
-    for (int l = threadIdx.x; l < q.L; l += 256) { const double x = q.u[l]; part += x * x; }
-    const double uu = block_sum_256(part, red);
-    const int c = threadIdx.x & 63, h = threadIdx.x >> 6;
-    const int k = blockIdx.x * 64 + c;
-    double acc = 0.0;
-    if (k < d) {
-        int l = h;
-        for (; l + 28 < q.L; l += 32) {            // eight loads in flight per thread
-            float rv[8], uv[8];
-#pragma unroll
-            for (int t = 0; t < 8; ++t) { rv[t] = q.R[(size_t)(l + 4 * t) * d + k]; uv[t] = q.u[l + 4 * t]; }
-#pragma unroll
-            for (int t = 0; t < 8; ++t) acc = fma((double)rv[t], (double)uv[t], acc);
-        }
-        for (; l < q.L; l += 4) acc = fma((double)q.R[(size_t)l * d + k], (double)q.u[l], acc);
+    for (int l = warp; l < nrow; l += NW) {
+        const T *x = (const T *)q.X + (size_t)(row0 + l) * q.ldx_in;
+        float *r = (l < ns ? sR : gR) + (size_t)l * dp;
+        for (int k = lane; k < dp; k += 32) r[k] = k < d ? to_f32(x[k]) : 0.f;
     }
-    if (h > 0) quarter[h - 1][c] = acc;
     __syncthreads();
-    if (h == 0 && k < d) q.v[k] = uu > 0.0 ? (float)((acc + quarter[0][c] + quarter[1][c] + quarter[2][c]) / uu) : 0.f;
-}
 
-// R <- R - u v^T, and the finished component: U[:, comp] = u / |u|, X'[comp, :] = v |u|.
-template <typename T>
-__global__ void __launch_bounds__(256) alt_deflate_kernel(const __grid_constant__ AltBatch batch, int d, int comp)
-{
-    pdl_trigger();
-    pdl_wait();
-    const AltSeq &q = batch.s[blockIdx.y];
-    if (comp >= q.r) return;
-    __shared__ double red[8];
-    double part = 0.0;
-    for (int l = threadIdx.x; l < q.L; l += 256) { const double x = q.u[l]; part += x * x; }
-    const double un = sqrt(block_sum_256(part, red));
-    if (blockIdx.x == 0) {
-        T *xp = (T *)q.Xp + (size_t)comp * q.ldx;
-        for (int k = threadIdx.x; k < d; k += 256) xp[k] = from_f32<T>((float)((double)q.v[k] * un));
+    for (int comp = 0; comp < q.r && alive; ++comp) {
+        double un = 0.0, vpart = 0.0;                          // vpart: this thread's share of |v|^2
+        for (int k = tid; k < dp; k += ALT_NT) {               // the start vector (vp still holds v of the last component)
+            const double v = k < d ? (double)q.v0[(size_t)comp * q.ldv + k] : 0.0;
+            vd[k] = v * WIDEN_SCALE;
+            vpart += v * v;
+        }
+        for (int j = 0; j < inner && alive; ++j, ++round) {
+            const bool deflate = j == 0 && comp > 0;
+            const double vv = block_sum<NW>(vpart, red);       // (its barriers also publish vd)
+            double usq = 0.0;
+            auto finish = [&](int l, double acc) {             // u of row l from the lanes' sums
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                const float u = vv > 0.0 ? (float)(acc / vv) : 0.f;
+                if (lane == 0) { uf[l] = u; ud[l] = (double)u * WIDEN_SCALE; }
+                usq += (double)u * (double)u;
+            };
+            auto dot = [&](double acc, float4 x, double2 va, double2 vb) {
+                acc = fma(widen(x.x), va.x, acc); acc = fma(widen(x.y), va.y, acc);
+                acc = fma(widen(x.z), vb.x, acc); return fma(widen(x.w), vb.y, acc);
+            };
+            auto subtract = [&](float4 &x, float u, float4 p) {
+                x.x = fmaf(-u, p.x, x.x); x.y = fmaf(-u, p.y, x.y); x.z = fmaf(-u, p.z, x.z); x.w = fmaf(-u, p.w, x.w);
+            };
+
+            // phase A: u = R v / |v|^2. Rows in shared memory, four of a warp together (v is read once for them)
+            for (int l0 = warp; l0 < ns; l0 += NW * 4) {
+                double acc[4] = {0.0, 0.0, 0.0, 0.0};
+                float *rp[4], up[4];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    const int l = l0 + NW * a;
+                    rp[a] = sR + (size_t)(l < ns ? l : l0) * dp;
+                    up[a] = deflate && l < ns ? uf[l] : 0.f;
+                }
+                for (int k = lane * 4; k < dp; k += 128) {
+                    const double2 va = *(const double2 *)(vd + k), vb = *(const double2 *)(vd + k + 2);
+                    float4 x[4];
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) x[a] = *(const float4 *)(rp[a] + k);
+                    if (deflate) {
+                        const float4 p = *(const float4 *)(vp + k);
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) {
+                            subtract(x[a], up[a], p);
+                            if (l0 + NW * a < ns) *(float4 *)(rp[a] + k) = x[a];
+                        }
+                    }
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) acc[a] = dot(acc[a], x[a], va, vb);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int a = 0; a < 4; ++a) if (l0 + NW * a < ns) finish(l0 + NW * a, acc[a]);
+            }
+            // rows in the workspace, one of a warp at a time, eight loads in flight
+            for (int l = ns + warp; l < nrow; l += NW) {
+                float *rp = gR + (size_t)l * dp;
+                const float up = deflate ? uf[l] : 0.f;
+                double acc = 0.0;
+                for (int k0 = lane * 4; k0 < dp; k0 += 1024) {
+                    float4 x[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) x[i] = k0 + 128 * i < dp ? *(const float4 *)(rp + k0 + 128 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int k = k0 + 128 * i;
+                        if (k >= dp) continue;
+                        if (deflate) { subtract(x[i], up, *(const float4 *)(vp + k)); *(float4 *)(rp + k) = x[i]; }
+                        acc = dot(acc, x[i], *(const double2 *)(vd + k), *(const double2 *)(vd + k + 2));
+                    }
+                }
+                __syncwarp();
+                finish(l, acc);
+            }
+            if (lane == 0) redu[warp] = usq;
+            __syncthreads();
+
+            // phase B: this CTA's part of R^T u, two columns a thread; the first rows from the workspace are fetched early
+            double *mine = q.part + ((size_t)(round & 1) * q.ncta + rank) * (dp + 4);
+            for (int k = tid * 2; k < dp; k += ALT_NT * 2) {
+                double a0 = 0.0, a1 = 0.0;
+                float2 g[4];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) g[a] = ns + a < nrow ? *(const float2 *)(gR + (size_t)(ns + a) * dp + k) : make_float2(0.f, 0.f);
+                const float *col = sR + k;
+                int l = 0;
+                for (; l + 8 <= ns; l += 8, col += 8 * (size_t)dp) {
+                    float2 x[8];
+#pragma unroll
+                    for (int a = 0; a < 8; ++a) x[a] = *(const float2 *)(col + a * (size_t)dp);
+#pragma unroll
+                    for (int a = 0; a < 8; ++a) { const double u = ud[l + a]; a0 = fma(widen(x[a].x), u, a0); a1 = fma(widen(x[a].y), u, a1); }
+                }
+                for (; l < ns; ++l, col += dp) { const float2 x = *(const float2 *)col; a0 = fma(widen(x.x), ud[l], a0); a1 = fma(widen(x.y), ud[l], a1); }
+#pragma unroll
+                for (int a = 0; a < 4; ++a) if (ns + a < nrow) { a0 = fma(widen(g[a].x), ud[ns + a], a0); a1 = fma(widen(g[a].y), ud[ns + a], a1); }
+#pragma unroll 4
+                for (l = ns + 4; l < nrow; ++l) { const float2 x = *(const float2 *)(gR + (size_t)l * dp + k); a0 = fma(widen(x.x), ud[l], a0); a1 = fma(widen(x.y), ud[l], a1); }
+                *(double2 *)(mine + k) = make_double2(a0, a1);
+            }
+            if (tid == 0) {
+                double s = 0.0;
+#pragma unroll
+                for (int i = 0; i < NW; ++i) s += redu[i];
+                mine[dp] = s;
+            }
+            alive = group_barrier(q.sync, ++gen, (unsigned)q.ncta, abort_flag) && alive;
+            if (!alive) break;
+            // v = R^T u / |u|^2 from the partial columns, in rank order
+            const size_t ps = (size_t)dp + 4;
+            const double *all = q.part + (size_t)(round & 1) * q.ncta * ps;
+            auto total = [&](int k) {                            // eight loads in flight
+                double s0 = 0.0;
+                for (int c = 0; c < q.ncta; c += 8) {
+                    double x[8];
+#pragma unroll
+                    for (int a = 0; a < 8; ++a) x[a] = c + a < q.ncta ? __ldcg(all + (size_t)(c + a) * ps + k) : 0.0;
+#pragma unroll
+                    for (int a = 0; a < 8; ++a) s0 += x[a];
+                }
+                return s0;
+            };
+            vpart = 0.0;
+            auto keep = [&](int k, float v) { vp[k] = v; vd[k] = (double)v * WIDEN_SCALE; vpart += (double)v * (double)v; };
+            if (q.ncta <= ALT_DIRECT) {
+                const double s0 = tid < dp ? total(tid) : 0.0, uu = total(dp);
+                un = uu;
+                if (tid < dp) keep(tid, uu > 0.0 ? (float)(s0 / uu) : 0.f);
+                for (int k = tid + ALT_NT; k < dp; k += ALT_NT) keep(k, uu > 0.0 ? (float)(total(k) / uu) : 0.f);
+            } else {                                             // a slice per CTA, then everybody reads the whole
+                const int per = (dp + q.ncta - 1) / q.ncta;
+                const double uu = total(dp);
+                un = uu;
+                for (int k = rank * per + tid; k < min(dp, (rank + 1) * per); k += ALT_NT) q.vbuf[k] = uu > 0.0 ? (float)(total(k) / uu) : 0.f;
+                alive = group_barrier(q.sync, ++gen, (unsigned)q.ncta, abort_flag) && alive;
+                if (!alive) break;
+                for (int k = tid; k < dp; k += ALT_NT) keep(k, __ldcg(q.vbuf + k));
+            }
+        }
+        if (!alive) break;
+        __syncthreads();
+        un = sqrt(un);
+        // the finished component: U[:, comp] = u / |u|, X'[comp, :] = v |u|
+        for (int l = tid; l < nrow; l += ALT_NT)
+            ((T *)q.U)[(size_t)(row0 + l) * q.ldu + comp] = from_f32<T>(un > 0.0 ? (float)((double)uf[l] / un) : 0.f);
+        for (int k = rank * ALT_NT + tid; k < d; k += q.ncta * ALT_NT)
+            ((T *)q.Xp)[(size_t)comp * q.ldx + k] = from_f32<T>((float)((double)vp[k] * un));
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int l = blockIdx.x * 8 + warp;
-    if (l >= q.L) return;
-    const float ul = q.u[l];
-    float *row = q.R + (size_t)l * d;
-    for (int k = lane; k < d; k += 32) row[k] = fmaf(-ul, q.v[k], row[k]);
-    if (lane == 0) ((T *)q.U)[(size_t)l * q.ldu + comp] = from_f32<T>(un > 0.0 ? (float)((double)ul / un) : 0.f);
+    if (!alive && rank == 0 && tid == 0) raise_status(status, ATP_ERR_TIMEOUT);
 }
 
-size_t alternating_workspace_bytes(const std::vector<SeqDims> &sd, int d)
+__global__ void alternating_init_kernel(const __grid_constant__ AltBatch batch)
+{
+    if (threadIdx.x < 64) batch.s[blockIdx.x].sync[threadIdx.x] = 0u;
+}
+
+// CTAs of each sequence of a launch (at most `total` together): in proportion to the rows, at least one, and not more than
+// leaves 16 rows (a row a warp) to a CTA.
+static std::vector<int> alternating_ctas(const std::vector<SeqDims> &sd, size_t i0, size_t i1, int total)
+{
+    double rows = 0;
+    for (size_t i = i0; i < i1; ++i) rows += sd[i].L;
+    const int spare = std::max(0, total - (int)(i1 - i0));
+    std::vector<int> c;
+    for (size_t i = i0; i < i1; ++i)
+        c.push_back(std::min(std::max(1, ceil_div(sd[i].L, 16)), 1 + (int)(rows > 0 ? spare * (sd[i].L / rows) : 0)));
+    return c;
+}
+
+struct AltScratch { float *R; double *part; float *vbuf; unsigned *sync; int ncta; };
+static void plan_alternating(Arena &ar, const std::vector<SeqDims> &sd, int d, int sm_count, std::vector<AltScratch> &out)
+{
+    const size_t dp = align_up((size_t)d, 4);
+    for (size_t i0 = 0; i0 < sd.size(); i0 += ALT_MAX) {
+        const size_t i1 = std::min(sd.size(), i0 + ALT_MAX);
+        const std::vector<int> c = alternating_ctas(sd, i0, i1, sm_count);
+        for (size_t i = i0; i < i1; ++i) {
+            AltScratch a;
+            a.ncta = c[i - i0];
+            a.R = ar.take<float>((size_t)sd[i].L * dp);
+            a.part = ar.take<double>((size_t)2 * a.ncta * (dp + 4));
+            a.vbuf = ar.take<float>(dp);
+            a.sync = ar.take<unsigned>(64);
+            out.push_back(a);
+        }
+    }
+}
+
+size_t alternating_workspace_bytes(const std::vector<SeqDims> &sd, int d, int sm_count)
 {
     Arena ar(nullptr, (size_t)-1);
-    for (auto &s : sd) { ar.take<float>((size_t)s.L * d); ar.take<float>(s.L); ar.take<float>(d); }
+    std::vector<AltScratch> sc;
+    plan_alternating(ar, sd, d, sm_count, sc);
     return ar.off;
 }
 
@@ -135,43 +288,52 @@ template <typename T>
 static atp_status alternating_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<SeqDims> &sd, const atp_mat *V0, int inner,
                                    atp_mat *U_r, atp_mat *X_r)
 {
-    const int d = (int)X->cols;
+    const int d = (int)X->cols, dp = (int)align_up((size_t)d, 4);
     Arena ar(ctx->workspace, ctx->workspace_bytes);
-    std::vector<AltSeq> seqs(sd.size());
-    for (size_t i = 0; i < sd.size(); ++i) {
-        AltSeq &q = seqs[i];
-        q.R = ar.take<float>((size_t)sd[i].L * d); q.u = ar.take<float>(sd[i].L); q.v = ar.take<float>(d);
-        q.v0 = (const float *)V0->data + (size_t)sd[i].rank0 * V0->ld;
-        q.U = (T *)U_r->data + (size_t)sd[i].row0 * U_r->ld;
-        q.Xp = (T *)X_r->data + (size_t)sd[i].rank0 * X_r->ld;
-        q.L = sd[i].L; q.r = sd[i].r; q.ldu = (int)U_r->ld; q.ldx = (int)X_r->ld; q.ldv = (int)V0->ld;
-        q.row0 = sd[i].row0;
-    }
-    if (ar.overflow) return ATP_ERR_WORKSPACE_TOO_SMALL;
+    std::vector<AltScratch> sc;
+    plan_alternating(ar, sd, d, ctx->sm_count, sc);
+    if (ar.overflow || !ctx->workspace) return ATP_ERR_WORKSPACE_TOO_SMALL;
+    constexpr int SMEM = 225 * 1024;       // of 227 KB a CTA may have: the rest is the kernel's static share
+    static PerDeviceOnce attr_once;
+    ATP_CUDA_OK(ctx, attr_once.run(ctx->device, [] {
+        return cudaFuncSetAttribute(alternating_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    }));
     for (size_t i0 = 0; i0 < sd.size(); i0 += ALT_MAX) {
         AltBatch b; b.count = (int)std::min<size_t>(ALT_MAX, sd.size() - i0);
-        int maxL = 0, maxr = 0;
-        for (int k = 0; k < b.count; ++k) { b.s[k] = seqs[i0 + k]; maxL = std::max(maxL, b.s[k].L); maxr = std::max(maxr, b.s[k].r); }
-        if (maxL == 0) continue;
-        const double mat_bytes = [&] { double s = 0; for (int k = 0; k < b.count; ++k) s += (double)b.s[k].L * d * 4; return s; }();
-        ATP_KERNEL(ctx, "alt_copy", 0, mat_bytes * (1.0 + sizeof(T) / 4.0));
-        alt_copy_kernel<T><<<dim3(std::min(1024, (int)(((size_t)maxL * d + 255) / 256)), b.count), 256, 0, ctx->stream>>>(
-            b, (const T *)X->data, (int)X->ld, d);
-        ATP_LAUNCHED(ctx);
-        const dim3 grows((maxL + 7) / 8, b.count), gcols((d + 63) / 64, b.count);
-        for (int comp = 0; comp < maxr; ++comp) {
-            for (int j = 0; j < inner; ++j) {
-                ATP_KERNEL(ctx, "alt_u", 0, mat_bytes);
-                launch_pdl(alt_u_kernel, grows, dim3(256), 0, ctx->stream, b, d, comp, (int)(j == 0));
-                ATP_LAUNCHED(ctx);
-                ATP_KERNEL(ctx, "alt_v", 0, mat_bytes);
-                launch_pdl(alt_v_kernel, gcols, dim3(256), 0, ctx->stream, b, d, comp);
-                ATP_LAUNCHED(ctx);
-            }
-            ATP_KERNEL(ctx, "alt_deflate", 0, 2.0 * mat_bytes);
-            launch_pdl(alt_deflate_kernel<T>, grows, dim3(256), 0, ctx->stream, b, d, comp);
-            ATP_LAUNCHED(ctx);
+        int next = 0, maxrows = 0;
+        double work = 0;
+        for (int k = 0; k < b.count; ++k) {
+            const SeqDims &s = sd[i0 + k];
+            const AltScratch &a = sc[i0 + k];
+            AltSeq &q = b.s[k];
+            q.X = (const T *)X->data + (size_t)s.row0 * X->ld; q.ldx_in = (int)X->ld;
+            q.R = a.R; q.part = a.part; q.vbuf = a.vbuf; q.sync = a.sync;
+            q.v0 = (const float *)V0->data + (size_t)s.rank0 * V0->ld; q.ldv = (int)V0->ld;
+            q.U = (T *)U_r->data + (size_t)s.row0 * U_r->ld; q.ldu = (int)U_r->ld;
+            q.Xp = (T *)X_r->data + (size_t)s.rank0 * X_r->ld; q.ldx = (int)X_r->ld;
+            q.L = s.L; q.r = s.r;
+            q.cta0 = next; q.ncta = a.ncta; q.rows = ceil_div(s.L, a.ncta);
+            next += a.ncta;
+            maxrows = std::max(maxrows, q.rows);
+            work += (double)s.r * s.L * d * 4;
         }
+        maxrows = (int)align_up((size_t)std::max(maxrows, 1), 2);
+        if (work == 0) continue;
+        // the vectors first, then as many rows of R as fit
+        const size_t fixed = (size_t)dp * 12 + (size_t)maxrows * 12 + 32;
+        if (fixed > SMEM) return ATP_ERR_INVALID_ARG;
+        int srows = (int)std::min<size_t>((SMEM - fixed) / ((size_t)dp * 4), (size_t)maxrows);
+        const size_t smem = fixed + (size_t)srows * dp * 4;
+        ATP_KERNEL(ctx, "alternating_init", 0, 0);
+        alternating_init_kernel<<<b.count, 64, 0, ctx->stream>>>(b);
+        ATP_LAUNCHED(ctx);
+        int dd = d, ddp = dp, mr = maxrows, in = inner;
+        int *status = ctx->dev_status;
+        void *args[] = {(void *)&b, (void *)&dd, (void *)&ddp, (void *)&srows, (void *)&mr, (void *)&in, (void *)&status};
+        // bytes: R once per round, written once per component (most of it in shared memory)
+        ATP_KERNEL(ctx, "alternating", work / 4 * (4.0 * inner + 2), work * (inner + 1));
+        ATP_CUDA_OK(ctx, cudaLaunchCooperativeKernel((const void *)alternating_kernel<T>, dim3(next), dim3(ALT_NT), args, smem, ctx->stream));
+        ATP_LAUNCHED(ctx);
     }
     return ATP_OK;
 }
@@ -207,10 +369,10 @@ __global__ void __launch_bounds__(256) svd_entropy_kernel(const __grid_constant_
     const int lo = batch.off[b], hi = batch.off[b + 1];
     double p = 0.0;
     for (int i = lo + threadIdx.x; i < hi; i += 256) p += (double)sigma[i];
-    const double tot = block_sum_256(p, red);
+    const double tot = block_sum<8>(p, red);
     p = 0.0;
     for (int i = lo + threadIdx.x; i < hi; i += 256) { const double s = (double)sigma[i] / tot; p += s * s; }
-    const double acc = block_sum_256(p, red);
+    const double acc = block_sum<8>(p, red);
     if (threadIdx.x == 0) {
         const double m = (tot > 0.0 && acc > 0.0) ? -log2(acc) : 0.0;
         mu[b] = (float)m;

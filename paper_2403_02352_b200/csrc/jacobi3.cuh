@@ -22,6 +22,7 @@
 // (zero diagonal entries are never rotated), the padding of Wt is the identity.
 #pragma once
 #include "common.cuh"
+#include "group_barrier.cuh"
 #include <mutex>
 #include <algorithm>
 
@@ -33,7 +34,6 @@ constexpr int NT = 256;           // threads per CTA
 constexpr int LDA = 68;           // shared-memory row stride (floats) of A-operand style tiles
 constexpr int LDB = 72;           // shared-memory row stride of B-operand style tiles
 constexpr int MAXSEQ = 32;        // sequences per launch
-constexpr unsigned SPIN_LIMIT = 1u << 22;
 
 struct Seq {
     float *G, *Wt, *Vbuf;         // G, Wt: np x np (ld = np); Vbuf: 2 x npairs x 64 x 64 (by step parity)
@@ -59,41 +59,7 @@ __device__ __forceinline__ void rr_pair(int nb, int step, int t, int &I, int &J)
     if (I > J) { const int x = I; I = J; J = x; }
 }
 
-// Group barrier number `gen` (1, 2, ...) of a group of `ncta` CTAs: every CTA adds one to the arrival
-// counter sync[0] (release); the last one to arrive publishes `gen` in sync[32] (another cache line, so that
-// the pollers do not slow the arrivals down); the others poll that word (acquire). Bounded: returns false when
-// the wait ran out or another CTA flagged an abort. Data that crosses the barrier is read with L2 loads.
-__device__ __forceinline__ bool group_barrier(unsigned *sync, unsigned gen, unsigned ncta, int *abort_flag,
-                                              unsigned limit = SPIN_LIMIT)
-{
-    __syncthreads();
-    __shared__ int ok_s;
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        if (ncta > 1) {
-            // release / acquire at GPU scope: the block barrier above orders the CTA's writes before thread 0's
-            // release, the one below orders its acquire before the CTA's later reads
-            unsigned old;
-            asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(sync) : "memory");
-            unsigned *flag = sync + 32;
-            if (old + 1u == gen * ncta) {
-                asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flag), "r"(gen) : "memory");
-            } else {
-                ok = 0;
-                for (unsigned i = 0; i < limit; ++i) {
-                    unsigned v;
-                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-                    if ((int)(v - gen) >= 0) { ok = 1; break; }
-                    if ((i & 1023u) == 1023u && *(volatile int *)abort_flag) break;
-                }
-                if (!ok) *(volatile int *)abort_flag = 1;
-            }
-        }
-        ok_s = ok;
-    }
-    __syncthreads();
-    return ok_s != 0;
-}
+using ::group_barrier;
 
 // ---- pivot phase -------------------------------------------------------------------------------
 // The 64 rows of a pivot block sit in 32 "even" and 32 "odd" slots. A phase of width M rotates, in M rounds, every

@@ -216,3 +216,40 @@ def test_basis_without_host_sync_matches_and_can_be_captured(ctx):
     ctx.use_current_stream()
     ctx.poll()
     assert torch.equal(out[0], U0) and torch.equal(out[1], X0) and torch.equal(out[2], s0)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("lengths,d,inner", [
+    ([1], 3, 1),                       # a row, fewer columns than a 16-byte piece
+    ([16, 17], 65, 2),                 # one and two CTAs per sequence, ragged columns
+    ([700], 300, 2),                   # more CTAs than sum the partial columns directly
+    ([250, 33, 90], 1030, 3),          # more columns than threads
+    ([700] * 3, 2048, 1),              # several rows per warp
+    ([90] * 34, 40, 2),                # two launches
+    ([1000] * 15, 1000, 1),            # rows that do not fit in shared memory
+])
+def test_alternating_basis_row_and_column_splits(ctx, dtype, lengths, d, inner):
+    """Algorithm 1 at the edges of its split of rows over CTAs and warps and of columns over threads, against a 64-bit
+    run on the GPU (R, u and v are stored in fp32 here: about 2^-22 per step, amplified by the following components)."""
+    rng = np.random.default_rng(sum(lengths) + d)
+    ranks = [min(3, L) for L in lengths]
+    Xs = [ai.finish(ai.planted_matrix(rng, L, d, 0.5 ** np.arange(min(L, d, 6)), 0.01)[0], dtype) for L in lengths]
+    V0 = rng.standard_normal((sum(ranks), d)).astype(np.float32).astype(np.float64)
+    U, Xr = _atp().atp_alternating_basis(ctx, to_dev(np.concatenate(Xs), dtype), to_dev(V0, "f32"), lengths, ranks, inner=inner)
+    ctx.poll()
+    U, Xr = to_np(U), to_np(Xr)
+    ro = ko = 0
+    tol = 1e-4 if dtype == "f32" else 2e-2
+    for X, L, r in zip(Xs, lengths, ranks):
+        R = X.copy()
+        for c in range(r):
+            v = V0[ko + c]
+            for _ in range(inner):
+                u = R @ v / (v @ v)
+                v = R.T @ u / (u @ u)
+            R = R - np.outer(u, v)
+            n = np.linalg.norm(u)
+            assert np.abs(U[ro:ro + L, c] - u / n).max() <= tol * np.abs(u / n).max()
+            assert np.abs(Xr[ko + c] - v * n).max() <= tol * np.abs(v * n).max()
+        ro += L
+        ko += r
