@@ -10,9 +10,9 @@
 // round of a component it applies the deflation of the component before on the way), phase B multiplies the same rows by u
 // column by column. The partial columns of the group's CTAs are summed in a fixed order around a group barrier. Dot
 // products accumulate in fp64, so that the only rounding of a step is the fp32 storage of u, v and R.
-// Bound by widening the elements to fp64 (three integer operations, about 32 elements a clock and SM, once per phase; the
-// conversion instruction runs at 16) and by the barrier and the partial sums of a round.
-// 16 sequences of 512 x 1024, r = 64, inner = 2: 5092 -> 1660 us (a chain of 320 launches that read R six times per
+// Bound by shared-memory reads and the widening of the elements to fp64 (half by the conversion instruction, 16 a clock and
+// SM, half by three integer operations each), and by the barrier and the partial sums of a round.
+// 16 sequences of 512 x 1024, r = 64, inner = 2: 5092 -> 1380 us (a chain of 320 launches that read R six times per
 // component from L2 before).
 #include "common.cuh"
 #include "group_barrier.cuh"
@@ -48,7 +48,7 @@ template <int W> __device__ __forceinline__ double block_sum(double x, double *r
 }
 
 // x * 2^-896 in fp64, exactly, by shifting the bits of x into place (the exponent field keeps its value, fp32 denormals
-// become fp64 denormals, zero stays zero). The other factor of a product carries 2^896.
+// become fp64 denormals, zero stays zero). A sum of products with it is multiplied by 2^896 at the end.
 __device__ __forceinline__ double widen(float x)
 {
     const int b = __float_as_int(x);
@@ -63,15 +63,15 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
 {
     extern __shared__ __align__(16) unsigned char altsm[];
     constexpr int NW = ALT_NT / 32;
-    __shared__ double red[NW], redu[NW];
+    __shared__ double red[NW], redu[NW], slice[ALT_NT];
     int si = 0;
 #pragma unroll 1
     for (int i = 1; i < batch.count; ++i) if ((int)blockIdx.x >= batch.s[i].cta0) si = i;
     const AltSeq &q = batch.s[si];
     const int rank = (int)blockIdx.x - q.cta0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (rank >= q.ncta || q.L <= 0) return;
-    double *vd = (double *)altsm, *ud = vd + dp;               // v and u of the current round, times WIDEN_SCALE
-    float *vp = (float *)(ud + maxrows), *uf = vp + dp;        // v of the last round, u in fp32
+    double *ud = (double *)altsm;                              // u of the current round
+    float *vc = (float *)(ud + maxrows), *vo = vc + dp, *uf = vo + dp;   // v of the current round and of the last one, u in fp32
     float *sR = (float *)(((uintptr_t)(uf + maxrows) + 15) & ~(uintptr_t)15);   // rows of R
     const int row0 = rank * q.rows, nrow = max(0, min(q.rows, q.L - row0)), ns = min(srows, nrow);
     float *gR = q.R + (size_t)row0 * dp;                       // rows ns .. nrow - 1 of this CTA
@@ -84,29 +84,51 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
         float *r = (l < ns ? sR : gR) + (size_t)l * dp;
         for (int k = lane; k < dp; k += 32) r[k] = k < d ? to_f32(x[k]) : 0.f;
     }
+    for (int l = tid; l < maxrows; l += ALT_NT) ud[l] = 0.0;
     __syncthreads();
 
     for (int comp = 0; comp < q.r && alive; ++comp) {
         double un = 0.0, vpart = 0.0;                          // vpart: this thread's share of |v|^2
-        for (int k = tid; k < dp; k += ALT_NT) {               // the start vector (vp still holds v of the last component)
-            const double v = k < d ? (double)q.v0[(size_t)comp * q.ldv + k] : 0.0;
-            vd[k] = v * WIDEN_SCALE;
-            vpart += v * v;
+        { float *t = vc; vc = vo; vo = t; }                    // vo: v of the last component; vc: the start vector
+        for (int k = tid; k < dp; k += ALT_NT) {
+            const float v = k < d ? q.v0[(size_t)comp * q.ldv + k] : 0.f;
+            vc[k] = v;
+            vpart += (double)v * (double)v;
         }
         for (int j = 0; j < inner && alive; ++j, ++round) {
             const bool deflate = j == 0 && comp > 0;
-            const double vv = block_sum<NW>(vpart, red);       // (its barriers also publish vd)
-            double usq = 0.0;
-            auto finish = [&](int l, double acc) {             // u of row l from the lanes' sums
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            for (int o = 16; o > 0; o >>= 1) vpart += __shfl_xor_sync(0xffffffffu, vpart, o);
+            if (lane == 0) red[warp] = vpart;
+            // a row that lives in the workspace is fetched before anything else (first 1024 columns)
+            float4 pre[8];
+            const int pl = ns + warp;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                pre[i] = pl < nrow && lane * 4 + 128 * i < dp ? *(const float4 *)(gR + (size_t)pl * dp + lane * 4 + 128 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            __syncthreads();                                   // v and the parts of |v|^2
+            double usq = 0.0, vv = -1.0;
+            auto norm_v = [&]() {                              // fixed order
+                if (vv < 0.0) {
+                    vv = 0.0;
+#pragma unroll
+                    for (int i = 0; i < NW; ++i) vv += red[i];
+                }
+            };
+            auto put_u = [&](int l, double acc) {              // u of row l, by one lane
                 const float u = vv > 0.0 ? (float)(acc / vv) : 0.f;
-                if (lane == 0) { uf[l] = u; ud[l] = (double)u * WIDEN_SCALE; }
+                uf[l] = u; ud[l] = (double)u;
                 usq += (double)u * (double)u;
             };
-            auto dot = [&](double acc, float4 x, double2 va, double2 vb) {
-                acc = fma(widen(x.x), va.x, acc); acc = fma(widen(x.y), va.y, acc);
-                acc = fma(widen(x.z), vb.x, acc); return fma(widen(x.w), vb.y, acc);
+            auto lanes_sum = [&](double acc, int from) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) if (o <= from) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                return acc;
+            };
+            // one sum with converted and one with shifted elements
+            auto dot = [&](double &a, double &w, float4 x, const double (&v)[4]) {
+                a = fma((double)x.x, v[0], a); w = fma(widen(x.y), v[1], w);
+                a = fma((double)x.z, v[2], a); w = fma(widen(x.w), v[3], w);
             };
             auto subtract = [&](float4 &x, float u, float4 p) {
                 x.x = fmaf(-u, p.x, x.x); x.y = fmaf(-u, p.y, x.y); x.z = fmaf(-u, p.z, x.z); x.w = fmaf(-u, p.w, x.w);
@@ -114,7 +136,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
 
             // phase A: u = R v / |v|^2. Rows in shared memory, four of a warp together (v is read once for them)
             for (int l0 = warp; l0 < ns; l0 += NW * 4) {
-                double acc[4] = {0.0, 0.0, 0.0, 0.0};
+                double acc[4] = {0.0, 0.0, 0.0, 0.0}, aw[4] = {0.0, 0.0, 0.0, 0.0};
                 float *rp[4], up[4];
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {
@@ -123,12 +145,13 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
                     up[a] = deflate && l < ns ? uf[l] : 0.f;
                 }
                 for (int k = lane * 4; k < dp; k += 128) {
-                    const double2 va = *(const double2 *)(vd + k), vb = *(const double2 *)(vd + k + 2);
+                    const float4 vf = *(const float4 *)(vc + k);
+                    const double v[4] = {vf.x, vf.y, vf.z, vf.w};
                     float4 x[4];
 #pragma unroll
                     for (int a = 0; a < 4; ++a) x[a] = *(const float4 *)(rp[a] + k);
                     if (deflate) {
-                        const float4 p = *(const float4 *)(vp + k);
+                        const float4 p = *(const float4 *)(vo + k);
 #pragma unroll
                         for (int a = 0; a < 4; ++a) {
                             subtract(x[a], up[a], p);
@@ -136,32 +159,45 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
                         }
                     }
 #pragma unroll
-                    for (int a = 0; a < 4; ++a) acc[a] = dot(acc[a], x[a], va, vb);
+                    for (int a = 0; a < 4; ++a) dot(acc[a], aw[a], x[a], v);
                 }
                 __syncwarp();
+                // the four sums over the lanes together: after two exchanges a quarter of the warp holds each row
 #pragma unroll
-                for (int a = 0; a < 4; ++a) if (l0 + NW * a < ns) finish(l0 + NW * a, acc[a]);
+                for (int a = 0; a < 4; ++a) acc[a] = fma(aw[a], WIDEN_SCALE, acc[a]);
+                const bool h1 = lane & 16, h0 = lane & 8;
+                const double p0 = (h1 ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, h1 ? acc[0] : acc[2], 16);
+                const double p1 = (h1 ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, h1 ? acc[1] : acc[3], 16);
+                const double t = lanes_sum((h0 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, h0 ? p0 : p1, 8), 4);
+                norm_v();
+                const int l = l0 + NW * (lane >> 3);
+                if ((lane & 7) == 0 && l < ns) put_u(l, t);
             }
             // rows in the workspace, one of a warp at a time, eight loads in flight
-            for (int l = ns + warp; l < nrow; l += NW) {
+            for (int l = pl; l < nrow; l += NW) {
                 float *rp = gR + (size_t)l * dp;
                 const float up = deflate ? uf[l] : 0.f;
-                double acc = 0.0;
+                double acc = 0.0, aw = 0.0;
                 for (int k0 = lane * 4; k0 < dp; k0 += 1024) {
-                    float4 x[8];
+                    if (l != pl || k0 >= 1024)
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) x[i] = k0 + 128 * i < dp ? *(const float4 *)(rp + k0 + 128 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int i = 0; i < 8; ++i) pre[i] = k0 + 128 * i < dp ? *(const float4 *)(rp + k0 + 128 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const int k = k0 + 128 * i;
                         if (k >= dp) continue;
-                        if (deflate) { subtract(x[i], up, *(const float4 *)(vp + k)); *(float4 *)(rp + k) = x[i]; }
-                        acc = dot(acc, x[i], *(const double2 *)(vd + k), *(const double2 *)(vd + k + 2));
+                        if (deflate) { subtract(pre[i], up, *(const float4 *)(vo + k)); *(float4 *)(rp + k) = pre[i]; }
+                        const float4 vf = *(const float4 *)(vc + k);
+                        const double v[4] = {vf.x, vf.y, vf.z, vf.w};
+                        dot(acc, aw, pre[i], v);
                     }
                 }
                 __syncwarp();
-                finish(l, acc);
+                acc = lanes_sum(fma(aw, WIDEN_SCALE, acc), 16);
+                norm_v();
+                if (lane == 0) put_u(l, acc);
             }
+            usq = lanes_sum(usq, 16);
             if (lane == 0) redu[warp] = usq;
             __syncthreads();
 
@@ -173,20 +209,24 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
 #pragma unroll
                 for (int a = 0; a < 4; ++a) g[a] = ns + a < nrow ? *(const float2 *)(gR + (size_t)(ns + a) * dp + k) : make_float2(0.f, 0.f);
                 const float *col = sR + k;
+                auto add = [&](float2 x, double u) { a0 = fma((double)x.x, u, a0); a1 = fma(widen(x.y), u, a1); };
                 int l = 0;
                 for (; l + 8 <= ns; l += 8, col += 8 * (size_t)dp) {
                     float2 x[8];
+                    double2 u[4];
 #pragma unroll
                     for (int a = 0; a < 8; ++a) x[a] = *(const float2 *)(col + a * (size_t)dp);
 #pragma unroll
-                    for (int a = 0; a < 8; ++a) { const double u = ud[l + a]; a0 = fma(widen(x[a].x), u, a0); a1 = fma(widen(x[a].y), u, a1); }
-                }
-                for (; l < ns; ++l, col += dp) { const float2 x = *(const float2 *)col; a0 = fma(widen(x.x), ud[l], a0); a1 = fma(widen(x.y), ud[l], a1); }
+                    for (int a = 0; a < 4; ++a) u[a] = *(const double2 *)(ud + l + 2 * a);
 #pragma unroll
-                for (int a = 0; a < 4; ++a) if (ns + a < nrow) { a0 = fma(widen(g[a].x), ud[ns + a], a0); a1 = fma(widen(g[a].y), ud[ns + a], a1); }
+                    for (int a = 0; a < 8; ++a) add(x[a], a & 1 ? u[a >> 1].y : u[a >> 1].x);
+                }
+                for (; l < ns; ++l, col += dp) add(*(const float2 *)col, ud[l]);
+#pragma unroll
+                for (int a = 0; a < 4; ++a) if (ns + a < nrow) add(g[a], ud[ns + a]);
 #pragma unroll 4
-                for (l = ns + 4; l < nrow; ++l) { const float2 x = *(const float2 *)(gR + (size_t)l * dp + k); a0 = fma(widen(x.x), ud[l], a0); a1 = fma(widen(x.y), ud[l], a1); }
-                *(double2 *)(mine + k) = make_double2(a0, a1);
+                for (l = ns + 4; l < nrow; ++l) add(*(const float2 *)(gR + (size_t)l * dp + k), ud[l]);
+                *(double2 *)(mine + k) = make_double2(a0, a1 * WIDEN_SCALE);
             }
             if (tid == 0) {
                 double s = 0.0;
@@ -199,33 +239,53 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
             // v = R^T u / |u|^2 from the partial columns, in rank order
             const size_t ps = (size_t)dp + 4;
             const double *all = q.part + (size_t)(round & 1) * q.ncta * ps;
-            auto total = [&](int k) {                            // eight loads in flight
-                double s0 = 0.0;
-                for (int c = 0; c < q.ncta; c += 8) {
-                    double x[8];
-#pragma unroll
-                    for (int a = 0; a < 8; ++a) x[a] = c + a < q.ncta ? __ldcg(all + (size_t)(c + a) * ps + k) : 0.0;
-#pragma unroll
-                    for (int a = 0; a < 8; ++a) s0 += x[a];
-                }
-                return s0;
-            };
+            double uu = 0.0;
+            for (int c = lane; c < q.ncta; c += 32) uu += __ldcg(all + (size_t)c * ps + dp);
             vpart = 0.0;
-            auto keep = [&](int k, float v) { vp[k] = v; vd[k] = (double)v * WIDEN_SCALE; vpart += (double)v * (double)v; };
-            if (q.ncta <= ALT_DIRECT) {
-                const double s0 = tid < dp ? total(tid) : 0.0, uu = total(dp);
-                un = uu;
-                if (tid < dp) keep(tid, uu > 0.0 ? (float)(s0 / uu) : 0.f);
-                for (int k = tid + ALT_NT; k < dp; k += ALT_NT) keep(k, uu > 0.0 ? (float)(total(k) / uu) : 0.f);
-            } else {                                             // a slice per CTA, then everybody reads the whole
-                const int per = (dp + q.ncta - 1) / q.ncta;
-                const double uu = total(dp);
-                un = uu;
-                for (int k = rank * per + tid; k < min(dp, (rank + 1) * per); k += ALT_NT) q.vbuf[k] = uu > 0.0 ? (float)(total(k) / uu) : 0.f;
+            auto keep = [&](int k, float v) { vc[k] = v; vpart += (double)v * (double)v; };
+            auto all_lanes = [&](double x) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                return x;
+            };
+            if (q.ncta <= ALT_DIRECT) {                          // two columns a thread, all loads in flight
+                bool first = true;
+                for (int k0 = 0; k0 < dp; k0 += ALT_NT * 2) {
+                    const int k = k0 + tid * 2;
+                    double2 x[ALT_DIRECT];
+#pragma unroll
+                    for (int c = 0; c < ALT_DIRECT; ++c)
+                        x[c] = c < q.ncta && k < dp ? __ldcg((const double2 *)(all + (size_t)c * ps + k)) : make_double2(0.0, 0.0);
+                    if (first) { uu = all_lanes(uu); first = false; }
+                    double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+                    for (int c = 0; c < ALT_DIRECT; ++c) { s0 += x[c].x; s1 += x[c].y; }
+                    if (k < dp) { keep(k, uu > 0.0 ? (float)(s0 / uu) : 0.f); keep(k + 1, uu > 0.0 ? (float)(s1 / uu) : 0.f); }
+                }
+            } else {                                             // a slice of columns per CTA, then everybody reads the whole
+                uu = all_lanes(uu);
+                const int per = (dp + q.ncta - 1) / q.ncta, c0 = rank * per, c1 = min(dp, c0 + per);
+                for (int k0 = c0; k0 < c1; k0 += 32) {           // 32 columns at a time, the partials dealt to the warps
+                    const int k = k0 + lane;
+                    double s0 = 0.0;
+                    if (k < c1)
+#pragma unroll 4
+                        for (int c = warp; c < q.ncta; c += NW) s0 += __ldcg(all + (size_t)c * ps + k);
+                    slice[tid] = s0;
+                    __syncthreads();
+                    if (warp == 0 && k < c1) {
+                        s0 = 0.0;
+#pragma unroll
+                        for (int i = 0; i < NW; ++i) s0 += slice[i * 32 + lane];
+                        q.vbuf[k] = uu > 0.0 ? (float)(s0 / uu) : 0.f;
+                    }
+                    __syncthreads();
+                }
                 alive = group_barrier(q.sync, ++gen, (unsigned)q.ncta, abort_flag) && alive;
                 if (!alive) break;
                 for (int k = tid; k < dp; k += ALT_NT) keep(k, __ldcg(q.vbuf + k));
             }
+            un = uu;
         }
         if (!alive) break;
         __syncthreads();
@@ -234,7 +294,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
         for (int l = tid; l < nrow; l += ALT_NT)
             ((T *)q.U)[(size_t)(row0 + l) * q.ldu + comp] = from_f32<T>(un > 0.0 ? (float)((double)uf[l] / un) : 0.f);
         for (int k = rank * ALT_NT + tid; k < d; k += q.ncta * ALT_NT)
-            ((T *)q.Xp)[(size_t)comp * q.ldx + k] = from_f32<T>((float)((double)vp[k] * un));
+            ((T *)q.Xp)[(size_t)comp * q.ldx + k] = from_f32<T>((float)((double)vc[k] * un));
     }
     if (!alive && rank == 0 && tid == 0) raise_status(status, ATP_ERR_TIMEOUT);
 }
@@ -293,7 +353,7 @@ static atp_status alternating_impl(atp_ctx *ctx, const atp_mat *X, const std::ve
     std::vector<AltScratch> sc;
     plan_alternating(ar, sd, d, ctx->sm_count, sc);
     if (ar.overflow || !ctx->workspace) return ATP_ERR_WORKSPACE_TOO_SMALL;
-    constexpr int SMEM = 225 * 1024;       // of 227 KB a CTA may have: the rest is the kernel's static share
+    constexpr int SMEM = 226 * 1024 - 512 * 8;       // of 227 KB a CTA may have: the rest is the kernel's static share
     static PerDeviceOnce attr_once;
     ATP_CUDA_OK(ctx, attr_once.run(ctx->device, [] {
         return cudaFuncSetAttribute(alternating_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
@@ -320,7 +380,7 @@ static atp_status alternating_impl(atp_ctx *ctx, const atp_mat *X, const std::ve
         maxrows = (int)align_up((size_t)std::max(maxrows, 1), 2);
         if (work == 0) continue;
         // the vectors first, then as many rows of R as fit
-        const size_t fixed = (size_t)dp * 12 + (size_t)maxrows * 12 + 32;
+        const size_t fixed = (size_t)dp * 8 + (size_t)maxrows * 12 + 32;
         if (fixed > SMEM) return ATP_ERR_INVALID_ARG;
         int srows = (int)std::min<size_t>((SMEM - fixed) / ((size_t)dp * 4), (size_t)maxrows);
         const size_t smem = fixed + (size_t)srows * dp * 4;
