@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(NT, 2)
 orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t seed, int *status)
 {
     extern __shared__ __align__(16) float osm[];
-    __shared__ __align__(16) double Gs[PB * PB];
+    __shared__ __align__(16) double Gs[PB * LDC];
     float *sA = osm, *sB = osm + BLK * LDB;                   // two tiles at stride LDB (covers LDA too)
     int si = 0;
 #pragma unroll 1
@@ -234,10 +234,26 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             if (!skip) switch (op) {
             case OP_PF: {
                 if (do_factor && rank == 0) {
-                    for (int e = tid; e < 4096; e += NT) Gs[e] = ordered_sum(sq.gpart2 + e, 4096, nrange);
+                    {   // all elements of a partial matrix in flight together
+                        double2 g[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) g[i] = make_double2(0.0, 0.0);
+                        for (int rg = 0; rg < nrange; ++rg) {
+                            double2 x[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) x[i] = __ldcg((const double2 *)(sq.gpart2 + (size_t)rg * 4096) + tid + i * NT);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) { g[i].x += x[i].x; g[i].y += x[i].y; }
+                        }
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            double *dst = Gs + ((tid + i * NT) >> 5) * LDC + ((tid + i * NT) & 31) * 2;
+                            dst[0] = g[i].x; dst[1] = g[i].y;
+                        }
+                    }
                     __syncthreads();
                     // a nearly orthonormal panel gets its factor from a short series instead of the factorisation
-                    if (!(series_ok && lowdin_64(Gs, w, sA, sq.W, sq.flags))) chol_invert_64(Gs, w, sq.W, sq.flags);
+                    if (!(series_ok && lowdin_64(Gs, w, sA, sq.W, sq.flags))) chol_invert_64(Gs, (double *)osm, w, sq.W, sq.flags);
                     __syncthreads();
                 } else if (first >= 0) {
                     for (int it = first; it < nj * KS; it += stride) {
@@ -269,8 +285,16 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             case OP_SUMUPD: {
                 for (int it = rank; it < nj * 4; it += ncta) {           // a quarter tile per job
                     const int jb = it >> 2;
-                    for (int e = (it & 3) * 1024 + tid; e < ((it & 3) + 1) * 1024; e += NT)
-                        sq.C[(size_t)jb * 4096 + e] = ordered_sum(sq.Cpart + (size_t)jb * KS * 4096 + e, 4096, KS);
+                    const float4 *src = (const float4 *)(sq.Cpart + (size_t)jb * KS * 4096) + (it & 3) * NT + tid;
+                    float4 c4 = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int ks = 0; ks < KS; ks += 8) {                 // in this order, eight loads in flight
+                        float4 x[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) x[q] = ks + q < KS ? __ldcg(src + (size_t)(ks + q) * 1024) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) { c4.x += x[q].x; c4.y += x[q].y; c4.z += x[q].z; c4.w += x[q].w; }
+                    }
+                    ((float4 *)(sq.C + (size_t)jb * 4096))[(it & 3) * NT + tid] = c4;
                 }
                 barrier();
                 if (!alive) break;

@@ -1,161 +1,169 @@
 // Cholesky factorisation and inversion of a 64 x 64 Gram matrix in fp64, on 256 threads of a CTA.
-// Gs (shared memory, 64 x 64 doubles, row-major) holds G = P^T P of a panel of n <= 64 columns. The
+// Gs (shared memory, 64 rows of 64 doubles at stride LDC) holds G = P^T P of a panel of n <= 64 columns. The
 // matrix is scaled to unit diagonal, factored D^-1 G D^-1 = L L^T and the factor inverted; the result
 // W = D^-1 L^-T (upper triangular, fp32, 64 x 64 row-major) goes to rinv, so that P W has orthonormal
 // columns. A column whose scaled pivot falls below 1e-10 (its part outside the span of the earlier
 // columns is below 1e-5 of its norm) is flagged as dependent in flags[0..63].
-// Right-looking by blocks of four columns, in registers: thread (br, bc) owns the 4 x 4 blocks of G
-// and of X (X starts as the identity and ends as L^-1) at rows 4 br, columns 4 bc. Block step jb:
-//   1. the owner of the diagonal block factors it (four pivots) and publishes L_bb and 1 / L_jj;
-//   2. the owners of the block column below it solve for their rows of L, the owners of block row jb of
-//      X apply L_bb^-1 to it; both publish;
-//   3. everybody below subtracts L_i L_k^T from G (columns right of jb) or L_i X_b from X (columns up
-//      to jb): 64 independent multiply-adds per thread.
-// Two barriers per four columns (named barrier 1, 256 threads: exactly the threads 0..255 must call).
-// Bound by the chain of 64 pivots (reciprocal root, scaling, next pivot) and the two barriers of a block step. The
-// published rows are stored column-wise (lc[c][row]), so that step 3 reads them in 16-byte pieces with at most two
-// lanes on a bank; row-wise they collided 16-fold, and the reciprocal root went through two fp32 conversions:
-// 40300 -> 34600 cycles.
+// Four panels of 16 columns. What bounds it is the chain of 64 pivots, so a panel's diagonal block is factored inside one
+// warp, without a barrier: lane i < 16 holds row i of the block, lane 16 + j column j of its inverse (which starts as the
+// identity); with m = (entry of column c) / L_cc in every lane, the right-looking step
+//     entry[k] -= m * m_k        (m_k: m of lane k, the k-th entry of column c of L)
+// is the update of the block in the lower lanes and the forward substitution for the inverse in the upper ones. The other
+// warps finish the trailing update of the panel before meanwhile (the block that is factored next goes first), then all
+// warps form the rows of L below the panel (A_21 X_11^T) and the blocks of the inverse left of it (-X_pp L_p,: X), in
+// strips of 8 x 16 on the fp64 matrix units (with scalar multiply-adds these were bound by shared-memory reads).
+// Cycles: 40300 (first form: 4 x 4 blocks per thread, 16-way bank conflicts) -> 34600 -> 16800.
 #pragma once
 #include "common.cuh"
 #include "jacobi3.cuh"
 
 constexpr int PB = 64;            // orthonormalisation panel width
 
-__device__ __noinline__ void chol_invert_64(const double *Gs, int n, float *rinv, int *flags)
+constexpr int LDC = 68;           // row stride (doubles) in shared memory: the fragments below are free of bank conflicts
+
+// acc (8 x 8 tiles n = 0, 1 of an 8 x 16 result) += sign * A B over K = 16 on the fp64 matrix units: A rows at a, stride LDC;
+// B[k][n] = b[k * LDC + n], or b[n * LDC + k] when B_T. Lane: row lane / 4, columns 8 t + 2 (lane % 4), + 1.
+template <bool B_T, bool NEG>
+__device__ __forceinline__ void dmma_8x16x16(const double *a, const double *b, double (&acc)[2][2])
 {
-    __shared__ double rs[PB];          // 1 / sqrt(diagonal of the Gram matrix)
-    __shared__ __align__(16) double lc[4][PB];    // block column jb of L (rows below the diagonal block), by column
-    __shared__ __align__(16) double xrow4[4][PB]; // block row jb of L^-1
-    __shared__ double Lbb[4][4];       // the factored diagonal block (strictly lower part)
-    __shared__ double rinv4[4];        // 1 / L_jj, 0 for a dependent column
-    __shared__ int dep[PB];
-    auto bar256 = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
-    const int tid = threadIdx.x;
-    const int br = tid >> 4, bc = tid & 15;
-    // One 4 x 4 block per thread: it holds the thread's block of G until block step jb = bc has consumed it, and
-    // the thread's block of X from then on (a block of G left of the current step is dead, a block of X right of
-    // it is still its initial identity / zero block), which halves the register need.
-    double blk[4][4];
+    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int k0 = 0; k0 < 16; k0 += 4) {
+        const double x = a[g * LDC + k0 + q], av = NEG ? -x : x;
 #pragma unroll
-        for (int b = 0; b < 4; ++b) blk[a][b] = Gs[(4 * br + a) * PB + 4 * bc + b];
-    auto to_x = [&]() {
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) blk[a][b] = (br == bc && a == b) ? 1.0 : 0.0;
-    };
-    if (br == bc) {
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const int i = 4 * br + a;
-            rs[i] = (i < n && blk[a][a] > 0.0) ? rsqrt(blk[a][a]) : 0.0;
-            dep[i] = 0;
+        for (int t = 0; t < 2; ++t) {
+            const double bv = B_T ? b[(8 * t + g) * LDC + k0 + q] : b[(k0 + q) * LDC + 8 * t + g];
+            asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+                : "+d"(acc[t][0]), "+d"(acc[t][1]) : "d"(av), "d"(bv));
         }
     }
-    bar256();
+}
+__device__ __forceinline__ void dmma_load(const double *c, double (&acc)[2][2])
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int t = 0; t < 2; ++t) { acc[t][0] = c[g * LDC + 8 * t + 2 * q]; acc[t][1] = c[g * LDC + 8 * t + 2 * q + 1]; }
+}
+__device__ __forceinline__ void dmma_store(double *c, const double (&acc)[2][2])
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const double ra = rs[4 * br + a], rb = rs[4 * bc + b];
-            blk[a][b] = (br == bc && a == b) ? (ra > 0.0 ? 1.0 : 0.0) : blk[a][b] * ra * rb;
-        }
-    const int nblk = (n + 3) >> 2;
-    for (int jb = 0; jb < nblk; ++jb) {
-        if (br == jb && bc == jb) {
-            // 1. the diagonal block, column by column; a dependent column gets a unit pivot and zeros below
-            double ri[4];
+    for (int t = 0; t < 2; ++t) { c[g * LDC + 8 * t + 2 * q] = acc[t][0]; c[g * LDC + 8 * t + 2 * q + 1] = acc[t][1]; }
+}
+// Gs is overwritten. work: 64 x LDC doubles of shared memory (ends as L^-1, lower triangle). 256 threads.
+__device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, float *rinv, int *flags)
+{
+    __shared__ double rs[PB];          // 1 / sqrt(diagonal of the Gram matrix)
+    __shared__ int dep[PB];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    double *X = work;
+    if (tid < PB) {
+        const double g = Gs[tid * (LDC + 1)];
+        rs[tid] = tid < n && g > 0.0 ? rsqrt(g) : 0.0;
+        dep[tid] = 0;
+    }
+    __syncthreads();
+    // D^-1 G D^-1 in place: unit diagonal (0 for a zero column); X = 0
+    for (int e = tid; e < PB * PB; e += 256) {
+        const int r = e >> 6, c = e & 63;
+        Gs[r * LDC + c] = r == c ? (rs[r] > 0.0 ? 1.0 : 0.0) : Gs[r * LDC + c] * rs[r] * rs[c];
+        X[r * LDC + c] = 0.0;
+    }
+    __syncthreads();
+    for (int p = 0; p < 4; ++p) {
+        const int b = 16 * p;
+        if (warp == 0) {
+            // the diagonal block: 16 dependent pivots. The next pivot comes from the current one and two entries that every
+            // lane already has (d - e^2 / piv), so the exchange of the multipliers is off the chain.
+            double e[16];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                double piv = blk[c][c];
+            for (int k = 0; k < 16; ++k) e[k] = lane < 16 ? Gs[(b + lane) * LDC + b + k] : (lane - 16 == k ? 1.0 : 0.0);
+            unsigned bad = 0u;
+            double piv = __shfl_sync(0xffffffffu, e[0], 0);
 #pragma unroll
-                for (int k = 0; k < c; ++k) piv = fma(-blk[c][k], blk[c][k], piv);
-                const bool bad = !(piv > 1e-10);
+            for (int c = 0; c < 16; ++c) {
+                // entries of the next column that its pivot needs, before this step's update
+                const double dn = c < 15 ? __shfl_sync(0xffffffffu, e[c < 15 ? c + 1 : 15], c < 15 ? c + 1 : 15) : 0.0;
+                const double en = c < 15 ? __shfl_sync(0xffffffffu, e[c], c < 15 ? c + 1 : 15) : 0.0;
+                const bool dep_c = !(piv > 1e-10);
                 // 1/sqrt from the hardware's 20-bit approximation and one Newton step: ~2^-40 relative, far below the
                 // fp32 precision the result is stored in
                 double y;
                 asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(piv));
                 y = fma(0.5 * y, fma(-piv * y, y, 1.0), y);
-                ri[c] = bad ? 0.0 : y;
-                if (bad && 4 * jb + c < n) dep[4 * jb + c] = 1;
+                const double ln = dep_c ? 0.0 : en * y;
+                piv = fma(-ln, ln, dn);
+                // a dependent column: unit pivot, zeros below; its row of the inverse keeps its scale
+                const double m = e[c] * (dep_c ? (lane < 16 ? 0.0 : 1.0) : y);
+                bad |= dep_c ? 1u << c : 0u;
+                e[c] = m;
 #pragma unroll
-                for (int r = c + 1; r < 4; ++r) {
-                    double v = blk[r][c];
-#pragma unroll
-                    for (int k = 0; k < c; ++k) v = fma(-blk[r][k], blk[c][k], v);
-                    blk[r][c] = v * ri[c];
-                }
+                for (int k = c + 1; k < 16; ++k) e[k] = fma(-m, __shfl_sync(0xffffffffu, m, k), e[k]);
             }
+            if (lane >= 16)
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                rinv4[r] = ri[r];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) Lbb[r][c] = (c < r) ? blk[r][c] : 0.0;
-            }
-            to_x();
-        }
-        bar256();
-        if (bc == jb && br > jb) {
-            // 2a. rows of L below the diagonal block: l_c = (g_c - sum_{k<c} l_k L_bb[c][k]) / L_cc
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                double l[4];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    double v = blk[a][c];
-#pragma unroll
-                    for (int k = 0; k < c; ++k) v = fma(-l[k], Lbb[c][k], v);
-                    l[c] = v * rinv4[c];
-                    lc[c][4 * br + a] = l[c];
-                }
-            }
-            to_x();
-        }
-        if (br == jb && bc <= jb) {
-            // 2b. block row jb of X: forward substitution with L_bb (a dependent column keeps its scale)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const double sc = rinv4[c] > 0.0 ? rinv4[c] : 1.0;
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    double v = blk[c][b];
-#pragma unroll
-                    for (int k = 0; k < c; ++k) v = fma(-Lbb[c][k], blk[k][b], v);
-                    blk[c][b] = v * sc;
-                    xrow4[c][4 * bc + b] = blk[c][b];
-                }
+                for (int k = 0; k < 16; ++k) X[(b + k) * LDC + b + lane - 16] = k >= lane - 16 ? e[k] : 0.0;
+            if (lane < 16 && b + lane < n && ((bad >> lane) & 1u)) dep[b + lane] = 1;
+        } else if (p > 0) {
+            // the rest of the trailing update of panel p - 1: blocks (bi, bj), bj <= bi, below the diagonal block of panel p
+            const int nb = 4 - p;
+            for (int t = warp - 1; t < (nb * (nb + 1) / 2 - 1) * 2; t += 7) {
+                int blk = (t >> 1) + 1, bi = 0;
+                while (blk > bi) { blk -= bi + 1; ++bi; }
+                const int r = b + 16 * bi + 8 * (t & 1), c = b + 16 * blk;
+                double acc[2][2];
+                dmma_load(Gs + r * LDC + c, acc);
+                dmma_8x16x16<true, true>(Gs + r * LDC + b - 16, Gs + c * LDC + b - 16, acc);
+                dmma_store(Gs + r * LDC + c, acc);
             }
         }
-        bar256();
-        if (br > jb && bc <= br) {
-            // 3. trailing update, one column of L (and its row of X) at a time
-            const double *rsrc = bc > jb ? &lc[0][4 * bc] : &xrow4[0][4 * bc];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const double2 a0 = *(const double2 *)&lc[c][4 * br], a1 = *(const double2 *)&lc[c][4 * br + 2];
-                const double2 b0 = *(const double2 *)(rsrc + c * PB), b1 = *(const double2 *)(rsrc + c * PB + 2);
-                const double la[4] = {a0.x, a0.y, a1.x, a1.y}, rb[4] = {b0.x, b0.y, b1.x, b1.y};
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) blk[a][b] = fma(-la[a], rb[b], blk[a][b]);
-            }
+        __syncthreads();
+        // strips of the rows of L below the panel, L = A X_pp^T (t < 2 (3 - p)), and of T = sum_k L_pk X_kq, q < p
+        double acc[2][2] = {};
+        const int nl = 2 * (3 - p), strip = warp;
+        double *dst = nullptr;
+        if (strip < nl) {
+            double *a = Gs + (b + 16 + 8 * strip) * LDC + b;
+            dmma_8x16x16<true, false>(a, X + b * LDC + b, acc);
+            dst = a;
+        } else if (strip < nl + 2 * p) {
+            const int s = strip - nl, q16 = (s >> 1) * 16, r = b + 8 * (s & 1);
+            for (int kb = q16; kb < b; kb += 16) dmma_8x16x16<false, false>(Gs + r * LDC + kb, X + kb * LDC + q16, acc);
+            dst = X + r * LDC + q16;
         }
+        __syncthreads();
+        if (dst) dmma_store(dst, acc);
+        __syncthreads();
+        // X_pq = -X_pp T (in place: every warp reads before the barrier); the diagonal block of the next panel
+#pragma unroll
+        for (int t = 0; t < 2; ++t) acc[t][0] = acc[t][1] = 0.0;
+        dst = nullptr;
+        if (strip < 2 * p) {
+            const int q16 = (strip >> 1) * 16, r = b + 8 * (strip & 1);
+            dmma_8x16x16<false, true>(X + r * LDC + b, X + b * LDC + q16, acc);
+            dst = X + r * LDC + q16;
+        } else if (p < 3 && strip >= 6) {
+            const int r = b + 16 + 8 * (strip - 6);
+            dmma_load(Gs + r * LDC + b + 16, acc);
+            dmma_8x16x16<true, true>(Gs + r * LDC + b, Gs + (b + 16) * LDC + b, acc);
+            dst = Gs + r * LDC + b + 16;
+        }
+        __syncthreads();
+        if (dst) dmma_store(dst, acc);
+        if (strip >= 6) asm volatile("bar.arrive 2, 96;" ::: "memory");          // warp 0 goes on with the diagonal block
+        else if (strip == 0) asm volatile("bar.sync 2, 96;" ::: "memory");
     }
-    if (bc > br || bc >= nblk) to_x();      // blocks that never became part of X: above the diagonal, beyond n
-    // W[k][c] = (L^-1)[c][k] / D_k ; this thread holds (L^-1)[4 br + a][4 bc + b]
+    __syncthreads();
+    // W[k][c] = (L^-1)[c][k] / D_k
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-        const int k = 4 * bc + b;
+    for (int i = 0; i < 4; ++i) {
+        const int f = tid + 256 * i, k = f & 63, c = (f >> 6) * 4;
         const double rk = rs[k];
         float4 w;
-        w.x = (float)(rk * blk[0][b]); w.y = (float)(rk * blk[1][b]); w.z = (float)(rk * blk[2][b]); w.w = (float)(rk * blk[3][b]);
-        *(float4 *)(rinv + k * PB + 4 * br) = w;
+        w.x = (float)(rk * X[c * LDC + k]); w.y = (float)(rk * X[(c + 1) * LDC + k]);
+        w.z = (float)(rk * X[(c + 2) * LDC + k]); w.w = (float)(rk * X[(c + 3) * LDC + k]);
+        *(float4 *)(rinv + k * PB + c) = w;
     }
-    bar256();
     if (tid < PB) flags[tid] = (tid < n) ? (dep[tid] || !(rs[tid] > 0.0)) : 0;
 }
 
@@ -177,7 +185,7 @@ __device__ __noinline__ bool lowdin_64(const double *Gs, int n, float *Es, float
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     bool bad = false;
     if (tid < PB) {
-        const double d = Gs[tid * PB + tid];
+        const double d = Gs[tid * (LDC + 1)];
         const bool pos = tid < n && d > 0.0;
         rsq[tid] = pos ? rsqrt(d) : 0.0;
         bad = tid < n && !pos;
@@ -189,8 +197,7 @@ __device__ __noinline__ bool lowdin_64(const double *Gs, int n, float *Es, float
     for (int i = 0; i < 4; ++i) {
         const int r = ty * 4 + i;
         const double sr = rsq[r];
-        const double2 g0 = *(const double2 *)&Gs[r * PB + tx * 4], g1 = *(const double2 *)&Gs[r * PB + tx * 4 + 2];
-        const double g[4] = {g0.x, g0.y, g1.x, g1.y};
+        const double *gr = Gs + r * LDC + tx * 4, g[4] = {gr[0], gr[1], gr[2], gr[3]};
         float e[4];
         sum[i] = 0.f;
 #pragma unroll
