@@ -586,7 +586,7 @@ static void plan_basis(Arena &ar, const std::vector<SeqDims> &sd, int d, int ove
             p.oCpart = ar.take<float>(sc.cpart * 4096); p.oC = ar.take<float>(sc.c * 4096);
             p.oDpart = ar.take<float>(sc.dpart * 4096); p.oW = ar.take<float>(4096);
             p.ogpart = ar.take<double>(sc.gpart * 4096); p.ogpart2 = ar.take<double>((size_t)orth::NRED * 4096);
-            p.flags = ar.take<int>(64); p.osync = ar.take<unsigned>(64 + (size_t)p.ocap);
+            p.flags = ar.take<int>(64); p.osync = ar.take<unsigned>(orth::SYNC_WORDS + (size_t)p.ocap);
         }
         p.np = jacobi_padded(rt);
         p.G = ar.take<float>((size_t)p.np * p.np);
@@ -846,6 +846,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
             // and a short second pass on it finishes the job (a one-sided Jacobi in two strokes).
             // Each pass is one persistent kernel that stops on its own convergence test: nothing is
             // read back by the host.
+            constexpr float LEFT = 0.3f;
             for (int pass = 0; pass < 2; ++pass) {
                 if constexpr (kBf16) {
                     hp.clear();
@@ -868,7 +869,10 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 const int nsw = pass == 0 ? nsw0 : std::max(1, max_sweeps - nsw0);
                 const float tolc = pass == 0 ? fmaxf(tol_conv, 1e-2f) : tol_conv;
                 // fp32 inputs: the block products stay on the fp32 units (the threshold is below split-precision rounding)
-                if ((st = j3::launch<kBf16>(ctx, jb, tolc, tolc * 0.1f, nsw, pass == 1)) != ATP_OK) return st;
+                // A sweep whose visits all stayed below tolc ends the pass, and so does a matrix that a sweep leaves below
+                // tolc (first pass) or LEFT * tolc (second: a sweep that ends by its visits still rotates what exceeds
+                // 0.1 * tolc on the way, so what it leaves is further down)
+                if ((st = j3::launch<kBf16>(ctx, jb, tolc, pass == 0 ? tolc : LEFT * tolc, tolc * 0.1f, nsw, pass == 1)) != ATP_OK) return st;
                 if (pass == 0) {
                     // Bt2 = Bt Wt^T (d x r~),  Y2 = Y Wt^T (L x r~);  Wt rows are the eigenvectors
                     if constexpr (kBf16) {

@@ -40,7 +40,7 @@ struct Seq {
     int *vflag;                   // 2 x npairs: the pair rotated in this step
     unsigned *sync;               // 64 words. [0]: arrivals at the group barrier (monotonic); [32]: last
                                   // barrier completed; [1..4]: largest scaled off-diagonal entry of a
-                                  // sweep, slot sweep % 4; [5]: sweeps used; [16..17]: work tickets of the update, [20..21]: pivot blocks fetched, both by step parity
+                                  // sweep, slot sweep % 4; [8..11]: the same over the whole matrix after the sweep; [5]: sweeps used; [16..17]: work tickets of the update, [20..21]: pivot blocks fetched, both by step parity
     int n, np, nb;                // size, padded size (multiple of 64), number of 32-row blocks (even)
     int cta0, ncta;               // the group of CTAs that owns this sequence
 };
@@ -859,9 +859,41 @@ __device__ bool apply_item(float *sm, const Seq &sq, const float *Vbuf, const in
 // status[0]: sticky device status word of the context; status[1]: abort flag of bounded waits.
 constexpr int MAXPAIRS = 72;                  // np <= 4608
 
+// This CTA's share (rows rank, rank + ncta, ...) of the largest |g_ij| / sqrt(g_ii g_jj), i < j. rs: np floats of shared memory.
+__device__ float matrix_max(float *rs, const Seq &sq, int rank)
+{
+    __shared__ float part[NT / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = sq.n, np = sq.np;
+#pragma unroll 4
+    for (int i = tid; i < np; i += NT) {
+        const float d = i < n ? __ldcg(sq.G + (size_t)i * np + i) : 0.f;
+        rs[i] = d > 0.f ? rsqrtf(d) : 0.f;
+    }
+    __syncthreads();
+    float mo = 0.f;
+    for (int i = rank * (NT / 32) + warp; i < n; i += sq.ncta * (NT / 32)) {
+        const float *row = sq.G + (size_t)i * np;
+        float m = 0.f;
+#pragma unroll 4
+        for (int j = (i & ~127) + lane * 4; j < n; j += 128) {
+            const float4 g = __ldcg((const float4 *)(row + j)), r = *(const float4 *)(rs + j);
+            m = fmaxf(m, fmaxf(j > i ? fabsf(g.x) * r.x : 0.f, j + 1 > i ? fabsf(g.y) * r.y : 0.f));
+            m = fmaxf(m, fmaxf(j + 2 > i ? fabsf(g.z) * r.z : 0.f, j + 3 > i ? fabsf(g.w) * r.w : 0.f));
+        }
+        mo = fmaxf(mo, m * rs[i]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mo = fmaxf(mo, __shfl_xor_sync(0xffffffffu, mo, o));
+    if (lane == 0) part[warp] = mo;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) mo = fmaxf(mo, part[w]);
+    return mo;
+}
+
 template <bool TENSOR>
 __global__ void __launch_bounds__(NT, 2)
-jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, float tol_rot, int max_sweeps,
+jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, float tol_left, float tol_rot, int max_sweeps,
                          int raise_not_converged, int *status)
 {
     extern __shared__ __align__(16) float j3sm[];
@@ -902,7 +934,7 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
 
     int sweep = 0;
     for (; sweep < max_sweeps && alive; ++sweep) {
-        if (rank == 0 && tid == 0) sq.sync[1 + (sweep + 2) % 4] = 0u;      // slot of sweep + 2, last read two sweeps ago
+        if (rank == 0 && tid == 0) sq.sync[1 + (sweep + 2) % 4] = sq.sync[8 + (sweep + 2) % 4] = 0u;   // slots of sweep + 2, last read two sweeps ago
         for (int step = 0; step < nsteps && alive; ++step, ++gstep) {
             const int par = (int)(gstep & 1u);
             const bool has_next = !(sweep == max_sweeps - 1 && step == nsteps - 1);
@@ -955,6 +987,13 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
         if (!alive) break;
         const float mo = __uint_as_float(*(volatile unsigned *)(sq.sync + 1 + sweep % 4));
         if (mo <= tol_conv) { converged = true; ++sweep; break; }
+        // The largest scaled off-diagonal entry of the matrix as the sweep has left it: a few microseconds, against a whole
+        // sweep (65 steps at n = 2112) to find the same by visiting every pair again.
+        const float left = matrix_max(j3sm, sq, rank);
+        if (tid == 0) atomicMax(sq.sync + 8 + sweep % 4, __float_as_uint(left));
+        alive = group_barrier(sq.sync, ++gen, (unsigned)sq.ncta, abort_flag);
+        if (!alive) break;
+        if (__uint_as_float(*(volatile unsigned *)(sq.sync + 8 + sweep % 4)) <= tol_left) { converged = true; ++sweep; break; }
     }
     if (rank == 0 && tid == 0) {
         if (!alive) raise_status(status, ATP_ERR_TIMEOUT);
@@ -986,7 +1025,7 @@ __global__ void init_kernel(const __grid_constant__ Batch batch, int *status)
 // CTA per block of the update, at least one) and launches the kernel cooperatively, so that all
 // groups are resident together and the group barriers cannot starve.
 template <bool TENSOR>
-static inline atp_status launch(atp_ctx *ctx, Batch &jb, float tol_conv, float tol_rot, int max_sweeps, bool raise_not_converged)
+static inline atp_status launch(atp_ctx *ctx, Batch &jb, float tol_conv, float tol_left, float tol_rot, int max_sweeps, bool raise_not_converged)
 {
     if (jb.count <= 0) return ATP_OK;
     static std::mutex mu;
@@ -1024,7 +1063,7 @@ static inline atp_status launch(atp_ctx *ctx, Batch &jb, float tol_conv, float t
     ATP_LAUNCHED(ctx);
     int *status = ctx->dev_status;
     int ms = max_sweeps, rn = raise_not_converged ? 1 : 0;
-    void *args[] = {(void *)&jb, (void *)&tol_conv, (void *)&tol_rot, (void *)&ms, (void *)&rn, (void *)&status};
+    void *args[] = {(void *)&jb, (void *)&tol_conv, (void *)&tol_left, (void *)&tol_rot, (void *)&ms, (void *)&rn, (void *)&status};
     // bytes: one read and one write of G and Wt (what the kernel must move at least; it runs from L2)
     ATP_KERNEL(ctx, "jacobi_persistent", 0, wsum * 16.0);
     ATP_CUDA_OK(ctx, cudaLaunchCooperativeKernel((const void *)jacobi_persistent_kernel<TENSOR>, dim3(next), dim3(NT), args, SMEM_BYTES, ctx->stream));

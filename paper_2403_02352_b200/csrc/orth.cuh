@@ -13,19 +13,22 @@
 // pass; see the panel program in the kernel.
 // Two repetitions give orthonormality to working precision (the second also repairs the explicit inverse,
 // which is only norm-wise stable). Each sequence owns a group of CTAs; the phases of a panel are separated by
-// the group's barrier (bounded spin, see jacobi3.cuh) instead of kernel boundaries, and every phase is a list
-// of independent 64 x 64 tile jobs dealt out round-robin. The 64^3 tile products run on the tensor cores in
-// split TF32 precision (three products, ~2^-21): plain TF32 is not enough even for the first repetition, because
-// what a projection leaves of an ill-conditioned panel is far below 2^-11 of the panel. fp32 inputs keep every
-// product on the fp32 units.
+// the group's barrier (bounded spin) instead of kernel boundaries, and every phase is a list
+// of independent 64 x 64 tile jobs dealt out round-robin. The tile products of the projections (most of the arithmetic) run on
+// the tensor cores from two fp16 parts per operand (split_mma.cuh), columns of the panel scaled by powers of two to a
+// common range; the products with the factor, whose rows differ by the ratio of the column norms, from two TF32 parts. Plain
+// TF32 is not enough even for the first repetition, because what a projection leaves of an ill-conditioned panel is far
+// below 2^-11 of the panel. fp32 inputs keep every product on the fp32 units.
 #pragma once
 #include "jacobi3.cuh"
 #include "panel_chol.cuh"
+#include "split_mma.cuh"
 
 namespace orth {
 
 using j3::BLK; using j3::NT; using j3::LDA; using j3::LDB;
 constexpr int MAXSEQ = 32;
+constexpr int SYNC_WORDS = 192;   // words of Seq::sync before the SM list
 constexpr int NRED = 8;           // second-level partial Gram sums (chunk ranges)
 
 struct Seq {
@@ -34,8 +37,9 @@ struct Seq {
     float *Cpart, *C, *Dpart, *W;             // tile scratch (see scratch_tiles)
     double *gpart, *gpart2;
     int *flags;
-    unsigned *sync;                           // 64 words: group barrier (jacobi3.cuh); then one word per CTA of the
-                                              // group (its SM)
+    unsigned *sync;                           // 64 words: group barrier; 2 x 64 words: largest entry of each column of the
+                                              // panel (as bits), before the first and before the second projection; then
+                                              // one word per CTA of the group (its SM)
     int cta0, ncta, index;                    // CTA group (on entry to launch(): ncta = the cap the scratch was
                                               // sized for); index of the sequence in its batch (noise stream)
 };
@@ -169,21 +173,67 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
     // rank 0's factorisation, which is a latency chain and slows down under a busy neighbour.
     unsigned smid;
     asm("mov.u32 %0, %%smid;" : "=r"(smid));
-    if (tid == 0) sq.sync[64 + rank] = smid;
+    if (tid == 0) sq.sync[SYNC_WORDS + rank] = smid;
+    // Largest entry of each column of panel pj over the row tiles first, first + stride, ... (bits of non-negative floats
+    // order like integers)
+    auto column_max = [&](int pj, int first, int stride) {
+        const int j0 = pj * 64, w = min(64, rt - j0), c = tid & 63;
+        float m = 0.f;
+        if (c < w)
+            for (int t = first; t < ntile; t += stride) {
+                const int r0 = t * 64 + (tid >> 6), r1 = min(n, (t + 1) * 64);
+#pragma unroll 8
+                for (int r = r0; r < r1; r += 4) m = fmaxf(m, fabsf(__ldcg(sq.M + (size_t)r * ld + j0 + c)));
+            }
+        if (m > 0.f) atomicMax(sq.sync + 64 + c, __float_as_uint(m));
+    };
+    if (TENSOR) column_max(0, rank, ncta);
     barrier();
     __shared__ int mate_s;
     if (tid == 0) mate_s = 1 << 30;
     __syncthreads();
     if (alive) {
-        const unsigned sm0 = __ldcg(sq.sync + 64);
+        const unsigned sm0 = __ldcg(sq.sync + SYNC_WORDS);
         for (int r = 1 + tid; r < ncta; r += NT)
-            if (__ldcg(sq.sync + 64 + r) == sm0) atomicMin(&mate_s, r);
+            if (__ldcg(sq.sync + SYNC_WORDS + r) == sm0) atomicMin(&mate_s, r);
     }
     __syncthreads();
     const int mate = mate_s < ncta ? mate_s : -1;
     const bool overlap = reps == 2 && ncta >= 4;
     const int nworkers = ncta - 1 - (mate > 0 ? 1 : 0);
     const int wid = (rank == 0 || rank == mate) ? -1 : rank - 1 - ((mate > 0 && rank > mate) ? 1 : 0);
+
+    // Scales of the panel's columns for the fp16 parts: entries of P, and of C = Q^T P, are below the column norm, i.e. below
+    // sqrt(n) times the largest entry of the column; after a first apply the columns have unit norm.
+    __shared__ __align__(16) float colscale[64], colinv[64];   // (read in 16-byte pieces)
+    int half_log_n = 0;
+    while ((1ll << (2 * half_log_n)) < n) ++half_log_n;
+    constexpr float QSCALE = 16384.f;                         // entries of the finished columns: at most 1
+    auto set_scales = [&](int slot) {                         // slot < 0: unit columns
+        if (TENSOR && tid < 64) {
+            const float2 sc = slot < 0 ? make_float2(8192.f, 1.f / 8192.f) : hs::scale_for(__ldcg(sq.sync + 64 + 64 * slot + tid), 15 - half_log_n);
+            colscale[tid] = sc.x;
+            colinv[tid] = sc.y * (1.f / QSCALE);
+        }
+        __syncthreads();
+    };
+    __half *hA = (__half *)osm, *hB = hA + 2 * hs::PLANE;      // the same shared memory as sA, sB
+    auto put_tile = [&](const TileRegs &tr, __half *dst, float4 sc) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int f = tid + i * NT;
+            const float4 v = tr.v[i];
+            hs::put4(dst, f >> 4, (f & 15) * 4, make_float4(v.x * sc.x, v.y * sc.y, v.z * sc.z, v.w * sc.w));
+        }
+    };
+    const float4 qs4 = make_float4(QSCALE, QSCALE, QSCALE, QSCALE);
+    auto unscale = [&](float (&acc)[4][4]) {
+        const int t2 = (tid & 3) * 2;
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[nt][e] *= colinv[n0 + nt * 8 + t2 + (e & 1)];
+    };
 
     // A panel is a short program of four kinds of passes, each written once below:
     //   PF      project (partial C over row ranges, jobs first, first + stride, ...) and / or, on rank 0, the factor
@@ -207,6 +257,8 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
         while (stage >= 0 && alive) {
             int op = OP_PF, first = -1, stride = 1, arep = 0;
             bool do_factor = false, series_ok = false, with_w = false, last = false, skip = false;
+            // which scales a projection uses: 0 the panel as it came, 1 after the first projection, -1 unit columns
+            const int scale_slot = stage <= 1 ? 0 : stage <= 4 ? 1 : stage < 30 ? -1 : rep == 0 ? 0 : -1;
             switch (stage) {
                 // overlapped order
                 case 0: op = OP_PF; first = rank; stride = ncta; skip = nj == 0; break;
@@ -233,6 +285,9 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             }
             if (!skip) switch (op) {
             case OP_PF: {
+                // beside the last factor of a panel the other CTAs note the column maxima of the next panel
+                const bool scan = TENSOR && do_factor && stage != 3 && (stage != 33 || rep == reps - 1) && pj + 1 < npanel;
+                if (scan && (rank > 0 || ncta == 1)) column_max(pj + 1, max(rank - 1, 0), max(ncta - 1, 1));
                 if (do_factor && rank == 0) {
                     {   // all elements of a partial matrix in flight together
                         double2 g[8];
@@ -256,6 +311,8 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                     if (!(series_ok && lowdin_64(Gs, w, sA, sq.W, sq.flags))) chol_invert_64(Gs, (double *)osm, w, sq.W, sq.flags);
                     __syncthreads();
                 } else if (first >= 0) {
+                    set_scales(scale_slot);
+                    const float4 ps4 = *(const float4 *)&colscale[(tid & 15) * 4];
                     for (int it = first; it < nj * KS; it += stride) {
                         const int jb = it / KS, ks = it - jb * KS;
                         float acc[4][4] = {};
@@ -266,17 +323,19 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                             fetch_tile(rb, sq.M + (size_t)t0 * 64 * ld + j0, ld, min(64, n - t0 * 64), w, vec);
                         }
                         for (int t = t0; t < t1; ++t) {
-                            stash_tile(ra, sA, LDB);
-                            stash_tile(rb, sB, LDB);
+                            if (TENSOR) { put_tile(ra, hA, qs4); put_tile(rb, hB, ps4); }
+                            else { stash_tile(ra, sA, LDB); stash_tile(rb, sB, LDB); }
                             __syncthreads();
                             if (t + 1 < t1) {                               // next tiles in flight during the product
                                 const int rv = min(64, n - (t + 1) * 64);
                                 fetch_tile(ra, sq.M + (size_t)(t + 1) * 64 * ld + jb * 64, ld, rv, 64, vec);
                                 fetch_tile(rb, sq.M + (size_t)(t + 1) * 64 * ld + j0, ld, rv, w, vec);
                             }
-                            tile_mac<P_FINE, true>(sA, LDB, sB, LDB, m0, n0, acc);
+                            if (TENSOR) hs::product64<true, false>(hA, hB, m0, n0, acc);
+                            else tile_mac<0, true>(sA, LDB, sB, LDB, m0, n0, acc);
                             __syncthreads();
                         }
+                        if (TENSOR) unscale(acc);
                         store_acc(sq.Cpart + (size_t)it * 4096, 64, m0, n0, acc);
                     }
                 }
@@ -298,6 +357,8 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                 }
                 barrier();
                 if (!alive) break;
+                set_scales(scale_slot);
+                const float4 ps4 = *(const float4 *)&colscale[(tid & 15) * 4];
                 for (int it = rank; it < ntile * G; it += ncta) {
                     const int t = it / G, g = it - t * G;
                     const int rv = min(64, n - t * 64);
@@ -309,21 +370,28 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                         fetch_tile(rb, sq.C + (size_t)jb0 * 4096, 64, 64, 64, true);
                     }
                     for (int jb = jb0; jb < jb1; ++jb) {
-                        stash_tile(ra, sA, LDA);
-                        stash_tile(rb, sB, LDB);
+                        if (TENSOR) { put_tile(ra, hA, qs4); put_tile(rb, hB, ps4); }
+                        else { stash_tile(ra, sA, LDA); stash_tile(rb, sB, LDB); }
                         __syncthreads();
                         if (jb + 1 < jb1) {
                             fetch_tile(ra, sq.M + (size_t)t * 64 * ld + (jb + 1) * 64, ld, rv, 64, vec);
                             fetch_tile(rb, sq.C + (size_t)(jb + 1) * 4096, 64, 64, 64, true);
                         }
-                        tile_mac<P_FINE, false>(sA, LDA, sB, LDB, m0, n0, acc);
+                        if (TENSOR) hs::product64<false, false>(hA, hB, m0, n0, acc);
+                        else tile_mac<0, false>(sA, LDA, sB, LDB, m0, n0, acc);
                         __syncthreads();
                     }
+                    if (TENSOR) unscale(acc);
                     store_acc(sq.Dpart + (size_t)it * 4096, 64, m0, n0, acc);
                 }
                 barrier();
             } break;
             case OP_GRAM: {
+                // the columns' largest entries go to slot 1 before a second projection of the same panel; otherwise slot 0 has
+                // been used and is cleared for the next panel (noted beside the factor that follows)
+                const bool note_max = TENSOR && stage == 2;
+                float cmax = 0.f;
+                if (TENSOR && !note_max && rank == 0 && tid < 64) sq.sync[64 + tid] = 0u;
                 for (int t = rank; t < ntile; t += ncta) {
                     const int rv = min(64, n - t * 64);
                     load_tile(sA, LDA, sq.M + (size_t)t * 64 * ld + j0, ld, rv, w, vec);
@@ -345,6 +413,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                                 const int e = e0 + q * NT, r = e >> 6, c = e & 63;
                                 const float v = sA[r * LDA + c] - sacc[q];
                                 sA[r * LDA + c] = (r < rv && c < w) ? v : 0.f;
+                                if (r < rv && c < w) cmax = fmaxf(cmax, fabsf(v));
                                 if (!with_w && r < rv && c < w) sq.M[((size_t)t * 64 + r) * ld + j0 + c] = v;
                             }
                         }
@@ -369,6 +438,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                     gram_tile_64(sA, LDA, Gs, sq.gpart + (size_t)t * 4096);
                     __syncthreads();
                 }
+                if (note_max && cmax > 0.f) atomicMax(sq.sync + 128 + (tid & 63), __float_as_uint(cmax));
                 barrier();
                 if (!alive) break;
                 // ordered sum of the partial Gram matrices: 16 element slices x (up to 8) chunk ranges
@@ -382,6 +452,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             default: {                                                   // OP_APPLY
                 const uint64_t nseed = seed + 7919ull * (uint64_t)(pj * 2 + arep);
                 const float rscale = rsqrtf((float)n * (1.f / 3.f));     // replacement columns of about unit norm
+                if (TENSOR && rank == 0 && tid < 64) sq.sync[128 + tid] = 0u;
                 int fl[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) fl[k] = __ldcg(sq.flags + (tid & 15) * 4 + k);
@@ -440,7 +511,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
 __global__ void init_kernel(const __grid_constant__ Batch batch)
 {
     const Seq &sq = batch.s[blockIdx.x];
-    if (threadIdx.x < 64 && sq.n > 0) sq.sync[threadIdx.x] = 0u;
+    if ((int)threadIdx.x < SYNC_WORDS && sq.n > 0) sq.sync[threadIdx.x] = 0u;
 }
 
 constexpr size_t SMEM_BYTES = (size_t)(2 * BLK * LDB) * sizeof(float);
@@ -474,7 +545,7 @@ static inline atp_status launch(atp_ctx *ctx, Batch &ob, int reps, uint64_t seed
     }
     if (next > total) return ATP_ERR_INVALID_ARG;      // cannot happen: shares sum to at most `total`
     ATP_KERNEL(ctx, "orth_init", 0, 0);
-    init_kernel<<<ob.count, 64, 0, ctx->stream>>>(ob);
+    init_kernel<<<ob.count, 256, 0, ctx->stream>>>(ob);
     ATP_LAUNCHED(ctx);
     int *status = ctx->dev_status;
     void *args[] = {(void *)&ob, (void *)&reps, (void *)&seed, (void *)&status};
