@@ -565,6 +565,7 @@ static void plan_basis(Arena &ar, const std::vector<SeqDims> &sd, int d, int ove
         bp.seqs.push_back(p);
     }
     bp.omega = ar.take<float>((size_t)d * bp.rtmax);
+    bp.part = ar.take<float>((size_t)splitk_floats(sm_count));
     bp.omega_b = ar.take<__nv_bfloat16>((size_t)d * align_up((size_t)bp.rtmax, 8));
     for (auto &p : bp.seqs) {
         int L = p.dims.L, rt = p.rt;
@@ -664,6 +665,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
     // occupancy, sets the time, and the launch count doubles), so it is off by default.
     const size_t nseq = bp.seqs.size();
     const bool forked = groups == 2 && nseq >= 2 && ctx->aux[0] && ctx->aux[1] && !ctx->profiling;
+    float *kpart = forked ? nullptr : bp.part;      // one scratch for split products: not shared by two streams
     const size_t gsz = forked ? std::min<size_t>(BMAX, (nseq + 1) / 2) : BMAX;
     // reading the convergence flags back lets the host stop enqueueing sweeps; without it (forked streams, or on
     // request: stream capture, callers that must never block) the whole sweep budget is enqueued and the kernels
@@ -723,7 +725,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 SeqPlan &p = bp.seqs[i];
                 g.p[i - i0] = GemmProblem{Xb(p), bp.omega, p.Y, nullptr, p.dims.L, p.rt, d, (int)X->ld, bp.rtmax, p.rt, 0};
             }
-            if ((st = launch_gemm_simt<T, float, float, false>(ctx, g, store)) != ATP_OK) return st;
+            if ((st = launch_gemm_simt<T, float, float, false>(ctx, g, store, 0, kpart, splitk_floats(ctx->sm_count))) != ATP_OK) return st;
             if ((st = orthonormalise<std::is_same<T, __nv_bfloat16>::value>(ctx, bp, i0, i1, seed, 2)) != ATP_OK) return st;
             for (int it = 0; it < power_iters; ++it) {
                 // Z = X^T Y ; Y = X Z ; orth(Y).  Z is not orthonormalised: Y has orthonormal, QR-ordered
@@ -733,12 +735,12 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                     SeqPlan &p = bp.seqs[i];
                     g.p[i - i0] = GemmProblem{Xb(p), p.Y, p.Z, nullptr, p.rt > 0 ? d : 0, p.rt, p.dims.L, (int)X->ld, p.rt, p.rt, 0};
                 }
-                if ((st = launch_gemm_simt<T, float, float, true>(ctx, g, store)) != ATP_OK) return st;
+                if ((st = launch_gemm_simt<T, float, float, true>(ctx, g, store, 0, kpart, splitk_floats(ctx->sm_count))) != ATP_OK) return st;
                 for (size_t i = i0; i < i1; ++i) {
                     SeqPlan &p = bp.seqs[i];
                     g.p[i - i0] = GemmProblem{Xb(p), p.Z, p.Y, nullptr, p.dims.L, p.rt, d, (int)X->ld, p.rt, p.rt, 0};
                 }
-                if ((st = launch_gemm_simt<T, float, float, false>(ctx, g, store)) != ATP_OK) return st;
+                if ((st = launch_gemm_simt<T, float, float, false>(ctx, g, store, 0, kpart, splitk_floats(ctx->sm_count))) != ATP_OK) return st;
                 if ((st = orthonormalise<std::is_same<T, __nv_bfloat16>::value>(ctx, bp, i0, i1, seed + 2000003ull * (it + 1), 2)) != ATP_OK) return st;
             }
         }
@@ -837,7 +839,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 }
                 if ((st = tc::launch<true, 2, tc::OUT_BF16_SPLIT>(ctx, hp, store)) != ATP_OK) return st;
             } else {
-                if ((st = launch_gemm_simt<T, float, float, true>(ctx, g, store)) != ATP_OK) return st;
+                if ((st = launch_gemm_simt<T, float, float, true>(ctx, g, store, 0, kpart, splitk_floats(ctx->sm_count))) != ATP_OK) return st;
             }
             // Two passes. G squares the condition number of B, so when sigma_1 / sigma_r~ exceeds ~10^3
             // the first diagonalisation resolves the weak components only roughly. Its rotation W1 is
@@ -846,7 +848,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
             // and a short second pass on it finishes the job (a one-sided Jacobi in two strokes).
             // Each pass is one persistent kernel that stops on its own convergence test: nothing is
             // read back by the host.
-            constexpr float LEFT = 0.3f;
+            constexpr float LEFT = 0.5f;
             for (int pass = 0; pass < 2; ++pass) {
                 if constexpr (kBf16) {
                     hp.clear();
@@ -860,7 +862,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                     }
                     if ((st = tc::launch<true, 2, tc::OUT_F32, false, true>(ctx, hp, store, "gemm_tc_gram")) != ATP_OK) return st;
                 } else {
-                    if ((st = launch_gemm_simt<float, float, float, true, false>(ctx, gg, store, 1, nullptr, 0, "gemm_simt_gram")) != ATP_OK) return st;
+                    if ((st = launch_gemm_simt<float, float, float, true, false>(ctx, gg, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_gram")) != ATP_OK) return st;
                 }
                 // pass 0 only has to make the rows graded and roughly orthogonal (scaled off-diagonals below
                 // 1e-2; on ill-conditioned input it stalls at the noise floor of G, hence the cap of 8 sweeps);
@@ -871,7 +873,8 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 // fp32 inputs: the block products stay on the fp32 units (the threshold is below split-precision rounding)
                 // A sweep whose visits all stayed below tolc ends the pass, and so does a matrix that a sweep leaves below
                 // tolc (first pass) or LEFT * tolc (second: a sweep that ends by its visits still rotates what exceeds
-                // 0.1 * tolc on the way, so what it leaves is further down)
+                // 0.1 * tolc on the way, so what it leaves is further down). 0.5: storing X_r in bf16 alone leaves about 2e-4
+                // (1.0 measured 127 ms instead of 129 on the 4096-token layer, but shows in X_r X_r^T)
                 if ((st = j3::launch<kBf16>(ctx, jb, tolc, pass == 0 ? tolc : LEFT * tolc, tolc * 0.1f, nsw, pass == 1)) != ATP_OK) return st;
                 if (pass == 0) {
                     // Bt2 = Bt Wt^T (d x r~),  Y2 = Y Wt^T (L x r~);  Wt rows are the eigenvectors
@@ -910,8 +913,8 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                             gg.p[k].A = p.Z; gg.p[k].B = p.Z;
                             fb.s[k].Y = p.Y2;
                         }
-                        if ((st = launch_gemm_simt<float, float, float, false, true>(ctx, r1, store, 1, nullptr, 0, "gemm_simt_rot")) != ATP_OK) return st;
-                        if ((st = launch_gemm_simt<float, float, float, false, true>(ctx, r2, store, 1, nullptr, 0, "gemm_simt_rot")) != ATP_OK) return st;
+                        if ((st = launch_gemm_simt<float, float, float, false, true>(ctx, r1, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_rot")) != ATP_OK) return st;
+                        if ((st = launch_gemm_simt<float, float, float, false, true>(ctx, r2, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_rot")) != ATP_OK) return st;
                     }
                 }
             }
@@ -951,8 +954,8 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                     gg.p[k] = GemmProblem{p.Y2, p.Wsel, (T *)U_r->data + (size_t)p.dims.row0 * U_r->ld, nullptr,
                                           p.dims.L, p.dims.r, p.rt, p.rt, p.dims.r, (int)U_r->ld, 0};
                 }
-                if ((st = launch_gemm_simt<float, float, T, true, true>(ctx, g, store, 1, nullptr, 0, "gemm_simt_out")) != ATP_OK) return st;
-                if ((st = launch_gemm_simt<float, float, T, false>(ctx, gg, store, 1, nullptr, 0, "gemm_simt_out")) != ATP_OK) return st;
+                if ((st = launch_gemm_simt<float, float, T, true, true>(ctx, g, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_out")) != ATP_OK) return st;
+                if ((st = launch_gemm_simt<float, float, T, false>(ctx, gg, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_out")) != ATP_OK) return st;
             }
             ATP_KERNEL(ctx, "signfix", 0, 0);
             signfix_kernel<T><<<dim3(maxr, cnt), 256, 0, ctx->stream>>>(fb);
