@@ -592,7 +592,7 @@ static void plan_basis(Arena &ar, const std::vector<SeqDims> &sd, int d, int ove
         p.np = jacobi_padded(rt);
         p.G = ar.take<float>((size_t)p.np * p.np);
         p.Wt = ar.take<float>((size_t)p.np * p.np);
-        p.Vbuf = ar.take<float>((size_t)2 * (p.np / 64 + 1) * 4096);
+        p.Vbuf = ar.take<float>((size_t)2 * (p.np / 64 + 1) * j3::VSTRIDE);
         p.vflag = ar.take<int>(2 * (p.np / 64) + 4);
         p.tpart = ar.take<float>((size_t)COLSUM_SLABS * std::max(rt, 1));
         {   // bf16 hi/lo operands of the tensor-core products around the rotation (bf16 inputs only)

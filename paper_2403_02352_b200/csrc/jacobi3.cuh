@@ -15,14 +15,14 @@
 //   apply : every 64 x 64 block (p, q) of G becomes Vt_p G_pq Vt_q^T (upper triangle computed, mirror
 //           stored), rows of Wt become Vt_p Wt, both in place. The pivot CTAs of the step read blocks of G as they
 //           were before the update; a counter of fetched pivot blocks holds the first store of every updating
-//           CTA back until they have them on chip. The 64^3 products run on the tensor cores in split
-//           precision (three TF32 mma products per fp32 product), which keeps fp32 accuracy; fp32 inputs use the
-//           fp32 units.
+//           CTA back until they have them on chip. The 64^3 products run on the tensor cores from two fp16 parts per operand
+//           (split_mma.cuh; see "published transforms" for the scaling); fp32 inputs use the fp32 units.
 // G and Wt are stored with a leading dimension padded to a multiple of 64; the padding of G is zero
 // (zero diagonal entries are never rotated), the padding of Wt is the identity.
 #pragma once
 #include "common.cuh"
 #include "group_barrier.cuh"
+#include "split_mma.cuh"
 #include <mutex>
 #include <algorithm>
 
@@ -34,9 +34,10 @@ constexpr int NT = 256;           // threads per CTA
 constexpr int LDA = 68;           // shared-memory row stride (floats) of A-operand style tiles
 constexpr int LDB = 72;           // shared-memory row stride of B-operand style tiles
 constexpr int MAXSEQ = 32;        // sequences per launch
+constexpr int VSTRIDE = 2 * BLK * BLK + 2 * BLK;   // floats of a published transform (see below)
 
 struct Seq {
-    float *G, *Wt, *Vbuf;         // G, Wt: np x np (ld = np); Vbuf: 2 x npairs x 64 x 64 (by step parity)
+    float *G, *Wt, *Vbuf;         // G, Wt: np x np (ld = np); Vbuf: 2 x npairs x VSTRIDE (by step parity)
     int *vflag;                   // 2 x npairs: the pair rotated in this step
     unsigned *sync;               // 64 words. [0]: arrivals at the group barrier (monotonic); [32]: last
                                   // barrier completed; [1..4]: largest scaled off-diagonal entry of a
@@ -97,6 +98,7 @@ struct PivotShared {
     float dn[2][3][32];           // oe of the first offset of warp w + 1, for warp w
     float sd[2][64];              // row factors d at the end of a phase (even slots, odd slots), by phase parity
     float red[4];
+    float d[64];                  // powers of two above the square roots of the diagonal
 };
 
 __device__ __forceinline__ float rsqrt_ftz(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
@@ -292,7 +294,7 @@ template <int M> __device__ __forceinline__ void inner_phase(float *As, PivotSha
     }
 }
 
-// The transform's share of a phase (warps 4..7): lane = columns l and l + 32, warp 4 + h = the rows of the pairs
+// The transform's share of a phase (warps 4..7): lane = columns 2 l and 2 l + 1, warp 4 + h = the rows of the pairs
 // 8 h .. 8 h + 7. Widths 32 and 16: ve / vo = even and odd rows in slot order; the odd row that leaves the quarter goes to
 // the next quarter of its group through shared memory. Widths <= 8: the 16 rows 16 h .. 16 h + 15 in v.
 __device__ __forceinline__ void rotate_rows(float b, float g, float2 &x, float2 &y)
@@ -394,6 +396,19 @@ template <int W> __device__ __forceinline__ float pivot_warp(float *As, PivotSha
     }
     return mo;
 }
+// Published transforms. fp32 inputs: Vt as 64 x 64 floats. Otherwise, for products from fp16 parts, with powers of two
+//     d_i >= sqrt(g_ii)  per row of the pivot block before the rotation,     s_i > max_k |vt_ik| d_k  per row of Vt:
+//   VS  = diag(1/s) Vt diag(d)  (entries below 1), 64 x 64 fp16 high parts, then the low parts, times V_SCALE: rotates G,
+//         whose blocks diag(1/d_p) G_pq diag(1/d_q) have entries of at most 1 however the rows are graded; the result is scaled
+//         back by s_p, s_q. What is left out is below 2^-35 s_i s_j, on top of 2^-22 of the entries themselves.
+//   VU  = Vt times V_SCALE in the same form: rotates the rows of Wt, whose entries are at most 1.
+//   d, s as 64 floats each (s = d where the pair was not rotated).
+constexpr float V_SCALE = 8192.f, G_SCALE = 1024.f, T_SCALE = 256.f;
+constexpr int V_VU = BLK * BLK, V_D = 2 * BLK * BLK, V_S = V_D + BLK;     // offsets in floats
+constexpr int LDV = 66;           // row stride of the transform in shared memory
+__device__ __forceinline__ float inv_pow2(float x) { return __uint_as_float(0x7f000000u - __float_as_uint(x)); }
+
+template <bool TENSOR>
 __device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *vout, bool &rotated)
 {
     __shared__ __align__(16) PivotShared sh;
@@ -401,6 +416,15 @@ __device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *
     float *As = sm, *Vs = sm + BLK * LDP;
     float mo;
     __syncthreads();
+    if (TENSOR && tid < BLK) {
+        // g < 2^(E - 126): d = 2^ceil((E - 126) / 2)
+        const float g = As[tid * (LDP + 1)];
+        const int e = g > 0.f ? min(max(((int)(__float_as_uint(g) >> 23) - 125) >> 1, -60), 63) : -60;
+        const float d = __int_as_float((127 + e) << 23);
+        sh.d[tid] = d;
+        vout[V_D + tid] = d;
+        vout[V_S + tid] = d;                                     // (overwritten below where rows are rotated)
+    }
     if (warp == 0) mo = pivot_warp<0>(As, sh, cross_only, tol_rot);
     else if (warp == 1) mo = pivot_warp<1>(As, sh, cross_only, tol_rot);
     else if (warp == 2) mo = pivot_warp<2>(As, sh, cross_only, tol_rot);
@@ -414,23 +438,39 @@ __device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int e = 8 * h + i, o = 32 + e;
-                ve[i] = make_float2(e == l ? 1.f : 0.f, e == l + 32 ? 1.f : 0.f);
-                vo[i] = make_float2(o == l ? 1.f : 0.f, o == l + 32 ? 1.f : 0.f);
+                ve[i] = make_float2(e == 2 * l ? 1.f : 0.f, e == 2 * l + 1 ? 1.f : 0.f);
+                vo[i] = make_float2(o == 2 * l ? 1.f : 0.f, o == 2 * l + 1 ? 1.f : 0.f);
             }
             transform_wide(ve, vo, sh, 32, h, (h - 1) & 3);
             __syncthreads();
             vo[0] = sh.vx[1][(h - 1) & 3][l];
 #pragma unroll
             for (int i = 0; i < 8; ++i) { scale_row(ve[i], sh.sd[0][8 * h + i]); scale_row(vo[i], sh.sd[0][32 + 8 * h + i]); }
-            auto put = [&](float *dst, int ld, int row, float2 v) { dst[row * ld + l] = v.x; dst[row * ld + l + 32] = v.y; };
-            auto get = [&](int row) { return make_float2(Vs[row * LDP + l], Vs[row * LDP + l + 32]); };
+            auto put = [&](int row, float2 v) { *(float2 *)(Vs + row * LDV + 2 * l) = v; };
+            auto get = [&](int row) { return *(const float2 *)(Vs + row * LDV + 2 * l); };
+            auto publish = [&](int row, float2 v) {
+                if (!TENSOR) { *(float2 *)(vout + row * BLK + 2 * l) = v; return; }
+                auto parts = [&](float *dst, float x, float y) {
+                    const __half2 hi = __floats2half2_rn(x, y);
+                    const float2 f = __half22float2(hi);
+                    ((__half2 *)dst)[row * 32 + l] = hi;
+                    ((__half2 *)dst)[2048 + row * 32 + l] = __floats2half2_rn(x - f.x, y - f.y);
+                };
+                parts(vout + V_VU, v.x * V_SCALE, v.y * V_SCALE);
+                const float x = v.x * sh.d[2 * l], y = v.y * sh.d[2 * l + 1];
+                const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fabsf(x), fabsf(y))));
+                const int e = min(max((int)(m >> 23), 20), 250);                  // largest entry < 2^(e - 126)
+                const float is = __int_as_float((266 - e) << 23);                 // V_SCALE * 2^(126 - e)
+                parts(vout, x * is, y * is);
+                if (l == 0) vout[V_S + row] = __int_as_float((e + 1) << 23);
+            };
             auto vbar = [] { asm volatile("bar.sync 1, 128;" ::: "memory"); };          // the warps of the transform
             if (cross_only) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) { put(vout, BLK, 8 * h + i, ve[i]); put(vout, BLK, 32 + 8 * h + i, vo[i]); }
+                for (int i = 0; i < 8; ++i) { publish(8 * h + i, ve[i]); publish(32 + 8 * h + i, vo[i]); }
             } else {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) { put(Vs, LDP, 8 * h + i, ve[i]); put(Vs, LDP, 32 + 8 * h + i, vo[i]); }
+                for (int i = 0; i < 8; ++i) { put(8 * h + i, ve[i]); put(32 + 8 * h + i, vo[i]); }
                 vbar();
                 const int e16 = 32 * (h >> 1) + 8 * (h & 1);     // width 16: even rows e16 + i, odd rows 16 further on
 #pragma unroll
@@ -442,7 +482,7 @@ __device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *
 #pragma unroll
                 for (int i = 0; i < 8; ++i) { scale_row(ve[i], sh.sd[1][8 * h + i]); scale_row(vo[i], sh.sd[1][32 + 8 * h + i]); }
 #pragma unroll
-                for (int i = 0; i < 8; ++i) { put(Vs, LDP, e16 + i, ve[i]); put(Vs, LDP, e16 + 16 + i, vo[i]); }
+                for (int i = 0; i < 8; ++i) { put(e16 + i, ve[i]); put(e16 + 16 + i, vo[i]); }
                 vbar();
                 float2 v[16];
 #pragma unroll
@@ -450,7 +490,7 @@ __device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *
                 transform_inner<8>(v, sh, h, 0); transform_inner<4>(v, sh, h, 1); transform_inner<2>(v, sh, h, 0);
                 transform_inner<1>(v, sh, h, 1);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) put(vout, BLK, 16 * h + i, v[i]);
+                for (int i = 0; i < 16; ++i) publish(16 * h + i, v[i]);
             }
         }
     }
@@ -474,46 +514,10 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// acc (this warp's 16 x 32 part of a 64 x 64 result, rows m0.., columns n0..) = As * Bop, K = 64, in
-// split precision: x = hi + lo with both parts in TF32, product = lo*hi + hi*lo + hi*hi (the lo*lo term
-// is below fp32 rounding). As[m][k] at stride LDA; Bop[k][n] = Bs[k * ldb + n], or Bs[n * ldb + k] when
-// B_TRANS. Strides LDA = 68 and LDB = 72 make every fragment load conflict-free.
-template <bool B_TRANS>
-__device__ __forceinline__ void product64(const float *As, const float *Bs, int ldb, int m0, int n0, float (&acc)[4][4])
-{
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[nt][i] = 0.f;
-#pragma unroll 2
-    for (int k0 = 0; k0 < BLK; k0 += 8) {
-        uint32_t ah[4], al[4];
-        split_tf32(As[(m0 + g) * LDA + k0 + t], ah[0], al[0]);
-        split_tf32(As[(m0 + g + 8) * LDA + k0 + t], ah[1], al[1]);
-        split_tf32(As[(m0 + g) * LDA + k0 + t + 4], ah[2], al[2]);
-        split_tf32(As[(m0 + g + 8) * LDA + k0 + t + 4], ah[3], al[3]);
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int n = n0 + nt * 8 + g;
-            uint32_t bh[2], bl[2];
-            if (B_TRANS) {
-                split_tf32(Bs[n * ldb + k0 + t], bh[0], bl[0]);
-                split_tf32(Bs[n * ldb + k0 + t + 4], bh[1], bl[1]);
-            } else {
-                split_tf32(Bs[(k0 + t) * ldb + n], bh[0], bl[0]);
-                split_tf32(Bs[(k0 + t + 4) * ldb + n], bh[1], bl[1]);
-            }
-            mma_tf32(acc[nt], al, bh);
-            mma_tf32(acc[nt], ah, bl);
-            mma_tf32(acc[nt], ah, bh);
-        }
-    }
-}
-
-// General form for other kernels: acc += op(A) * op(B) over K = 64, NPASS = 3 (split precision, as above) or
+// acc (this warp's 16 x 32 part of a 64 x 64 result, rows m0.., columns n0..) += op(A) * op(B), K = 64, NPASS = 3 (split
+// precision: x = hi + lo with both parts in TF32, product = lo*hi + hi*lo + hi*hi; the lo*lo term is below fp32 rounding) or
 // 1 (plain TF32, ~2^-11 relative per term). A_TRANS: A[m][k] = As[k * lda + m] (use stride LDB = 72);
-// otherwise As[m * lda + k] (stride LDA = 68). B as in product64.
+// otherwise As[m * lda + k] (stride LDA = 68). B[k][n] = Bs[k * ldb + n], or Bs[n * ldb + k] when B_TRANS.
 template <bool A_TRANS, bool B_TRANS, int NPASS>
 __device__ __forceinline__ void product64_acc(const float *As, int lda, const float *Bs, int ldb, int m0, int n0, float (&acc)[4][4])
 {
@@ -588,7 +592,6 @@ __device__ __forceinline__ void product64_fma(const float *As, const float *Bs, 
 //       [   (mirror)    W2 X22 W2^T ]
 // in three 64^3 products: [W1 X11; W2 X22] and W1 X12 first, then the multiplication by [W1; W2]^T from the
 // right. The result lands in As = sm (stride LDP). So the chain of pivot solves never waits for the update.
-template <bool TENSOR>
 __device__ void pivot_form(float *sm, const Seq &sq, const float *Gsrc, const float *Vcur, int step, int p1, int h1, int f1, int p2, int h2, int f2, unsigned *fetched)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -602,7 +605,7 @@ __device__ void pivot_form(float *sm, const Seq &sq, const float *Gsrc, const fl
         const bool up = i < JB;
         const int row = (up ? h1 : h2) * JB + (i & (JB - 1));
         float4 w;
-        if (up ? f1 : f2) w = __ldcg((const float4 *)(Vcur + (size_t)(up ? p1 : p2) * BLK * BLK + row * BLK + c));
+        if (up ? f1 : f2) w = __ldcg((const float4 *)(Vcur + (size_t)(up ? p1 : p2) * VSTRIDE + row * BLK + c));
         else w = make_float4(row == c ? 1.f : 0.f, row == c + 1 ? 1.f : 0.f, row == c + 2 ? 1.f : 0.f, row == c + 3 ? 1.f : 0.f);
         *(float4 *)(Wc + i * LDA + c) = w;
         const size_t r1 = (size_t)glob_of_loc(I1, J1, i) * np, r2 = (size_t)glob_of_loc(I2, J2, i) * np;
@@ -614,13 +617,10 @@ __device__ void pivot_form(float *sm, const Seq &sq, const float *Gsrc, const fl
     if (tid == 0) atomicAdd(fetched, 1u);                       // the old blocks are on chip: the update may overwrite them
     const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32;
     const bool up = m0 < JB;
-    const bool on_tensor = TENSOR;
     float accd[4][4], acco[4][4];
-    if (on_tensor) product64<false>(Wc, up ? S1 : S2, LDB, m0, n0, accd);
-    else product64_fma<false>(Wc, up ? S1 : S2, LDB, m0, n0, accd);
+    product64_fma<false>(Wc, up ? S1 : S2, LDB, m0, n0, accd);
     if (up) {
-        if (on_tensor) product64<false>(Wc, S3, LDB, m0, n0, acco);
-        else product64_fma<false>(Wc, S3, LDB, m0, n0, acco);
+        product64_fma<false>(Wc, S3, LDB, m0, n0, acco);
     }
     __syncthreads();
 #pragma unroll
@@ -637,8 +637,7 @@ __device__ void pivot_form(float *sm, const Seq &sq, const float *Gsrc, const fl
     const bool lower_left = !up && n0 == 0;                     // mirror of the upper right part
     if (!lower_left) {
         const float *Ta = (up && n0 != 0) ? S2 : S1;
-        if (on_tensor) product64<true>(Ta, Wc, LDA, m0, n0, accd);
-        else product64_fma<true>(Ta, Wc, LDA, m0, n0, accd);
+        product64_fma<true>(Ta, Wc, LDA, m0, n0, accd);
     }
     __syncthreads();
     float *As = sm;
@@ -650,6 +649,109 @@ __device__ void pivot_form(float *sm, const Seq &sq, const float *Gsrc, const fl
                 const int i = m0 + g + (e >> 1) * 8, j = n0 + nt * 8 + 2 * t + (e & 1);
                 As[i * LDP + j] = accd[nt][e];
                 if (up && n0 != 0) As[j * LDP + i] = accd[nt][e];
+            }
+    }
+}
+
+
+// four values as two fp16 parts, kept inside fp16's range (a scaled entry of G beyond 1 is rounding noise of a row whose
+// diagonal entry is noise itself)
+__device__ __forceinline__ void put4_clamped(__half *tile, int row, int c, float4 v, float4 cs, float rs)
+{
+    auto k = [&](float x, float s) { return fminf(fmaxf(x * s * rs, -60000.f), 60000.f); };
+    hs::put4(tile, row, c, make_float4(k(v.x, cs.x), k(v.y, cs.y), k(v.z, cs.z), k(v.w, cs.w)));
+}
+__device__ __forceinline__ float4 inv_pow2_4(float4 v) { return make_float4(inv_pow2(v.x), inv_pow2(v.y), inv_pow2(v.z), inv_pow2(v.w)); }
+// accumulator of a product, times k, as fp16 parts of the same 64 x 64 tile position
+__device__ __forceinline__ void put_acc(__half *tile, int m0, int n0, const float (&acc)[4][4], float k)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float x = fminf(fmaxf(acc[nt][2 * e] * k, -60000.f), 60000.f), y = fminf(fmaxf(acc[nt][2 * e + 1] * k, -60000.f), 60000.f);
+            const __half2 hi = __floats2half2_rn(x, y);
+            const float2 f = __half22float2(hi);
+            __half *dst = tile + (m0 + g + 8 * e) * hs::LDH + n0 + nt * 8 + 2 * t;
+            *(__half2 *)dst = hi;
+            *(__half2 *)(dst + hs::PLANE) = __floats2half2_rn(x - f.x, y - f.y);
+        }
+}
+// rows of a published transform (64 x 64, high parts then low parts) to a tile; 256 threads
+__device__ __forceinline__ void load_parts(__half *tile, const float *src)
+{
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int f = threadIdx.x + it * NT, plane = f >> 9, r = (f >> 3) & 63, c = (f & 7) * 8;
+        *(uint4 *)(tile + plane * hs::PLANE + r * hs::LDH + c) = __ldcg((const uint4 *)src + f);
+    }
+}
+
+// The same with the products from fp16 parts. With the scaled transforms and blocks of "published transforms", N is formed
+// as diag(s) [V'1 X'11 V'1^T ...] diag(s), s the scales of the 64 rows taken.
+__device__ void pivot_form_half(float *sm, const Seq &sq, const float *Gsrc, const float *Vcur, int step, int p1, int h1, int f1, int p2, int h2, int f2, unsigned *fetched)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    __half *Wc = (__half *)sm, *S1 = Wc + 2 * hs::PLANE, *S2 = S1 + 2 * hs::PLANE, *S3 = S2 + 2 * hs::PLANE;
+    __shared__ float srow[BLK];
+    int I1, J1, I2, J2;
+    rr_pair(sq.nb, step, p1, I1, J1);
+    rr_pair(sq.nb, step, p2, I2, J2);
+    const int np = sq.np;
+    const float *P1 = Vcur + (size_t)p1 * VSTRIDE, *P2 = Vcur + (size_t)p2 * VSTRIDE;
+    if (tid < BLK) srow[tid] = tid < JB ? __ldcg(P1 + V_S + h1 * JB + tid) : __ldcg(P2 + V_S + h2 * JB + tid - JB);
+    const int c = (tid & 15) * 4;
+    const float4 c1 = inv_pow2_4(__ldcg((const float4 *)(P1 + V_D + c))), c2 = inv_pow2_4(__ldcg((const float4 *)(P2 + V_D + c)));
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int i = (tid >> 4) + 16 * it;
+        const size_t r1 = (size_t)glob_of_loc(I1, J1, i) * np, r2 = (size_t)glob_of_loc(I2, J2, i) * np;
+        const float4 x1 = __ldcg((const float4 *)(Gsrc + r1 + glob_of_loc(I1, J1, c)));
+        const float4 x2 = __ldcg((const float4 *)(Gsrc + r2 + glob_of_loc(I2, J2, c)));
+        const float4 x3 = __ldcg((const float4 *)(Gsrc + r1 + glob_of_loc(I2, J2, c)));
+        const float d1 = inv_pow2(__ldcg(P1 + V_D + i)) * G_SCALE, d2 = inv_pow2(__ldcg(P2 + V_D + i)) * G_SCALE;
+        const bool up = i < JB;
+        const int row = (up ? h1 : h2) * JB + (i & (JB - 1));
+        if (up ? f1 : f2) {
+            const uint2 *src = (const uint2 *)(up ? P1 : P2) + (row * BLK + c) / 4;
+            *(uint2 *)(Wc + i * hs::LDH + c) = __ldcg(src);
+            *(uint2 *)(Wc + hs::PLANE + i * hs::LDH + c) = __ldcg(src + BLK * BLK / 4);
+        } else
+            hs::put4(Wc, i, c, make_float4(row == c ? V_SCALE : 0.f, row == c + 1 ? V_SCALE : 0.f, row == c + 2 ? V_SCALE : 0.f, row == c + 3 ? V_SCALE : 0.f));
+        put4_clamped(S1, i, c, x1, c1, d1);
+        put4_clamped(S2, i, c, x2, c2, d2);
+        put4_clamped(S3, i, c, x3, c2, d1);
+    }
+    __syncthreads();
+    if (tid == 0) atomicAdd(fetched, 1u);                       // the old blocks are on chip: the update may overwrite them
+    const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32;
+    const bool up = m0 < JB;
+    float accd[4][4] = {}, acco[4][4] = {};
+    hs::product64<false, false>(Wc, up ? S1 : S2, m0, n0, accd);
+    if (up) hs::product64<false, false>(Wc, S3, m0, n0, acco);
+    __syncthreads();
+    constexpr float k1 = T_SCALE / (V_SCALE * G_SCALE), k2 = 1.f / (T_SCALE * V_SCALE);
+    put_acc(S1, m0, n0, accd, k1);
+    if (up) put_acc(S2, m0, n0, acco, k1);
+    __syncthreads();
+    const bool lower_left = !up && n0 == 0;                     // mirror of the upper right part
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) accd[nt][e] = 0.f;
+    if (!lower_left) hs::product64<false, true>((up && n0 != 0) ? S2 : S1, Wc, m0, n0, accd);
+    __syncthreads();
+    float *As = sm;
+    if (!lower_left) {
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = m0 + g + (e >> 1) * 8, j = n0 + nt * 8 + 2 * t + (e & 1);
+                const float v = accd[nt][e] * k2 * srow[i] * srow[j];
+                As[i * LDP + j] = v;
+                if (up && n0 != 0) As[j * LDP + i] = v;
             }
     }
 }
@@ -697,7 +799,6 @@ __device__ bool wait_fetched(Fetched &f)
     return f.ok;
 }
 
-template <bool TENSOR>
 __device__ bool g_strip(float *sm, const Seq &sq, float *G, const float *Vbuf, const int *vflag, int step, int p, int q0, int cnt, Fetched &fetched)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -720,7 +821,7 @@ __device__ bool g_strip(float *sm, const Seq &sq, float *G, const float *Vbuf, c
 #pragma unroll
         for (int it = 0; it < 4; ++it) {
             const int f = tid + it * NT, i = f >> 4, c = (f & 15) * 4;
-            *(float4 *)(Vp + i * LDA + c) = __ldcg((const float4 *)(Vbuf + (size_t)p * BLK * BLK + i * BLK + c));
+            *(float4 *)(Vp + i * LDA + c) = __ldcg((const float4 *)(Vbuf + (size_t)p * VSTRIDE + i * BLK + c));
         }
     }
     fetch(q0);
@@ -739,22 +840,20 @@ __device__ bool g_strip(float *sm, const Seq &sq, float *G, const float *Vbuf, c
         for (int it = 0; it < 4; ++it) {
             const int f = tid + it * NT, i = f >> 4, c = (f & 15) * 4;
             *(float4 *)(blk_dst + i * blk_ld + c) = x[it];
-            if (fq) *(float4 *)(Vq + i * LDA + c) = __ldcg((const float4 *)(Vbuf + (size_t)q * BLK * BLK + i * BLK + c));
+            if (fq) *(float4 *)(Vq + i * LDA + c) = __ldcg((const float4 *)(Vbuf + (size_t)q * VSTRIDE + i * BLK + c));
         }
         __syncthreads();
         if (j + 1 < cnt) fetch(q + 1);
         float acc[4][4];
         if (fp) {
-            if (TENSOR) product64<false>(Vp, Bk, LDB, m0, n0, acc);  // T = Vt_p * block
-            else product64_fma<false>(Vp, Bk, LDB, m0, n0, acc);
+            product64_fma<false>(Vp, Bk, LDB, m0, n0, acc);
             if (fq) {
                 store_tile_acc(Tm, LDA, m0, n0, acc);
                 __syncthreads();
             }
         }
         if (fq) {                                                // out = T * Vt_q^T
-            if (TENSOR) product64<true>(Tm, Vq, LDA, m0, n0, acc);
-            else product64_fma<true>(Tm, Vq, LDA, m0, n0, acc);
+            product64_fma<true>(Tm, Vq, LDA, m0, n0, acc);
         }
         if (!wait_fetched(fetched)) return false;
         const int gr0 = glob_of_loc(Ip, Jp, m0 + g), gr1 = glob_of_loc(Ip, Jp, m0 + g + 8);
@@ -773,7 +872,6 @@ __device__ bool g_strip(float *sm, const Seq &sq, float *G, const float *Vbuf, c
     return true;
 }
 
-template <bool TENSOR>
 __device__ void wt_strip(float *sm, const Seq &sq, const float *Vbuf, const int *vflag, int step, int p, int c0, int cnt)
 {
     if (!__ldcg(vflag + p)) return;
@@ -793,7 +891,7 @@ __device__ void wt_strip(float *sm, const Seq &sq, const float *Vbuf, const int 
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
         const int f = tid + it * NT, i = f >> 4, c = (f & 15) * 4;
-        *(float4 *)(Vp + i * LDA + c) = __ldcg((const float4 *)(Vbuf + (size_t)p * BLK * BLK + i * BLK + c));
+        *(float4 *)(Vp + i * LDA + c) = __ldcg((const float4 *)(Vbuf + (size_t)p * VSTRIDE + i * BLK + c));
     }
     fetch(c0);
     const int gr0 = glob_of_loc(Ip, Jp, m0 + g), gr1 = glob_of_loc(Ip, Jp, m0 + g + 8);
@@ -806,8 +904,7 @@ __device__ void wt_strip(float *sm, const Seq &sq, const float *Vbuf, const int 
         __syncthreads();
         if (j + 1 < cnt) fetch(c0 + j + 1);
         float acc[4][4];
-        if (TENSOR) product64<false>(Vp, Bk, LDB, m0, n0, acc);
-        else product64_fma<false>(Vp, Bk, LDB, m0, n0, acc);
+        product64_fma<false>(Vp, Bk, LDB, m0, n0, acc);
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
             const int gc = (c0 + j) * BLK + n0 + nt * 8 + 2 * t;
@@ -816,6 +913,114 @@ __device__ void wt_strip(float *sm, const Seq &sq, const float *Vbuf, const int 
         }
         __syncthreads();                                         // the B tile is reused by the next chunk
     }
+}
+
+// One block (p, q) of G, products from fp16 parts: with V' and the scaled block G' of "published transforms",
+//   G_pq <- diag(s_p) V'_p G' V'_q^T diag(s_q)     (V' the identity and s = d for a pair that was not rotated).
+__device__ bool g_block_half(float *sm, const Seq &sq, float *G, const float *Vbuf, const int *vflag, int step, int p, int q, Fetched &fetched)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32, np = sq.np;
+    __half *Vp = (__half *)sm, *Vq = Vp + 2 * hs::PLANE, *Bk = Vq + 2 * hs::PLANE;
+    __shared__ float sp[BLK], sqv[BLK];
+    const int fp = __ldcg(vflag + p), fq = __ldcg(vflag + q);
+    if (!fp && !fq) return true;                                 // unchanged block
+    int Ip, Jp, Iq, Jq;
+    rr_pair(sq.nb, step, p, Ip, Jp);
+    rr_pair(sq.nb, step, q, Iq, Jq);
+    const float *Pp = Vbuf + (size_t)p * VSTRIDE, *Pq = Vbuf + (size_t)q * VSTRIDE;
+    const int c = (tid & 15) * 4;
+    float4 x[4];
+    float d[4];
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int i = (tid >> 4) + 16 * it;
+        x[it] = __ldcg((const float4 *)(G + (size_t)glob_of_loc(Ip, Jp, i) * np + glob_of_loc(Iq, Jq, c)));
+        d[it] = __ldcg(Pp + V_D + i);
+    }
+    const float4 cs = inv_pow2_4(__ldcg((const float4 *)(Pq + V_D + c)));
+    if (tid < BLK) sp[tid] = __ldcg(Pp + V_S + tid);
+    else if (tid < 2 * BLK) sqv[tid - BLK] = __ldcg(Pq + V_S + tid - BLK);
+    if (fp) load_parts(Vp, Pp);
+    if (fq) load_parts(Vq, Pq);
+#pragma unroll
+    for (int it = 0; it < 4; ++it) put4_clamped(Bk, (tid >> 4) + 16 * it, c, x[it], cs, inv_pow2(d[it]) * G_SCALE);
+    __syncthreads();
+    float acc[4][4] = {};
+    float k = 1.f / (V_SCALE * G_SCALE);
+    if (fp) hs::product64<false, false>(Vp, Bk, m0, n0, acc);
+    if (fq) {
+        if (fp) {
+            __syncthreads();
+            put_acc(Bk, m0, n0, acc, T_SCALE * k);
+            __syncthreads();
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
+            k = 1.f / (V_SCALE * T_SCALE);
+        }
+        hs::product64<false, true>(Bk, Vq, m0, n0, acc);
+    }
+    if (!wait_fetched(fetched)) return false;
+    const int gr0 = glob_of_loc(Ip, Jp, m0 + g), gr1 = glob_of_loc(Ip, Jp, m0 + g + 8);
+    const float s0 = sp[m0 + g] * k, s1 = sp[m0 + g + 8] * k;
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+        const int lc = n0 + nt * 8 + 2 * t, gc = glob_of_loc(Iq, Jq, lc);        // gc, gc + 1 are contiguous
+        const float q0 = sqv[lc], q1 = sqv[lc + 1];
+        const float v0 = acc[nt][0] * s0 * q0, v1 = acc[nt][1] * s0 * q1, v2 = acc[nt][2] * s1 * q0, v3 = acc[nt][3] * s1 * q1;
+        *(float2 *)(G + (size_t)gr0 * np + gc) = make_float2(v0, v1);
+        *(float2 *)(G + (size_t)gr1 * np + gc) = make_float2(v2, v3);
+        if (q != p) {                                            // mirror block
+            G[(size_t)gc * np + gr0] = v0; G[(size_t)(gc + 1) * np + gr0] = v1;
+            G[(size_t)gc * np + gr1] = v2; G[(size_t)(gc + 1) * np + gr1] = v3;
+        }
+    }
+    __syncthreads();                                             // tiles are reused by the next block
+    return true;
+}
+
+// Column chunks c0 .. c0 + cnt - 1 of the rows of pair p of Wt, products from fp16 parts.
+__device__ void wt_strip_half(float *sm, const Seq &sq, const float *Vbuf, const int *vflag, int step, int p, int c0, int cnt)
+{
+    if (!__ldcg(vflag + p)) return;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32, np = sq.np;
+    __half *Vp = (__half *)sm, *Bk = Vp + 2 * hs::PLANE;
+    int Ip, Jp;
+    rr_pair(sq.nb, step, p, Ip, Jp);
+    float4 x[4];
+    auto fetch = [&](int chunk) {
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            const int f = tid + it * NT, i = f >> 4, c = (f & 15) * 4;
+            x[it] = __ldcg((const float4 *)(sq.Wt + (size_t)glob_of_loc(Ip, Jp, i) * np + chunk * BLK + c));
+        }
+    };
+    fetch(c0);
+    load_parts(Vp, Vbuf + (size_t)p * VSTRIDE + V_VU);
+    const int gr0 = glob_of_loc(Ip, Jp, m0 + g), gr1 = glob_of_loc(Ip, Jp, m0 + g + 8);
+    for (int j = 0; j < cnt; ++j) {
+        __half *B = Bk + (j & 1) * 2 * hs::PLANE;                // two tiles: one barrier per chunk
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            const int f = tid + it * NT;
+            hs::put4(B, f >> 4, (f & 15) * 4, make_float4(x[it].x * V_SCALE, x[it].y * V_SCALE, x[it].z * V_SCALE, x[it].w * V_SCALE));
+        }
+        __syncthreads();
+        if (j + 1 < cnt) fetch(c0 + j + 1);
+        float acc[4][4] = {};
+        hs::product64<false, false>(Vp, B, m0, n0, acc);
+        constexpr float k = 1.f / (V_SCALE * V_SCALE);
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt) {
+            const int gc = (c0 + j) * BLK + n0 + nt * 8 + 2 * t;
+            *(float2 *)(sq.Wt + (size_t)gr0 * np + gc) = make_float2(acc[nt][0] * k, acc[nt][1] * k);
+            *(float2 *)(sq.Wt + (size_t)gr1 * np + gc) = make_float2(acc[nt][2] * k, acc[nt][3] * k);
+        }
+    }
+    __syncthreads();
 }
 
 // Work items of the update: first the strips of G (row by row of the upper triangle), then the strips of Wt.
@@ -836,11 +1041,17 @@ __device__ bool apply_item(float *sm, const Seq &sq, const float *Vbuf, const in
             idx -= n; ++p;
         }
         const int q0 = p + idx * SEG_G;
-        return g_strip<TENSOR>(sm, sq, sq.G, Vbuf, vflag, step, p, q0, min(SEG_G, npairs - q0), fetched);
+        if (TENSOR) {
+            for (int q = q0; q < min(q0 + SEG_G, npairs); ++q)
+                if (!g_block_half(sm, sq, sq.G, Vbuf, vflag, step, p, q, fetched)) return false;
+            return true;
+        }
+        return g_strip(sm, sq, sq.G, Vbuf, vflag, step, p, q0, min(SEG_G, npairs - q0), fetched);
     } else {
         idx -= items_g;
         const int nseg = (nw + SEG_W - 1) / SEG_W, p = idx / nseg, c0 = (idx - p * nseg) * SEG_W;
-        wt_strip<TENSOR>(sm, sq, Vbuf, vflag, step, p, c0, min(SEG_W, nw - c0));
+        if (TENSOR) wt_strip_half(sm, sq, Vbuf, vflag, step, p, c0, min(SEG_W, nw - c0));
+        else wt_strip(sm, sq, Vbuf, vflag, step, p, c0, min(SEG_W, nw - c0));
     }
     return true;
 }
@@ -915,7 +1126,7 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
     // rotates the block held in shared memory for pair pr of (sweep, step); publishes to parity par
     auto pivot_finish = [&](int sweep, int step, int pr, int par) {
         bool rotated;
-        const float mo = pivot_rotate(j3sm, step > 0, tol_rot, sq.Vbuf + ((size_t)par * npairs + pr) * BLK * BLK, rotated);
+        const float mo = pivot_rotate<TENSOR>(j3sm, step > 0, tol_rot, sq.Vbuf + ((size_t)par * npairs + pr) * VSTRIDE, rotated);
         if (tid == 0) {
             sq.vflag[par * npairs + pr] = rotated ? 1 : 0;
             atomicMax(sq.sync + 1 + sweep % 4, __float_as_uint(mo));
@@ -939,7 +1150,7 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
             const int par = (int)(gstep & 1u);
             const bool has_next = !(sweep == max_sweeps - 1 && step == nsteps - 1);
             const int nstep = step + 1 == nsteps ? 0 : step + 1, nsweep = sweep + (step + 1 == nsteps ? 1 : 0);
-            const float *Vcur = sq.Vbuf + (size_t)par * npairs * BLK * BLK;
+            const float *Vcur = sq.Vbuf + (size_t)par * npairs * VSTRIDE;
             const int *fcur = sq.vflag + par * npairs;
             // a step in which no pair was rotated needs no update
             const bool any_rot = __syncthreads_or(tid < npairs && __ldcg(fcur + tid) != 0) != 0;
@@ -965,7 +1176,8 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
                         pivot_load(j3sm, sq.G, sq.np, I2, J2);
                         __syncthreads();
                         if (tid == 0) atomicAdd(sq.sync + 20 + par, 1u);
-                    } else pivot_form<TENSOR>(j3sm, sq, sq.G, Vcur, step, p1, h1, f1, p2, h2, f2, sq.sync + 20 + par);
+                    } else if (TENSOR) pivot_form_half(j3sm, sq, sq.G, Vcur, step, p1, h1, f1, p2, h2, f2, sq.sync + 20 + par);
+                    else pivot_form(j3sm, sq, sq.G, Vcur, step, p1, h1, f1, p2, h2, f2, sq.sync + 20 + par);
                     pivot_finish(nsweep, nstep, pr, par ^ 1);
                 }
             }
