@@ -390,35 +390,47 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                 // the columns' largest entries go to slot 1 before a second projection of the same panel; otherwise slot 0 has
                 // been used and is cleared for the next panel (noted beside the factor that follows)
                 const bool note_max = TENSOR && stage == 2;
-                float cmax = 0.f;
+                float4 cmax = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (TENSOR && !note_max && rank == 0 && tid < 64) sq.sync[64 + tid] = 0u;
                 for (int t = rank; t < ntile; t += ncta) {
                     const int rv = min(64, n - t * 64);
-                    load_tile(sA, LDA, sq.M + (size_t)t * 64 * ld + j0, ld, rv, w, vec);
-                    if (with_w) load_tile(sB, LDB, sq.W, 64, 64, 64, true);
-                    __syncthreads();
+                    TileRegs ra;
+                    fetch_tile(ra, sq.M + (size_t)t * 64 * ld + j0, ld, rv, w, vec);
                     if (nj > 0) {
-                        for (int e0 = tid; e0 < 4096; e0 += 4 * NT) {            // four elements, 4 G loads in flight
-                            float sacc[4] = {0.f, 0.f, 0.f, 0.f};
-                            const float *dp = sq.Dpart + (size_t)t * G * 4096 + e0;
-                            for (int g = 0; g < G; ++g) {
-                                float x[4];
+                        const float4 *dp = (const float4 *)(sq.Dpart + (size_t)t * G * 4096) + tid;
+                        float4 d[4];
 #pragma unroll
-                                for (int q = 0; q < 4; ++q) x[q] = __ldcg(dp + (size_t)g * 4096 + q * NT);
+                        for (int i = 0; i < 4; ++i) d[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int g = 0; g < G; g += 2) {                 // in this order, eight loads in flight
+                            float4 x[8];
 #pragma unroll
-                                for (int q = 0; q < 4; ++q) sacc[q] += x[q];
-                            }
+                            for (int q = 0; q < 8; ++q)
+                                x[q] = g + (q >> 2) < G ? __ldcg(dp + (size_t)(g + (q >> 2)) * 1024 + (q & 3) * NT) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int e = e0 + q * NT, r = e >> 6, c = e & 63;
-                                const float v = sA[r * LDA + c] - sacc[q];
-                                sA[r * LDA + c] = (r < rv && c < w) ? v : 0.f;
-                                if (r < rv && c < w) cmax = fmaxf(cmax, fabsf(v));
-                                if (!with_w && r < rv && c < w) sq.M[((size_t)t * 64 + r) * ld + j0 + c] = v;
+                            for (int q = 0; q < 8; ++q) { float4 &a = d[q & 3]; a.x += x[q].x; a.y += x[q].y; a.z += x[q].z; a.w += x[q].w; }
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {                    // (rows and columns beyond the tile are zero in both)
+                            float4 &v = ra.v[i];
+                            v.x -= d[i].x; v.y -= d[i].y; v.z -= d[i].z; v.w -= d[i].w;
+                            cmax.x = fmaxf(cmax.x, fabsf(v.x)); cmax.y = fmaxf(cmax.y, fabsf(v.y));
+                            cmax.z = fmaxf(cmax.z, fabsf(v.z)); cmax.w = fmaxf(cmax.w, fabsf(v.w));
+                            const int f = tid + i * NT, r = f >> 4, c = (f & 15) * 4;
+                            if (!with_w && r < rv) {
+                                float *dm = sq.M + ((size_t)t * 64 + r) * ld + j0 + c;
+                                if (vec && c + 3 < w) *(float4 *)dm = v;
+                                else {
+                                    if (c < w) dm[0] = v.x;
+                                    if (c + 1 < w) dm[1] = v.y;
+                                    if (c + 2 < w) dm[2] = v.z;
+                                    if (c + 3 < w) dm[3] = v.w;
+                                }
                             }
                         }
-                        __syncthreads();
                     }
+                    stash_tile(ra, sA, LDA);
+                    if (with_w) load_tile(sB, LDB, sq.W, 64, 64, 64, true);
+                    __syncthreads();
                     if (with_w) {
                         float acc[4][4] = {};
                         tile_mac<P_FINE, false>(sA, LDA, sB, LDB, m0, n0, acc);
@@ -438,7 +450,16 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                     gram_tile_64(sA, LDA, Gs, sq.gpart + (size_t)t * 4096);
                     __syncthreads();
                 }
-                if (note_max && cmax > 0.f) atomicMax(sq.sync + 128 + (tid & 63), __float_as_uint(cmax));
+                if (note_max) {
+                    unsigned *cm = (unsigned *)colinv;                       // (free between the projections)
+                    if (tid < 64) cm[tid] = 0u;
+                    __syncthreads();
+                    const float m[4] = {cmax.x, cmax.y, cmax.z, cmax.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) atomicMax(cm + (tid & 15) * 4 + k, __float_as_uint(m[k]));
+                    __syncthreads();
+                    if (tid < 64 && cm[tid] > 0u) atomicMax(sq.sync + 128 + tid, cm[tid]);
+                }
                 barrier();
                 if (!alive) break;
                 // ordered sum of the partial Gram matrices: 16 element slices x (up to 8) chunk ranges
