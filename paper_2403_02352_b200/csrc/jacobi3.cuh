@@ -804,7 +804,7 @@ __device__ bool g_strip(float *sm, const Seq &sq, float *G, const float *Vbuf, c
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32, np = sq.np;
     float *Vp = sm, *Vq = sm + BLK * LDA, *Tm = sm + 2 * BLK * LDA, *Bk = sm + 3 * BLK * LDA;
-    const int fp = __ldcg(vflag + p);
+    const int fp = vflag[p];
     int Ip, Jp;
     rr_pair(sq.nb, step, p, Ip, Jp);
     float4 x[4];
@@ -826,7 +826,7 @@ __device__ bool g_strip(float *sm, const Seq &sq, float *G, const float *Vbuf, c
     }
     fetch(q0);
     for (int j = 0; j < cnt; ++j) {
-        const int q = q0 + j, fq = __ldcg(vflag + q);
+        const int q = q0 + j, fq = vflag[q];
         int Iq, Jq;
         rr_pair(sq.nb, step, q, Iq, Jq);
         if (!fp && !fq) {                                        // unchanged block
@@ -874,7 +874,7 @@ __device__ bool g_strip(float *sm, const Seq &sq, float *G, const float *Vbuf, c
 
 __device__ void wt_strip(float *sm, const Seq &sq, const float *Vbuf, const int *vflag, int step, int p, int c0, int cnt)
 {
-    if (!__ldcg(vflag + p)) return;
+    if (!vflag[p]) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32, np = sq.np;
     float *Vp = sm, *Bk = sm + 3 * BLK * LDA;
@@ -923,7 +923,7 @@ __device__ bool g_block_half(float *sm, const Seq &sq, float *G, const float *Vb
     const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32, np = sq.np;
     __half *Vp = (__half *)sm, *Vq = Vp + 2 * hs::PLANE, *Bk = Vq + 2 * hs::PLANE;
     __shared__ float sp[BLK], sqv[BLK];
-    const int fp = __ldcg(vflag + p), fq = __ldcg(vflag + q);
+    const int fp = vflag[p], fq = vflag[q];
     if (!fp && !fq) return true;                                 // unchanged block
     int Ip, Jp, Iq, Jq;
     rr_pair(sq.nb, step, p, Ip, Jp);
@@ -984,7 +984,7 @@ __device__ bool g_block_half(float *sm, const Seq &sq, float *G, const float *Vb
 // Column chunks c0 .. c0 + cnt - 1 of the rows of pair p of Wt, products from fp16 parts.
 __device__ void wt_strip_half(float *sm, const Seq &sq, const float *Vbuf, const int *vflag, int step, int p, int c0, int cnt)
 {
-    if (!__ldcg(vflag + p)) return;
+    if (!vflag[p]) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32, np = sq.np;
     __half *Vp = (__half *)sm, *Bk = Vp + 2 * hs::PLANE;
@@ -1109,6 +1109,7 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
 {
     extern __shared__ __align__(16) float j3sm[];
     __shared__ short pair_of[2 * MAXPAIRS];       // block -> 2 * pair + half, for the current step
+    __shared__ int flag_s[MAXPAIRS];              // the pairs rotated in the current step
     __shared__ int ticket_s;
     int si = 0;
 #pragma unroll 1
@@ -1152,8 +1153,10 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
             const int nstep = step + 1 == nsteps ? 0 : step + 1, nsweep = sweep + (step + 1 == nsteps ? 1 : 0);
             const float *Vcur = sq.Vbuf + (size_t)par * npairs * VSTRIDE;
             const int *fcur = sq.vflag + par * npairs;
-            // a step in which no pair was rotated needs no update
-            const bool any_rot = __syncthreads_or(tid < npairs && __ldcg(fcur + tid) != 0) != 0;
+            // a step in which no pair was rotated needs no update (the flags are read once: an L2 round trip per use otherwise)
+            const int my_flag = tid < npairs ? __ldcg(fcur + tid) : 0;
+            if (tid < npairs) flag_s[tid] = my_flag;
+            const bool any_rot = __syncthreads_or(my_flag != 0) != 0;
             if (rank == 0 && tid == 0) {                                  // tickets and fetch count of the next step
                 sq.sync[16 + (par ^ 1)] = 0u;
                 sq.sync[20 + (par ^ 1)] = 0u;
@@ -1171,7 +1174,7 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
                     int I2, J2;
                     rr_pair(sq.nb, nstep, pr, I2, J2);
                     const int p1 = pair_of[I2] >> 1, h1 = pair_of[I2] & 1, p2 = pair_of[J2] >> 1, h2 = pair_of[J2] & 1;
-                    const int f1 = __ldcg(fcur + p1), f2 = __ldcg(fcur + p2);
+                    const int f1 = flag_s[p1], f2 = flag_s[p2];
                     if (!f1 && !f2) {
                         pivot_load(j3sm, sq.G, sq.np, I2, J2);
                         __syncthreads();
@@ -1181,14 +1184,20 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
                     pivot_finish(nsweep, nstep, pr, par ^ 1);
                 }
             }
-            // 2. the update, by tickets (the next one is requested while a block is processed)
-            if (tid == 0) ticket_s = any_rot ? (int)atomicAdd(sq.sync + 16 + par, 1u) : total;
-            __syncthreads();
-            int t = ticket_s;
+            // 2. the update: the CTAs without a pivot take the first items by rank, everything else goes by tickets (the next
+            // one is requested while a block is processed)
+            const int fixed = has_next ? max(sq.ncta - npairs, 0) : sq.ncta, mine = has_next ? rank - npairs : rank;
+            int t = total;
+            if (any_rot && mine >= 0) t = mine;
+            else if (any_rot) {
+                if (tid == 0) ticket_s = fixed + (int)atomicAdd(sq.sync + 16 + par, 1u);
+                __syncthreads();
+                t = ticket_s;
+            }
             while (t < total && alive) {
                 int tn = 0;
-                if (tid == 0) tn = (int)atomicAdd(sq.sync + 16 + par, 1u);
-                alive = apply_item<TENSOR>(j3sm, sq, Vcur, fcur, step, t, npairs, items_g, nw, fetched);
+                if (tid == 0) tn = fixed + (int)atomicAdd(sq.sync + 16 + par, 1u);
+                alive = apply_item<TENSOR>(j3sm, sq, Vcur, flag_s, step, t, npairs, items_g, nw, fetched);
                 __syncthreads();
                 if (tid == 0) ticket_s = tn;
                 __syncthreads();
