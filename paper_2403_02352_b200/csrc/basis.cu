@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(256) signfix_kernel(const __grid_constant__ Fi
 struct SeqPlan {
     SeqDims dims; int rt, np, npanel_L, npanel_d; unsigned *jsync; float *tpart;
     __nv_bfloat16 *Bth, *Btl, *Y2h, *Y2l, *Wth, *Wtl, *Wsh, *Wsl;
-    float *oCpart, *oC, *oDpart, *oW; double *ogpart, *ogpart2; unsigned *osync; int ocap;
+    __half *oqh, *oql; float *oCpart, *oC, *oDpart, *oW; double *ogpart, *ogpart2; unsigned *osync; int ocap;
     __nv_bfloat16 *Yb, *Yl, *Zb, *Zl; float *Y2; float *Y, *Z, *BW, *Wsel, *tsum, *sig, *Cc, *rinv, *G, *Wt, *Vbuf; double *gpart; int *ord, *flags, *conv, *vflag, *needfix; unsigned *maxoff;
 };
 struct BasisPlan {
@@ -584,6 +584,8 @@ static void plan_basis(Arena &ar, const std::vector<SeqDims> &sd, int d, int ove
         {   // tile scratch of the orthonormalisation kernel
             p.ocap = orth::max_ctas_per_seq(sm_count, (int)std::min<size_t>(sd.size(), BMAX));
             const orth::Scratch sc = orth::scratch_tiles(L, rt, p.ocap);
+            const size_t ldq = align_up((size_t)std::max(rt, 1), 64);
+            p.oqh = ar.take<__half>((size_t)L * ldq); p.oql = ar.take<__half>((size_t)L * ldq);
             p.oCpart = ar.take<float>(sc.cpart * 4096); p.oC = ar.take<float>(sc.c * 4096);
             p.oDpart = ar.take<float>(sc.dpart * 4096); p.oW = ar.take<float>(4096);
             p.ogpart = ar.take<double>(sc.gpart * 4096); p.ogpart2 = ar.take<double>((size_t)orth::NRED * 4096);
@@ -628,7 +630,7 @@ static atp_status orthonormalise(atp_ctx *ctx, BasisPlan &bp, size_t i0, size_t 
     for (size_t i = i0; i < i1; ++i) {
         SeqPlan &p = bp.seqs[i];
         ob.s[i - i0] = orth::Seq{p.Y, p.dims.L, p.rt, p.rt, TENSOR ? p.Yb : nullptr, TENSOR ? p.Yl : nullptr,
-                                 (int)align_up((size_t)std::max(p.rt, 1), 8), p.oCpart, p.oC, p.oDpart, p.oW, p.ogpart, p.ogpart2,
+                                 (int)align_up((size_t)std::max(p.rt, 1), 8), p.oqh, p.oql, (int)align_up((size_t)std::max(p.rt, 1), 64), p.oCpart, p.oC, p.oDpart, p.oW, p.ogpart, p.ogpart2,
                                  p.flags, p.osync, 0, p.ocap, 0};
     }
     return orth::launch<TENSOR>(ctx, ob, reps, seed);

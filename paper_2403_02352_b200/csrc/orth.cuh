@@ -16,7 +16,9 @@
 // the group's barrier (bounded spin) instead of kernel boundaries, and every phase is a list
 // of independent 64 x 64 tile jobs dealt out round-robin. The tile products of the projections (most of the arithmetic) run on
 // the tensor cores from two fp16 parts per operand (split_mma.cuh), columns of the panel scaled by powers of two to a
-// common range; the products with the factor, whose rows differ by the ratio of the column norms, from two TF32 parts. Plain
+// common range. The finished columns are kept as such parts: their tiles go to shared memory by cp.async, without a
+// conversion, two of them for every tile of the panel (or of C), which is fetched and cut once for two products (from fp32
+// tiles, one product per pair of fetched and cut tiles, 32768 x 1088 took 4920 us instead of 3710). The products with the factor, whose rows differ by the ratio of the column norms, from two TF32 parts. Plain
 // TF32 is not enough even for the first repetition, because what a projection leaves of an ill-conditioned panel is far
 // below 2^-11 of the panel. fp32 inputs keep every product on the fp32 units.
 #pragma once
@@ -34,6 +36,7 @@ constexpr int NRED = 8;           // second-level partial Gram sums (chunk range
 struct Seq {
     float *M; int n, rt, ld;                  // the iterate: n x rt, fp32, leading dimension ld
     __nv_bfloat16 *hi, *lo; int ldh;          // nullable: the finished columns also go out as a bf16 hi/lo pair
+    __half *qh, *ql; int ldq;                 // bf16 inputs: the finished columns times QSCALE as two fp16 parts, n x ldq
     float *Cpart, *C, *Dpart, *W;             // tile scratch (see scratch_tiles)
     double *gpart, *gpart2;
     int *flags;
@@ -51,7 +54,7 @@ struct Scratch { size_t cpart, c, dpart, gpart; };
 static inline Scratch scratch_tiles(int n, int rt, int ncta)
 {
     const size_t nt = (size_t)(n + 63) / 64, nj = (size_t)(rt + 63) / 64;
-    return Scratch{(size_t)ncta + nj + 1, nj + 1, (size_t)ncta + nt + 1, nt + 1};
+    return Scratch{2 * (size_t)ncta + nj + 2, nj + 1, 2 * (size_t)ncta + nt + 2, nt + 1};   // (jobs make pairs of tiles)
 }
 
 // 64 x 64 tile of a row-major fp32 matrix, zero beyond rv rows / cv columns, in two halves so that the loads of
@@ -149,8 +152,8 @@ __global__ void __launch_bounds__(NT, 2)
 orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t seed, int *status)
 {
     extern __shared__ __align__(16) float osm[];
-    __shared__ __align__(16) double Gs[PB * LDC];
     float *sA = osm, *sB = osm + BLK * LDB;                   // two tiles at stride LDB (covers LDA too)
+    double *Gs = (double *)(osm + 2 * BLK * LDB);             // 64 x LDC, behind them
     int si = 0;
 #pragma unroll 1
     for (int i = 1; i < batch.count; ++i) if ((int)blockIdx.x >= batch.s[i].cta0) si = i;
@@ -217,7 +220,19 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
         }
         __syncthreads();
     };
-    __half *hA = (__half *)osm, *hB = hA + 2 * hs::PLANE;      // the same shared memory as sA, sB
+    // Tiles of fp16 parts: two buffers of two tiles of finished columns, one tile of the panel or of C; the first four take
+    // the place of sA, sB and Gs.
+    auto htile = [&](int k) { return (__half *)osm + (size_t)k * 2 * hs::PLANE; };
+    auto async_q = [&](__half *dst, int t, int jb) {           // rows of tile t, columns of panel jb
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int f = tid + i * NT, plane = f >> 9, r = (f >> 3) & 63, c = (f & 7) * 8, row = t * 64 + r;
+            const __half *src = (plane ? sq.ql : sq.qh) + (size_t)(row < n ? row : 0) * sq.ldq + jb * 64 + c;
+            const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + plane * hs::PLANE + r * hs::LDH + c);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(row < n ? 16 : 0) : "memory");
+        }
+    };
+    auto async_commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
     auto put_tile = [&](const TileRegs &tr, __half *dst, float4 sc) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -226,7 +241,6 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             hs::put4(dst, f >> 4, (f & 15) * 4, make_float4(v.x * sc.x, v.y * sc.y, v.z * sc.z, v.w * sc.w));
         }
     };
-    const float4 qs4 = make_float4(QSCALE, QSCALE, QSCALE, QSCALE);
     auto unscale = [&](float (&acc)[4][4]) {
         const int t2 = (tid & 3) * 2;
 #pragma unroll
@@ -248,9 +262,11 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
     enum { OP_PF, OP_SUMUPD, OP_GRAM, OP_APPLY };
     for (int pj = 0; pj < npanel && alive; ++pj) {
         const int j0 = pj * 64, w = min(64, rt - j0), nj = pj;            // nj finished panels
-        const int KS = nj > 0 ? max(1, min(ntile, (ncta + nj - 1) / nj)) : 1;
+        // jobs of the projections: (columns, row range) and (rows, column range), by pairs of tiles with TENSOR
+        const int nc = TENSOR ? (nj + 1) / 2 : nj, nr = TENSOR ? (ntile + 1) / 2 : ntile;
+        const int KS = nj > 0 ? max(1, min(ntile, (ncta + nc - 1) / nc)) : 1;
         const int tper = (ntile + KS - 1) / KS;
-        const int G = nj > 0 ? max(1, min(nj, (ncta + ntile - 1) / ntile)) : 1;
+        const int G = nj > 0 ? max(1, min(nj, (ncta + nr - 1) / nr)) : 1;
         const int jper = nj > 0 ? (nj + G - 1) / G : 1;
         const int nrange = max(1, min(8, ntile / 64)), cper = (ntile + nrange - 1) / nrange;
         int stage = overlap ? 0 : 30, rep = 0;
@@ -313,7 +329,41 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                 } else if (first >= 0) {
                     set_scales(scale_slot);
                     const float4 ps4 = *(const float4 *)&colscale[(tid & 15) * 4];
-                    for (int it = first; it < nj * KS; it += stride) {
+                    if constexpr (TENSOR) for (int it = first; it < nc * KS; it += stride) {
+                        const int jb = it / KS * 2, ks = it - jb / 2 * KS;
+                        const bool two = jb + 1 < nj;
+                        float acc[2][4][4] = {};
+                        const int t0 = ks * tper, t1 = min(ntile, (ks + 1) * tper);
+                        TileRegs rb;
+                        auto issue = [&](int t) {
+                            __half *dst = htile(2 * ((t - t0) & 1));
+                            async_q(dst, t, jb);
+                            if (two) async_q(dst + 2 * hs::PLANE, t, jb + 1);
+                        };
+                        if (t0 < t1) {
+                            issue(t0);
+                            fetch_tile(rb, sq.M + (size_t)t0 * 64 * ld + j0, ld, min(64, n - t0 * 64), w, vec);
+                        }
+                        async_commit();
+                        for (int t = t0; t < t1; ++t) {
+                            put_tile(rb, htile(4), ps4);
+                            if (t + 1 < t1) issue(t + 1);                   // next tiles in flight during the products
+                            async_commit();
+                            asm volatile("cp.async.wait_group 1;" ::: "memory");
+                            __syncthreads();
+                            if (t + 1 < t1) fetch_tile(rb, sq.M + (size_t)(t + 1) * 64 * ld + j0, ld, min(64, n - (t + 1) * 64), w, vec);
+                            const __half *q = htile(2 * ((t - t0) & 1));
+                            hs::product64<true, false>(q, htile(4), m0, n0, acc[0]);
+                            if (two) hs::product64<true, false>(q + 2 * hs::PLANE, htile(4), m0, n0, acc[1]);
+                            __syncthreads();
+                        }
+                        unscale(acc[0]);
+                        store_acc(sq.Cpart + (size_t)(jb * KS + ks) * 4096, 64, m0, n0, acc[0]);
+                        if (two) {
+                            unscale(acc[1]);
+                            store_acc(sq.Cpart + (size_t)((jb + 1) * KS + ks) * 4096, 64, m0, n0, acc[1]);
+                        }
+                    } else for (int it = first; it < nj * KS; it += stride) {
                         const int jb = it / KS, ks = it - jb * KS;
                         float acc[4][4] = {};
                         const int t0 = ks * tper, t1 = min(ntile, (ks + 1) * tper);
@@ -323,19 +373,17 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                             fetch_tile(rb, sq.M + (size_t)t0 * 64 * ld + j0, ld, min(64, n - t0 * 64), w, vec);
                         }
                         for (int t = t0; t < t1; ++t) {
-                            if (TENSOR) { put_tile(ra, hA, qs4); put_tile(rb, hB, ps4); }
-                            else { stash_tile(ra, sA, LDB); stash_tile(rb, sB, LDB); }
+                            stash_tile(ra, sA, LDB);
+                            stash_tile(rb, sB, LDB);
                             __syncthreads();
                             if (t + 1 < t1) {                               // next tiles in flight during the product
                                 const int rv = min(64, n - (t + 1) * 64);
                                 fetch_tile(ra, sq.M + (size_t)(t + 1) * 64 * ld + jb * 64, ld, rv, 64, vec);
                                 fetch_tile(rb, sq.M + (size_t)(t + 1) * 64 * ld + j0, ld, rv, w, vec);
                             }
-                            if (TENSOR) hs::product64<true, false>(hA, hB, m0, n0, acc);
-                            else tile_mac<0, true>(sA, LDB, sB, LDB, m0, n0, acc);
+                            tile_mac<0, true>(sA, LDB, sB, LDB, m0, n0, acc);
                             __syncthreads();
                         }
-                        if (TENSOR) unscale(acc);
                         store_acc(sq.Cpart + (size_t)it * 4096, 64, m0, n0, acc);
                     }
                 }
@@ -359,7 +407,41 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                 if (!alive) break;
                 set_scales(scale_slot);
                 const float4 ps4 = *(const float4 *)&colscale[(tid & 15) * 4];
-                for (int it = rank; it < ntile * G; it += ncta) {
+                if constexpr (TENSOR) for (int it = rank; it < nr * G; it += ncta) {
+                    const int t = it / G * 2, g = it - t / 2 * G;
+                    const bool two = t + 1 < ntile;
+                    float acc[2][4][4] = {};
+                    const int jb0 = g * jper, jb1 = min(nj, (g + 1) * jper);
+                    TileRegs rb;
+                    auto issue = [&](int jb) {
+                        __half *dst = htile(2 * ((jb - jb0) & 1));
+                        async_q(dst, t, jb);
+                        if (two) async_q(dst + 2 * hs::PLANE, t + 1, jb);
+                    };
+                    if (jb0 < jb1) {
+                        issue(jb0);
+                        fetch_tile(rb, sq.C + (size_t)jb0 * 4096, 64, 64, 64, true);
+                    }
+                    async_commit();
+                    for (int jb = jb0; jb < jb1; ++jb) {
+                        put_tile(rb, htile(4), ps4);
+                        if (jb + 1 < jb1) issue(jb + 1);
+                        async_commit();
+                        asm volatile("cp.async.wait_group 1;" ::: "memory");
+                        __syncthreads();
+                        if (jb + 1 < jb1) fetch_tile(rb, sq.C + (size_t)(jb + 1) * 4096, 64, 64, 64, true);
+                        const __half *q = htile(2 * ((jb - jb0) & 1));
+                        hs::product64<false, false>(q, htile(4), m0, n0, acc[0]);
+                        if (two) hs::product64<false, false>(q + 2 * hs::PLANE, htile(4), m0, n0, acc[1]);
+                        __syncthreads();
+                    }
+                    unscale(acc[0]);
+                    store_acc(sq.Dpart + (size_t)(t * G + g) * 4096, 64, m0, n0, acc[0]);
+                    if (two) {
+                        unscale(acc[1]);
+                        store_acc(sq.Dpart + (size_t)((t + 1) * G + g) * 4096, 64, m0, n0, acc[1]);
+                    }
+                } else for (int it = rank; it < ntile * G; it += ncta) {
                     const int t = it / G, g = it - t * G;
                     const int rv = min(64, n - t * 64);
                     float acc[4][4] = {};
@@ -370,18 +452,16 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                         fetch_tile(rb, sq.C + (size_t)jb0 * 4096, 64, 64, 64, true);
                     }
                     for (int jb = jb0; jb < jb1; ++jb) {
-                        if (TENSOR) { put_tile(ra, hA, qs4); put_tile(rb, hB, ps4); }
-                        else { stash_tile(ra, sA, LDA); stash_tile(rb, sB, LDB); }
+                        stash_tile(ra, sA, LDA);
+                        stash_tile(rb, sB, LDB);
                         __syncthreads();
                         if (jb + 1 < jb1) {
                             fetch_tile(ra, sq.M + (size_t)t * 64 * ld + (jb + 1) * 64, ld, rv, 64, vec);
                             fetch_tile(rb, sq.C + (size_t)(jb + 1) * 4096, 64, 64, 64, true);
                         }
-                        if (TENSOR) hs::product64<false, false>(hA, hB, m0, n0, acc);
-                        else tile_mac<0, false>(sA, LDA, sB, LDB, m0, n0, acc);
+                        tile_mac<0, false>(sA, LDA, sB, LDB, m0, n0, acc);
                         __syncthreads();
                     }
-                    if (TENSOR) unscale(acc);
                     store_acc(sq.Dpart + (size_t)it * 4096, 64, m0, n0, acc);
                 }
                 barrier();
@@ -506,6 +586,15 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                         float *dm = sq.M + (size_t)grow * ld + j0 + c;
                         if (vec && c + 3 < w) *(float4 *)dm = make_float4(v[0], v[1], v[2], v[3]);
                         else for (int k = 0; k < 4 && c + k < w; ++k) dm[k] = v[k];
+                        if (TENSOR && last && pj + 1 < npanel) {             // (the last panel is projected against by nobody)
+                            const __half2 h0 = __floats2half2_rn(v[0] * QSCALE, v[1] * QSCALE), h1 = __floats2half2_rn(v[2] * QSCALE, v[3] * QSCALE);
+                            const float2 f0 = __half22float2(h0), f1 = __half22float2(h1);
+                            const __half2 l0 = __floats2half2_rn(v[0] * QSCALE - f0.x, v[1] * QSCALE - f0.y);
+                            const __half2 l1 = __floats2half2_rn(v[2] * QSCALE - f1.x, v[3] * QSCALE - f1.y);
+                            const size_t at = (size_t)grow * sq.ldq + j0 + c;
+                            *(uint2 *)(sq.qh + at) = make_uint2(*(const uint32_t *)&h0, *(const uint32_t *)&h1);
+                            *(uint2 *)(sq.ql + at) = make_uint2(*(const uint32_t *)&l0, *(const uint32_t *)&l1);
+                        }
                         if (last && sq.hi) {
                             // the pair's rows are padded to multiples of 8 columns; what lies beyond rt is never read
                             *(uint2 *)(sq.hi + (size_t)grow * sq.ldh + j0 + c) = *(const uint2 *)h;
@@ -535,7 +624,9 @@ __global__ void init_kernel(const __grid_constant__ Batch batch)
     if ((int)threadIdx.x < SYNC_WORDS && sq.n > 0) sq.sync[threadIdx.x] = 0u;
 }
 
-constexpr size_t SMEM_BYTES = (size_t)(2 * BLK * LDB) * sizeof(float);
+// two fp32 tiles and the Gram matrix, or five tiles of fp16 parts
+template <bool TENSOR> constexpr size_t SMEM_BYTES = TENSOR ? 5 * hs::TILE_BYTES : (size_t)(2 * BLK * LDB) * sizeof(float) + (size_t)PB * LDC * sizeof(double);
+static_assert((size_t)(2 * BLK * LDB) * sizeof(float) + (size_t)PB * LDC * sizeof(double) <= 5 * hs::TILE_BYTES, "Gram matrix behind the tiles");
 
 // Largest number of CTAs a launch hands to one sequence (workspace sizing and launch agree on it).
 static inline int max_ctas_per_seq(int sm_count, int nseq) { return std::max(1, 2 * sm_count / std::max(nseq, 1)); }
@@ -546,10 +637,10 @@ static inline atp_status launch(atp_ctx *ctx, Batch &ob, int reps, uint64_t seed
     if (ob.count <= 0) return ATP_OK;
     static PerDeviceOnce attr_once;
     ATP_CUDA_OK(ctx, attr_once.run(ctx->device, [] {
-        return cudaFuncSetAttribute(orth_persistent_kernel<TENSOR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+        return cudaFuncSetAttribute(orth_persistent_kernel<TENSOR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES<TENSOR>);
     }));
     int occ = 0;
-    ATP_CUDA_OK(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, orth_persistent_kernel<TENSOR>, NT, SMEM_BYTES));
+    ATP_CUDA_OK(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, orth_persistent_kernel<TENSOR>, NT, SMEM_BYTES<TENSOR>));
     if (occ < 1) return ATP_ERR_CUDA;
     const int total = ctx->sm_count * std::min(occ, 2);
     double wsum = 0;
@@ -572,7 +663,7 @@ static inline atp_status launch(atp_ctx *ctx, Batch &ob, int reps, uint64_t seed
     void *args[] = {(void *)&ob, (void *)&reps, (void *)&seed, (void *)&status};
     // bytes: one read and one write of every iterate
     ATP_KERNEL(ctx, "orth_persistent", 0, wsum * 8.0);
-    ATP_CUDA_OK(ctx, cudaLaunchCooperativeKernel((const void *)orth_persistent_kernel<TENSOR>, dim3(next), dim3(NT), args, SMEM_BYTES, ctx->stream));
+    ATP_CUDA_OK(ctx, cudaLaunchCooperativeKernel((const void *)orth_persistent_kernel<TENSOR>, dim3(next), dim3(NT), args, SMEM_BYTES<TENSOR>, ctx->stream));
     ATP_LAUNCHED(ctx);
     return ATP_OK;
 }
