@@ -18,9 +18,11 @@
 // the tensor cores from two fp16 parts per operand (split_mma.cuh), columns of the panel scaled by powers of two to a
 // common range. The finished columns are kept as such parts: their tiles go to shared memory by cp.async, without a
 // conversion, two of them for every tile of the panel (or of C), which is fetched and cut once for two products (from fp32
-// tiles, one product per pair of fetched and cut tiles, 32768 x 1088 took 4920 us instead of 3710). The products with the factor, whose rows differ by the ratio of the column norms, from two TF32 parts. Plain
-// TF32 is not enough even for the first repetition, because what a projection leaves of an ill-conditioned panel is far
-// below 2^-11 of the panel. fp32 inputs keep every product on the fp32 units.
+// tiles, one product per pair of fetched and cut tiles, 32768 x 1088 took 4920 us instead of 3710). The products
+// with the factor run the same way: the panel's columns scaled as before, the factor's rows by the inverse and all of it to
+// its largest entry. Plain TF32 is not enough even for the first repetition, because what a projection leaves of an
+// ill-conditioned panel is far below 2^-11 of the panel.
+// fp32 inputs keep every product on the fp32 units.
 #pragma once
 #include "jacobi3.cuh"
 #include "panel_chol.cuh"
@@ -30,7 +32,7 @@ namespace orth {
 
 using j3::BLK; using j3::NT; using j3::LDA; using j3::LDB;
 constexpr int MAXSEQ = 32;
-constexpr int SYNC_WORDS = 192;   // words of Seq::sync before the SM list
+constexpr int SYNC_WORDS = 256;   // words of Seq::sync before the SM list
 constexpr int NRED = 8;           // second-level partial Gram sums (chunk ranges)
 
 struct Seq {
@@ -40,9 +42,9 @@ struct Seq {
     float *Cpart, *C, *Dpart, *W;             // tile scratch (see scratch_tiles)
     double *gpart, *gpart2;
     int *flags;
-    unsigned *sync;                           // 64 words: group barrier; 2 x 64 words: largest entry of each column of the
-                                              // panel (as bits), before the first and before the second projection; then
-                                              // one word per CTA of the group (its SM)
+    unsigned *sync;                           // 64 words: group barrier; 3 x 64 words: largest entry of each column of the
+                                              // panel (as bits), before the first projection (by panel parity) and before
+                                              // the second; then one word per CTA of the group (its SM)
     int cta0, ncta, index;                    // CTA group (on entry to launch(): ncta = the cap the scratch was
                                               // sized for); index of the sequence in its batch (noise stream)
 };
@@ -88,12 +90,6 @@ __device__ __forceinline__ void stash_tile(const TileRegs &tr, float *dst, int l
         *(float4 *)(dst + r * lds + c) = tr.v[i];             // lds is a multiple of 4 floats: 16-byte aligned
     }
 }
-__device__ __forceinline__ void load_tile(float *dst, int lds, const float *src, int ld, int rv, int cv, bool vec)
-{
-    TileRegs tr;
-    fetch_tile(tr, src, ld, rv, cv, vec);
-    stash_tile(tr, dst, lds);
-}
 
 // sum of base[0], base[stride], ..., base[(count - 1) stride] in that order, eight loads in flight
 template <typename T>
@@ -112,24 +108,20 @@ __device__ __forceinline__ T ordered_sum(const T *base, size_t stride, int count
     return s;
 }
 
-// acc += op(A) B on the units chosen by PREC: 0 fp32 FMA, 1 plain TF32, 3 split TF32.
-template <int PREC, bool A_TRANS>
+// acc += op(A) B on the fp32 units (fp32 inputs).
+template <bool A_TRANS>
 __device__ __forceinline__ void tile_mac(const float *As, int lda, const float *Bs, int ldb, int m0, int n0, float (&acc)[4][4])
 {
-    if (PREC == 3) j3::product64_acc<A_TRANS, false, 3>(As, lda, Bs, ldb, m0, n0, acc);
-    else if (PREC == 1) j3::product64_acc<A_TRANS, false, 1>(As, lda, Bs, ldb, m0, n0, acc);
-    else {
-        const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll 4
-        for (int k = 0; k < BLK; ++k) {
-            const float a0 = A_TRANS ? As[k * lda + m0 + g] : As[(m0 + g) * lda + k];
-            const float a1 = A_TRANS ? As[k * lda + m0 + g + 8] : As[(m0 + g + 8) * lda + k];
+    for (int k = 0; k < BLK; ++k) {
+        const float a0 = A_TRANS ? As[k * lda + m0 + g] : As[(m0 + g) * lda + k];
+        const float a1 = A_TRANS ? As[k * lda + m0 + g + 8] : As[(m0 + g + 8) * lda + k];
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const float2 b = *(const float2 *)(Bs + k * ldb + n0 + nt * 8 + 2 * t);
-                acc[nt][0] = fmaf(a0, b.x, acc[nt][0]); acc[nt][1] = fmaf(a0, b.y, acc[nt][1]);
-                acc[nt][2] = fmaf(a1, b.x, acc[nt][2]); acc[nt][3] = fmaf(a1, b.y, acc[nt][3]);
-            }
+        for (int nt = 0; nt < 4; ++nt) {
+            const float2 b = *(const float2 *)(Bs + k * ldb + n0 + nt * 8 + 2 * t);
+            acc[nt][0] = fmaf(a0, b.x, acc[nt][0]); acc[nt][1] = fmaf(a0, b.y, acc[nt][1]);
+            acc[nt][2] = fmaf(a1, b.x, acc[nt][2]); acc[nt][3] = fmaf(a1, b.y, acc[nt][3]);
         }
     }
 }
@@ -167,9 +159,6 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
     int *abort_flag = status + 1;
     unsigned gen = 0;
     bool alive = true;
-    // Every product needs fp32-like accuracy: a panel of an ill-conditioned iterate lies almost entirely in the span
-    // of the finished columns, and what the projection leaves (1e-4 of the panel or less) is the information kept.
-    constexpr int P_FINE = TENSOR ? 3 : 0;
     auto barrier = [&]() { alive = j3::group_barrier(sq.sync, ++gen, (unsigned)ncta, abort_flag) && alive; };
 
     // The CTA that shares an SM with rank 0 (if it belongs to this group) stays out of the work that runs beside
@@ -188,7 +177,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
 #pragma unroll 8
                 for (int r = r0; r < r1; r += 4) m = fmaxf(m, fabsf(__ldcg(sq.M + (size_t)r * ld + j0 + c)));
             }
-        if (m > 0.f) atomicMax(sq.sync + 64 + c, __float_as_uint(m));
+        if (m > 0.f) atomicMax(sq.sync + 64 + 64 * (pj & 1) + c, __float_as_uint(m));
     };
     if (TENSOR) column_max(0, rank, ncta);
     barrier();
@@ -208,6 +197,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
 
     // Scales of the panel's columns for the fp16 parts: entries of P, and of C = Q^T P, are below the column norm, i.e. below
     // sqrt(n) times the largest entry of the column; after a first apply the columns have unit norm.
+    __shared__ unsigned wmax[NT / 32];
     __shared__ __align__(16) float colscale[64], colinv[64];   // (read in 16-byte pieces)
     int half_log_n = 0;
     while ((1ll << (2 * half_log_n)) < n) ++half_log_n;
@@ -241,6 +231,46 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             hs::put4(dst, f >> 4, (f & 15) * 4, make_float4(v.x * sc.x, v.y * sc.y, v.z * sc.z, v.w * sc.w));
         }
     };
+    // P <- P W on a tile: P (fp32, in registers) times W, result in acc. W's rows undo the column scales.
+    auto times_factor = [&](const TileRegs &tr, float (&acc)[4][4]) {
+        TileRegs rw;
+        fetch_tile(rw, sq.W, 64, 64, 64, true);
+        if constexpr (!TENSOR) {
+            stash_tile(tr, sA, LDA);
+            stash_tile(rw, sB, LDB);
+            __syncthreads();
+            tile_mac<false>(sA, LDA, sB, LDB, m0, n0, acc);
+        } else {
+            float rs[4], m = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                rs[i] = colinv[(tid >> 4) + 16 * i] * QSCALE;
+                const float4 v = rw.v[i];
+                m = fmaxf(m, rs[i] * fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+            }
+            const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+            if ((tid & 31) == 0) wmax[warp] = mb;
+            put_tile(tr, htile(0), *(const float4 *)&colscale[(tid & 15) * 4]);
+            __syncthreads();
+            unsigned all = wmax[0];
+#pragma unroll
+            for (int k = 1; k < NT / 32; ++k) all = max(all, wmax[k]);
+            const float2 sc = hs::scale_for(all, 15);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float k = rs[i] * sc.x;
+                const float4 v = rw.v[i];
+                hs::put4(htile(1), (tid >> 4) + 16 * i, (tid & 15) * 4, make_float4(v.x * k, v.y * k, v.z * k, v.w * k));
+            }
+            __syncthreads();
+            hs::product64<false, false>(htile(0), htile(1), m0, n0, acc);
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[nt][e] *= sc.y;
+        }
+        __syncthreads();
+    };
     auto unscale = [&](float (&acc)[4][4]) {
         const int t2 = (tid & 3) * 2;
 #pragma unroll
@@ -273,8 +303,8 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
         while (stage >= 0 && alive) {
             int op = OP_PF, first = -1, stride = 1, arep = 0;
             bool do_factor = false, series_ok = false, with_w = false, last = false, skip = false;
-            // which scales a projection uses: 0 the panel as it came, 1 after the first projection, -1 unit columns
-            const int scale_slot = stage <= 1 ? 0 : stage <= 4 ? 1 : stage < 30 ? -1 : rep == 0 ? 0 : -1;
+            // which scales the panel's columns have: pj & 1 the panel as it came, 2 after the first projection, -1 unit columns
+            const int scale_slot = stage <= 1 ? pj & 1 : stage <= 5 || stage == 20 ? 2 : stage < 30 ? -1 : rep == 0 ? pj & 1 : -1;
             switch (stage) {
                 // overlapped order
                 case 0: op = OP_PF; first = rank; stride = ncta; skip = nj == 0; break;
@@ -303,6 +333,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             case OP_PF: {
                 // beside the last factor of a panel the other CTAs note the column maxima of the next panel
                 const bool scan = TENSOR && do_factor && stage != 3 && (stage != 33 || rep == reps - 1) && pj + 1 < npanel;
+                if (TENSOR && !do_factor && rank == 0 && tid < 64) sq.sync[192 + tid] = 0u;   // (used up by the panel before)
                 if (scan && (rank > 0 || ncta == 1)) column_max(pj + 1, max(rank - 1, 0), max(ncta - 1, 1));
                 if (do_factor && rank == 0) {
                     {   // all elements of a partial matrix in flight together
@@ -381,7 +412,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                                 fetch_tile(ra, sq.M + (size_t)(t + 1) * 64 * ld + jb * 64, ld, rv, 64, vec);
                                 fetch_tile(rb, sq.M + (size_t)(t + 1) * 64 * ld + j0, ld, rv, w, vec);
                             }
-                            tile_mac<0, true>(sA, LDB, sB, LDB, m0, n0, acc);
+                            tile_mac<true>(sA, LDB, sB, LDB, m0, n0, acc);
                             __syncthreads();
                         }
                         store_acc(sq.Cpart + (size_t)it * 4096, 64, m0, n0, acc);
@@ -459,7 +490,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                             fetch_tile(ra, sq.M + (size_t)t * 64 * ld + (jb + 1) * 64, ld, rv, 64, vec);
                             fetch_tile(rb, sq.C + (size_t)(jb + 1) * 4096, 64, 64, 64, true);
                         }
-                        tile_mac<0, false>(sA, LDA, sB, LDB, m0, n0, acc);
+                        tile_mac<false>(sA, LDA, sB, LDB, m0, n0, acc);
                         __syncthreads();
                     }
                     store_acc(sq.Dpart + (size_t)it * 4096, 64, m0, n0, acc);
@@ -467,11 +498,12 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                 barrier();
             } break;
             case OP_GRAM: {
-                // the columns' largest entries go to slot 1 before a second projection of the same panel; otherwise slot 0 has
-                // been used and is cleared for the next panel (noted beside the factor that follows)
+                // the columns' largest entries are noted before a second projection of the same panel; the slot of the panel
+                // before this one is cleared for the next panel (noted beside the factor that follows)
                 const bool note_max = TENSOR && stage == 2;
                 float4 cmax = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (TENSOR && !note_max && rank == 0 && tid < 64) sq.sync[64 + tid] = 0u;
+                if (TENSOR && rank == 0 && tid < 64) sq.sync[64 + 64 * ((pj + 1) & 1) + tid] = 0u;
+                if (TENSOR && with_w) set_scales(scale_slot);
                 for (int t = rank; t < ntile; t += ncta) {
                     const int rv = min(64, n - t * 64);
                     TileRegs ra;
@@ -493,8 +525,6 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                         for (int i = 0; i < 4; ++i) {                    // (rows and columns beyond the tile are zero in both)
                             float4 &v = ra.v[i];
                             v.x -= d[i].x; v.y -= d[i].y; v.z -= d[i].z; v.w -= d[i].w;
-                            cmax.x = fmaxf(cmax.x, fabsf(v.x)); cmax.y = fmaxf(cmax.y, fabsf(v.y));
-                            cmax.z = fmaxf(cmax.z, fabsf(v.z)); cmax.w = fmaxf(cmax.w, fabsf(v.w));
                             const int f = tid + i * NT, r = f >> 4, c = (f & 15) * 4;
                             if (!with_w && r < rv) {
                                 float *dm = sq.M + ((size_t)t * 64 + r) * ld + j0 + c;
@@ -508,13 +538,18 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                             }
                         }
                     }
-                    stash_tile(ra, sA, LDA);
-                    if (with_w) load_tile(sB, LDB, sq.W, 64, 64, 64, true);
-                    __syncthreads();
-                    if (with_w) {
-                        float acc[4][4] = {};
-                        tile_mac<P_FINE, false>(sA, LDA, sB, LDB, m0, n0, acc);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 v = ra.v[i];
+                        cmax.x = fmaxf(cmax.x, fabsf(v.x)); cmax.y = fmaxf(cmax.y, fabsf(v.y));
+                        cmax.z = fmaxf(cmax.z, fabsf(v.z)); cmax.w = fmaxf(cmax.w, fabsf(v.w));
+                    }
+                    if (!with_w) {
+                        stash_tile(ra, sA, LDA);
                         __syncthreads();
+                    } else {
+                        float acc[4][4] = {};
+                        times_factor(ra, acc);
                         const int lane = tid & 31, g = lane >> 2, tq = lane & 3;
 #pragma unroll
                         for (int nt = 0; nt < 4; ++nt)
@@ -538,7 +573,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
 #pragma unroll
                     for (int k = 0; k < 4; ++k) atomicMax(cm + (tid & 15) * 4 + k, __float_as_uint(m[k]));
                     __syncthreads();
-                    if (tid < 64 && cm[tid] > 0u) atomicMax(sq.sync + 128 + tid, cm[tid]);
+                    if (tid < 64 && cm[tid] > 0u) atomicMax(sq.sync + 192 + tid, cm[tid]);
                 }
                 barrier();
                 if (!alive) break;
@@ -553,18 +588,16 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             default: {                                                   // OP_APPLY
                 const uint64_t nseed = seed + 7919ull * (uint64_t)(pj * 2 + arep);
                 const float rscale = rsqrtf((float)n * (1.f / 3.f));     // replacement columns of about unit norm
-                if (TENSOR && rank == 0 && tid < 64) sq.sync[128 + tid] = 0u;
+                if (TENSOR) set_scales(scale_slot);
                 int fl[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) fl[k] = __ldcg(sq.flags + (tid & 15) * 4 + k);
                 for (int t = rank; t < ntile; t += ncta) {
                     const int rv = min(64, n - t * 64);
-                    load_tile(sA, LDA, sq.M + (size_t)t * 64 * ld + j0, ld, rv, w, vec);
-                    load_tile(sB, LDB, sq.W, 64, 64, 64, true);
-                    __syncthreads();
+                    TileRegs ra;
+                    fetch_tile(ra, sq.M + (size_t)t * 64 * ld + j0, ld, rv, w, vec);
                     float acc[4][4] = {};
-                    tile_mac<P_FINE, false>(sA, LDA, sB, LDB, m0, n0, acc);
-                    __syncthreads();
+                    times_factor(ra, acc);
                     store_acc(sA, LDA, m0, n0, acc);
                     __syncthreads();
                     // out row by row, four columns a thread (the flags are read once, before any store)
