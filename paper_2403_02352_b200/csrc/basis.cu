@@ -866,12 +866,13 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 } else {
                     if ((st = launch_gemm_simt<float, float, float, true, false>(ctx, gg, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_gram")) != ATP_OK) return st;
                 }
-                // pass 0 only has to make the rows graded and roughly orthogonal (scaled off-diagonals below
-                // 3e-2; 1e-2 takes a sweep more on most inputs and saves none in the second pass, 1e-1 one more there; on ill-conditioned input it stalls at the noise floor of G, hence the cap of 8 sweeps);
-                // the second pass continues the same iteration on the rotated data with the rest of the budget
+                // pass 0 only has to make the rows graded and roughly orthogonal (on ill-conditioned input it stalls at the
+                // noise floor of G, hence the cap of 8 sweeps); the second pass continues the same iteration on the rotated
+                // data with the rest of the budget. bf16: scaled off-diagonals below 3e-2 (1e-2 costs most inputs a sweep here
+                // and saves none there, 1e-1 costs one there); fp32: 1e-2 (3e-2 leaves the result at 8e-7 instead of 5e-7).
                 const int nsw0 = std::min(8, (max_sweeps + 1) / 2);
                 const int nsw = pass == 0 ? nsw0 : std::max(1, max_sweeps - nsw0);
-                const float tolc = pass == 0 ? fmaxf(tol_conv, 3e-2f) : tol_conv, tolr = pass == 0 ? 1e-3f : 0.1f * tol_conv;
+                const float tolc = pass == 0 ? (kBf16 ? 3e-2f : 1e-2f) : tol_conv, tolr = pass == 0 ? 1e-3f : 0.1f * tol_conv;
                 // fp32 inputs: the block products stay on the fp32 units (the threshold is below split-precision rounding)
                 // A sweep whose visits all stayed below tolc ends the pass, and so does a matrix that a sweep leaves below
                 // tolc (first pass) or LEFT * tolc (second: a sweep that ends by its visits still rotates what exceeds
