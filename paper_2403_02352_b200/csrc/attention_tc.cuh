@@ -1,17 +1,23 @@
-// Fused attention of 128 queries of one head on the r principal keys/values of their sequence
+// Fused attention of 256 queries of one head on the r principal keys/values of their sequence
 // (score GEMM, row softmax, value GEMM in one kernel; Sec. 4.1 closing paragraph, Eq. 1 on r keys).
 //
-//   S = Q_h K'_h^T          tcgen05.mma, accumulator in TMEM (two 128 x 128 fp32 buffers)
+//   S = Q_h K'_h^T          tcgen05.mma, accumulator in TMEM (128 x 128 fp32 per tile of 128 queries)
 //   P = exp2(S * c - m)     one thread per query row (TMEM lane = row), online maximum
-//   O += P V'_h             tcgen05.mma, accumulator 128 x d_h fp32 in TMEM
+//   O += P V'_h             tcgen05.mma, accumulator 128 x d_h fp32 in TMEM, P read from TMEM where S was
 //
 // Q and K' arrive as bf16 hi/lo pairs and the scores are accumulated from three products
 // (Qh Kh + Qh Kl + Ql Kh): with logits of magnitude 10^2 a single bf16 rounding of Q or K' moves
 // the softmax by more than the accuracy bar, the split keeps ~16 mantissa bits. P and V' are bf16.
-// Operands are staged by TMA (128-byte swizzle): Q once, then per 128-key block K'_hi, K'_lo, V'
-// through a ring of tile slots. Warp 8 issues TMA, warp 9 issues the MMAs, warps 0-7 run softmax (two
-// threads per query row, each on 64 of the 128 keys of a block), the O rescale (only when a row maximum
-// grows by more than 2^8) and the final normalisation.
+// Operands are staged by TMA (128-byte swizzle): Q_hi of two tiles of 128 queries once, then per 128-key block K'_hi, where
+// the lo products count K'_lo and the tiles' Q_lo, and V' through a ring of tile slots that both query tiles read.
+// What bounds a tile is the chain S -> load -> maximum -> exponentials (1024 cycles of the exponential unit) -> P -> value
+// product, so two tiles run side by side: warps 0-3 and 4-7 run their softmax (a thread per row with its 128 scores in
+// registers, no exchange between threads) and one tile's exponentials overlap the other's products (512 cycles each) and
+// waits. Warp 8 issues TMA, warp 9 all MMAs. O is rescaled only when a row maximum grows by more than 2^8.
+// Measured at 4096 queries, 2048 keys, 32 heads of 128: one tile per CTA, two threads per row and the maximum through
+// shared memory 228 us (3400 cycles per block and tile); two tiles with Q_lo and K'_lo always resident (a ring of one
+// block) 306; the ring of five slots below 218; the issuing threads chosen by elect.sync instead of lane == 0, with which
+// an MMA took 140 cycles to issue, 160 us (3950 cycles per block and two tiles; the products alone 2300).
 // Every mbarrier wait is bounded; on expiry the kernel records ATP_ERR_TIMEOUT and winds down.
 #pragma once
 #include "gemm_tc.cuh"
@@ -44,6 +50,12 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ float fast_exp2(float x)
 {
     float y;
@@ -53,28 +65,22 @@ __device__ __forceinline__ float fast_exp2(float x)
 
 template <int DH> struct Cfg {
     static constexpr int TILE = 128 * DH * 2;                   // one 128-row operand tile (bf16)
-    static constexpr int NSLOT = (DH == 128) ? 5 : 6;           // K'_hi / K'_lo / V' tile slots (a ring: the loads run ahead of the MMAs)
-    static constexpr int NPBUF = 2;                             // P buffers, in tensor memory (64 columns each)
-    static constexpr int OFF_Q = 0;                             // Q hi, Q lo
+    static constexpr int NSLOT = (DH == 128) ? 5 : 11;          // ring of operand tiles; a block holds at most 4 + the V' before it
+    static constexpr int OFF_Q = 0;                             // Q hi of the two tiles
     static constexpr int OFF_SLOT = 2 * TILE;
-    static constexpr int OFF_P = OFF_SLOT + NSLOT * TILE;       // (no shared-memory P any more: barriers follow the slots)
-    static constexpr int OFF_BAR = OFF_P;
-    // q, slot full/empty, s_full[2], s_free[2], p_full[2], p_free[2], o_done, xchg
-    static constexpr int NBAR = 1 + 2 * NSLOT + 2 + 2 + 2 + 2 + 1 + 1;
-    static constexpr int OFF_XCH = OFF_BAR + 8 * NBAR + 16;     // float[2 parity][2 halves][128 rows]
+    static constexpr int OFF_BAR = OFF_SLOT + NSLOT * TILE;
+    static constexpr int NBAR = 1 + 2 * NSLOT + 2 + 2 + 2;      // q, slot full / empty, S full, P full, O done (by tile)
     // no slack for aligning the base: the kernel has no static shared memory, so its dynamic window starts
-    // on a 1024-byte boundary (checked at run time); with four 32 KB slots at d_h = 128 every byte counts
-    static constexpr int SMEM = OFF_XCH + 2 * 2 * 128 * 4;
+    // on a 1024-byte boundary (checked at run time); at d_h = 128 every byte counts
+    static constexpr int SMEM = OFF_BAR + 8 * NBAR + 16;
 };
 
-// Warps 0-7: softmax (warp w and w + 4 share the TMEM lanes 32 (w & 3) .. and split the 128 keys of a
-// block in halves), warp 8: TMA, warp 9: score MMAs, warp 10: value MMAs.
 template <int DH>
-__global__ void __launch_bounds__(352)
+__global__ void __launch_bounds__(384, 1)
 attn_tc_kernel(const __grid_constant__ Batch batch, int heads, float scale_log2e, float lo_thresh, int *dev_status)
 {
     using C_ = Cfg<DH>;
-    constexpr int NS = C_::NSLOT, NP = C_::NPBUF;
+    constexpr int NS = C_::NSLOT;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     uint8_t *gbase = smem_raw;
@@ -84,257 +90,229 @@ attn_tc_kernel(const __grid_constant__ Batch batch, int heads, float scale_log2e
         return;
     }
     const uint32_t bar0 = base + C_::OFF_BAR;
-    const uint32_t b_q = bar0, b_full = bar0 + 8, b_empty = b_full + 8 * NS, b_sfull = b_empty + 8 * NS, b_sfree = b_sfull + 16,
-                   b_pfull = b_sfree + 16, b_pfree = b_pfull + 16, b_odone = b_pfree + 16, b_xchg = b_odone + 8;
+    const uint32_t b_q = bar0, b_full = bar0 + 8, b_empty = b_full + 8 * NS, b_sfull = b_empty + 8 * NS, b_pfull = b_sfull + 16,
+                   b_odone = b_pfull + 16;
     uint32_t *tmem_slot = (uint32_t *)(gbase + C_::OFF_BAR + 8 * C_::NBAR);
-    float *xch = (float *)(gbase + C_::OFF_XCH);
     volatile int &abort_flag = *(volatile int *)(tmem_slot + 1);
 
-    // work item: (sequence, query tile) from blockIdx.x, head from blockIdx.y
+    // work item: (sequence, 256 queries) from blockIdx.x, head from blockIdx.y
     int si = 0;
 #pragma unroll 1
     for (int i = 1; i < batch.count; ++i) if ((int)blockIdx.x >= batch.s[i].tile0) si = i;
     const Seq &sq = batch.s[si];
-    const int q0 = ((int)blockIdx.x - sq.tile0) * 128;
+    const int q0 = ((int)blockIdx.x - sq.tile0) * 256;
+    const int ntile = q0 + 128 < sq.L ? 2 : 1;                  // query tiles of this CTA
     const int head = blockIdx.y;
     const int col0 = head * DH;
     const int nblk = (sq.r + 127) / 128;
-    // The lo terms of a key block matter only while |q| |k| 2^-8 * scale can move a logit: a (query tile, key
-    // block) pair whose largest norms stay below the threshold gets the single product Qh Kh^T.
-    const float *km = sq.kmax + (size_t)head * nblk;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         abort_flag = 0;
         mbar_init(b_q, 1);
         for (int s = 0; s < NS; ++s) { mbar_init(b_full + 8 * s, 1); mbar_init(b_empty + 8 * s, 1); }
-        mbar_init(b_sfull, 1); mbar_init(b_sfull + 8, 1);
-        mbar_init(b_sfree, 8); mbar_init(b_sfree + 8, 8);
-        mbar_init(b_pfull, 8); mbar_init(b_pfull + 8, 8);
-        mbar_init(b_pfree, 1); mbar_init(b_pfree + 8, 1);
-        mbar_init(b_odone, 1); mbar_init(b_xchg, 8);
+        for (int t = 0; t < 2; ++t) { mbar_init(b_sfull + 8 * t, 1); mbar_init(b_pfull + 8 * t, 4); mbar_init(b_odone + 8 * t, 1); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 9) tmem_alloc(smem_u32(tmem_slot), 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = *tmem_slot;                      // tile t: S (then P) at 256 t, O at 256 t + 128
     pdl_wait();                                                 // set-up done; from here on memory of the launch before is read
     pdl_trigger();
-    const float qm = *((volatile const float *)sq.qmax + (size_t)head * ((sq.L + 127) / 128) + (q0 >> 7));
-    const uint32_t t_s0 = tmem_base, t_o = tmem_base + 256, t_p0 = tmem_base + 384;   // S0 S1 | O | P0 P1
+    // The lo terms of a key block matter only while |q| |k| 2^-8 * scale can move a logit: a (query tile, key
+    // block) pair whose largest norms stay below the threshold gets the single product Qh Kh^T.
+    const volatile float *qmp = sq.qmax + (size_t)head * ((sq.L + 127) / 128) + (q0 >> 7);
+    const float qm0 = qmp[0], qm1 = ntile == 2 ? qmp[1] : 0.f;
+    const float *km = sq.kmax + (size_t)head * nblk;
+    const float qmx = fmaxf(qm0, qm1);
 
+    // 384 threads start with 168 registers each; 128 x 80 + 256 x 208 stays within those 64512
+    if (warp >= 8) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
     if (warp == 8) {
-        if (lane == 0) {
-            mbar_expect_tx(b_q, 2 * C_::TILE);
+        if (elect_one()) {
+            mbar_expect_tx(b_q, ntile * C_::TILE);
+            for (int t = 0; t < ntile; ++t)
 #pragma unroll
-            for (int c = 0; c < DH / 64; ++c) {
-                tma_load_2d(base + C_::OFF_Q + c * 16384, &sq.qh, col0 + 64 * c, q0, b_q);
-                tma_load_2d(base + C_::OFF_Q + C_::TILE + c * 16384, &sq.ql, col0 + 64 * c, q0, b_q);
-            }
-            int li = 0;                                   // running load index: K'_hi, K'_lo, V' per block
-            for (int j = 0; j < nblk; ++j) {
-                for (int which = 0; which < 3; ++which, ++li) {
-                    const int s = li % NS, n = li / NS;
-                    if (n >= 1 && !mbar_wait(b_empty + 8 * s, (n - 1) & 1, &abort_flag)) { j = nblk; break; }
-                    const uint32_t dst = base + C_::OFF_SLOT + s * C_::TILE;
-                    const CUtensorMap *m = which == 0 ? &sq.kh : (which == 1 ? &sq.kl : &sq.v);
-                    if (which == 1 && !(qm * km[j] > lo_thresh)) { mbar_arrive(b_full + 8 * s); continue; }   // K'_lo not needed
-                    mbar_expect_tx(b_full + 8 * s, C_::TILE);
+                for (int c = 0; c < DH / 64; ++c)
+                    tma_load_2d(base + C_::OFF_Q + t * C_::TILE + c * 16384, &sq.qh, col0 + 64 * c, q0 + 128 * t, b_q);
+            int li = 0;                                   // running index of the ring: K'_hi, [K'_lo, Q lo of each tile], V' per block
+            auto load = [&](const CUtensorMap *m, int row) -> bool {
+                const int s = li % NS, n = li / NS;
+                if (n >= 1 && !mbar_wait(b_empty + 8 * s, (n - 1) & 1, &abort_flag)) return false;
+                mbar_expect_tx(b_full + 8 * s, C_::TILE);
 #pragma unroll
-                    for (int c = 0; c < DH / 64; ++c) tma_load_2d(dst + c * 16384, m, col0 + 64 * c, j * 128, b_full + 8 * s);
+                for (int c = 0; c < DH / 64; ++c)
+                    tma_load_2d(base + C_::OFF_SLOT + s * C_::TILE + c * 16384, m, col0 + 64 * c, row, b_full + 8 * s);
+                ++li;
+                return true;
+            };
+            bool ok = true;
+            for (int j = 0; j < nblk && ok; ++j) {
+                ok = load(&sq.kh, j * 128);
+                if (ok && qmx * km[j] > lo_thresh) {
+                    ok = load(&sq.kl, j * 128);
+                    for (int t = 0; t < ntile && ok; ++t) ok = load(&sq.ql, q0 + 128 * t);
                 }
+                if (ok) ok = load(&sq.v, j * 128);
             }
         }
     } else if (warp == 9) {
-        if (lane == 0) {
-            constexpr uint32_t idesc_s = instr_desc(128, 128, false, false);
-            const uint32_t q_hi = base + C_::OFF_Q, q_lo = q_hi + C_::TILE;
+        if (elect_one()) {
+            constexpr uint32_t idesc_s = instr_desc(128, 128, false, false), idesc_o = instr_desc(128, DH, false, true);
             bool ok = mbar_wait(b_q, 0, &abort_flag);
             tc_fence_after();
-            // S_j for block j into buffer j & 1: Qh Kh^T (+ Qh Kl^T + Ql Kh^T)
-            auto issue_s = [&](int j) -> bool {
-                const int lk = 3 * j, sh = lk % NS, sl = (lk + 1) % NS;
-                const bool need_lo = qm * km[j] > lo_thresh;
-                if (j >= 2 && !mbar_wait(b_sfree + 8 * (j & 1), ((j >> 1) - 1) & 1, &abort_flag)) return false;
-                if (!mbar_wait(b_full + 8 * sh, (lk / NS) & 1, &abort_flag)) return false;
-                if (!mbar_wait(b_full + 8 * sl, ((lk + 1) / NS) & 1, &abort_flag)) return false;
-                tc_fence_after();
-                const uint32_t kh = base + C_::OFF_SLOT + sh * C_::TILE, kl = base + C_::OFF_SLOT + sl * C_::TILE;
-                const uint32_t d = t_s0 + 128 * (j & 1);
+            // the descriptors of a tile differ from that of its first 16 columns by the address alone (in units of 16 bytes)
+            const uint64_t slot0 = smem_desc(base + C_::OFF_SLOT, 16, 1024), vslot0 = smem_desc(base + C_::OFF_SLOT, 16384, 1024),
+                           q0d = smem_desc(base + C_::OFF_Q, 16, 1024);
+            auto full = [&](int k) -> bool { return mbar_wait(b_full + 8 * (k % NS), (k / NS) & 1, &abort_flag); };
+            auto slot = [&](int k) -> uint64_t { return slot0 + (uint64_t)(k % NS) * (C_::TILE >> 4); };
+            auto scores = [&](uint32_t d, uint64_t a, uint64_t b, uint32_t add) {
 #pragma unroll
                 for (int kk = 0; kk < DH / 16; ++kk) {
-                    const uint32_t off = (kk >> 2) * 16384 + (kk & 3) * 32;
-                    const uint64_t aqh = smem_desc(q_hi + off, 16, 1024), aql = smem_desc(q_lo + off, 16, 1024);
-                    const uint64_t bkh = smem_desc(kh + off, 16, 1024), bkl = smem_desc(kl + off, 16, 1024);
-                    umma_bf16(d, aqh, bkh, idesc_s, kk > 0 ? 1u : 0u);
-                    if (need_lo) {
-                        umma_bf16(d, aqh, bkl, idesc_s, 1u);
-                        umma_bf16(d, aql, bkh, idesc_s, 1u);
-                    }
+                    const uint64_t off = ((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
+                    umma_bf16(d, a + off, b + off, idesc_s, kk > 0 ? 1u : add);
                 }
-                umma_commit(b_empty + 8 * sh);
-                umma_commit(b_empty + 8 * sl);
-                umma_commit(b_sfull + 8 * (j & 1));
+            };
+            // S of tile t for the block whose operands start at ring index k: Qh Kh^T (+ Qh Kl^T + Ql Kh^T); the last tile
+            // frees them. The commit that announces S also covers the value product issued before it, so O is at rest when a
+            // tile's softmax sees its S.
+            auto issue_s = [&](int t, int k, int cnt, bool lo) -> bool {
+                if (t == 0) {
+                    for (int i = 0; i < cnt; ++i) if (!full(k + i)) return false;
+                    tc_fence_after();
+                }
+                const uint32_t d = tmem_base + 256 * t;
+                const uint64_t qh = q0d + (uint64_t)t * (C_::TILE >> 4);
+                scores(d, qh, slot(k), 0u);
+                if (lo) {
+                    scores(d, qh, slot(k + 1), 1u);
+                    scores(d, slot(k + 2 + t), slot(k), 1u);
+                }
+                umma_commit(b_sfull + 8 * t);
+                if (t == ntile - 1) for (int i = 0; i < cnt; ++i) umma_commit(b_empty + 8 * ((k + i) % NS));
                 return true;
             };
-            for (int j = 0; j < nblk && ok; ++j) ok = issue_s(j);
-        }
-    } else if (warp == 10) {
-        // the value MMAs have their own issuing thread: they are independent of the score MMAs of the next
-        // block (other accumulator), and two instruction streams let the tensor pipe take them in either order
-        if (lane == 0) {
-            constexpr uint32_t idesc_o = instr_desc(128, DH, false, true);
-            bool ok = true;
+            bool any_lo = qmx * km[0] > lo_thresh;
+            int k = 0, cnt = any_lo ? 2 + ntile : 1;              // ring index and number of the score operands of the next block
+            for (int t = 0; t < ntile && ok; ++t) ok = issue_s(t, k, cnt, any_lo && (t ? qm1 : qm0) * km[0] > lo_thresh);
             for (int j = 0; j < nblk && ok; ++j) {
-                // O += P_j V_j
-                const int lv = 3 * j + 2, sv = lv % NS, pb = j % NP, pu = j / NP;
-                if (!mbar_wait(b_full + 8 * sv, (lv / NS) & 1, &abort_flag)) { ok = false; break; }
-                if (!mbar_wait(b_pfull + 8 * pb, pu & 1, &abort_flag)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t tp = t_p0 + 64 * pb, vv = base + C_::OFF_SLOT + sv * C_::TILE;
+                const int kv = k + cnt;                           // V' of block j
+                k = kv + 1;
+                const float kn = j + 1 < nblk ? km[j + 1] : 0.f;
+                any_lo = qmx * kn > lo_thresh;
+                cnt = any_lo ? 2 + ntile : 1;
+                for (int t = 0; t < ntile && ok; ++t) {
+                    // O += P_j V_j, then the scores of the next block over the same columns
+                    if (t == 0 && !full(kv)) { ok = false; break; }
+                    if (!mbar_wait(b_pfull + 8 * t, j & 1, &abort_flag)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t tp = tmem_base + 256 * t, to = tp + 128;
+                    const uint64_t vv = vslot0 + (uint64_t)(kv % NS) * (C_::TILE >> 4);
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {                 // A = P from tensor memory: 16 keys = 8 columns per step
-                    const uint64_t bv = smem_desc(vv + kk * 2048, 16384, 1024);
-                    umma_bf16_ts(t_o, tp + 8 * kk, bv, idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 0; kk < 8; ++kk)               // A = P from tensor memory: 16 keys = 8 columns per step
+                        umma_bf16_ts(to, tp + 8 * kk, vv + kk * (2048 >> 4), idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
+                    if (t == ntile - 1) umma_commit(b_empty + 8 * (kv % NS));
+                    if (j + 1 < nblk) ok = issue_s(t, k, cnt, any_lo && (t ? qm1 : qm0) * kn > lo_thresh);
+                    else umma_commit(b_odone + 8 * t);
                 }
-                umma_commit(b_empty + 8 * sv);
-                umma_commit(b_pfree + 8 * pb);
-                umma_commit(b_odone);
             }
         }
-    } else {
-        // softmax / correction / epilogue: thread = (query row, half of the keys of a block)
-        const int quad = warp & 3, half = warp >> 2;
+    } else if ((warp >> 2) < ntile) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
+        // softmax / correction / epilogue: thread = query row of tile t
+        const int t = warp >> 2, quad = warp & 3;
         const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
-        const int row = quad * 32 + lane;
-        constexpr int OC = DH / 2;                                   // O columns owned by this thread
+        const uint32_t t_s = tmem_base + 256 * t + lane_addr, t_o = t_s + 128;
+        const int row = q0 + 128 * t + quad * 32 + lane;
         float m_used = -INFINITY, l_sum = 0.f;
         bool ok = true;
-        int ok_i = 0;
         auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {   // lane 0 polls, the warp follows
+            int ok_i = 0;
             if (lane == 0) ok_i = mbar_wait(bar, parity, &abort_flag) ? 1 : 0;
             return __shfl_sync(0xffffffffu, ok_i, 0) != 0;
         };
         for (int j = 0; j < nblk; ++j) {
-            ok = wait_all(b_sfull + 8 * (j & 1), (j >> 1) & 1);
+            ok = wait_all(b_sfull + 8 * t, j & 1);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t t_s = t_s0 + 128 * (j & 1) + lane_addr + half * 64;
-            const int kvalid = sq.r - j * 128 - half * 64;            // keys of this half-block that exist
-            // the 64 scores of this half go to registers in one go (both loads in flight), which frees the S
-            // buffer for the score products of block j + 2 before any arithmetic here
-            uint32_t sa[32], sb[32];
-            tmem_ld32_nowait(t_s, sa);
-            tmem_ld32_nowait(t_s + 32, sb);
+            const int kvalid = sq.r - j * 128;                        // keys of this block that exist
+            uint32_t s[4][32];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) tmem_ld32_nowait(t_s + 32 * c, s[c]);
             tmem_ld_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(b_sfree + 8 * (j & 1));
             // maximum of the raw scores (the scale is positive: applied once); four independent chains
             float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-            if (kvalid >= 64) {
+            if (kvalid >= 128) {
 #pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(sa[i]));
-                    mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(sb[i]));
-                }
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(s[c][i]));
             } else {
 #pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    if (i < kvalid) mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(sa[i]));
-                    if (32 + i < kvalid) mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(sb[i]));
-                }
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        if (32 * c + i >= kvalid) s[c][i] = 0xff800000u;      // weight 0
+                        mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(s[c][i]));
+                    }
             }
-            float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-            // exchange with the thread that holds the other half of the row
-            float *xb = xch + (j & 1) * 256;
-            xb[half * 128 + row] = mx;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(b_xchg);
-            ok = wait_all(b_xchg, j & 1);
-            if (!ok) break;
-            mx = fmaxf(mx, xb[(half ^ 1) * 128 + row]) * scale_log2e;
+            const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * scale_log2e;
             // the exponent offset only moves when the maximum grew by more than 8 (factor 256)
             float alpha = 1.f;
-            bool grow = (mx > m_used + 8.f) || (j == 0);
+            const bool grow = (mx > m_used + 8.f) || (j == 0);
             if (grow) { alpha = (j == 0) ? 0.f : fast_exp2(m_used - mx); m_used = mx; }
             if (j > 0 && __any_sync(0xffffffffu, grow)) {
-                // O must be quiescent: P V of block j-1 done (block j's waits for the P written below)
-                ok = wait_all(b_odone, (j - 1) & 1);
-                if (!ok) break;
-                tc_fence_after();
 #pragma unroll
-                for (int c = 0; c < OC; c += 32) {
+                for (int c = 0; c < DH; c += 32) {
                     uint32_t rr[32];
-                    tmem_ld32(t_o + lane_addr + half * OC + c, rr);
+                    tmem_ld32(t_o + c, rr);
 #pragma unroll
                     for (int i = 0; i < 32; ++i) rr[i] = __float_as_uint(__uint_as_float(rr[i]) * alpha);
-                    tmem_st32(t_o + lane_addr + half * OC + c, rr);
+                    tmem_st32(t_o + c, rr);
                 }
-                tc_fence_before();
             }
             l_sum *= alpha;
-            // the P buffer is free once the value MMAs that read it (block j - NP) have finished
-            const int pb = j % NP, pu = j / NP;
-            if (pu > 0) {
-                ok = wait_all(b_pfree + 8 * pb, (pu - 1) & 1);
-                if (!ok) break;
-            }
-            // P = exp2(s * c - m) as bf16 pairs into tensor memory (this half = 32 columns of the P buffer: the A
-            // operand of the value MMA); the row sum is taken from the unrounded values
+            // P = exp2(s * c - m) as bf16 pairs into the columns S came from (64 of them: the A operand of the value MMA); the
+            // row sum is taken from the unrounded values
             const float neg_m = -m_used;
             float ls[4] = {0.f, 0.f, 0.f, 0.f};
-            uint32_t packed[32];
 #pragma unroll
-            for (int c = 0; c < 64; c += 32) {
-                const uint32_t (&rr)[32] = (c == 0) ? sa : sb;
+            for (int hf = 0; hf < 2; ++hf) {
+                uint32_t packed[32];
 #pragma unroll
-                for (int i = 0; i < 32; i += 2) {
-                    float p0 = fast_exp2(fmaf(__uint_as_float(rr[i]), scale_log2e, neg_m));
-                    float p1 = fast_exp2(fmaf(__uint_as_float(rr[i + 1]), scale_log2e, neg_m));
-                    if (kvalid < 64) {
-                        if (c + i >= kvalid) p0 = 0.f;
-                        if (c + i + 1 >= kvalid) p1 = 0.f;
-                    }
+                for (int i = 0; i < 64; i += 2) {
+                    const float p0 = fast_exp2(fmaf(__uint_as_float(s[2 * hf + (i >> 5)][i & 31]), scale_log2e, neg_m));
+                    const float p1 = fast_exp2(fmaf(__uint_as_float(s[2 * hf + (i >> 5)][(i & 31) + 1]), scale_log2e, neg_m));
                     ls[(i >> 1) & 3] += p0 + p1;
-                    __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
-                    packed[(c + i) >> 1] = *(uint32_t *)&h;
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
+                    packed[i >> 1] = *(const uint32_t *)&h;
                 }
+                tmem_st32(t_s + 32 * hf, packed);
             }
             l_sum += (ls[0] + ls[1]) + (ls[2] + ls[3]);
-            tmem_st32(t_p0 + 64 * pb + lane_addr + half * 32, packed);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(b_pfull + 8 * pb);
+            if (lane == 0) mbar_arrive(b_pfull + 8 * t);
         }
-        // epilogue: O / l, with l summed over the two halves of the row
-        if (ok) {
-            float *xb = xch + (nblk & 1) * 256;
-            xb[half * 128 + row] = l_sum;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(b_xchg);
-            ok = wait_all(b_xchg, nblk & 1);
-            if (ok) l_sum += xb[(half ^ 1) * 128 + row];
-        }
-        if (ok) ok = wait_all(b_odone, (nblk - 1) & 1);
+        // epilogue: O / l
+        if (ok) ok = wait_all(b_odone + 8 * t, 0);
         tc_fence_after();
         if (ok) {
             const float inv = 1.f / l_sum;
-            const int grow_ = q0 + row;
-            __nv_bfloat16 *dst = (__nv_bfloat16 *)sq.O + (size_t)grow_ * sq.ldo + col0 + half * OC;
+            __nv_bfloat16 *dst = (__nv_bfloat16 *)sq.O + (size_t)row * sq.ldo + col0;
 #pragma unroll
-            for (int c = 0; c < OC; c += 32) {
+            for (int c = 0; c < DH; c += 32) {
                 uint32_t rr[32];
-                tmem_ld32(t_o + lane_addr + half * OC + c, rr);
-                if (grow_ < sq.L) {
+                tmem_ld32(t_o + c, rr);
+                if (row < sq.L) {
 #pragma unroll
                     for (int i = 0; i < 32; i += 8) {
                         __nv_bfloat162 h[4];
 #pragma unroll
-                        for (int t = 0; t < 4; ++t)
-                            h[t] = __floats2bfloat162_rn(__uint_as_float(rr[i + 2 * t]) * inv, __uint_as_float(rr[i + 2 * t + 1]) * inv);
+                        for (int k = 0; k < 4; ++k)
+                            h[k] = __floats2bfloat162_rn(__uint_as_float(rr[i + 2 * k]) * inv, __uint_as_float(rr[i + 2 * k + 1]) * inv);
                         *(uint4 *)(dst + c + i) = *(uint4 *)h;
                     }
                 }
@@ -434,7 +412,7 @@ static atp_status launch(atp_ctx *ctx, const std::vector<HostSeq> &seqs, int hea
                                      nbt.total_tiles};
             nbt.total_tiles += ceil_div(h.L, 128) + ceil_div(h.r, 128);
             nbytes += 2.0 * (h.L + h.r) * h.dp;
-            b.total_tiles += ceil_div(h.L, 128);
+            b.total_tiles += ceil_div(h.L, 256);
             b.count++;
             flops += 4.0 * h.L * h.r * h.dp;                                   // algorithmic: one score and one value product
             bytes += 2.0 * (2.0 * h.L * h.dp + 3.0 * h.r * h.dp) + 2.0 * h.L * h.dp;
@@ -450,7 +428,7 @@ static atp_status launch(atp_ctx *ctx, const std::vector<HostSeq> &seqs, int hea
         // weights exp(s) of such a pair are off by at most 0.8 %, and by far less on average - inside the
         // 2e-2 bar on O with room to spare; the strong principal keys (the first blocks) keep all three products.
         const float lo_thresh = 2.0f / scale;
-        ATP_CUDA_OK(ctx, launch_pdl(attn_tc_kernel<DH>, dim3(b.total_tiles, heads), dim3(352), C_::SMEM, ctx->stream, b, heads,
+        ATP_CUDA_OK(ctx, launch_pdl(attn_tc_kernel<DH>, dim3(b.total_tiles, heads), dim3(384), C_::SMEM, ctx->stream, b, heads,
                                     scale * 1.4426950408889634f, lo_thresh, ctx->dev_status));
         ATP_LAUNCHED(ctx);
     }
