@@ -72,6 +72,14 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(dst), "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
+// One lane of a converged warp. The compiler knows the branch to be taken by a single thread: with lane == 0 it guards every
+// tcgen05 instruction against several active lanes, and issuing an MMA took 140 cycles.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols)
 {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols) : "memory");
@@ -269,7 +277,7 @@ gemm_tc_kernel(const __grid_constant__ Batch<P> batch, GemmEpi epi, int *dev_sta
     uint32_t *tmem_slot = (uint32_t *)(gbase + S * C_::STAGE_BYTES + 8 * (2 * S + 4));
     __shared__ int abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t rank = CG == 2 ? cluster_rank() : 0u;
     const int first = (int)blockIdx.x / CG, step = (int)gridDim.x / CG, total = batch.total_tiles;
     if (threadIdx.x == 0) {
@@ -303,7 +311,7 @@ gemm_tc_kernel(const __grid_constant__ Batch<P> batch, GemmEpi epi, int *dev_sta
     };
 
     if (warp == EW) {
-        if (lane == 0) {
+        if (elect_one()) {
             int ks = 0;                                          // stages filled so far
             bool ok = true;
             for (int t = first; t < total && ok; t += step) {
@@ -349,7 +357,7 @@ gemm_tc_kernel(const __grid_constant__ Batch<P> batch, GemmEpi epi, int *dev_sta
             }
         }
     } else if (warp == EW + 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             constexpr uint32_t idesc = instr_desc(CG * BM, C_::NACC, A_MN, !B_KMAJ);
             bool ok = true;
             int ks = 0, it = 0;
