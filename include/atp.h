@@ -171,7 +171,7 @@ ATP_API atp_status atp_input_norm(atp_ctx *ctx, const atp_mat *X, const atp_mat 
  * one-sided on the rows themselves with opts->jacobi_block = 1) - not by a full SVD - so
  * the subspace is the optimal one up to the range finder's error; opts->power_iters trades passes
  * over X for that. The Jacobi sweeps stop on a device-side convergence test (largest scaled
- * off-diagonal <= 1e-6 for f32, 3e-5 for bf16); opts->max_sweeps bounds them, and a sequence that
+ * off-diagonal <= 1e-6 for f32, 3e-4 for bf16); opts->max_sweeps bounds them, and a sequence that
  * has not converged by then raises ATP_ERR_NOT_CONVERGED on the device status word.
  * Sign of each component: sum of the column of U_r >= 0; if that sum is within 1e-6*sqrt(L_b) of
  * zero, the largest-magnitude entry of the row of X_r is positive.
