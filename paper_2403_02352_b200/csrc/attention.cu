@@ -231,7 +231,7 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
             const int ldq = (int)align_up((size_t)dp, 8);
             // rotary positions: K = U_r K' is rotated in the epilogue of its GEMM and goes back as K'_rot = U_r^T K. K' and K
             // travel as bf16 triples (24 mantissa bits, so nothing is lost against fp32); the scratch of the fp32 path holds them.
-            // Q is rotated in the epilogue of the GEMM that makes it. (8 x 1024 ragged, 32 heads of 128: 1749 -> 543 us; the
+            // Q is rotated in the epilogue of the GEMM that makes it. (8 x 1024 ragged, 32 heads of 128: 1749 -> 560 us; the
             // two extra contractions ran on the fp32 units, the angles were formed again for every head.)
             __nv_bfloat16 *K1[3] = {(__nv_bfloat16 *)pl.Kp, (__nv_bfloat16 *)pl.Qp, (__nv_bfloat16 *)pl.Vp};
             __nv_bfloat16 *Kr[3] = {(__nv_bfloat16 *)pl.Q, (__nv_bfloat16 *)pl.Q + (size_t)tl * ldq, (__nv_bfloat16 *)pl.Kf};

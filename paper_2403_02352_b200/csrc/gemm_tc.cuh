@@ -73,7 +73,8 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
                  ::"r"(dst), "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
 // One lane of a converged warp. The compiler knows the branch to be taken by a single thread: with lane == 0 it guards every
-// tcgen05 instruction against several active lanes, and issuing an MMA took 140 cycles.
+// tcgen05 instruction against several active lanes, and issuing an MMA took 140 cycles (SwiGLU of 4096 rows at r 2048: 586 ->
+// 555 us). Fetching the tensor maps ahead of the first copy (prefetch.tensormap) gave nothing measurable.
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
@@ -524,12 +525,6 @@ struct HostProblem {
     const void *B3 = nullptr;     // third part of B
     void *C3 = nullptr;           // third part of C
 };
-
-static inline bool operands_ok(const HostProblem &h)
-{
-    auto al = [](const void *p) { return ((uintptr_t)p & 15) == 0; };
-    return al(h.A) && al(h.B) && (!h.B2 || al(h.B2)) && (h.lda % 8 == 0) && (h.ldb % 8 == 0) && h.M > 0 && h.N > 0 && h.K > 0;
-}
 
 template <int CG, bool A_MN, int NB, int OUT, bool B_KMAJ, bool SPLIT_A, bool DUAL, int P>
 static atp_status launch_form(atp_ctx *ctx, const HostProblem *probs, int count, GemmEpi epi, const char *tag)

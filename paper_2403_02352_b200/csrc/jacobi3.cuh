@@ -9,7 +9,7 @@
 //   pivot : per pair, the 64 x 64 pivot block is rotated on chip by cyclic Jacobi (first step of a sweep: all
 //           2016 pairs of its 64 rows once, in 63 rounds; other steps: the 1024 pairs across its two blocks, in
 //           32 rounds). The block lives in registers (see "pivot phase" below); a round is a rotation per row
-//           pair, two block barriers and a shift of the pairing. The accumulated row transform Vt (64 x 64)
+//           pair, one block barrier and a shift of the pairing. The accumulated row transform Vt (64 x 64)
 //           is published. The pivot block of the NEXT step is formed on chip from the matrix before this step's
 //           update (pivot_form), so the chain of pivot solves runs beside the update and never waits for it.
 //   apply : every 64 x 64 block (p, q) of G becomes Vt_p G_pq Vt_q^T (upper triangle computed, mirror
@@ -499,61 +499,7 @@ __device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *
 }
 
 // ---- apply phase -------------------------------------------------------------------------------
-// x = hi + lo + (less than 2^-21 |x|) with hi and lo in TF32 (low 13 mantissa bits zero): hi is x cut to TF32, lo
-// the remainder cut the same way. Two logic operations and one subtraction; the cvt.rna.tf32 conversion would
-// round instead of cut, but it is a slow-path instruction and bounded the whole product (2997 -> 2273 cycles).
-__device__ __forceinline__ void split_tf32(float x, uint32_t &hi, uint32_t &lo)
-{
-    hi = __float_as_uint(x) & 0xffffe000u;
-    lo = __float_as_uint(x - __uint_as_float(hi)) & 0xffffe000u;
-}
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2])
-{
-    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-// acc (this warp's 16 x 32 part of a 64 x 64 result, rows m0.., columns n0..) += op(A) * op(B), K = 64, NPASS = 3 (split
-// precision: x = hi + lo with both parts in TF32, product = lo*hi + hi*lo + hi*hi; the lo*lo term is below fp32 rounding) or
-// 1 (plain TF32, ~2^-11 relative per term). A_TRANS: A[m][k] = As[k * lda + m] (use stride LDB = 72);
-// otherwise As[m * lda + k] (stride LDA = 68). B[k][n] = Bs[k * ldb + n], or Bs[n * ldb + k] when B_TRANS.
-template <bool A_TRANS, bool B_TRANS, int NPASS>
-__device__ __forceinline__ void product64_acc(const float *As, int lda, const float *Bs, int ldb, int m0, int n0, float (&acc)[4][4])
-{
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-#pragma unroll 2
-    for (int k0 = 0; k0 < BLK; k0 += 8) {
-        float af[4];
-        if (A_TRANS) {
-            af[0] = As[(k0 + t) * lda + m0 + g]; af[1] = As[(k0 + t) * lda + m0 + g + 8];
-            af[2] = As[(k0 + t + 4) * lda + m0 + g]; af[3] = As[(k0 + t + 4) * lda + m0 + g + 8];
-        } else {
-            af[0] = As[(m0 + g) * lda + k0 + t]; af[1] = As[(m0 + g + 8) * lda + k0 + t];
-            af[2] = As[(m0 + g) * lda + k0 + t + 4]; af[3] = As[(m0 + g + 8) * lda + k0 + t + 4];
-        }
-        uint32_t ah[4], al[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (NPASS == 3) split_tf32(af[i], ah[i], al[i]);
-            else { ah[i] = __float_as_uint(af[i]); al[i] = 0u; }
-        }
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int n = n0 + nt * 8 + g;
-            float b0, b1;
-            if (B_TRANS) { b0 = Bs[n * ldb + k0 + t]; b1 = Bs[n * ldb + k0 + t + 4]; }
-            else { b0 = Bs[(k0 + t) * ldb + n]; b1 = Bs[(k0 + t + 4) * ldb + n]; }
-            uint32_t bh[2], bl[2];
-            if (NPASS == 3) { split_tf32(b0, bh[0], bl[0]); split_tf32(b1, bh[1], bl[1]); }
-            else { bh[0] = __float_as_uint(b0); bh[1] = __float_as_uint(b1); }
-            if (NPASS == 3) { mma_tf32(acc[nt], al, bh); mma_tf32(acc[nt], ah, bl); }
-            mma_tf32(acc[nt], ah, bh);
-        }
-    }
-}
-
-// The same product on the fp32 FMA units, with the ownership layout of the tensor-core version (this
+// A 64^3 product on the fp32 FMA units: B[k][n] = Bs[k * ldb + n], or Bs[n * ldb + k] when B_TRANS; rows of A at stride LDA (this
 // thread: rows m0 + g and m0 + g + 8, columns n0 + 8 nt + 2 t, + 1). Used for fp32 inputs, whose
 // convergence threshold (1e-6) sits below the rounding of the split-precision product (~2^-21).
 template <bool B_TRANS>

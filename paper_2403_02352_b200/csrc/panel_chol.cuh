@@ -175,6 +175,27 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, flo
 }
 
 
+// acc (a warp's 16 x 32 part of a 64 x 64 result, rows m0.., columns n0..) += E E, TF32 parts of the entries (2^-10), E symmetric:
+// thread holds rows m0 + g, + 8, columns n0 + 8 nt + 2 t, + 1.
+__device__ __forceinline__ void square64_tf32(const float *Es, int ld, int m0, int n0, float (&acc)[4][4])
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+#pragma unroll 2
+    for (int k0 = 0; k0 < 64; k0 += 8) {
+        uint32_t a[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = __float_as_uint(Es[(k0 + t + 4 * (i >> 1)) * ld + m0 + g + 8 * (i & 1)]);
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt) {
+            float (&d)[4] = acc[nt];
+            const int n = n0 + nt * 8 + g;
+            const uint32_t b0 = __float_as_uint(Es[(k0 + t) * ld + n]), b1 = __float_as_uint(Es[(k0 + t + 4) * ld + n]);
+            asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+        }
+    }
+}
+
 // Orthonormalising factor of a panel that is already close to orthonormal (the second Gram-Schmidt repetition):
 // with the Gram matrix scaled to unit diagonal, D^-1/2 G D^-1/2 = I + E, the symmetric factor
 //   W = D^-1/2 (I - E/2 + 3/8 E^2)          (P W has orthonormal columns up to 5/16 |E|^3)
@@ -225,7 +246,7 @@ __device__ __noinline__ bool lowdin_64(const double *Gs, int n, float *Es, float
     // E^2 (E is symmetric); this warp: rows m0 .. + 15, columns n0 .. + 31
     const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32;
     float acc[4][4] = {};
-    j3::product64_acc<true, false, 1>(Es, LDE, Es, LDE, m0, n0, acc);
+    square64_tf32(Es, LDE, m0, n0, acc);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int r = m0 + g + 8 * h;
