@@ -95,10 +95,9 @@ class ClockSampler:
 
 ALT_INNER = 2        # rounds per component of Algorithm 1, as the paper runs it
 
-# DRAM bytes (read + write) of one launch of the dominant kernels, from one ncu pass on the same command
-# (profiles/ncu_metrics_llama7b_bf16_r2048.md); other workloads / kernels: no capture, null.
-NCU_DRAM_BYTES_PER_LAUNCH = {("llama7b_bf16", 2048, "jacobi_persistent"): 33.7e6,
-                             ("llama7b_bf16", 2048, "orth_persistent"): 67.2e6}
+# DRAM bytes (read + write) of one launch of the dominant kernel, from an ncu capture of the same workload
+# (mean of the two passes of a rotation); other workloads / kernels: no capture, null.
+NCU_DRAM_BYTES_PER_LAUNCH = {("bert_large_bf16", 256, "jacobi_persistent"): 12.0e6}
 
 
 def alt_start_vectors(w, seed):
