@@ -103,6 +103,12 @@ struct PivotShared {
 
 __device__ __forceinline__ float rsqrt_ftz(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
+// 2^-e for x in [2^e, 2^(e+1)), from the exponent field (kept to normal numbers)
+__device__ __forceinline__ float inv_exponent(float x)
+{
+    return __uint_as_float(0x7f000000u - min(max(__float_as_uint(x) & 0x7f800000u, 0x01000000u), 0x7e800000u));
+}
+
 // The rotations of the pairs of warp 0, one per lane, with the row factors of the pair (and their reciprocals) and the
 // two diagonal entries.
 struct Rotor {
@@ -112,21 +118,23 @@ struct Rotor {
     // identity when the entry is already small against its diagonal. With a = g_qq - g_pp, b = 2 g_pq,
     // r = sqrt(a^2 + b^2):
     //   cos 2t = |a| / r,  c = sqrt((1 + cos 2t) / 2),  tan t = sign(a) b / (2 r c^2)      (|t| <= pi/4).
-    // What does not depend on eo (it arrives last) comes first; the squares are kept in range by a power of two chosen
-    // from the diagonal. Returns (beta, gamma) and advances the factors and the diagonal.
+    // What does not depend on eo (it arrives last) comes first. The squares are taken of entries scaled by the power of two
+    // that brings the larger diagonal entry into [1, 2): an entry worth rotating is then far above the flush to zero of the
+    // approximate reciprocal root (1 / 0 times 0 otherwise), whatever the scale of the matrix. Returns (beta, gamma) and
+    // advances the factors and the diagonal.
     __device__ __forceinline__ float2 next(float eo, float tol2)
     {
-        const float w = de * dod, dp = fmaxf(gpp, 0.f), dq = fmaxf(gqq, 0.f), md = fmaxf(dp, dq);
-        const float sc = md < 1e-18f ? 0x1p60f : (md > 1e18f ? 0x1p-60f : 1.f);
+        const float w = de * dod, dp = fmaxf(gpp, 0.f), dq = fmaxf(gqq, 0.f);
+        const float sc = inv_exponent(fmaxf(fabsf(gpp), fabsf(gqq)));
         const float a = (gqq - gpp) * sc, a2 = a * a, ah = 0.5f * fabsf(a), sgw = copysignf(sc, a) * w;
-        const float thr = tol2 * dp * dq, scw = 2.f * sc * w, kb = dod * ie, kg = de * io;
-        const float b = eo * scw;
-        const float r2 = fmaf(b, b, a2);
+        const float thr = fmaxf(4.f * tol2 * (dp * sc) * (dq * sc), 0x1p-120f), scw = 2.f * sc * w, kb = dod * ie, kg = de * io;
+        const float b = eo * scw, b2 = b * b;
+        const float r2 = b2 + a2;
         const float rh = rsqrt_ftz(r2);
         const float c2 = fmaf(ah, rh, 0.5f);
         const float rc = rsqrt_ftz(c2);
         const float gpq = eo * w;
-        const bool on = gpq * gpq > thr && r2 > 0.f;
+        const bool on = b2 > thr;
         const float t = on ? (eo * sgw) * rh * (rc * rc) : 0.f;
         const float2 out = make_float2(t * kb, t * kg);
         gpp = fmaf(-t, gpq, gpp); gqq = fmaf(t, gpq, gqq);
