@@ -138,7 +138,10 @@ struct Rotor {
         const float t = on ? (eo * sgw) * rh * (rc * rc) : 0.f;
         const float2 out = make_float2(t * kb, t * kg);
         gpp = fmaf(-t, gpq, gpp); gqq = fmaf(t, gpq, gqq);
-        const float c = on ? c2 * rc : 1.f, ic = on ? rc : 1.f;
+        // c = 1 / sqrt(1 + t^2) for the t that is applied: one Newton step from c0 = cos t above. The bias of the approximate
+        // roots in c^2 (1 + t^2) would add up over the rotations of a row.
+        const float c0 = on ? c2 * rc : 1.f, cc = c0 * c0, ch = 0.5f * c0;
+        const float q2 = fmaf(t, t, 1.f), c = fmaf(ch, fmaf(-cc, q2, 1.f), c0), ic = q2 * c;
         de *= c; dod *= c; ie *= ic; io *= ic;
         ie = ie * fmaf(-de, ie, 2.f); io = io * fmaf(-dod, io, 2.f);      // keeps d * (1 / d) = 1 to the last bit or so
         return out;
