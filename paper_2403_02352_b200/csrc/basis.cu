@@ -850,7 +850,6 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
             // and a short second pass on it finishes the job (a one-sided Jacobi in two strokes).
             // Each pass is one persistent kernel that stops on its own convergence test: nothing is
             // read back by the host.
-            constexpr float LEFT = 0.5f;
             for (int pass = 0; pass < 2; ++pass) {
                 if constexpr (kBf16) {
                     hp.clear();
@@ -874,11 +873,11 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 const int nsw = pass == 0 ? nsw0 : std::max(1, max_sweeps - nsw0);
                 const float tolc = pass == 0 ? (kBf16 ? 3e-2f : 1e-2f) : tol_conv, tolr = pass == 0 ? 1e-3f : 0.1f * tol_conv;
                 // fp32 inputs: the block products stay on the fp32 units (the threshold is below split-precision rounding)
-                // A sweep whose visits all stayed below tolc ends the pass, and so does a matrix that a sweep leaves below
-                // tolc (first pass) or LEFT * tolc (second: a sweep that ends by its visits still rotates what exceeds
-                // 0.1 * tolc on the way, so what it leaves is further down). 0.5: storing X_r in bf16 alone leaves about 2e-4
-                // (1.0 measured 127 ms instead of 129 on the 4096-token layer, but shows in X_r X_r^T)
-                if ((st = j3::launch<kBf16>(ctx, jb, tolc, pass == 0 ? tolc : LEFT * tolc, tolr, nsw, pass == 1)) != ATP_OK) return st;
+                // A sweep whose visits all stayed below tolc ends the pass; what exceeded tolr was rotated on the way, so such a
+                // sweep leaves the matrix at about tolr. A look at the whole matrix ends a pass as well: the second where it
+                // finds the same, nothing above tolr (at half of tolc it left off-diagonals of 1.5e-4 instead of 3e-5 in bf16,
+                // 4e-7 instead of 1e-7 in fp32), the first at tolc.
+                if ((st = j3::launch<kBf16>(ctx, jb, tolc, pass == 0 ? tolc : tolr, tolr, nsw, pass == 1)) != ATP_OK) return st;
                 if (pass == 0) {
                     // Bt2 = Bt Wt^T (d x r~),  Y2 = Y Wt^T (L x r~);  Wt rows are the eigenvectors
                     if constexpr (kBf16) {
