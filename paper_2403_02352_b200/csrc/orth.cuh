@@ -33,6 +33,7 @@ namespace orth {
 using j3::BLK; using j3::NT; using j3::LDA; using j3::LDB;
 constexpr int MAXSEQ = 32;
 constexpr int SYNC_WORDS = 256;   // words of Seq::sync before the SM list
+constexpr int EXTRA = 3;          // repetitions of a panel beyond those asked for
 constexpr int NRED = 8;           // second-level partial Gram sums (chunk ranges)
 
 struct Seq {
@@ -288,7 +289,12 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
     // projection is taken of the panel BEFORE the first factor is applied ((P - Q Q^T P) W = P W - Q Q^T (P W)), so
     // it runs beside rank 0's factorisation, and the first APPLY folds into the second GRAM pass:
     //   PF(project) SUMUPD GRAM | PF(project beside factor) SUMUPD GRAM(with W) | PF(series factor) APPLY.
-    // A panel with dependent columns (their replacements must still be projected) returns to the classic order.
+    // A panel with dependent columns (their replacements must still be projected) returns to the classic order, and so does an
+    // ill-conditioned one: W enlarges what rounding leaves of the finished columns in P - Q Q^T P by 1 / sqrt(least pivot),
+    // and in this order nothing is projected after W. For the same reason a panel whose last factor was not benign (dependent
+    // columns, a small pivot, little left of a column by the projection) gets another repetition, up to EXTRA of them.
+    // (512 x 768, r 128, a spectrum that falls to 1e-6 of noise: X - U U^T X 1.5e-6 sigma_1 instead of 5e-4; 300 x 1000,
+    // r 250, 1e-4 of noise: U^T U - I 4e-6 instead of 0.3.)
     enum { OP_PF, OP_SUMUPD, OP_GRAM, OP_APPLY };
     for (int pj = 0; pj < npanel && alive; ++pj) {
         const int j0 = pj * 64, w = min(64, rt - j0), nj = pj;            // nj finished panels
@@ -315,24 +321,24 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                 case 5: op = OP_GRAM; with_w = true; break;
                 case 6: op = OP_PF; do_factor = true; series_ok = true; break;
                 case 7: op = OP_APPLY; arep = 1; last = true; break;
-                // dependent columns found by the first factor: classic remainder
+                // dependent columns or a small pivot found by the first factor: classic remainder (rep counts its repetitions)
                 case 20: op = OP_APPLY; arep = 0; break;
                 case 21: op = OP_PF; first = rank; stride = ncta; skip = nj == 0; break;
                 case 22: op = OP_SUMUPD; skip = nj == 0; break;
                 case 23: op = OP_GRAM; break;
                 case 24: op = OP_PF; do_factor = true; series_ok = true; break;
-                case 25: op = OP_APPLY; arep = 1; last = true; break;
+                case 25: op = OP_APPLY; arep = 1 + rep; last = true; break;
                 // classic order, any number of repetitions
                 case 30: op = OP_PF; first = rank; stride = ncta; skip = nj == 0; break;
                 case 31: op = OP_SUMUPD; skip = nj == 0; break;
                 case 32: op = OP_GRAM; break;
                 case 33: op = OP_PF; do_factor = true; series_ok = rep > 0; break;
-                default: op = OP_APPLY; arep = rep; last = rep == reps - 1; break;      // 34
+                default: op = OP_APPLY; arep = rep; last = rep >= reps - 1; break;      // 34
             }
             if (!skip) switch (op) {
             case OP_PF: {
                 // beside the last factor of a panel the other CTAs note the column maxima of the next panel
-                const bool scan = TENSOR && do_factor && stage != 3 && (stage != 33 || rep == reps - 1) && pj + 1 < npanel;
+                const bool scan = TENSOR && do_factor && stage != 3 && (stage != 33 || rep >= reps - 1) && pj + 1 < npanel;
                 if (TENSOR && !do_factor && rank == 0 && tid < 64) sq.sync[192 + tid] = 0u;   // (used up by the panel before)
                 if (scan && (rank > 0 || ncta == 1)) column_max(pj + 1, max(rank - 1, 0), max(ncta - 1, 1));
                 if (do_factor && rank == 0) {
@@ -586,12 +592,12 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                 barrier();
             } break;
             default: {                                                   // OP_APPLY
-                const uint64_t nseed = seed + 7919ull * (uint64_t)(pj * 2 + arep);
+                const uint64_t nseed = seed + 7919ull * (uint64_t)(pj * 2 + (arep & 1)) + 0x51ED270Bull * (uint64_t)(arep >> 1);
                 const float rscale = rsqrtf((float)n * (1.f / 3.f));     // replacement columns of about unit norm
                 if (TENSOR) set_scales(scale_slot);
                 int fl[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) fl[k] = __ldcg(sq.flags + (tid & 15) * 4 + k);
+                for (int k = 0; k < 4; ++k) fl[k] = __ldcg(sq.flags + (tid & 15) * 4 + k) & 1;
                 for (int t = rank; t < ntile; t += ncta) {
                     const int rv = min(64, n - t * 64);
                     TileRegs ra;
@@ -640,11 +646,13 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             } break;
             }
             // next stage
-            if (stage == 3) {
-                const bool dependent = __syncthreads_or(alive && tid < w && __ldcg(sq.flags + tid) != 0) != 0;
-                stage = dependent ? 20 : 4;
-            } else if (stage == 7 || stage == 25) stage = -1;
-            else if (stage == 34) { ++rep; stage = rep < reps ? 30 : -1; }
+            if (stage == 3 || stage == 7 || stage == 25 || stage == 34) {
+                // (lengths count from the second factor on: the panel had unit columns then)
+                const bool again = __syncthreads_or(alive && tid < w && (__ldcg(sq.flags + tid) & (stage == 3 ? 5 : 7)) != 0) != 0;
+                if (stage == 3) stage = again ? 20 : 4;
+                else if (stage == 34) { ++rep; stage = rep < reps || (again && rep < reps + EXTRA) ? 30 : -1; }
+                else stage = again && rep++ < EXTRA ? 21 : -1;
+            }
             else ++stage;
         }
     }

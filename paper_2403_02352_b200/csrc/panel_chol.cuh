@@ -3,7 +3,10 @@
 // matrix is scaled to unit diagonal, factored D^-1 G D^-1 = L L^T and the factor inverted; the result
 // W = D^-1 L^-T (upper triangular, fp32, 64 x 64 row-major) goes to rinv, so that P W has orthonormal
 // columns. A column whose scaled pivot falls below 1e-10 (its part outside the span of the earlier
-// columns is below 1e-5 of its norm) is flagged as dependent in flags[0..63].
+// columns is below 1e-5 of its norm) is flagged as dependent: bit 0 of its word in flags[0..63]. Bit 1: the column is shorter
+// than SHRUNK; where it had unit length before the projection, what rounding left of the finished columns in it is no longer
+// small against it. Bit 2: its scaled pivot is below ILL_PIVOT^2, so W enlarges a rounding error of the panel more than
+// 1 / ILL_PIVOT times.
 // Four panels of 16 columns. What bounds it is the chain of 64 pivots, so a panel's diagonal block is factored inside one
 // warp, without a barrier: lane i < 16 holds row i of the block, lane 16 + j column j of its inverse (which starts as the
 // identity); with m = (entry of column c) / L_cc in every lane, the right-looking step
@@ -18,6 +21,7 @@
 #include "jacobi3.cuh"
 
 constexpr int PB = 64;            // orthonormalisation panel width
+constexpr double ILL_PIVOT = 0x1p-5, SHRUNK = 0.25;
 
 constexpr int LDC = 68;           // row stride (doubles) in shared memory: the fragments below are free of bank conflicts
 
@@ -171,7 +175,9 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, flo
         w.z = (float)(rk * X[(c + 2) * LDC + k]); w.w = (float)(rk * X[(c + 3) * LDC + k]);
         *(float4 *)(rinv + k * PB + c) = w;
     }
-    if (tid < PB) flags[tid] = (tid < n) ? (dep[tid] || !(rs[tid] > 0.0)) : 0;
+    // (the diagonal of L^-1 holds the reciprocal square roots of the pivots)
+    if (tid < PB)
+        flags[tid] = tid >= n ? 0 : (dep[tid] || !(rs[tid] > 0.0) ? 1 : 0) | (rs[tid] > 1.0 / SHRUNK ? 2 : 0) | (X[tid * (LDC + 1)] > 1.0 / ILL_PIVOT ? 4 : 0);
 }
 
 
@@ -200,7 +206,7 @@ __device__ __forceinline__ void square64_tf32(const float *Es, int ld, int m0, i
 // with the Gram matrix scaled to unit diagonal, D^-1/2 G D^-1/2 = I + E, the symmetric factor
 //   W = D^-1/2 (I - E/2 + 3/8 E^2)          (P W has orthonormal columns up to 5/16 |E|^3)
 // needs one 64^3 product instead of a factorisation and its chain of 64 dependent pivots. Taken only when every
-// diagonal entry is positive and the largest absolute row sum of E is at most LOWDIN_LIMIT (then the neglected
+// column has kept SHRUNK of its unit length and the largest absolute row sum of E is at most LOWDIN_LIMIT (then the neglected
 // term is below 4e-8); otherwise nothing is written and the caller factors the matrix. Returns the decision
 // (block-uniform). Es: a 64 x LDE fp32 tile of shared memory; 256 threads.
 // E^2 is at most 2.5e-5, so plain TF32 products (2^-10 relative) leave an error near 1e-8. Thread = 4 x 4 block: a row sum
@@ -214,9 +220,9 @@ __device__ __noinline__ bool lowdin_64(const double *Gs, int n, float *Es, float
     bool bad = false;
     if (tid < PB) {
         const double d = Gs[tid * (LDC + 1)];
-        const bool pos = tid < n && d > 0.0;
-        rsq[tid] = pos ? rsqrt(d) : 0.0;
-        bad = tid < n && !pos;
+        const bool kept = tid < n && d >= SHRUNK * SHRUNK;
+        rsq[tid] = kept ? rsqrt(d) : 0.0;
+        bad = tid < n && !kept;
     }
     __syncthreads();
     float sum[4];
