@@ -12,7 +12,7 @@
 // products accumulate in fp64, so that the only rounding of a step is the fp32 storage of u, v and R.
 // Bound by shared-memory reads and the widening of the elements to fp64 (half by the conversion instruction, 16 a clock and
 // SM, half by three integer operations each), and by the barrier and the partial sums of a round.
-// 16 sequences of 512 x 1024, r = 64, inner = 2: 5092 -> 1380 us (a chain of 320 launches that read R six times per
+// 16 sequences of 512 x 1024, r = 64, inner = 2: 5092 -> 1398 us (a chain of 320 launches that read R six times per
 // component from L2 before).
 #include "common.cuh"
 #include "group_barrier.cuh"
@@ -47,8 +47,10 @@ template <int W> __device__ __forceinline__ double block_sum(double x, double *r
     return s;
 }
 
-// x * 2^-896 in fp64, exactly, by shifting the bits of x into place (the exponent field keeps its value, fp32 denormals
-// become fp64 denormals, zero stays zero). A sum of products with it is multiplied by 2^896 at the end.
+// x * 2^-896 in fp64, exactly, by shifting the bits of a finite x into place (the exponent field keeps its value, fp32
+// denormals become fp64 denormals, zero stays zero). The other factor of a product is scaled by 2^896 (an fp32 value times
+// 2^896 is an fp64 number), so the products and their sums are those of the converted values, whatever their size. Inf and NaN
+// would come out as numbers: a warp with such rows takes their dot products again with conversions alone.
 __device__ __forceinline__ double widen(float x)
 {
     const int b = __float_as_int(x);
@@ -71,18 +73,23 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
     const int rank = (int)blockIdx.x - q.cta0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (rank >= q.ncta || q.L <= 0) return;
     double *ud = (double *)altsm;                              // u of the current round
-    float *vc = (float *)(ud + maxrows), *vo = vc + dp, *uf = vo + dp;   // v of the current round and of the last one, u in fp32
-    float *sR = (float *)(((uintptr_t)(uf + maxrows) + 15) & ~(uintptr_t)15);   // rows of R
+    float *vc = (float *)(ud + maxrows), *vo = vc + dp;        // v of the current round and of the last one
+    float *sR = vo + dp;                                       // rows of R
     const int row0 = rank * q.rows, nrow = max(0, min(q.rows, q.L - row0)), ns = min(srows, nrow);
     float *gR = q.R + (size_t)row0 * dp;                       // rows ns .. nrow - 1 of this CTA
     int *abort_flag = status + 1;
     unsigned gen = 0, round = 0;
     bool alive = true;
 
+    float seen = 0.f;                                          // NaN once this lane has seen Inf or NaN in R
     for (int l = warp; l < nrow; l += NW) {
         const T *x = (const T *)q.X + (size_t)(row0 + l) * q.ldx_in;
         float *r = (l < ns ? sR : gR) + (size_t)l * dp;
-        for (int k = lane; k < dp; k += 32) r[k] = k < d ? to_f32(x[k]) : 0.f;
+        for (int k = lane; k < dp; k += 32) {
+            const float v = k < d ? to_f32(x[k]) : 0.f;
+            seen = fmaf(v, 0.f, seen);
+            r[k] = v;
+        }
     }
     for (int l = tid; l < maxrows; l += ALT_NT) ud[l] = 0.0;
     __syncthreads();
@@ -117,7 +124,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
             };
             auto put_u = [&](int l, double acc) {              // u of row l, by one lane
                 const float u = vv > 0.0 ? (float)(acc / vv) : 0.f;
-                uf[l] = u; ud[l] = (double)u;
+                ud[l] = (double)u;
                 usq += (double)u * (double)u;
             };
             auto lanes_sum = [&](double acc, int from) {
@@ -126,10 +133,15 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
                 return acc;
             };
             // one sum with converted and one with shifted elements
+            auto factors = [&](double (&v)[4], int k) {
+                const float4 f = *(const float4 *)(vc + k);
+                v[0] = f.x; v[1] = (double)f.y * WIDEN_SCALE; v[2] = f.z; v[3] = (double)f.w * WIDEN_SCALE;
+            };
             auto dot = [&](double &a, double &w, float4 x, const double (&v)[4]) {
                 a = fma((double)x.x, v[0], a); w = fma(widen(x.y), v[1], w);
                 a = fma((double)x.z, v[2], a); w = fma(widen(x.w), v[3], w);
             };
+            auto see = [&](float4 x) { seen = fmaf(x.w, 0.f, fmaf(x.y, 0.f, seen)); };       // (the shifted elements)
             auto subtract = [&](float4 &x, float u, float4 p) {
                 x.x = fmaf(-u, p.x, x.x); x.y = fmaf(-u, p.y, x.y); x.z = fmaf(-u, p.z, x.z); x.w = fmaf(-u, p.w, x.w);
             };
@@ -142,11 +154,11 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
                 for (int a = 0; a < 4; ++a) {
                     const int l = l0 + NW * a;
                     rp[a] = sR + (size_t)(l < ns ? l : l0) * dp;
-                    up[a] = deflate && l < ns ? uf[l] : 0.f;
+                    up[a] = deflate && l < ns ? (float)ud[l] : 0.f;
                 }
                 for (int k = lane * 4; k < dp; k += 128) {
-                    const float4 vf = *(const float4 *)(vc + k);
-                    const double v[4] = {vf.x, vf.y, vf.z, vf.w};
+                    double v[4];
+                    factors(v, k);
                     float4 x[4];
 #pragma unroll
                     for (int a = 0; a < 4; ++a) x[a] = *(const float4 *)(rp[a] + k);
@@ -155,7 +167,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
 #pragma unroll
                         for (int a = 0; a < 4; ++a) {
                             subtract(x[a], up[a], p);
-                            if (l0 + NW * a < ns) *(float4 *)(rp[a] + k) = x[a];
+                            if (l0 + NW * a < ns) { *(float4 *)(rp[a] + k) = x[a]; see(x[a]); }
                         }
                     }
 #pragma unroll
@@ -164,7 +176,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
                 __syncwarp();
                 // the four sums over the lanes together: after two exchanges a quarter of the warp holds each row
 #pragma unroll
-                for (int a = 0; a < 4; ++a) acc[a] = fma(aw[a], WIDEN_SCALE, acc[a]);
+                for (int a = 0; a < 4; ++a) acc[a] += aw[a];
                 const bool h1 = lane & 16, h0 = lane & 8;
                 const double p0 = (h1 ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, h1 ? acc[0] : acc[2], 16);
                 const double p1 = (h1 ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, h1 ? acc[1] : acc[3], 16);
@@ -176,7 +188,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
             // rows in the workspace, one of a warp at a time, eight loads in flight
             for (int l = pl; l < nrow; l += NW) {
                 float *rp = gR + (size_t)l * dp;
-                const float up = deflate ? uf[l] : 0.f;
+                const float up = deflate ? (float)ud[l] : 0.f;
                 double acc = 0.0, aw = 0.0;
                 for (int k0 = lane * 4; k0 < dp; k0 += 1024) {
                     if (l != pl || k0 >= 1024)
@@ -186,16 +198,27 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
                     for (int i = 0; i < 8; ++i) {
                         const int k = k0 + 128 * i;
                         if (k >= dp) continue;
-                        if (deflate) { subtract(pre[i], up, *(const float4 *)(vo + k)); *(float4 *)(rp + k) = pre[i]; }
-                        const float4 vf = *(const float4 *)(vc + k);
-                        const double v[4] = {vf.x, vf.y, vf.z, vf.w};
+                        if (deflate) { subtract(pre[i], up, *(const float4 *)(vo + k)); *(float4 *)(rp + k) = pre[i]; see(pre[i]); }
+                        double v[4];
+                        factors(v, k);
                         dot(acc, aw, pre[i], v);
                     }
                 }
                 __syncwarp();
-                acc = lanes_sum(fma(aw, WIDEN_SCALE, acc), 16);
+                acc = lanes_sum(acc + aw, 16);
                 norm_v();
                 if (lane == 0) put_u(l, acc);
+            }
+            if (__any_sync(0xffffffffu, seen != 0.f)) {          // (the whole warp again)
+                usq = 0.0;
+                for (int l = warp; l < nrow; l += NW) {
+                    const float *row = (l < ns ? sR : gR) + (size_t)l * dp;
+                    double acc = 0.0;
+                    for (int k = lane; k < dp; k += 32) acc = fma((double)row[k], (double)vc[k], acc);
+                    acc = lanes_sum(acc, 16);
+                    norm_v();
+                    if (lane == 0) put_u(l, acc);
+                }
             }
             usq = lanes_sum(usq, 16);
             if (lane == 0) redu[warp] = usq;
@@ -209,7 +232,8 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
 #pragma unroll
                 for (int a = 0; a < 4; ++a) g[a] = ns + a < nrow ? *(const float2 *)(gR + (size_t)(ns + a) * dp + k) : make_float2(0.f, 0.f);
                 const float *col = sR + k;
-                auto add = [&](float2 x, double u) { a0 = fma((double)x.x, u, a0); a1 = fma(widen(x.y), u, a1); };
+                // (a row with Inf or NaN has an infinite or NaN u, so its shifted elements need no care here)
+                auto add = [&](float2 x, double u) { a0 = fma((double)x.x, u, a0); a1 = fma(widen(x.y), u * WIDEN_SCALE, a1); };
                 int l = 0;
                 for (; l + 8 <= ns; l += 8, col += 8 * (size_t)dp) {
                     float2 x[8];
@@ -226,7 +250,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
                 for (int a = 0; a < 4; ++a) if (ns + a < nrow) add(g[a], ud[ns + a]);
 #pragma unroll 4
                 for (l = ns + 4; l < nrow; ++l) add(*(const float2 *)(gR + (size_t)l * dp + k), ud[l]);
-                *(double2 *)(mine + k) = make_double2(a0, a1 * WIDEN_SCALE);
+                *(double2 *)(mine + k) = make_double2(a0, a1);
             }
             if (tid == 0) {
                 double s = 0.0;
@@ -292,7 +316,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
         un = sqrt(un);
         // the finished component: U[:, comp] = u / |u|, X'[comp, :] = v |u|
         for (int l = tid; l < nrow; l += ALT_NT)
-            ((T *)q.U)[(size_t)(row0 + l) * q.ldu + comp] = from_f32<T>(un > 0.0 ? (float)((double)uf[l] / un) : 0.f);
+            ((T *)q.U)[(size_t)(row0 + l) * q.ldu + comp] = from_f32<T>(un > 0.0 ? (float)(ud[l] / un) : 0.f);
         for (int k = rank * ALT_NT + tid; k < d; k += q.ncta * ALT_NT)
             ((T *)q.Xp)[(size_t)comp * q.ldx + k] = from_f32<T>((float)((double)vc[k] * un));
     }
@@ -380,7 +404,7 @@ static atp_status alternating_impl(atp_ctx *ctx, const atp_mat *X, const std::ve
         maxrows = (int)align_up((size_t)std::max(maxrows, 1), 2);
         if (work == 0) continue;
         // the vectors first, then as many rows of R as fit
-        const size_t fixed = (size_t)dp * 8 + (size_t)maxrows * 12 + 32;
+        const size_t fixed = (size_t)dp * 8 + (size_t)maxrows * 8 + 32;
         if (fixed > SMEM) return ATP_ERR_INVALID_ARG;
         int srows = (int)std::min<size_t>((SMEM - fixed) / ((size_t)dp * 4), (size_t)maxrows);
         const size_t smem = fixed + (size_t)srows * dp * 4;
