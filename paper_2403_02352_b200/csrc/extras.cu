@@ -25,6 +25,7 @@ struct AltSeq {
     float *R;                      // rows of the deflated matrix that do not fit in shared memory (L x dp)
     double *part;                  // partial columns: 2 (by round parity) x ncta x (dp + 4)
     float *vbuf;                   // v of a round, where it is summed in slices
+    double *vecs;                  // u, v and the last v of every CTA, where they do not fit in shared memory
     unsigned *sync;                // words of the group barrier
     const float *v0;               // start vectors of this sequence (r x d, row stride ldv)
     void *U, *Xp;                  // outputs: U (L x r), X' (r x d)
@@ -58,8 +59,9 @@ __device__ __forceinline__ double widen(float x)
 }
 constexpr double WIDEN_SCALE = 0x1p896;
 
-// dp: d rounded up to 4 (row stride of R; columns d .. dp - 1 are zero); srows: rows of a CTA kept in shared memory
-template <typename T>
+// dp: d rounded up to 4 (row stride of R; columns d .. dp - 1 are zero); srows: rows of a CTA kept in shared memory.
+// FAR: the vectors do not fit in shared memory either (alternating_fixed), they lie in the workspace; srows = 0 then.
+template <typename T, bool FAR>
 __global__ void __launch_bounds__(ALT_NT, 1)
 alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int srows, int maxrows, int inner, int *status)
 {
@@ -72,9 +74,9 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
     const AltSeq &q = batch.s[si];
     const int rank = (int)blockIdx.x - q.cta0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (rank >= q.ncta || q.L <= 0) return;
-    double *ud = (double *)altsm;                              // u of the current round
+    double *ud = FAR ? q.vecs + (size_t)rank * (maxrows + dp) : (double *)altsm;   // u of the current round
     float *vc = (float *)(ud + maxrows), *vo = vc + dp;        // v of the current round and of the last one
-    float *sR = vo + dp;                                       // rows of R
+    float *sR = FAR ? nullptr : vo + dp;                       // rows of R
     const int row0 = rank * q.rows, nrow = max(0, min(q.rows, q.L - row0)), ns = min(srows, nrow);
     float *gR = q.R + (size_t)row0 * dp;                       // rows ns .. nrow - 1 of this CTA
     int *abort_flag = status + 1;
@@ -341,16 +343,26 @@ static std::vector<int> alternating_ctas(const std::vector<SeqDims> &sd, size_t 
     return c;
 }
 
-struct AltScratch { float *R; double *part; float *vbuf; unsigned *sync; int ncta; };
+// Shared memory of a CTA, and what its vectors take of it: u of at most `rows` rows in fp64, two v of dp floats.
+constexpr int ALT_SMEM = 226 * 1024 - 512 * 8;   // of 227 KB a CTA may have: the rest is the kernel's static share
+static size_t alternating_fixed(int dp, int rows) { return (size_t)dp * 8 + align_up((size_t)std::max(rows, 1), 2) * 8 + 32; }
+
+struct AltScratch { float *R; double *part; float *vbuf; double *vecs; unsigned *sync; int ncta, maxrows; };
 static void plan_alternating(Arena &ar, const std::vector<SeqDims> &sd, int d, int sm_count, std::vector<AltScratch> &out)
 {
     const size_t dp = align_up((size_t)d, 4);
     for (size_t i0 = 0; i0 < sd.size(); i0 += ALT_MAX) {
         const size_t i1 = std::min(sd.size(), i0 + ALT_MAX);
         const std::vector<int> c = alternating_ctas(sd, i0, i1, sm_count);
+        int rows = 1;
+        for (size_t i = i0; i < i1; ++i) rows = std::max(rows, ceil_div(sd[i].L, c[i - i0]));
+        rows = (int)align_up((size_t)rows, 2);
+        const bool far = alternating_fixed((int)dp, rows) > (size_t)ALT_SMEM;
         for (size_t i = i0; i < i1; ++i) {
             AltScratch a;
             a.ncta = c[i - i0];
+            a.maxrows = rows;
+            a.vecs = far ? ar.take<double>((size_t)a.ncta * (rows + dp)) : nullptr;
             a.R = ar.take<float>((size_t)sd[i].L * dp);
             a.part = ar.take<double>((size_t)2 * a.ncta * (dp + 4));
             a.vbuf = ar.take<float>(dp);
@@ -377,37 +389,35 @@ static atp_status alternating_impl(atp_ctx *ctx, const atp_mat *X, const std::ve
     std::vector<AltScratch> sc;
     plan_alternating(ar, sd, d, ctx->sm_count, sc);
     if (ar.overflow || !ctx->workspace) return ATP_ERR_WORKSPACE_TOO_SMALL;
-    constexpr int SMEM = 226 * 1024 - 512 * 8;       // of 227 KB a CTA may have: the rest is the kernel's static share
     static PerDeviceOnce attr_once;
     ATP_CUDA_OK(ctx, attr_once.run(ctx->device, [] {
-        return cudaFuncSetAttribute(alternating_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        return cudaFuncSetAttribute(alternating_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ALT_SMEM);
     }));
     for (size_t i0 = 0; i0 < sd.size(); i0 += ALT_MAX) {
         AltBatch b; b.count = (int)std::min<size_t>(ALT_MAX, sd.size() - i0);
-        int next = 0, maxrows = 0;
+        int next = 0;
         double work = 0;
         for (int k = 0; k < b.count; ++k) {
             const SeqDims &s = sd[i0 + k];
             const AltScratch &a = sc[i0 + k];
             AltSeq &q = b.s[k];
             q.X = (const T *)X->data + (size_t)s.row0 * X->ld; q.ldx_in = (int)X->ld;
-            q.R = a.R; q.part = a.part; q.vbuf = a.vbuf; q.sync = a.sync;
+            q.R = a.R; q.part = a.part; q.vbuf = a.vbuf; q.vecs = a.vecs; q.sync = a.sync;
             q.v0 = (const float *)V0->data + (size_t)s.rank0 * V0->ld; q.ldv = (int)V0->ld;
             q.U = (T *)U_r->data + (size_t)s.row0 * U_r->ld; q.ldu = (int)U_r->ld;
             q.Xp = (T *)X_r->data + (size_t)s.rank0 * X_r->ld; q.ldx = (int)X_r->ld;
             q.L = s.L; q.r = s.r;
             q.cta0 = next; q.ncta = a.ncta; q.rows = ceil_div(s.L, a.ncta);
             next += a.ncta;
-            maxrows = std::max(maxrows, q.rows);
             work += (double)s.r * s.L * d * 4;
         }
-        maxrows = (int)align_up((size_t)std::max(maxrows, 1), 2);
         if (work == 0) continue;
         // the vectors first, then as many rows of R as fit
-        const size_t fixed = (size_t)dp * 8 + (size_t)maxrows * 8 + 32;
-        if (fixed > SMEM) return ATP_ERR_INVALID_ARG;
-        int srows = (int)std::min<size_t>((SMEM - fixed) / ((size_t)dp * 4), (size_t)maxrows);
-        const size_t smem = fixed + (size_t)srows * dp * 4;
+        const int maxrows = sc[i0].maxrows;
+        const size_t fixed = alternating_fixed(dp, maxrows);
+        const bool far = fixed > (size_t)ALT_SMEM;
+        int srows = far ? 0 : (int)std::min<size_t>((ALT_SMEM - fixed) / ((size_t)dp * 4), (size_t)maxrows);
+        const size_t smem = far ? 0 : fixed + (size_t)srows * dp * 4;
         ATP_KERNEL(ctx, "alternating_init", 0, 0);
         alternating_init_kernel<<<b.count, 64, 0, ctx->stream>>>(b);
         ATP_LAUNCHED(ctx);
@@ -416,7 +426,8 @@ static atp_status alternating_impl(atp_ctx *ctx, const atp_mat *X, const std::ve
         void *args[] = {(void *)&b, (void *)&dd, (void *)&ddp, (void *)&srows, (void *)&mr, (void *)&in, (void *)&status};
         // bytes: R once per round, written once per component (most of it in shared memory)
         ATP_KERNEL(ctx, "alternating", work / 4 * (4.0 * inner + 2), work * (inner + 1));
-        ATP_CUDA_OK(ctx, cudaLaunchCooperativeKernel((const void *)alternating_kernel<T>, dim3(next), dim3(ALT_NT), args, smem, ctx->stream));
+        const void *kern = far ? (const void *)alternating_kernel<T, true> : (const void *)alternating_kernel<T, false>;
+        ATP_CUDA_OK(ctx, cudaLaunchCooperativeKernel(kern, dim3(next), dim3(ALT_NT), args, smem, ctx->stream));
         ATP_LAUNCHED(ctx);
     }
     return ATP_OK;

@@ -80,3 +80,32 @@ def test_overflow_of_the_deflation():
         assert (U.isfinite() == u.isfinite()).all() and (W.isfinite() == w.isfinite()).all()
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("lengths,d", [
+    ([48, 70], 28376), ([48, 70], 28408),      # the vectors of a CTA just fit in shared memory / no longer do
+    ([5, 33], 40008), ([64], 60000),           # long rows
+    ([80000] * 32, 16),                        # many rows to a CTA: u alone is near the shared memory
+    ([130000] * 32, 8),                        # and beyond it
+])
+def test_vectors_beyond_shared_memory(lengths, d, dtype):
+    import paper_2403_02352_b200 as atp
+    g = torch.Generator(device="cuda").manual_seed(d)
+    ranks = [2] * len(lengths)
+    X = torch.randn((sum(lengths), d), generator=g, device="cuda").to(dtype)
+    V0 = torch.randn((sum(ranks), d), generator=g, device="cuda")
+    c = atp.Context(0)
+    try:
+        U, W = atp.atp_alternating_basis(c, X, V0, lengths, ranks)
+        c.poll()
+        eps = 4e-6 if dtype == torch.float32 else 2.0 ** -8          # bf16: the outputs' own rounding
+        row = 0
+        for b, L in enumerate(lengths):
+            if b in (0, len(lengths) - 1):
+                u, w = algorithm1(X[row:row + L], V0[2 * b:2 * b + 2], 2, 2)
+                assert (U[row:row + L].float() - u).norm() <= eps * u.norm()
+                assert (W[2 * b:2 * b + 2].float() - w).norm() <= eps * w.norm()
+            row += L
+    finally:
+        c.close()
