@@ -225,10 +225,10 @@ ATP_API atp_status atp_profile_stop(atp_ctx *ctx, char *buf, size_t cap, size_t 
 
 /*
  * Self-tests of the library's own bookkeeping (no counterpart in the paper; used by the test suite).
- * atp_selftest_wait_timeout enqueues a kernel whose inter-CTA barrier can never complete (it expects
- * a second CTA that does not exist) with a short wait limit: the kernel gives up and raises
- * ATP_ERR_TIMEOUT on the status word, which the next atp_poll_device_status returns; the context stays
- * usable. It needs a workspace of at least 256 bytes.
+ * atp_selftest_wait_timeout enqueues a kernel of two CTAs that meet at the inter-CTA barrier, one of them
+ * with a short wait limit, the other only after that has run out: ATP_ERR_TIMEOUT is on the status word,
+ * which the next atp_poll_device_status returns; the context stays usable. It needs a workspace of at
+ * least 256 bytes.
  * atp_selftest_per_device_once runs the once-per-device set-up helper (kernel attributes, symbol
  * addresses) through a fixed script on the host and returns how often the guarded step ran (7).
  */

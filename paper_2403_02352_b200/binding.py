@@ -196,7 +196,7 @@ class Context:
             _check(lib.atp_set_workspace(self._h, C.c_void_p(t.data_ptr()), t.numel() * t.element_size()), "atp_set_workspace")
 
     def selftest_wait_timeout(self):
-        """Enqueues a kernel whose barrier cannot complete; the next poll() raises ATP_ERR_TIMEOUT."""
+        """Enqueues a kernel one of whose CTAs gives up a barrier; the next poll() raises ATP_ERR_TIMEOUT."""
         self.ensure_workspace(256)
         _check(lib.atp_selftest_wait_timeout(self._h), "atp_selftest_wait_timeout")
 

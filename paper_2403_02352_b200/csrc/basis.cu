@@ -1057,8 +1057,12 @@ extern "C" atp_status atp_basis_workspace_bytes(atp_ctx *ctx, const atp_seqs *se
 // Self-tests of the bookkeeping around the kernels (used by the test suite).
 __global__ void wait_timeout_kernel(unsigned *sync, int *status)
 {
-    // a group barrier that expects two CTAs while only this one exists: the flag it polls is never set
-    if (!j3::group_barrier(sync, 1u, 2u, status + 1, 1u << 12) && threadIdx.x == 0) raise_status(status, ATP_ERR_TIMEOUT);
+    // a group barrier of two CTAs: the second comes at once and gives up at its limit, the first only then (or after a limit
+    // of its own), and finds the barrier complete
+    if (blockIdx.x == 0) {
+        for (unsigned i = 0; i < SPIN_LIMIT && !*(volatile int *)(status + 1); ++i);
+        group_barrier(sync, 1u, 2u, status + 1);
+    } else group_barrier(sync, 1u, 2u, status + 1, 1u << 12);
 }
 
 extern "C" atp_status atp_selftest_wait_timeout(atp_ctx *ctx)
@@ -1068,7 +1072,7 @@ extern "C" atp_status atp_selftest_wait_timeout(atp_ctx *ctx)
     ATP_CUDA_OK(ctx, cudaSetDevice(ctx->device));
     ATP_CUDA_OK(ctx, cudaMemsetAsync(ctx->workspace, 0, 64 * sizeof(unsigned), ctx->stream));
     ATP_KERNEL(ctx, "wait_timeout", 0, 0);
-    wait_timeout_kernel<<<1, 32, 0, ctx->stream>>>((unsigned *)ctx->workspace, ctx->dev_status);
+    wait_timeout_kernel<<<2, 32, 0, ctx->stream>>>((unsigned *)ctx->workspace, ctx->dev_status);
     ATP_LAUNCHED(ctx);
     return ATP_OK;
 }

@@ -322,7 +322,6 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
         for (int k = rank * ALT_NT + tid; k < d; k += q.ncta * ALT_NT)
             ((T *)q.Xp)[(size_t)comp * q.ldx + k] = from_f32<T>((float)((double)vc[k] * un));
     }
-    if (!alive && rank == 0 && tid == 0) raise_status(status, ATP_ERR_TIMEOUT);
 }
 
 __global__ void alternating_init_kernel(const __grid_constant__ AltBatch batch)

@@ -748,7 +748,7 @@ __device__ bool wait_fetched(Fetched &f)
             if (*(volatile const unsigned *)f.count >= f.target) { ok = 1; break; }
             if ((i & 1023u) == 1023u && *(volatile int *)f.abort_flag) break;
         }
-        if (!ok) *(volatile int *)f.abort_flag = 1;
+        if (!ok) wait_ran_out(f.abort_flag);
         ok_s = ok;
     }
     __syncthreads();
@@ -1174,8 +1174,7 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
         if (__uint_as_float(*(volatile unsigned *)(sq.sync + 8 + sweep % 4)) <= tol_left) { converged = true; ++sweep; break; }
     }
     if (rank == 0 && tid == 0) {
-        if (!alive) raise_status(status, ATP_ERR_TIMEOUT);
-        else if (!converged && raise_not_converged) raise_status(status, ATP_ERR_NOT_CONVERGED);
+        if (alive && !converged && raise_not_converged) raise_status(status, ATP_ERR_NOT_CONVERGED);
         sq.sync[5] = (unsigned)sweep;
     }
 }

@@ -656,7 +656,6 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
             else ++stage;
         }
     }
-    if (rank == 0 && tid == 0 && !alive) raise_status(status, ATP_ERR_TIMEOUT);
 }
 
 __global__ void init_kernel(const __grid_constant__ Batch batch)

@@ -47,7 +47,7 @@ def test_sweep_limit_raises_not_converged_once_and_leaves_the_context_usable(ctx
 def test_bounded_wait_that_runs_out_raises_timeout(ctx):
     atp = _atp()
     from paper_2403_02352_b200 import binding as B
-    ctx.selftest_wait_timeout()               # a barrier between CTAs whose partner does not exist, short limit
+    ctx.selftest_wait_timeout()               # a barrier that one CTA gives up and the other then finds complete
     with pytest.raises(atp.AtpError) as e:
         ctx.poll()
     assert e.value.code == B.ERR_TIMEOUT
