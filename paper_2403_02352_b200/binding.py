@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from array import array
 from itertools import accumulate
 from typing import Optional, Sequence
 
@@ -132,8 +133,8 @@ def mat(t: Optional[torch.Tensor]) -> Optional[Mat]:
 
 
 class SeqDesc:
-    """Host arrays of a packed batch (kept alive for the duration of a call). One ctypes buffer holds the three arrays:
-    row offsets, ranks, rank offsets."""
+    """Host arrays of a packed batch (kept alive for the duration of a call). One buffer of 32-bit integers holds the three
+    arrays: row offsets, ranks, rank offsets (a number that does not fit raises OverflowError)."""
 
     def __init__(self, lengths: Sequence[int], ranks: Sequence[int]):
         self.lengths = [int(x) for x in lengths]
@@ -145,8 +146,8 @@ class SeqDesc:
         rows.extend(accumulate(self.lengths))
         offs.extend(accumulate(self.ranks))
         self.total_rows, self.total_rank = rows[-1], offs[-1]
-        self._buf = (C.c_int32 * (3 * n + 2))(*rows, *self.ranks, *offs)
-        at = C.addressof(self._buf)
+        self._buf = array("i", rows + self.ranks + offs)
+        at = self._buf.buffer_info()[0]
         self.c = Seqs(n, at, at + 4 * (n + 1), at + 4 * (2 * n + 1))
 
 
