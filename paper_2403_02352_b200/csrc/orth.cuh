@@ -361,7 +361,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                     }
                     __syncthreads();
                     // a nearly orthonormal panel gets its factor from a short series instead of the factorisation
-                    if (!(series_ok && lowdin_64(Gs, w, sA, sq.W, sq.flags))) chol_invert_64(Gs, (double *)osm, w, sq.W, sq.flags);
+                    if (!(series_ok && lowdin_64(Gs, w, sA, (__half *)sB, sq.W, sq.flags))) chol_invert_64(Gs, (double *)osm, w, sq.W, sq.flags);
                     __syncthreads();
                 } else if (first >= 0) {
                     set_scales(scale_slot);

@@ -19,6 +19,7 @@
 #pragma once
 #include "common.cuh"
 #include "jacobi3.cuh"
+#include "split_mma.cuh"
 
 constexpr int PB = 64;            // orthonormalisation panel width
 constexpr double ILL_PIVOT = 0x1p-5, SHRUNK = 0.25;
@@ -182,39 +183,19 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, flo
 }
 
 
-// acc (a warp's 16 x 32 part of a 64 x 64 result, rows m0.., columns n0..) += E E, TF32 parts of the entries (2^-10), E symmetric:
-// thread holds rows m0 + g, + 8, columns n0 + 8 nt + 2 t, + 1.
-__device__ __forceinline__ void square64_tf32(const float *Es, int ld, int m0, int n0, float (&acc)[4][4])
-{
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-#pragma unroll 2
-    for (int k0 = 0; k0 < 64; k0 += 8) {
-        uint32_t a[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = __float_as_uint(Es[(k0 + t + 4 * (i >> 1)) * ld + m0 + g + 8 * (i & 1)]);
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            float (&d)[4] = acc[nt];
-            const int n = n0 + nt * 8 + g;
-            const uint32_t b0 = __float_as_uint(Es[(k0 + t) * ld + n]), b1 = __float_as_uint(Es[(k0 + t + 4) * ld + n]);
-            asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-        }
-    }
-}
-
 // Orthonormalising factor of a panel that is already close to orthonormal (the second Gram-Schmidt repetition):
 // with the Gram matrix scaled to unit diagonal, D^-1/2 G D^-1/2 = I + E, the symmetric factor
 //   W = D^-1/2 (I - E/2 + 3/8 E^2)          (P W has orthonormal columns up to 5/16 |E|^3)
 // needs one 64^3 product instead of a factorisation and its chain of 64 dependent pivots. Taken only when every
 // column has kept SHRUNK of its unit length and the largest absolute row sum of E is at most LOWDIN_LIMIT (then the neglected
 // term is below 4e-8); otherwise nothing is written and the caller factors the matrix. Returns the decision
-// (block-uniform). Es: a 64 x LDE fp32 tile of shared memory; 256 threads.
-// E^2 is at most 2.5e-5, so plain TF32 products (2^-10 relative) leave an error near 1e-8. Thread = 4 x 4 block: a row sum
-// is complete within half a warp. 11600 -> 3300 cycles (per-element reductions, atomics and an fp32 product before).
+// (block-uniform). Es: a 64 x LDE fp32 tile of shared memory, Eh: a tile of fp16 parts; 256 threads.
+// E^2 comes from two fp16 parts of E, E_SCALE E = hi + lo to 2^-25, so it is as good as an fp32 product (from one TF32 part, as
+// before, it was off by 2^-10: 1e-8 in W). Thread = 4 x 4 block: a row sum is complete within half a warp.
 constexpr float LOWDIN_LIMIT = 5e-3f;
 constexpr int LDE = 72;
-__device__ __noinline__ bool lowdin_64(const double *Gs, int n, float *Es, float *rinv, int *flags)
+constexpr float E_SCALE = 0x1p20f;                               // an entry is at most LOWDIN_LIMIT: below 5300 then
+__device__ __noinline__ bool lowdin_64(const double *Gs, int n, float *Es, __half *Eh, float *rinv, int *flags)
 {
     __shared__ double rsq[PB];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -250,10 +231,16 @@ __device__ __noinline__ bool lowdin_64(const double *Gs, int n, float *Es, float
 #pragma unroll
     for (int i = 0; i < 4; ++i) bad |= !(sum[i] <= LOWDIN_LIMIT);
     if (__syncthreads_or(bad)) return false;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4 e = *(const float4 *)&Es[(ty * 4 + i) * LDE + tx * 4];
+        hs::put4(Eh, ty * 4 + i, tx * 4, make_float4(e.x * E_SCALE, e.y * E_SCALE, e.z * E_SCALE, e.w * E_SCALE));
+    }
+    __syncthreads();
     // E^2 (E is symmetric); this warp: rows m0 .. + 15, columns n0 .. + 31
     const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32;
     float acc[4][4] = {};
-    square64_tf32(Es, LDE, m0, n0, acc);
+    hs::product64<false, false>(Eh, Eh, m0, n0, acc);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int r = m0 + g + 8 * h;
@@ -264,7 +251,7 @@ __device__ __noinline__ bool lowdin_64(const double *Gs, int n, float *Es, float
             float w[2];
 #pragma unroll
             for (int k = 0; k < 2; ++k)
-                w[k] = r < n && c + k < n ? sr * ((r == c + k ? 1.f : 0.f) - 0.5f * Es[r * LDE + c + k] + 0.375f * acc[nt][2 * h + k]) : 0.f;
+                w[k] = r < n && c + k < n ? sr * ((r == c + k ? 1.f : 0.f) - 0.5f * Es[r * LDE + c + k] + 0.375f / (E_SCALE * E_SCALE) * acc[nt][2 * h + k]) : 0.f;
             *(float2 *)(rinv + r * PB + c) = make_float2(w[0], w[1]);
         }
     }
