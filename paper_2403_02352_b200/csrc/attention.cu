@@ -175,7 +175,9 @@ static void plan_attn(Arena &ar, int64_t tr, int64_t tl, int64_t dp, int64_t nse
     p.Qh = ar.take<__nv_bfloat16>((size_t)tl * align_up((size_t)dp, 8));
     p.Ql = ar.take<__nv_bfloat16>((size_t)tl * align_up((size_t)dp, 8));
     p.nrm = ar.take<float>((size_t)(tl / 128 + nseq) * dp + (size_t)(tr / 128 + nseq) * dp);    // per head norms: query tiles, key blocks
-    p.tab = ar.take<float2>((size_t)tl * 64);                                  // rotary (cos, sin) per row and pair (d_h <= 128)
+    // rotary (cos, sin) per row and pair of a head (d_h <= 128): 4 d_h bytes a row, where there is room in a buffer that the path
+    // leaves free otherwise - behind the third part of K in Kf, or in Qh - if there are two heads or more
+    p.tab = dp < 256 ? ar.take<float2>((size_t)tl * 64) : nullptr;
 }
 size_t attention_workspace_bytes(const std::vector<SeqDims> &seqs, int64_t dp)
 {
@@ -194,13 +196,14 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
                                  atp_mat *O)
 {
     const int d = (int)X_r->cols, dp = (int)WQ->cols, dh = dp / heads;
-    const bool rope = rope_base > 0.f;
+    const bool rope = rope_base > 0.f, tensor = std::is_same<T, __nv_bfloat16>::value && (dh == 64 || dh == 128);
     int64_t tr = 0, tl = 0;
     for (auto &s : seqs) { tr += s.r; tl += s.L; }
     Arena ar(ctx->workspace, ctx->workspace_bytes);
     AttnPlan pl;
     plan_attn(ar, tr, tl, dp, (int64_t)seqs.size(), pl);
     if (ar.overflow || !ctx->workspace) return ATP_ERR_WORKSPACE_TOO_SMALL;
+    if (!pl.tab) pl.tab = tensor ? (float2 *)((__nv_bfloat16 *)pl.Kf + (size_t)tl * align_up((size_t)dp, 8)) : (float2 *)pl.Qh;
     atp_status st;
     GemmEpi store{EPI_STORE, nullptr};
     auto make_rope_table = [&]() -> atp_status {
@@ -225,7 +228,7 @@ static atp_status attention_impl(atp_ctx *ctx, const atp_mat *X, const atp_mat *
         return flush();
     };
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-        if (dh == 64 || dh == 128) {
+        if (tensor) {
             // bf16, head width 64 or 128: everything on the tensor cores. K' and Q are produced as
             // bf16 hi/lo pairs by the GEMM epilogues, V' as bf16; the fused kernel does the rest.
             const int ldq = (int)align_up((size_t)dp, 8);

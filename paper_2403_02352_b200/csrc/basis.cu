@@ -545,16 +545,17 @@ struct SeqPlan {
     __nv_bfloat16 *Yb, *Yl, *Zb, *Zl; float *Y2; float *Y, *Z, *BW, *Wsel, *tsum, *sig, *Cc, *rinv, *G, *Wt, *Vbuf; double *gpart; int *ord, *flags, *conv, *vflag, *needfix; unsigned *maxoff;
 };
 struct BasisPlan {
-    std::vector<SeqPlan> seqs; float *omega; __nv_bfloat16 *omega_b; float *part; size_t part_stride, part_group; int group = 0; int rtmax; int splits;
+    std::vector<SeqPlan> seqs; float *omega; __nv_bfloat16 *omega_b; float *part; size_t part_stride; int group = 0; int rtmax;
 };
 
 // Size of the Jacobi matrices: rt rounded up to a whole number of 64-row block pairs.
 static int jacobi_padded(int rt) { return rt <= 0 ? 0 : (rt + 63) / 64 * 64; }
 
-static void plan_basis(Arena &ar, const std::vector<SeqDims> &sd, int d, int oversample, int sm_count, BasisPlan &bp)
+// Each input type reserves what its own path touches (BW and Wsel in both: the one-sided variant keeps its rows there).
+static void plan_basis(Arena &ar, const std::vector<SeqDims> &sd, int d, int oversample, int sm_count, bool bf16, BasisPlan &bp)
 {
     bp.seqs.clear(); bp.rtmax = 0;
-    int maxdim = d; size_t maxpart = 0;
+    int maxdim = d;
     for (auto &s : sd) {
         SeqPlan p; p.dims = s;
         int m = std::min(s.L, d);
@@ -564,18 +565,23 @@ static void plan_basis(Arena &ar, const std::vector<SeqDims> &sd, int d, int ove
         maxdim = std::max(maxdim, s.L);
         bp.seqs.push_back(p);
     }
-    bp.omega = ar.take<float>((size_t)d * bp.rtmax);
-    bp.part = ar.take<float>((size_t)splitk_floats(sm_count));
-    bp.omega_b = ar.take<__nv_bfloat16>((size_t)d * align_up((size_t)bp.rtmax, 8));
+    auto take_f32 = [&](size_t n) { return bf16 ? nullptr : ar.take<float>(n); };
+    auto take_bf16 = [&](size_t n) { return bf16 ? ar.take<__nv_bfloat16>(n) : nullptr; };
+    bp.omega = take_f32((size_t)d * bp.rtmax);
+    bp.omega_b = take_bf16((size_t)d * align_up((size_t)bp.rtmax, 8));
+    // partial results of the products that are split along K (of at most maxdim rows, rtmax columns, maxdim / 96 parts)
+    const size_t all_parts = (size_t)(maxdim / 96) * std::min<size_t>(sd.size(), BMAX) * maxdim * bp.rtmax;
+    bp.part_stride = bf16 ? 0 : std::min(splitk_floats(sm_count), all_parts);
+    bp.part = bp.part_stride > 0 ? ar.take<float>(bp.part_stride) : nullptr;
     for (auto &p : bp.seqs) {
         int L = p.dims.L, rt = p.rt;
         p.Y = ar.take<float>((size_t)L * rt);
-        p.Z = ar.take<float>((size_t)d * rt);
-        p.Yb = ar.take<__nv_bfloat16>((size_t)L * align_up((size_t)rt, 8));
-        p.Yl = ar.take<__nv_bfloat16>((size_t)L * align_up((size_t)rt, 8));
-        p.Zb = ar.take<__nv_bfloat16>((size_t)d * align_up((size_t)rt, 8));
-        p.Zl = ar.take<__nv_bfloat16>((size_t)d * align_up((size_t)rt, 8));
-        p.Y2 = ar.take<float>((size_t)L * rt);
+        p.Z = take_f32((size_t)d * rt);
+        p.Yb = take_bf16((size_t)L * align_up((size_t)rt, 8));
+        p.Yl = take_bf16((size_t)L * align_up((size_t)rt, 8));
+        p.Zb = take_bf16((size_t)d * align_up((size_t)rt, 8));
+        p.Zl = take_bf16((size_t)d * align_up((size_t)rt, 8));
+        p.Y2 = take_f32((size_t)L * rt);
         p.BW = ar.take<float>((size_t)rt * (d + rt));
         p.Wsel = ar.take<float>((size_t)rt * p.dims.r);
         p.tsum = ar.take<float>(rt);
@@ -583,9 +589,9 @@ static void plan_basis(Arena &ar, const std::vector<SeqDims> &sd, int d, int ove
         p.ord = ar.take<int>(rt);
         {   // tile scratch of the orthonormalisation kernel
             p.ocap = orth::max_ctas_per_seq(sm_count, (int)std::min<size_t>(sd.size(), BMAX));
-            const orth::Scratch sc = orth::scratch_tiles(L, rt, p.ocap);
+            const orth::Scratch sc = orth::scratch_tiles(L, rt, p.ocap, bf16);
             const size_t ldq = align_up((size_t)std::max(rt, 1), 64);
-            p.oqh = ar.take<__half>((size_t)L * ldq); p.oql = ar.take<__half>((size_t)L * ldq);
+            p.oqh = bf16 ? ar.take<__half>((size_t)L * ldq) : nullptr; p.oql = bf16 ? ar.take<__half>((size_t)L * ldq) : nullptr;
             p.oCpart = ar.take<float>(sc.cpart * 4096); p.oC = ar.take<float>(sc.c * 4096);
             p.oDpart = ar.take<float>(sc.dpart * 4096); p.oW = ar.take<float>(4096);
             p.ogpart = ar.take<double>(sc.gpart * 4096); p.ogpart2 = ar.take<double>((size_t)orth::NRED * 4096);
@@ -599,24 +605,23 @@ static void plan_basis(Arena &ar, const std::vector<SeqDims> &sd, int d, int ove
         p.tpart = ar.take<float>((size_t)COLSUM_SLABS * std::max(rt, 1));
         {   // bf16 hi/lo operands of the tensor-core products around the rotation (bf16 inputs only)
             const size_t ldr = align_up((size_t)std::max(rt, 1), 8), ldw = align_up((size_t)std::max(p.dims.r, 1), 8);
-            p.Bth = ar.take<__nv_bfloat16>((size_t)d * ldr); p.Btl = ar.take<__nv_bfloat16>((size_t)d * ldr);
-            p.Y2h = ar.take<__nv_bfloat16>((size_t)L * ldr); p.Y2l = ar.take<__nv_bfloat16>((size_t)L * ldr);
-            p.Wth = ar.take<__nv_bfloat16>((size_t)p.np * p.np); p.Wtl = ar.take<__nv_bfloat16>((size_t)p.np * p.np);
-            p.Wsh = ar.take<__nv_bfloat16>((size_t)std::max(rt, 1) * ldw); p.Wsl = ar.take<__nv_bfloat16>((size_t)std::max(rt, 1) * ldw);
+            p.Bth = take_bf16((size_t)d * ldr); p.Btl = take_bf16((size_t)d * ldr);
+            p.Y2h = take_bf16((size_t)L * ldr); p.Y2l = take_bf16((size_t)L * ldr);
+            p.Wth = take_bf16((size_t)p.np * p.np); p.Wtl = take_bf16((size_t)p.np * p.np);
+            p.Wsh = take_bf16((size_t)std::max(rt, 1) * ldw); p.Wsl = take_bf16((size_t)std::max(rt, 1) * ldw);
         }
         p.jsync = ar.take<unsigned>(64);
         p.needfix = ar.take<int>(std::max(p.dims.r, 1));
         p.maxoff = ar.take<unsigned>(1);
         p.conv = ar.take<int>(1);
-        maxpart = std::max(maxpart, (size_t)rt * PB);
     }
 }
 
-size_t basis_workspace_bytes(const std::vector<SeqDims> &sd, int d, int oversample, int sm_count)
+size_t basis_workspace_bytes(const std::vector<SeqDims> &sd, int d, int oversample, int sm_count, bool bf16)
 {
     Arena ar(nullptr, (size_t)-1);
     BasisPlan bp;
-    plan_basis(ar, sd, d, oversample, sm_count, bp);
+    plan_basis(ar, sd, d, oversample, sm_count, bf16, bp);
     return ar.off;
 }
 
@@ -643,7 +648,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
     const int d = (int)X->cols;
     Arena ar(ctx->workspace, ctx->workspace_bytes);
     BasisPlan bp;
-    plan_basis(ar, sd, d, oversample, ctx->sm_count, bp);
+    plan_basis(ar, sd, d, oversample, ctx->sm_count, std::is_same<T, __nv_bfloat16>::value, bp);
     if (ar.overflow || !ctx->workspace) return ATP_ERR_WORKSPACE_TOO_SMALL;
     atp_status st;
     if (X->dtype == ATP_BF16) {
@@ -727,7 +732,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 SeqPlan &p = bp.seqs[i];
                 g.p[i - i0] = GemmProblem{Xb(p), bp.omega, p.Y, nullptr, p.dims.L, p.rt, d, (int)X->ld, bp.rtmax, p.rt, 0};
             }
-            if ((st = launch_gemm_simt<T, float, float, false>(ctx, g, store, 0, kpart, splitk_floats(ctx->sm_count))) != ATP_OK) return st;
+            if ((st = launch_gemm_simt<T, float, float, false>(ctx, g, store, 0, kpart, bp.part_stride)) != ATP_OK) return st;
             if ((st = orthonormalise<std::is_same<T, __nv_bfloat16>::value>(ctx, bp, i0, i1, seed, 2)) != ATP_OK) return st;
             for (int it = 0; it < power_iters; ++it) {
                 // Z = X^T Y ; Y = X Z ; orth(Y).  Z is not orthonormalised: Y has orthonormal, QR-ordered
@@ -737,12 +742,12 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                     SeqPlan &p = bp.seqs[i];
                     g.p[i - i0] = GemmProblem{Xb(p), p.Y, p.Z, nullptr, p.rt > 0 ? d : 0, p.rt, p.dims.L, (int)X->ld, p.rt, p.rt, 0};
                 }
-                if ((st = launch_gemm_simt<T, float, float, true>(ctx, g, store, 0, kpart, splitk_floats(ctx->sm_count))) != ATP_OK) return st;
+                if ((st = launch_gemm_simt<T, float, float, true>(ctx, g, store, 0, kpart, bp.part_stride)) != ATP_OK) return st;
                 for (size_t i = i0; i < i1; ++i) {
                     SeqPlan &p = bp.seqs[i];
                     g.p[i - i0] = GemmProblem{Xb(p), p.Z, p.Y, nullptr, p.dims.L, p.rt, d, (int)X->ld, p.rt, p.rt, 0};
                 }
-                if ((st = launch_gemm_simt<T, float, float, false>(ctx, g, store, 0, kpart, splitk_floats(ctx->sm_count))) != ATP_OK) return st;
+                if ((st = launch_gemm_simt<T, float, float, false>(ctx, g, store, 0, kpart, bp.part_stride)) != ATP_OK) return st;
                 if ((st = orthonormalise<std::is_same<T, __nv_bfloat16>::value>(ctx, bp, i0, i1, seed + 2000003ull * (it + 1), 2)) != ATP_OK) return st;
             }
         }
@@ -841,7 +846,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 }
                 if ((st = tc::launch<true, 2, tc::OUT_BF16_SPLIT>(ctx, hp, store)) != ATP_OK) return st;
             } else {
-                if ((st = launch_gemm_simt<T, float, float, true>(ctx, g, store, 0, kpart, splitk_floats(ctx->sm_count))) != ATP_OK) return st;
+                if ((st = launch_gemm_simt<T, float, float, true>(ctx, g, store, 0, kpart, bp.part_stride)) != ATP_OK) return st;
             }
             // Two passes. G squares the condition number of B, so when sigma_1 / sigma_r~ exceeds ~10^3
             // the first diagonalisation resolves the weak components only roughly. Its rotation W1 is
@@ -863,7 +868,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                     }
                     if ((st = tc::launch<true, 2, tc::OUT_F32, false, true>(ctx, hp, store, "gemm_tc_gram")) != ATP_OK) return st;
                 } else {
-                    if ((st = launch_gemm_simt<float, float, float, true, false>(ctx, gg, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_gram")) != ATP_OK) return st;
+                    if ((st = launch_gemm_simt<float, float, float, true, false>(ctx, gg, store, 0, kpart, bp.part_stride, "gemm_simt_gram")) != ATP_OK) return st;
                 }
                 // pass 0 only has to make the rows graded and roughly orthogonal (on ill-conditioned input it stalls at the
                 // noise floor of G, hence the cap of 8 sweeps); the second pass continues the same iteration on the rotated
@@ -915,8 +920,8 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                             gg.p[k].A = p.Z; gg.p[k].B = p.Z;
                             fb.s[k].Y = p.Y2;
                         }
-                        if ((st = launch_gemm_simt<float, float, float, false, true>(ctx, r1, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_rot")) != ATP_OK) return st;
-                        if ((st = launch_gemm_simt<float, float, float, false, true>(ctx, r2, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_rot")) != ATP_OK) return st;
+                        if ((st = launch_gemm_simt<float, float, float, false, true>(ctx, r1, store, 0, kpart, bp.part_stride, "gemm_simt_rot")) != ATP_OK) return st;
+                        if ((st = launch_gemm_simt<float, float, float, false, true>(ctx, r2, store, 0, kpart, bp.part_stride, "gemm_simt_rot")) != ATP_OK) return st;
                     }
                 }
             }
@@ -956,8 +961,8 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                     gg.p[k] = GemmProblem{p.Y2, p.Wsel, (T *)U_r->data + (size_t)p.dims.row0 * U_r->ld, nullptr,
                                           p.dims.L, p.dims.r, p.rt, p.rt, p.dims.r, (int)U_r->ld, 0};
                 }
-                if ((st = launch_gemm_simt<float, float, T, true, true>(ctx, g, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_out")) != ATP_OK) return st;
-                if ((st = launch_gemm_simt<float, float, T, false>(ctx, gg, store, 0, kpart, splitk_floats(ctx->sm_count), "gemm_simt_out")) != ATP_OK) return st;
+                if ((st = launch_gemm_simt<float, float, T, true, true>(ctx, g, store, 0, kpart, bp.part_stride, "gemm_simt_out")) != ATP_OK) return st;
+                if ((st = launch_gemm_simt<float, float, T, false>(ctx, gg, store, 0, kpart, bp.part_stride, "gemm_simt_out")) != ATP_OK) return st;
             }
             ATP_KERNEL(ctx, "signfix", 0, 0);
             signfix_kernel<T><<<dim3(maxr, cnt), 256, 0, ctx->stream>>>(fb);
@@ -1012,7 +1017,7 @@ extern "C" atp_status atp_principal_basis(atp_ctx *ctx, const atp_mat *X, const 
 }
 
 // ------------------------------------------------------------------------------------------------
-size_t linear_workspace_bytes(const std::vector<SeqDims> &seqs, int64_t d_out);
+size_t linear_workspace_bytes(const std::vector<SeqDims> &seqs, int64_t d_out, bool bf16);
 size_t attention_workspace_bytes(const std::vector<SeqDims> &seqs, int64_t dp);
 
 static atp_status workspace_bytes_impl(atp_ctx *ctx, int op, const atp_seqs *seqs, int64_t d, int64_t d_out,
@@ -1027,9 +1032,9 @@ static atp_status workspace_bytes_impl(atp_ctx *ctx, int op, const atp_seqs *seq
     if (st != ATP_OK) return st;
     if (d < 1 || d > 0x7fffffff) return ATP_ERR_INVALID_ARG;
     switch (op) {
-        case ATP_OP_BASIS: *bytes = basis_workspace_bytes(sd, (int)d, oversample, ctx->sm_count) + 256; return ATP_OK;
+        case ATP_OP_BASIS: *bytes = basis_workspace_bytes(sd, (int)d, oversample, ctx->sm_count, dtype == ATP_BF16) + 256; return ATP_OK;
         case ATP_OP_ATTENTION: if (d_out < 1) return ATP_ERR_INVALID_ARG; *bytes = attention_workspace_bytes(sd, d_out) + 256; return ATP_OK;
-        case ATP_OP_LINEAR: if (d_out < 1) return ATP_ERR_INVALID_ARG; *bytes = linear_workspace_bytes(sd, d_out) + 256; return ATP_OK;
+        case ATP_OP_LINEAR: if (d_out < 1) return ATP_ERR_INVALID_ARG; *bytes = linear_workspace_bytes(sd, d_out, dtype == ATP_BF16) + 256; return ATP_OK;
         case ATP_OP_ALTERNATING: *bytes = alternating_workspace_bytes(sd, (int)d, ctx->sm_count) + 256; return ATP_OK;
         default: return ATP_ERR_INVALID_ARG;
     }

@@ -22,7 +22,7 @@ constexpr int ALT_NT = 512;        // threads per CTA
 constexpr int ALT_DIRECT = 16;     // up to this many CTAs in a group every CTA sums the partial columns itself
 struct AltSeq {
     const void *X;                 // first row of the sequence in the packed input
-    float *R;                      // rows of the deflated matrix that do not fit in shared memory (L x dp)
+    float *R;                      // rows of the deflated matrix that do not fit in shared memory (of each CTA, dp floats a row)
     double *part;                  // partial columns: 2 (by round parity) x ncta x (dp + 4)
     float *vbuf;                   // v of a round, where it is summed in slices
     double *vecs;                  // u, v and the last v of every CTA, where they do not fit in shared memory
@@ -78,7 +78,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
     float *vc = (float *)(ud + maxrows), *vo = vc + dp;        // v of the current round and of the last one
     float *sR = FAR ? nullptr : vo + dp;                       // rows of R
     const int row0 = rank * q.rows, nrow = max(0, min(q.rows, q.L - row0)), ns = min(srows, nrow);
-    float *gR = q.R + (size_t)row0 * dp;                       // rows ns .. nrow - 1 of this CTA
+    float *gR = q.R + ((ptrdiff_t)rank * max(q.rows - srows, 0) - ns) * (ptrdiff_t)dp;   // rows ns .. nrow - 1 of this CTA
     int *abort_flag = status + 1;
     unsigned gen = 0, round = 0;
     bool alive = true;
@@ -346,7 +346,7 @@ static std::vector<int> alternating_ctas(const std::vector<SeqDims> &sd, size_t 
 constexpr int ALT_SMEM = 226 * 1024 - 512 * 8;   // of 227 KB a CTA may have: the rest is the kernel's static share
 static size_t alternating_fixed(int dp, int rows) { return (size_t)dp * 8 + align_up((size_t)std::max(rows, 1), 2) * 8 + 32; }
 
-struct AltScratch { float *R; double *part; float *vbuf; double *vecs; unsigned *sync; int ncta, maxrows; };
+struct AltScratch { float *R; double *part; float *vbuf; double *vecs; unsigned *sync; int ncta, maxrows, srows; };
 static void plan_alternating(Arena &ar, const std::vector<SeqDims> &sd, int d, int sm_count, std::vector<AltScratch> &out)
 {
     const size_t dp = align_up((size_t)d, 4);
@@ -356,13 +356,16 @@ static void plan_alternating(Arena &ar, const std::vector<SeqDims> &sd, int d, i
         int rows = 1;
         for (size_t i = i0; i < i1; ++i) rows = std::max(rows, ceil_div(sd[i].L, c[i - i0]));
         rows = (int)align_up((size_t)rows, 2);
-        const bool far = alternating_fixed((int)dp, rows) > (size_t)ALT_SMEM;
+        // the vectors first, then as many rows of R as fit
+        const size_t fixed = alternating_fixed((int)dp, rows);
+        const bool far = fixed > (size_t)ALT_SMEM;
+        const int srows = far ? 0 : (int)std::min<size_t>((ALT_SMEM - fixed) / (dp * 4), (size_t)rows);
         for (size_t i = i0; i < i1; ++i) {
             AltScratch a;
             a.ncta = c[i - i0];
-            a.maxrows = rows;
+            a.maxrows = rows; a.srows = srows;
             a.vecs = far ? ar.take<double>((size_t)a.ncta * (rows + dp)) : nullptr;
-            a.R = ar.take<float>((size_t)sd[i].L * dp);
+            a.R = ar.take<float>((size_t)a.ncta * std::max(ceil_div(sd[i].L, a.ncta) - srows, 0) * dp);
             a.part = ar.take<double>((size_t)2 * a.ncta * (dp + 4));
             a.vbuf = ar.take<float>(dp);
             a.sync = ar.take<unsigned>(64);
@@ -411,12 +414,10 @@ static atp_status alternating_impl(atp_ctx *ctx, const atp_mat *X, const std::ve
             work += (double)s.r * s.L * d * 4;
         }
         if (work == 0) continue;
-        // the vectors first, then as many rows of R as fit
         const int maxrows = sc[i0].maxrows;
-        const size_t fixed = alternating_fixed(dp, maxrows);
-        const bool far = fixed > (size_t)ALT_SMEM;
-        int srows = far ? 0 : (int)std::min<size_t>((ALT_SMEM - fixed) / ((size_t)dp * 4), (size_t)maxrows);
-        const size_t smem = far ? 0 : fixed + (size_t)srows * dp * 4;
+        const bool far = alternating_fixed(dp, maxrows) > (size_t)ALT_SMEM;
+        int srows = sc[i0].srows;
+        const size_t smem = far ? 0 : alternating_fixed(dp, maxrows) + (size_t)srows * dp * 4;
         ATP_KERNEL(ctx, "alternating_init", 0, 0);
         alternating_init_kernel<<<b.count, 64, 0, ctx->stream>>>(b);
         ATP_LAUNCHED(ctx);

@@ -18,17 +18,17 @@ static size_t plan_linear(Arena &ar, int64_t total_rank, int64_t total_rows, int
         p.T = ar.take<float>((size_t)total_rank * d_out);
         if (swiglu) p.Tg = ar.take<float>((size_t)total_rank * d_out);
     }
-    if (swiglu) p.Yg = ar.take<float>((size_t)total_rows * d_out);
+    if (swiglu && !bf16) p.Yg = ar.take<float>((size_t)total_rows * d_out);
     return ar.off;
 }
 
-size_t linear_workspace_bytes(const std::vector<SeqDims> &seqs, int64_t d_out)
+size_t linear_workspace_bytes(const std::vector<SeqDims> &seqs, int64_t d_out, bool bf16)
 {
     int64_t tr = 0, tl = 0;
     for (auto &s : seqs) { tr += s.r; tl += s.L; }
     Arena ar(nullptr, (size_t)-1);
     LinearPlan p;
-    return plan_linear(ar, tr, tl, d_out, true, false, p);      // sized for the fp32 SwiGLU case (the largest one)
+    return plan_linear(ar, tr, tl, d_out, true, bf16, p);       // sized for SwiGLU (the largest one)
 }
 
 template <typename T>

@@ -52,12 +52,18 @@ struct Seq {
 struct Batch { Seq s[MAXSEQ]; int count; };
 
 // Number of 64 x 64 fp32 tiles of Cpart / C / Dpart, fp64 tiles of gpart, for a sequence of n rows and rt
-// columns handled by at most `ncta` CTAs.
+// columns handled by at most `ncta` CTAs: the partial results of the panel that has most (see KS and G in the kernel).
 struct Scratch { size_t cpart, c, dpart, gpart; };
-static inline Scratch scratch_tiles(int n, int rt, int ncta)
+static inline Scratch scratch_tiles(int n, int rt, int ncta, bool tensor)
 {
-    const size_t nt = (size_t)(n + 63) / 64, nj = (size_t)(rt + 63) / 64;
-    return Scratch{2 * (size_t)ncta + nj + 2, nj + 1, 2 * (size_t)ncta + nt + 2, nt + 1};   // (jobs make pairs of tiles)
+    const int nt = (n + 63) / 64, np = (rt + 63) / 64, nr = tensor ? (nt + 1) / 2 : nt;
+    Scratch s{1, (size_t)np + 1, 1, (size_t)nt + 1};
+    for (int nj = 1; nj < np && nt > 0; ++nj) {
+        const int nc = tensor ? (nj + 1) / 2 : nj;
+        s.cpart = std::max(s.cpart, (size_t)nj * std::min(nt, (ncta + nc - 1) / nc));
+        s.dpart = std::max(s.dpart, (size_t)nt * std::min(nj, (ncta + nr - 1) / nr));
+    }
+    return s;
 }
 
 // 64 x 64 tile of a row-major fp32 matrix, zero beyond rv rows / cv columns, in two halves so that the loads of
