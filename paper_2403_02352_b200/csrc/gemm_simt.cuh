@@ -21,11 +21,10 @@ struct GemmBatch {
 
 enum GemmEpiKind {
     EPI_STORE = 0,        // C = A B
-    EPI_D_MINUS = 1,      // C = D - A B
-    EPI_BIAS = 2,         // C = A B + bias
-    EPI_BIAS_GELU = 3,    // C = gelu_erf(A B + bias)
-    EPI_SILU_D_MUL = 4,   // C = silu(D) * (A B)
-    EPI_ROPE = 5          // pairs of columns of A B turned by (cos, sin) from D (tensor-core GEMM only)
+    EPI_BIAS = 1,         // C = A B + bias
+    EPI_BIAS_GELU = 2,    // C = gelu_erf(A B + bias)
+    EPI_SILU_D_MUL = 3,   // C = silu(D) * (A B)
+    EPI_ROPE = 4          // pairs of columns of A B turned by (cos, sin) from D (tensor-core GEMM only)
 };
 struct GemmEpi {
     int kind;
@@ -135,7 +134,6 @@ gemm_simt_kernel(const __grid_constant__ GemmBatch batch, GemmEpi epi, int split
             if (n >= pr.N) continue;
             float v = acc[i][j];
             switch (epi.kind) {
-                case EPI_D_MINUS: v = pr.D[(size_t)m * pr.ldd + n] - v; break;
                 case EPI_BIAS: if (epi.bias) v += epi.bias[n]; break;
                 case EPI_BIAS_GELU: if (epi.bias) v += epi.bias[n]; v = gelu_erf_f(v); break;
                 case EPI_SILU_D_MUL: v = silu_f(pr.D[(size_t)m * pr.ldd + n]) * v; break;

@@ -39,9 +39,10 @@ constexpr int VSTRIDE = 2 * BLK * BLK + 2 * BLK;   // floats of a published tran
 struct Seq {
     float *G, *Wt, *Vbuf;         // G, Wt: np x np (ld = np); Vbuf: 2 x npairs x VSTRIDE (by step parity)
     int *vflag;                   // 2 x npairs: the pair rotated in this step
-    unsigned *sync;               // 64 words. [0]: arrivals at the group barrier (monotonic); [32]: last
-                                  // barrier completed; [1..4]: largest scaled off-diagonal entry of a
-                                  // sweep, slot sweep % 4; [8..11]: the same over the whole matrix after the sweep; [5]: sweeps used; [16..17]: work tickets of the update, [20..21]: pivot blocks fetched, both by step parity
+    unsigned *sync;               // 64 words. [0]: arrivals at the group barrier (monotonic); largest scaled off-diagonal
+                                  // entry, slot sweep % 4: [1..4] met in a sweep, [8..11] in the whole matrix after it;
+                                  // [5]: sweeps used; by step parity: [16..17] work tickets of the update, [20..21] pivot
+                                  // blocks fetched
     int n, np, nb;                // size, padded size (multiple of 64), number of 32-row blocks (even)
     int cta0, ncta;               // the group of CTAs that owns this sequence
 };
@@ -713,14 +714,13 @@ __device__ void pivot_form_half(float *sm, const Seq &sq, const float *Gsrc, con
     }
 }
 
-// The update of a step is cut into strips. A strip of G: blocks (p, q0 .. q0 + cnt - 1) of the upper triangle,
-// updated in place together with their mirrors; a strip of Wt: the rows of pair p, column chunks
-// c0 .. c0 + cnt - 1 of 64, in place. The pivot CTAs of the same step read blocks of G as they were before the
-// update: before its first store of a step a CTA makes sure that all of them have fetched theirs (Fetched). Along a strip Vt_p stays in shared memory and
-// the next block is fetched into registers while the current one is multiplied. Short strips win at r~ = 2112: with
-// 296 CTAs a step has only a few items per CTA, and the last ones to finish set the time of the step (strips of
-// 2 + 3 blocks: 39.9 us per step, 1 + 2: 37.3 us).
-constexpr int SEG_G = 1, SEG_W = 2;
+// The update of a step is cut into items: a block (p, q), p <= q, of G, updated in place together with its mirror, or two
+// 64-column chunks of the rows of pair p of Wt, in place. The pivot CTAs of the same step read blocks of G as they were before
+// the update: before its first store of a step a CTA makes sure that all of them have fetched theirs (Fetched). Single blocks
+// rather than rows of them: at r~ = 2112 a step has about four items for each of 296 CTAs, and the last ones to finish set its
+// time (24 us; most of an item is the latency of its loads). The chunks of Wt share Vt_p, and the second one is fetched into
+// registers during the product of the first.
+constexpr int SEG_W = 2;
 
 __device__ __forceinline__ void store_tile_acc(float *dst, int ld, int m0, int n0, const float (&acc)[4][4])
 {
@@ -756,76 +756,50 @@ __device__ bool wait_fetched(Fetched &f)
     return f.ok;
 }
 
-__device__ bool g_strip(float *sm, const Seq &sq, float *G, const float *Vbuf, const int *vflag, int step, int p, int q0, int cnt, Fetched &fetched)
+// One block (p, q) of G on the fp32 units: Vt_p G_pq Vt_q^T.
+__device__ bool g_block(float *sm, const Seq &sq, float *G, const float *Vbuf, const int *vflag, int step, int p, int q, Fetched &fetched)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32, np = sq.np;
     float *Vp = sm, *Vq = sm + BLK * LDA, *Tm = sm + 2 * BLK * LDA, *Bk = sm + 3 * BLK * LDA;
-    const int fp = vflag[p];
-    int Ip, Jp;
+    const int fp = vflag[p], fq = vflag[q];
+    if (!fp && !fq) return true;                                 // unchanged block
+    int Ip, Jp, Iq, Jq;
     rr_pair(sq.nb, step, p, Ip, Jp);
-    float4 x[4];
-    auto fetch = [&](int q) {
-        int Iq, Jq;
-        rr_pair(sq.nb, step, q, Iq, Jq);
+    rr_pair(sq.nb, step, q, Iq, Jq);
+    // the block goes to the B tile when a row transform comes first, else straight to the T tile
+    float *blk_dst = fp ? Bk : Tm;
+    const int blk_ld = fp ? LDB : LDA;
 #pragma unroll
-        for (int it = 0; it < 4; ++it) {
-            const int f = tid + it * NT, i = f >> 4, c = (f & 15) * 4;
-            x[it] = __ldcg((const float4 *)(G + (size_t)glob_of_loc(Ip, Jp, i) * np + glob_of_loc(Iq, Jq, c)));
-        }
-    };
+    for (int it = 0; it < 4; ++it) {
+        const int f = tid + it * NT, i = f >> 4, c = (f & 15) * 4;
+        *(float4 *)(blk_dst + i * blk_ld + c) = __ldcg((const float4 *)(G + (size_t)glob_of_loc(Ip, Jp, i) * np + glob_of_loc(Iq, Jq, c)));
+        if (fp) *(float4 *)(Vp + i * LDA + c) = __ldcg((const float4 *)(Vbuf + (size_t)p * VSTRIDE + i * BLK + c));
+        if (fq) *(float4 *)(Vq + i * LDA + c) = __ldcg((const float4 *)(Vbuf + (size_t)q * VSTRIDE + i * BLK + c));
+    }
+    __syncthreads();
+    float acc[4][4];
     if (fp) {
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {
-            const int f = tid + it * NT, i = f >> 4, c = (f & 15) * 4;
-            *(float4 *)(Vp + i * LDA + c) = __ldcg((const float4 *)(Vbuf + (size_t)p * VSTRIDE + i * BLK + c));
+        product64_fma<false>(Vp, Bk, LDB, m0, n0, acc);
+        if (fq) {
+            store_tile_acc(Tm, LDA, m0, n0, acc);
+            __syncthreads();
         }
     }
-    fetch(q0);
-    for (int j = 0; j < cnt; ++j) {
-        const int q = q0 + j, fq = vflag[q];
-        int Iq, Jq;
-        rr_pair(sq.nb, step, q, Iq, Jq);
-        if (!fp && !fq) {                                        // unchanged block
-            if (j + 1 < cnt) fetch(q + 1);
-            continue;
-        }
-        // the block goes to the B tile when a row transform comes first, else straight to the T tile
-        float *blk_dst = fp ? Bk : Tm;
-        const int blk_ld = fp ? LDB : LDA;
+    if (fq) product64_fma<true>(Tm, Vq, LDA, m0, n0, acc);       // out = T * Vt_q^T
+    if (!wait_fetched(fetched)) return false;
+    const int gr0 = glob_of_loc(Ip, Jp, m0 + g), gr1 = glob_of_loc(Ip, Jp, m0 + g + 8);
 #pragma unroll
-        for (int it = 0; it < 4; ++it) {
-            const int f = tid + it * NT, i = f >> 4, c = (f & 15) * 4;
-            *(float4 *)(blk_dst + i * blk_ld + c) = x[it];
-            if (fq) *(float4 *)(Vq + i * LDA + c) = __ldcg((const float4 *)(Vbuf + (size_t)q * VSTRIDE + i * BLK + c));
+    for (int nt = 0; nt < 4; ++nt) {
+        const int gc = glob_of_loc(Iq, Jq, n0 + nt * 8 + 2 * t);         // gc, gc + 1 are contiguous
+        *(float2 *)(G + (size_t)gr0 * np + gc) = make_float2(acc[nt][0], acc[nt][1]);
+        *(float2 *)(G + (size_t)gr1 * np + gc) = make_float2(acc[nt][2], acc[nt][3]);
+        if (q != p) {                                            // mirror block
+            G[(size_t)gc * np + gr0] = acc[nt][0]; G[(size_t)(gc + 1) * np + gr0] = acc[nt][1];
+            G[(size_t)gc * np + gr1] = acc[nt][2]; G[(size_t)(gc + 1) * np + gr1] = acc[nt][3];
         }
-        __syncthreads();
-        if (j + 1 < cnt) fetch(q + 1);
-        float acc[4][4];
-        if (fp) {
-            product64_fma<false>(Vp, Bk, LDB, m0, n0, acc);
-            if (fq) {
-                store_tile_acc(Tm, LDA, m0, n0, acc);
-                __syncthreads();
-            }
-        }
-        if (fq) {                                                // out = T * Vt_q^T
-            product64_fma<true>(Tm, Vq, LDA, m0, n0, acc);
-        }
-        if (!wait_fetched(fetched)) return false;
-        const int gr0 = glob_of_loc(Ip, Jp, m0 + g), gr1 = glob_of_loc(Ip, Jp, m0 + g + 8);
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int gc = glob_of_loc(Iq, Jq, n0 + nt * 8 + 2 * t);     // gc, gc + 1 are contiguous
-            *(float2 *)(G + (size_t)gr0 * np + gc) = make_float2(acc[nt][0], acc[nt][1]);
-            *(float2 *)(G + (size_t)gr1 * np + gc) = make_float2(acc[nt][2], acc[nt][3]);
-            if (q != p) {                                        // mirror block
-                G[(size_t)gc * np + gr0] = acc[nt][0]; G[(size_t)(gc + 1) * np + gr0] = acc[nt][1];
-                G[(size_t)gc * np + gr1] = acc[nt][2]; G[(size_t)(gc + 1) * np + gr1] = acc[nt][3];
-            }
-        }
-        __syncthreads();                                         // tiles are reused by the next block
     }
+    __syncthreads();                                             // tiles are reused by the next block
     return true;
 }
 
@@ -980,36 +954,20 @@ __device__ void wt_strip_half(float *sm, const Seq &sq, const float *Vbuf, const
     __syncthreads();
 }
 
-// Work items of the update: first the strips of G (row by row of the upper triangle), then the strips of Wt.
-__host__ __device__ __forceinline__ int strips_of_g(int npairs)
-{
-    int n = 0;
-    for (int p = 0; p < npairs; ++p) n += (npairs - p + SEG_G - 1) / SEG_G;
-    return n;
-}
+// Work items of the update: first the blocks of G (row by row of the upper triangle), then the chunks of Wt.
+__host__ __device__ __forceinline__ int blocks_of_g(int npairs) { return npairs * (npairs + 1) / 2; }
 template <bool TENSOR>
 __device__ bool apply_item(float *sm, const Seq &sq, const float *Vbuf, const int *vflag, int step, int idx, int npairs, int items_g, int nw, Fetched &fetched)
 {
     if (idx < items_g) {
         int p = 0;
-        for (;;) {
-            const int n = (npairs - p + SEG_G - 1) / SEG_G;
-            if (idx < n) break;
-            idx -= n; ++p;
-        }
-        const int q0 = p + idx * SEG_G;
-        if (TENSOR) {
-            for (int q = q0; q < min(q0 + SEG_G, npairs); ++q)
-                if (!g_block_half(sm, sq, sq.G, Vbuf, vflag, step, p, q, fetched)) return false;
-            return true;
-        }
-        return g_strip(sm, sq, sq.G, Vbuf, vflag, step, p, q0, min(SEG_G, npairs - q0), fetched);
-    } else {
-        idx -= items_g;
-        const int nseg = (nw + SEG_W - 1) / SEG_W, p = idx / nseg, c0 = (idx - p * nseg) * SEG_W;
-        if (TENSOR) wt_strip_half(sm, sq, Vbuf, vflag, step, p, c0, min(SEG_W, nw - c0));
-        else wt_strip(sm, sq, Vbuf, vflag, step, p, c0, min(SEG_W, nw - c0));
+        while (idx >= npairs - p) { idx -= npairs - p; ++p; }
+        return TENSOR ? g_block_half(sm, sq, sq.G, Vbuf, vflag, step, p, p + idx, fetched) : g_block(sm, sq, sq.G, Vbuf, vflag, step, p, p + idx, fetched);
     }
+    idx -= items_g;
+    const int nseg = (nw + SEG_W - 1) / SEG_W, p = idx / nseg, c0 = (idx - p * nseg) * SEG_W;
+    if (TENSOR) wt_strip_half(sm, sq, Vbuf, vflag, step, p, c0, min(SEG_W, nw - c0));
+    else wt_strip(sm, sq, Vbuf, vflag, step, p, c0, min(SEG_W, nw - c0));
     return true;
 }
 
@@ -1075,7 +1033,7 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
     const int rank = (int)blockIdx.x - sq.cta0, tid = threadIdx.x;
     if (rank >= sq.ncta || sq.np <= 0) return;
     const int npairs = sq.nb / 2, nw = sq.np / BLK;
-    const int items_g = strips_of_g(npairs), total = items_g + npairs * ((nw + SEG_W - 1) / SEG_W);
+    const int items_g = blocks_of_g(npairs), total = items_g + npairs * ((nw + SEG_W - 1) / SEG_W);
     const int nsteps = sq.nb - 1;
     int *abort_flag = status + 1;
     unsigned gen = 0, gstep = 0;
@@ -1226,8 +1184,7 @@ static inline atp_status launch(atp_ctx *ctx, Batch &jb, float tol_conv, float t
     for (int i = 0; i < jb.count; ++i) {
         Seq &q = jb.s[i];
         const int npairs = q.nb / 2;
-        int items = npairs * ((q.np / BLK + SEG_W - 1) / SEG_W);                 // strips of the update
-        for (int pp = 0; pp < npairs; ++pp) items += (npairs - pp + SEG_G - 1) / SEG_G;
+        const int items = blocks_of_g(npairs) + npairs * ((q.np / BLK + SEG_W - 1) / SEG_W);     // of the update
         int c = (int)((double)total * ((double)q.np * q.np / wsum));
         c = std::max(1, std::min(c, std::max(items, 1)));
         if (q.np <= 0) c = 1;
