@@ -872,8 +872,9 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 }
                 // pass 0 only has to make the rows graded and roughly orthogonal (on ill-conditioned input it stalls at the
                 // noise floor of G, hence the cap of 8 sweeps); the second pass continues the same iteration on the rotated
-                // data with the rest of the budget. bf16: scaled off-diagonals below 3e-2 (1e-2 costs most inputs a sweep here
-                // and saves none there, 1e-1 costs one there); fp32: 1e-2 (3e-2 leaves the result at 8e-7 instead of 5e-7).
+                // data with the rest of the budget. bf16: scaled off-diagonals below 3e-2 (3 + 4 or 5 sweeps on the extractions
+                // of a layer, against 5 + 3 where the first pass ended by its visits at 1e-2; 1e-1 costs one in the second);
+                // fp32: 1e-2 (3e-2 leaves the result at 8e-7 instead of 5e-7).
                 const int nsw0 = std::min(8, (max_sweeps + 1) / 2);
                 const int nsw = pass == 0 ? nsw0 : std::max(1, max_sweeps - nsw0);
                 const float tolc = pass == 0 ? (kBf16 ? 3e-2f : 1e-2f) : tol_conv, tolr = pass == 0 ? 1e-3f : 0.1f * tol_conv;

@@ -573,7 +573,17 @@ static atp_status launch_form(atp_ctx *ctx, const HostProblem *probs, int count,
 
 // Pairs of CTAs (256 x 256 tiles) or single ones (128 x 128 tiles, 128 x 64 gated): the form with the smaller number of
 // waves times the time of a stage of one tile. A stage takes a pair about 560 cycles whatever runs beside it; a single CTA
-// about 330 when it has the L2 path to itself (all tiles in one wave), 500 when every SM loads at the full rate.
+// about 330 when it has the L2 path to itself (all tiles in one wave), 500 when every SM loads at the full rate. The weights
+// are those of one product; with two or three a stage takes both forms longer by about the same factor. All pairs / all
+// single / as chosen, us a launch:
+//   one product, linear layer (mean of its two launches) 512 rows, r 256, 1024 -> 1024  14.9 / 11.7 / 12.4
+//                4096 rows, r 2048, 4096 -> 4096  54.6 / 61.4 / 58.1;  gated, -> 11008  244 / 292 / 238
+//   two          Q = U_r Q', 1024 x 1024 x 256  16.9 / 11.0 / 10.8;  2048 x 4096 x 512  25.6 / 25.1 / 26.5
+//                4096 x 4096 x 2048  95.4 / 106 / 95.8
+//   three        rotary keys, 1024 x 1024 x 256  25.7 / 17.6 / 17.8;  4096 x 4096 x 2048  141 / 167 / 140
+//                Gram matrix, 576 x 576 x 2048  40.1 / 27.0 / 26.0;  2112 x 2112 x 4096  127 / 86.5 / 85.7
+// Over 24 such calls the choice is within 8 % of the better form, but for 1024 rows, r 256, 4096 columns (one product 35.3
+// against 32.3, two 16.9 against 14.9).
 template <bool DUAL>
 static inline bool choose_pairs(const HostProblem *probs, int count, int sm_count)
 {
