@@ -78,7 +78,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
     float *vc = (float *)(ud + maxrows), *vo = vc + dp;        // v of the current round and of the last one
     float *sR = FAR ? nullptr : vo + dp;                       // rows of R
     const int row0 = rank * q.rows, nrow = max(0, min(q.rows, q.L - row0)), ns = min(srows, nrow);
-    float *gR = q.R + ((ptrdiff_t)rank * max(q.rows - srows, 0) - ns) * (ptrdiff_t)dp;   // rows ns .. nrow - 1 of this CTA
+    float *gR = q.R + (size_t)rank * max(q.rows - srows, 0) * dp;   // rows ns .. nrow - 1 of this CTA
     int *abort_flag = status + 1;
     unsigned gen = 0, round = 0;
     bool alive = true;
@@ -86,7 +86,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
     float seen = 0.f;                                          // NaN once this lane has seen Inf or NaN in R
     for (int l = warp; l < nrow; l += NW) {
         const T *x = (const T *)q.X + (size_t)(row0 + l) * q.ldx_in;
-        float *r = (l < ns ? sR : gR) + (size_t)l * dp;
+        float *r = (l < ns ? sR + (size_t)l * dp : gR + (size_t)(l - ns) * dp);
         for (int k = lane; k < dp; k += 32) {
             const float v = k < d ? to_f32(x[k]) : 0.f;
             seen = fmaf(v, 0.f, seen);
@@ -114,7 +114,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
             const int pl = ns + warp;
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-                pre[i] = pl < nrow && lane * 4 + 128 * i < dp ? *(const float4 *)(gR + (size_t)pl * dp + lane * 4 + 128 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                pre[i] = pl < nrow && lane * 4 + 128 * i < dp ? *(const float4 *)(gR + (size_t)(pl - ns) * dp + lane * 4 + 128 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
             __syncthreads();                                   // v and the parts of |v|^2
             double usq = 0.0, vv = -1.0;
             auto norm_v = [&]() {                              // fixed order
@@ -189,7 +189,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
             }
             // rows in the workspace, one of a warp at a time, eight loads in flight
             for (int l = pl; l < nrow; l += NW) {
-                float *rp = gR + (size_t)l * dp;
+                float *rp = gR + (size_t)(l - ns) * dp;
                 const float up = deflate ? (float)ud[l] : 0.f;
                 double acc = 0.0, aw = 0.0;
                 for (int k0 = lane * 4; k0 < dp; k0 += 1024) {
@@ -214,7 +214,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
             if (__any_sync(0xffffffffu, seen != 0.f)) {          // (the whole warp again)
                 usq = 0.0;
                 for (int l = warp; l < nrow; l += NW) {
-                    const float *row = (l < ns ? sR : gR) + (size_t)l * dp;
+                    const float *row = (l < ns ? sR + (size_t)l * dp : gR + (size_t)(l - ns) * dp);
                     double acc = 0.0;
                     for (int k = lane; k < dp; k += 32) acc = fma((double)row[k], (double)vc[k], acc);
                     acc = lanes_sum(acc, 16);
@@ -232,7 +232,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
                 double a0 = 0.0, a1 = 0.0;
                 float2 g[4];
 #pragma unroll
-                for (int a = 0; a < 4; ++a) g[a] = ns + a < nrow ? *(const float2 *)(gR + (size_t)(ns + a) * dp + k) : make_float2(0.f, 0.f);
+                for (int a = 0; a < 4; ++a) g[a] = ns + a < nrow ? *(const float2 *)(gR + (size_t)a * dp + k) : make_float2(0.f, 0.f);
                 const float *col = sR + k;
                 // (a row with Inf or NaN has an infinite or NaN u, so its shifted elements need no care here)
                 auto add = [&](float2 x, double u) { a0 = fma((double)x.x, u, a0); a1 = fma(widen(x.y), u * WIDEN_SCALE, a1); };
@@ -251,7 +251,7 @@ alternating_kernel(const __grid_constant__ AltBatch batch, int d, int dp, int sr
 #pragma unroll
                 for (int a = 0; a < 4; ++a) if (ns + a < nrow) add(g[a], ud[ns + a]);
 #pragma unroll 4
-                for (l = ns + 4; l < nrow; ++l) add(*(const float2 *)(gR + (size_t)l * dp + k), ud[l]);
+                for (l = ns + 4; l < nrow; ++l) add(*(const float2 *)(gR + (size_t)(l - ns) * dp + k), ud[l]);
                 *(double2 *)(mine + k) = make_double2(a0, a1);
             }
             if (tid == 0) {
