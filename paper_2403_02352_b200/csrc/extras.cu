@@ -12,7 +12,7 @@
 // products accumulate in fp64, so that the only rounding of a step is the fp32 storage of u, v and R.
 // Bound by shared-memory reads and the widening of the elements to fp64 (half by the conversion instruction, 16 a clock and
 // SM, half by three integer operations each), and by the barrier and the partial sums of a round.
-// 16 sequences of 512 x 1024, r = 64, inner = 2: 5092 -> 1398 us (a chain of 320 launches that read R six times per
+// 16 sequences of 512 x 1024, r = 64, inner = 2: 5092 -> 1360 us (a chain of 320 launches that read R six times per
 // component from L2 before).
 #include "common.cuh"
 #include "group_barrier.cuh"
