@@ -123,7 +123,7 @@ def test_end_to_end_on_gap_inputs_of_each_workload(ctx, name):
     print(f"T3 {name}: err(U_r X_r) {worst_p:.2e}  err(O) {worst_o:.2e}  signs {agree}/{total}")
     assert agree == total
     # U_r X_r is sign- and rotation-free: storage precision. O multiplies the basis error by logits of order
-    # 10^2 before the exponential, so its end-to-end bar is looser than the stage bar (tolerances).
+    # 10^2 before the exponential, so its end-to-end bar is looser than the stage bar.
     assert worst_p <= (1e-5 if dt == "f32" else 2e-2)
     assert worst_o <= (2e-3 if dt == "f32" else 1e-1)
 
