@@ -34,7 +34,7 @@ constexpr int NT = 256;           // threads per CTA
 constexpr int LDA = 68;           // shared-memory row stride (floats) of A-operand style tiles
 constexpr int LDB = 72;           // shared-memory row stride of B-operand style tiles
 constexpr int MAXSEQ = 32;        // sequences per launch
-constexpr int VSTRIDE = 2 * BLK * BLK + 2 * BLK;   // floats of a published transform (see below)
+constexpr int VSTRIDE = 2 * BLK * BLK + 2 * BLK + 2 * JB * JB;   // floats of a published transform (see below)
 
 struct Seq {
     float *G, *Wt, *Vbuf;         // G, Wt: np x np (ld = np); Vbuf: 2 x npairs x VSTRIDE (by step parity)
@@ -55,10 +55,22 @@ constexpr size_t SMEM_BYTES = (size_t)4 * SLOT * sizeof(float);
 
 __device__ __forceinline__ void rr_pair(int nb, int step, int t, int &I, int &J)
 {
-    const int m = nb - 1;
-    if (t == 0) { I = m; J = step % m; }
-    else { I = (step + t) % m; J = (step - t + m) % m; }
+    const int m = nb - 1;                    // 0 <= step < m, 0 <= t < nb / 2
+    if (t == 0) { I = m; J = step; }
+    else { I = step + t; J = step - t; I -= I >= m ? m : 0; J += J < 0 ? m : 0; }
     if (I > J) { const int x = I; I = J; J = x; }
+}
+// The pair t that block b is in at a step, its two blocks and which of them b is.
+__device__ __forceinline__ void rr_locate(int nb, int step, int b, int &t, int &h, int &I, int &J)
+{
+    const int m = nb - 1;
+    int x = b - step, other;
+    x += x < 0 ? m : 0;
+    if (b == m) { t = 0; other = step; }
+    else if (x == 0) { t = 0; other = m; }
+    else if (x < nb / 2) { t = x; other = step - t; other += other < 0 ? m : 0; }
+    else { t = m - x; other = step + t; other -= other >= m ? m : 0; }
+    I = min(b, other); J = max(b, other); h = b == J;
 }
 
 using ::group_barrier;
@@ -170,25 +182,23 @@ template <int W> struct Band {
     __device__ __forceinline__ float load(const float *As)
     {
         const int k = threadIdx.x & 31;
-        const float de = fmaxf(As[k * (LDP + 1)], 0.f), dd = fmaxf(As[(32 + k) * (LDP + 1)], 0.f);
-        float mo = 0.f;
-        auto see = [&](float g, float d0, float d1) {
-            const float d2 = d0 * d1;
-            if (d2 > 0.f) mo = fmaxf(mo, fabsf(g) * rsqrtf(d2));
-        };
+        const float de = As[k * (LDP + 1)], dd = As[(32 + k) * (LDP + 1)];
+        const float re = de > 0.f ? rsqrtf(de) : 0.f, ro = dd > 0.f ? rsqrtf(dd) : 0.f;
+        float me = 0.f, mo = 0.f;                                // in the even rows and in the odd ones, without re and ro
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
             const int l = (k + D0 + i) & 31;
             ee[i] = As[k * LDP + l]; eo[i] = As[k * LDP + 32 + l];
             oe[i] = As[(32 + k) * LDP + l]; oo[i] = As[(32 + k) * LDP + 32 + l];
-            const float le = fmaxf(As[l * (LDP + 1)], 0.f), lo = fmaxf(As[(32 + l) * (LDP + 1)], 0.f);
-            if (D0 + i > 0) { see(ee[i], de, le); see(oo[i], dd, lo); }
-            see(eo[i], de, lo); see(oe[i], dd, le);
+            const float le = __shfl_sync(0xffffffffu, re, l), lo = __shfl_sync(0xffffffffu, ro, l);
+            if (D0 + i > 0) { me = fmaxf(me, fabsf(ee[i]) * le); mo = fmaxf(mo, fabsf(oo[i]) * lo); }
+            me = fmaxf(me, fabsf(eo[i]) * lo); mo = fmaxf(mo, fabsf(oe[i]) * le);
         }
+        mo = fmaxf(me * re, mo * ro);
         return mo;
     }
-    // the 32 rounds; with `store` the diagonal quadrants (both blocks after the cross rotations) go back to As
-    __device__ __forceinline__ void rounds(float *As, PivotShared &sh, float tol2, bool store)
+    // the 32 rounds; the diagonal quadrants (both blocks after the cross rotations) go back to As
+    __device__ __forceinline__ void rounds(float *As, PivotShared &sh, float tol2)
     {
         const int k = threadIdx.x & 31, km = (k - 1) & 31;
         float2 own = make_float2(0.f, 0.f), nxt = own;           // warp 0: rotations of the pairs k and k + 1
@@ -233,15 +243,13 @@ template <int W> struct Band {
             if (W == 3) oe[ND - 1] = wrap;
             __syncthreads();
         }
-        if (store) {
-            const float de = sh.sd[0][k], dd = sh.sd[0][32 + k];
+        const float de = sh.sd[0][k], dd = sh.sd[0][32 + k];
 #pragma unroll
-            for (int i = 0; i < ND; ++i) {
-                const int l = (k + D0 + i) & 31;
-                const float e = ee[i] * de * sh.sd[0][l], o = oo[i] * dd * sh.sd[0][32 + l];
-                As[k * LDP + l] = e; As[l * LDP + k] = e;
-                As[(32 + k) * LDP + 32 + l] = o; As[(32 + l) * LDP + 32 + k] = o;
-            }
+        for (int i = 0; i < ND; ++i) {
+            const int l = (k + D0 + i) & 31;
+            const float e = ee[i] * de * sh.sd[0][l], o = oo[i] * dd * sh.sd[0][32 + l];
+            As[k * LDP + l] = e; As[l * LDP + k] = e;
+            As[(32 + k) * LDP + 32 + l] = o; As[(32 + l) * LDP + 32 + k] = o;
         }
     }
 };
@@ -384,7 +392,7 @@ __device__ void pivot_load(float *sm, const float *G, int np, int I, int J)
 // vout. cross_only: the 32 rounds that pair the two blocks' rows; otherwise all 63 rounds. Returns the largest
 // scaled off-diagonal entry found in the block before rotating (block-uniform); when it is <= tol_rot nothing is
 // rotated or published.
-template <int W> __device__ __forceinline__ float pivot_warp(float *As, PivotShared &sh, bool cross_only, float tol_rot)
+template <int W> __device__ __forceinline__ float pivot_warp(float *As, PivotShared &sh, bool cross_only, float tol_rot, float *quad)
 {
     const float tol2 = tol_rot * tol_rot;
     Band<W> band;
@@ -395,8 +403,17 @@ template <int W> __device__ __forceinline__ float pivot_warp(float *As, PivotSha
     __syncthreads();
     mo = fmaxf(fmaxf(sh.red[0], sh.red[1]), fmaxf(sh.red[2], sh.red[3]));
     if (!(mo > tol_rot)) return mo;
-    band.rounds(As, sh, tol2, !cross_only);
-    if (!cross_only) {
+    band.rounds(As, sh, tol2);
+    if (cross_only) {
+        asm volatile("bar.sync 3, 128;" ::: "memory");           // these four warps
+        const int f = threadIdx.x & 127;
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            const int q = it >> 1, e = (f + (it & 1) * 128) * 4;
+            const float *src = As + (q * JB + (e >> 5)) * LDP + q * JB + (e & 31);
+            *(float4 *)(quad + q * JB * JB + e) = make_float4(src[0], src[1], src[2], src[3]);
+        }
+    } else {
         __syncthreads();
         if (W == 0) {
             inner_phase<16>(As, sh, tol2, 1); inner_phase<8>(As, sh, tol2, 0); inner_phase<4>(As, sh, tol2, 1);
@@ -415,8 +432,9 @@ template <int W> __device__ __forceinline__ float pivot_warp(float *As, PivotSha
 //         back by s_p, s_q. What is left out is below 2^-35 s_i s_j, on top of 2^-22 of the entries themselves.
 //   VU  = Vt times V_SCALE in the same form: rotates the rows of Wt, whose entries are at most 1.
 //   d, s as 64 floats each (s = d where the pair was not rotated).
+// Behind them, for every input and where the 32 rounds alone were done: the two 32 x 32 diagonal blocks of the rotated pivot block.
 constexpr float V_SCALE = 8192.f, G_SCALE = 1024.f, T_SCALE = 256.f;
-constexpr int V_VU = BLK * BLK, V_D = 2 * BLK * BLK, V_S = V_D + BLK;     // offsets in floats
+constexpr int V_VU = BLK * BLK, V_D = 2 * BLK * BLK, V_S = V_D + BLK, V_Q = V_S + BLK;     // offsets in floats
 constexpr int LDV = 66;           // row stride of the transform in shared memory
 __device__ __forceinline__ float inv_pow2(float x) { return __uint_as_float(0x7f000000u - __float_as_uint(x)); }
 
@@ -437,10 +455,10 @@ __device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *
         vout[V_D + tid] = d;
         vout[V_S + tid] = d;                                     // (overwritten below where rows are rotated)
     }
-    if (warp == 0) mo = pivot_warp<0>(As, sh, cross_only, tol_rot);
-    else if (warp == 1) mo = pivot_warp<1>(As, sh, cross_only, tol_rot);
-    else if (warp == 2) mo = pivot_warp<2>(As, sh, cross_only, tol_rot);
-    else if (warp == 3) mo = pivot_warp<3>(As, sh, cross_only, tol_rot);
+    if (warp == 0) mo = pivot_warp<0>(As, sh, cross_only, tol_rot, vout + V_Q);
+    else if (warp == 1) mo = pivot_warp<1>(As, sh, cross_only, tol_rot, vout + V_Q);
+    else if (warp == 2) mo = pivot_warp<2>(As, sh, cross_only, tol_rot, vout + V_Q);
+    else if (warp == 3) mo = pivot_warp<3>(As, sh, cross_only, tol_rot, vout + V_Q);
     else {
         const int h = warp - 4;
         __syncthreads();
@@ -621,11 +639,12 @@ __device__ __forceinline__ void put4_clamped(__half *tile, int row, int c, float
 }
 __device__ __forceinline__ float4 inv_pow2_4(float4 v) { return make_float4(inv_pow2(v.x), inv_pow2(v.y), inv_pow2(v.z), inv_pow2(v.w)); }
 // accumulator of a product, times k, as fp16 parts of the same 64 x 64 tile position
-__device__ __forceinline__ void put_acc(__half *tile, int m0, int n0, const float (&acc)[4][4], float k)
+template <int NTILE>
+__device__ __forceinline__ void put_acc(__half *tile, int m0, int n0, const float (&acc)[NTILE][4], float k)
 {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
+    for (int nt = 0; nt < NTILE; ++nt)
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const float x = fminf(fmaxf(acc[nt][2 * e] * k, -60000.f), 60000.f), y = fminf(fmaxf(acc[nt][2 * e + 1] * k, -60000.f), 60000.f);
@@ -711,6 +730,138 @@ __device__ void pivot_form_half(float *sm, const Seq &sq, const float *Gsrc, con
                 As[i * LDP + j] = v;
                 if (up && n0 != 0) As[j * LDP + i] = v;
             }
+    }
+}
+
+// The same where the current step did the 32 cross rounds only: the diagonal blocks of N are then those of the rotated pivot
+// blocks, published with the transforms (or still in G, where the pair was not rotated), and W1 X12 W2^T is all that is left
+// to form: one block of G to fetch instead of three, a quarter of the arithmetic (5400 -> 3300 cycles of a step at r~ = 1088 in
+// bf16, 15500 -> 9000 at r~ = 192 in fp32; jacobi_persistent of one 32768 x 1088 iterate 4730 -> 3740 us).
+template <bool TENSOR>
+__device__ void pivot_form_cross(float *sm, const Seq &sq, const float *Vcur, int step, int b1, int b2, const int *flags, unsigned *fetched)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, np = sq.np;
+    __shared__ float srow[BLK];
+    int p1, h1, I1, J1, p2, h2, I2, J2;
+    rr_locate(sq.nb, step, b1, p1, h1, I1, J1);
+    rr_locate(sq.nb, step, b2, p2, h2, I2, J2);
+    const int f1 = flags[p1], f2 = flags[p2];
+    const float *P1 = Vcur + (size_t)p1 * VSTRIDE, *P2 = Vcur + (size_t)p2 * VSTRIDE;
+    float *As = sm;                                              // slot 0; the operands live in the others
+    const int c = (tid & 15) * 4;
+    float4 x[4], q[2];
+#pragma unroll
+    for (int it = 0; it < 4; ++it)
+        x[it] = __ldcg((const float4 *)(sq.G + (size_t)glob_of_loc(I1, J1, (tid >> 4) + 16 * it) * np + glob_of_loc(I2, J2, c)));
+    const int qi = tid >> 3, qc = (tid & 7) * 4;
+    q[0] = __ldcg((const float4 *)(f1 ? P1 + V_Q + h1 * JB * JB + qi * JB + qc : sq.G + (size_t)(b1 * JB + qi) * np + b1 * JB + qc));
+    q[1] = __ldcg((const float4 *)(f2 ? P2 + V_Q + h2 * JB * JB + qi * JB + qc : sq.G + (size_t)(b2 * JB + qi) * np + b2 * JB + qc));
+    if constexpr (TENSOR) {
+        __half *Wc = (__half *)(sm + SLOT), *S = (__half *)(sm + 2 * SLOT);
+        const float4 cs = inv_pow2_4(__ldcg((const float4 *)(P2 + V_D + c)));
+        float d[4];
+        uint4 w[4];
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            d[it] = __ldcg(P1 + V_D + (tid >> 4) + 16 * it);
+            const int r = (tid >> 3) + 32 * (it & 1), e = (tid & 7) * 8, row = ((it & 1) ? h2 : h1) * JB + (r & (JB - 1));
+            if ((it & 1) ? f2 : f1) w[it] = __ldcg((const uint4 *)(((it & 1) ? P2 : P1) + (it >> 1) * (BLK * BLK / 2) + (row * BLK + e) / 2));
+            else {                                               // V_SCALE times the identity (0x7000: 8192 in fp16)
+                uint32_t u[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) u[k] = it < 2 && (row - e) >> 1 == k ? ((row & 1) ? 0x70000000u : 0x7000u) : 0u;
+                w[it] = make_uint4(u[0], u[1], u[2], u[3]);
+            }
+        }
+        if (tid < BLK) srow[tid] = tid < JB ? __ldcg(P1 + V_S + h1 * JB + tid) : __ldcg(P2 + V_S + h2 * JB + tid - JB);
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            *(uint4 *)(Wc + (it >> 1) * hs::PLANE + ((tid >> 3) + 32 * (it & 1)) * hs::LDH + (tid & 7) * 8) = w[it];
+            put4_clamped(S, (tid >> 4) + 16 * it, c, x[it], cs, inv_pow2(d[it]) * G_SCALE);
+        }
+    } else {
+        float *Wc = sm + SLOT, *S = sm + 2 * SLOT;
+        float4 w[4];
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            const int r = (tid >> 4) + 16 * it, row = (it < 2 ? h1 : h2) * JB + (r & (JB - 1));
+            if (it < 2 ? f1 : f2) w[it] = __ldcg((const float4 *)((it < 2 ? P1 : P2) + row * BLK + c));
+            else w[it] = make_float4(row == c ? 1.f : 0.f, row == c + 1 ? 1.f : 0.f, row == c + 2 ? 1.f : 0.f, row == c + 3 ? 1.f : 0.f);
+        }
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            *(float4 *)(Wc + ((tid >> 4) + 16 * it) * LDA + c) = w[it];
+            *(float4 *)(S + ((tid >> 4) + 16 * it) * LDB + c) = x[it];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        float *dst = As + (k * JB + qi) * LDP + k * JB + qc;
+        dst[0] = q[k].x; dst[1] = q[k].y; dst[2] = q[k].z; dst[3] = q[k].w;
+    }
+    __syncthreads();
+    if (tid == 0) atomicAdd(fetched, 1u);                       // the old blocks are on chip: the update may overwrite them
+    if constexpr (TENSOR) {
+        __half *Wc = (__half *)(sm + SLOT), *S = (__half *)(sm + 2 * SLOT), *T = (__half *)(sm + 3 * SLOT);
+        const int g = lane >> 2, t = lane & 3;
+        {   // T = W1 X12: 32 x 64, a 16 x 16 part per warp
+            const int m0 = (warp & 1) * 16, n0 = (warp >> 1) * 16;
+            float acc[2][4] = {};
+            hs::product16<false>(Wc, S, m0, n0, acc);
+            constexpr float k1 = T_SCALE / (V_SCALE * G_SCALE);
+            put_acc(T, m0, n0, acc, k1);
+        }
+        __syncthreads();
+        if (warp < 4) {   // T W2^T: 32 x 32
+            const int m0 = (warp & 1) * 16, n0 = (warp >> 1) * 16;
+            float acc[2][4] = {};
+            hs::product16<true>(T, Wc + JB * hs::LDH, m0, n0, acc);
+            constexpr float k2 = 1.f / (T_SCALE * V_SCALE);
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int i = m0 + g + (e >> 1) * 8, j = JB + n0 + nt * 8 + 2 * t + (e & 1);
+                    const float v = acc[nt][e] * k2 * srow[i] * srow[j];
+                    As[i * LDP + j] = v;
+                    As[j * LDP + i] = v;
+                }
+        }
+    } else {
+        const float *Wc = sm + SLOT, *S = sm + 2 * SLOT;
+        float *T = sm + 3 * SLOT;
+        {   // two rows, four columns a thread
+            const int r = (tid >> 4) * 2;
+            float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+#pragma unroll 4
+            for (int k = 0; k < BLK; ++k) {
+                const float4 b = *(const float4 *)(S + k * LDB + c);
+                const float u = Wc[r * LDA + k], v = Wc[(r + 1) * LDA + k];
+                a0.x = fmaf(u, b.x, a0.x); a0.y = fmaf(u, b.y, a0.y); a0.z = fmaf(u, b.z, a0.z); a0.w = fmaf(u, b.w, a0.w);
+                a1.x = fmaf(v, b.x, a1.x); a1.y = fmaf(v, b.y, a1.y); a1.z = fmaf(v, b.z, a1.z); a1.w = fmaf(v, b.w, a1.w);
+            }
+            *(float4 *)(T + r * LDA + c) = a0;
+            *(float4 *)(T + (r + 1) * LDA + c) = a1;
+        }
+        __syncthreads();
+        const int r = tid >> 3, j0 = tid & 7;                    // columns j0, j0 + 8, ...: rows of W2 without bank conflicts
+        float acc[4] = {};
+#pragma unroll 4
+        for (int k = 0; k < BLK; k += 4) {
+            const float4 a = *(const float4 *)(T + r * LDA + k);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float4 b = *(const float4 *)(Wc + (JB + j0 + 8 * e) * LDA + k);
+                acc[e] = fmaf(a.x, b.x, acc[e]); acc[e] = fmaf(a.y, b.y, acc[e]);
+                acc[e] = fmaf(a.z, b.z, acc[e]); acc[e] = fmaf(a.w, b.w, acc[e]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int j = JB + j0 + 8 * e;
+            As[r * LDP + j] = acc[e];
+            As[j * LDP + r] = acc[e];
+        }
     }
 }
 
@@ -1023,7 +1174,6 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
                          int raise_not_converged, int *status)
 {
     extern __shared__ __align__(16) float j3sm[];
-    __shared__ short pair_of[2 * MAXPAIRS];       // block -> 2 * pair + half, for the current step
     __shared__ int flag_s[MAXPAIRS];              // the pairs rotated in the current step
     __shared__ int ticket_s;
     int si = 0;
@@ -1079,22 +1229,18 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
             Fetched fetched{sq.sync + 20 + par, has_next ? (unsigned)npairs : 0u, abort_flag, false};
             // 1. pivots of the next step
             if (has_next && rank < npairs) {
-                if (tid < npairs) {
-                    int I, J;
-                    rr_pair(sq.nb, step, tid, I, J);
-                    pair_of[I] = (short)(2 * tid); pair_of[J] = (short)(2 * tid + 1);
-                }
-                __syncthreads();
                 for (int pr = rank; pr < npairs; pr += sq.ncta) {
-                    int I2, J2;
-                    rr_pair(sq.nb, nstep, pr, I2, J2);
-                    const int p1 = pair_of[I2] >> 1, h1 = pair_of[I2] & 1, p2 = pair_of[J2] >> 1, h2 = pair_of[J2] & 1;
+                    int b1, b2, p1, h1, p2, h2, I, J;
+                    rr_pair(sq.nb, nstep, pr, b1, b2);
+                    rr_locate(sq.nb, step, b1, p1, h1, I, J);
+                    rr_locate(sq.nb, step, b2, p2, h2, I, J);
                     const int f1 = flag_s[p1], f2 = flag_s[p2];
                     if (!f1 && !f2) {
-                        pivot_load(j3sm, sq.G, sq.np, I2, J2);
+                        pivot_load(j3sm, sq.G, sq.np, b1, b2);
                         __syncthreads();
                         if (tid == 0) atomicAdd(sq.sync + 20 + par, 1u);
-                    } else if (TENSOR) pivot_form_half(j3sm, sq, sq.G, Vcur, step, p1, h1, f1, p2, h2, f2, sq.sync + 20 + par);
+                    } else if (step > 0) pivot_form_cross<TENSOR>(j3sm, sq, Vcur, step, b1, b2, flag_s, sq.sync + 20 + par);
+                    else if (TENSOR) pivot_form_half(j3sm, sq, sq.G, Vcur, step, p1, h1, f1, p2, h2, f2, sq.sync + 20 + par);
                     else pivot_form(j3sm, sq, sq.G, Vcur, step, p1, h1, f1, p2, h2, f2, sq.sync + 20 + par);
                     pivot_finish(nsweep, nstep, pr, par ^ 1);
                 }

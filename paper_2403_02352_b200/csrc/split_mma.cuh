@@ -65,6 +65,30 @@ __device__ __forceinline__ void product64(const __half *At, const __half *Bt, in
     }
 }
 
+// The same for a 16 x 16 part of the result and A = At.
+template <bool B_T>
+__device__ __forceinline__ void product16(const __half *At, const __half *Bt, int m0, int n0, float (&acc)[2][4])
+{
+    const int lane = threadIdx.x & 31, l8 = lane & 7, b3 = (lane >> 3) & 1, b4 = lane >> 4;
+    const uint32_t a0 = (uint32_t)__cvta_generic_to_shared(At) + 2 * ((m0 + l8 + 8 * b3) * LDH + 8 * b4);
+    const uint32_t b0 = (uint32_t)__cvta_generic_to_shared(Bt) + 2 * (B_T ? (n0 + l8 + 8 * b4) * LDH + 8 * b3 : (l8 + 8 * b3) * LDH + n0 + 8 * b4);
+    constexpr uint32_t BS = 2 * (B_T ? 16 : 16 * LDH);
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+        uint32_t ah[4], al[4], bh[4], bl[4];
+        ldsm4<false>(a0 + ks * 32, ah);
+        ldsm4<false>(a0 + ks * 32 + 2 * PLANE, al);
+        ldsm4<!B_T>(b0 + ks * BS, bh);
+        ldsm4<!B_T>(b0 + ks * BS + 2 * PLANE, bl);
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) mma_f16(acc[nt], al, bh[2 * nt], bh[2 * nt + 1]);
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) mma_f16(acc[nt], ah, bl[2 * nt], bl[2 * nt + 1]);
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) mma_f16(acc[nt], ah, bh[2 * nt], bh[2 * nt + 1]);
+    }
+}
+
 // Power of two s with |x| s < 2^top for every |x| <= max (max given by its bits), and its inverse.
 __device__ __forceinline__ float2 scale_for(unsigned max_bits, int top)
 {
