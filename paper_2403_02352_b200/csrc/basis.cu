@@ -610,7 +610,7 @@ static void plan_basis(Arena &ar, const std::vector<SeqDims> &sd, int d, int ove
             p.Wth = take_bf16((size_t)p.np * p.np); p.Wtl = take_bf16((size_t)p.np * p.np);
             p.Wsh = take_bf16((size_t)std::max(rt, 1) * ldw); p.Wsl = take_bf16((size_t)std::max(rt, 1) * ldw);
         }
-        p.jsync = ar.take<unsigned>(64);
+        p.jsync = ar.take<unsigned>(j3::SYNC_WORDS + (size_t)2 * sm_count);
         p.needfix = ar.take<int>(std::max(p.dims.r, 1));
         p.maxoff = ar.take<unsigned>(1);
         p.conv = ar.take<int>(1);
@@ -825,7 +825,7 @@ static atp_status basis_impl(atp_ctx *ctx, const atp_mat *X, const std::vector<S
                 const int ldr = (int)align_up((size_t)std::max(p.rt, 1), 8), ldw = (int)align_up((size_t)std::max(p.dims.r, 1), 8);
                 g.p[k] = GemmProblem{Xb(p), p.Y, p.BW, nullptr, p.rt > 0 ? d : 0, p.rt, p.dims.L, (int)X->ld, p.rt, p.rt, 0};
                 gg.p[k] = GemmProblem{p.BW, p.BW, p.G, nullptr, p.rt, p.rt, p.rt > 0 ? d : 0, p.rt, p.rt, p.np, 0};
-                jb.s[k] = j3::Seq{p.G, p.Wt, p.Vbuf, p.vflag, p.jsync, p.rt, p.np, p.np / j3::JB, 0, 0};
+                jb.s[k] = j3::Seq{p.G, p.Wt, p.Vbuf, p.vflag, p.jsync, p.rt, p.np, p.np / j3::JB, 0, 0, 0, 0};
                 fb.s[k] = Fin2Seq{p.G, p.Wt, p.Y, p.sig, p.ord, p.tsum, p.Wsel, p.needfix,
                                   (T *)X_r->data + (size_t)p.dims.rank0 * X_r->ld, (T *)U_r->data + (size_t)p.dims.row0 * U_r->ld,
                                   sigma ? sigma + p.dims.rank0 : nullptr, p.rt, p.dims.r, d, p.dims.L, kBf16 ? ldr : p.rt, (int)X_r->ld, (int)U_r->ld, p.np,

@@ -34,6 +34,7 @@ constexpr int NT = 256;           // threads per CTA
 constexpr int LDA = 68;           // shared-memory row stride (floats) of A-operand style tiles
 constexpr int LDB = 72;           // shared-memory row stride of B-operand style tiles
 constexpr int MAXSEQ = 32;        // sequences per launch
+constexpr int SYNC_WORDS = 64;    // words of Seq::sync before the list of SMs (which the first sequence of a launch holds)
 constexpr int VSTRIDE = 2 * BLK * BLK + 2 * BLK + 2 * JB * JB;   // floats of a published transform (see below)
 
 struct Seq {
@@ -42,11 +43,17 @@ struct Seq {
     unsigned *sync;               // 64 words. [0]: arrivals at the group barrier (monotonic); largest scaled off-diagonal
                                   // entry, slot sweep % 4: [1..4] met in a sweep, [8..11] in the whole matrix after it;
                                   // [5]: sweeps used; by step parity: [16..17] work tickets of the update, [20..21] pivot
-                                  // blocks fetched
+                                  // blocks fetched; [32]: arrivals of the whole launch
     int n, np, nb;                // size, padded size (multiple of 64), number of 32-row blocks (even)
-    int cta0, ncta;               // the group of CTAs that owns this sequence
+    int ncta, npu;                // CTAs that own this sequence; those of them that solve pivot blocks
+    int pivot0, worker0;          // numbers of the first of its pivot CTAs and of the first of the others (see seat_of)
 };
-struct Batch { Seq s[MAXSEQ]; int count; };
+struct Batch {
+    Seq s[MAXSEQ]; int count;
+    int pivots;                   // pivot CTAs of all sequences
+    bool seated;                  // two CTAs to an SM: roles by seat_of, else by block number
+    unsigned *grid_sync, *smids;  // arrivals of all CTAs of the launch (zero at the start); the SM of each of them
+};
 
 // Bytes of dynamic shared memory: four tile slots of 64 x LDB floats (pivot phase: the old blocks and the
 // transforms the pivot block is formed from, then A and Vt; apply phase: Vt_p, Vt_q, T and the G block).
@@ -735,7 +742,7 @@ __device__ void pivot_form_half(float *sm, const Seq &sq, const float *Gsrc, con
 
 // The same where the current step did the 32 cross rounds only: the diagonal blocks of N are then those of the rotated pivot
 // blocks, published with the transforms (or still in G, where the pair was not rotated), and W1 X12 W2^T is all that is left
-// to form: one block of G to fetch instead of three, a quarter of the arithmetic (5400 -> 3300 cycles of a step at r~ = 1088 in
+// to form: one block of G to fetch instead of three, a quarter of the arithmetic (10000 -> 6500 cycles of a step at r~ = 1088 in
 // bf16, 15500 -> 9000 at r~ = 192 in fp32; jacobi_persistent of one 32768 x 1088 iterate 4730 -> 3740 us).
 template <bool TENSOR>
 __device__ void pivot_form_cross(float *sm, const Seq &sq, const float *Vcur, int step, int b1, int b2, const int *flags, unsigned *fetched)
@@ -1134,7 +1141,54 @@ __device__ bool apply_item(float *sm, const Seq &sq, const float *Vbuf, const in
 // blocks it forms its pivot block from. Vt and the rotated-flags are double buffered by step parity, because
 // the pivots of step s+1 publish while the update of step s still reads.
 // status[0]: sticky device status word of the context; status[1]: abort flag of bounded waits.
+constexpr int MATE_ITEMS = 2;
 constexpr int MAXPAIRS = 72;                  // np <= 4608
+
+// Number of this CTA in the order in which roles are given out: pivot solves go to CTAs on SMs of their own (two of them on one
+// SM, or one beside a CTA of the update, take 13000 cycles for their 32 rounds instead of 9400, and blocks that follow one
+// another do share an SM). First come the CTAs with the lowest block number of their SM, then the second CTAs of the SMs without
+// a pivot, last those beside a pivot; numbers that no sequence uses leave the kernel. -1: the wait for the other CTAs ran out.
+constexpr int MAXGRID = 1024;
+__device__ int seat_of(const Batch &batch, int *abort_flag)
+{
+    __shared__ int first[MAXGRID];
+    __shared__ unsigned prim[MAXGRID / 32], away[MAXGRID / 32], beside[MAXGRID / 32];
+    const int tid = threadIdx.x, n = (int)gridDim.x, n32 = (n + 31) & ~31;
+    unsigned sm;
+    asm("mov.u32 %0, %%smid;" : "=r"(sm));
+    if (tid == 0) batch.smids[blockIdx.x] = sm;
+    for (int i = tid; i < MAXGRID; i += NT) first[i] = n;
+    if (!group_barrier(batch.grid_sync, 1u, (unsigned)n, abort_flag)) return -1;
+    auto sm_of = [&](int b) { return (int)(__ldcg(batch.smids + b) % MAXGRID); };
+    auto below = [](const unsigned *mask, int b) {               // bits set below b
+        int c = __popc(mask[b >> 5] & ((1u << (b & 31)) - 1u));
+        for (int k = 0; k < b >> 5; ++k) c += __popc(mask[k]);
+        return c;
+    };
+    for (int b = tid; b < n; b += NT) atomicMin(&first[sm_of(b)], b);
+    __syncthreads();
+    for (int b = tid; b < n32; b += NT) {
+        const unsigned m = __ballot_sync(0xffffffffu, b < n && first[sm_of(b)] == b);
+        if ((tid & 31) == 0) prim[b >> 5] = m;
+    }
+    __syncthreads();
+    for (int b = tid; b < n32; b += NT) {
+        const bool second = b < n && !(prim[b >> 5] >> (b & 31) & 1u), near = second && below(prim, first[sm_of(b)]) < batch.pivots;
+        const unsigned m = __ballot_sync(0xffffffffu, second && !near), m2 = __ballot_sync(0xffffffffu, near);
+        if ((tid & 31) == 0) { away[b >> 5] = m; beside[b >> 5] = m2; }
+    }
+    __syncthreads();
+    const int b = (int)blockIdx.x;
+    int seat = below(prim, b);
+    if (!(prim[b >> 5] >> (b & 31) & 1u)) {
+        const bool far = away[b >> 5] >> (b & 31) & 1u;
+        int before = 0;                                          // all the CTAs of the classes before
+        for (int k = 0; k < n32 / 32; ++k) before += __popc(prim[k]) + (far ? 0 : __popc(away[k]));
+        seat = before + below(far ? away : beside, b);
+    }
+    __syncthreads();
+    return seat;
+}
 
 // This CTA's share (rows rank, rank + ncta, ...) of the largest |g_ij| / sqrt(g_ii g_jj), i < j. rs: np floats of shared memory.
 __device__ float matrix_max(float *rs, const Seq &sq, int rank)
@@ -1176,12 +1230,19 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
     extern __shared__ __align__(16) float j3sm[];
     __shared__ int flag_s[MAXPAIRS];              // the pairs rotated in the current step
     __shared__ int ticket_s;
-    int si = 0;
+    int si = -1, rank = 0;
+    const int seat = batch.seated ? seat_of(batch, status + 1) : (int)blockIdx.x;
+    if (seat < 0) return;
 #pragma unroll 1
-    for (int i = 1; i < batch.count; ++i) if ((int)blockIdx.x >= batch.s[i].cta0) si = i;
+    for (int i = 0; i < batch.count; ++i) {                      // pivot CTAs are the first ones of their sequence
+        const int p = seat - batch.s[i].pivot0, w = seat - batch.s[i].worker0, npu = batch.s[i].npu;
+        if (p >= 0 && p < npu) { si = i; rank = p; }
+        else if (w >= 0 && w < batch.s[i].ncta - npu) { si = i; rank = npu + w; }
+    }
+    if (si < 0) return;
     const Seq &sq = batch.s[si];
-    const int rank = (int)blockIdx.x - sq.cta0, tid = threadIdx.x;
-    if (rank >= sq.ncta || sq.np <= 0) return;
+    const int tid = threadIdx.x;
+    if (sq.np <= 0) return;
     const int npairs = sq.nb / 2, nw = sq.np / BLK;
     const int items_g = blocks_of_g(npairs), total = items_g + npairs * ((nw + SEG_W - 1) / SEG_W);
     const int nsteps = sq.nb - 1;
@@ -1297,9 +1358,7 @@ __global__ void init_kernel(const __grid_constant__ Batch batch, int *status)
         else if (!isfinite(sq.G[e])) bad = true;
     }
     if (__syncthreads_or(bad) && threadIdx.x == 0) raise_status(status, ATP_ERR_RANGE);
-    if (blockIdx.x == 0 && sq.np > 0) {
-        if (threadIdx.x < 64) sq.sync[threadIdx.x] = 0u;
-    }
+    if (blockIdx.x == 0 && threadIdx.x < SYNC_WORDS) sq.sync[threadIdx.x] = 0u;
 }
 
 // Host side: hands every sequence a group of CTAs in proportion to the size of its update (at most one
@@ -1322,22 +1381,47 @@ static inline atp_status launch(atp_ctx *ctx, Batch &jb, float tol_conv, float t
             if (dv >= 0 && dv < 64) occ_dev[dv] = occ;
         } else occ = occ_dev[dv];
     }
-    const int total = ctx->sm_count * std::min(occ, 2);
+    const int per_sm = std::min(occ, 2), total = ctx->sm_count * per_sm;
     double wsum = 0;
-    for (int i = 0; i < jb.count; ++i) wsum += (double)jb.s[i].np * jb.s[i].np;
+    int pairs = 0, all_items = 0, items[MAXSEQ];
+    for (int i = 0; i < jb.count; ++i) {
+        const Seq &q = jb.s[i];
+        const int npairs = q.nb / 2;
+        wsum += (double)q.np * q.np;
+        pairs += npairs;
+        items[i] = q.np > 0 ? blocks_of_g(npairs) + npairs * ((q.np / BLK + SEG_W - 1) / SEG_W) : 0;     // of the update
+        all_items += items[i];
+    }
     if (wsum <= 0) return ATP_OK;
-    int next = 0;
+    // Every pair a CTA of its own and the rest of the CTAs in proportion to the items of the update, if all pairs find an SM
+    // each; the CTAs beside them stay away as long as the others have at most MATE_ITEMS items each.
+    const bool own = pairs <= ctx->sm_count;
+    auto share = [&](int workers, int i) { return (int)std::min<double>(items[i], (double)workers * items[i] / all_items); };
+    bool apart = own && per_sm == 2;
+    for (int i = 0; i < jb.count; ++i) apart = apart && items[i] <= MATE_ITEMS * share(total - 2 * pairs, i);
+    int used = 0;
+    jb.pivots = 0;
     for (int i = 0; i < jb.count; ++i) {
         Seq &q = jb.s[i];
         const int npairs = q.nb / 2;
-        const int items = blocks_of_g(npairs) + npairs * ((q.np / BLK + SEG_W - 1) / SEG_W);     // of the update
-        int c = (int)((double)total * ((double)q.np * q.np / wsum));
-        c = std::max(1, std::min(c, std::max(items, 1)));
-        if (q.np <= 0) c = 1;
-        q.cta0 = next; q.ncta = c;
-        next += c;
+        if (own) { q.npu = npairs; q.ncta = npairs + share(total - (apart ? 2 : 1) * pairs, i); }
+        else {
+            q.ncta = 1 + (int)std::min<double>(items[i], (total - jb.count) * ((double)q.np * q.np / wsum));      // (at most `total` together)
+            q.npu = std::min(npairs, q.ncta);
+        }
+        if (q.np <= 0) q.npu = q.ncta = 0;
+        q.pivot0 = jb.pivots;
+        jb.pivots += q.npu;
+        used += q.ncta;
     }
-    if (next > total) return ATP_ERR_INVALID_ARG;      // cannot happen: shares sum to at most `total`
+    for (int i = 0, next = jb.pivots; i < jb.count; ++i) {
+        jb.s[i].worker0 = next;
+        next += jb.s[i].ncta - jb.s[i].npu;
+    }
+    jb.seated = apart && used > ctx->sm_count && total <= MAXGRID;
+    const int grid = jb.seated ? total : used;
+    jb.grid_sync = jb.s[0].sync + 32;
+    jb.smids = jb.s[0].sync + SYNC_WORDS;
     ATP_KERNEL(ctx, "jacobi_init", 0, wsum * 4.0);
     init_kernel<<<dim3(std::max(64, 4 * ctx->sm_count / jb.count), jb.count), 256, 0, ctx->stream>>>(jb, ctx->dev_status);
     ATP_LAUNCHED(ctx);
@@ -1346,7 +1430,7 @@ static inline atp_status launch(atp_ctx *ctx, Batch &jb, float tol_conv, float t
     void *args[] = {(void *)&jb, (void *)&tol_conv, (void *)&tol_left, (void *)&tol_rot, (void *)&ms, (void *)&rn, (void *)&status};
     // bytes: one read and one write of G and Wt (what the kernel must move at least; it runs from L2)
     ATP_KERNEL(ctx, "jacobi_persistent", 0, wsum * 16.0);
-    ATP_CUDA_OK(ctx, cudaLaunchCooperativeKernel((const void *)jacobi_persistent_kernel<TENSOR>, dim3(next), dim3(NT), args, SMEM_BYTES, ctx->stream));
+    ATP_CUDA_OK(ctx, cudaLaunchCooperativeKernel((const void *)jacobi_persistent_kernel<TENSOR>, dim3(grid), dim3(NT), args, SMEM_BYTES, ctx->stream));
     ATP_LAUNCHED(ctx);
     return ATP_OK;
 }
