@@ -57,7 +57,7 @@ struct Scratch { size_t cpart, c, dpart, gpart; };
 static inline Scratch scratch_tiles(int n, int rt, int ncta, bool tensor)
 {
     const int nt = (n + 63) / 64, np = (rt + 63) / 64, nr = tensor ? (nt + 1) / 2 : nt;
-    Scratch s{1, (size_t)np + 1, 1, (size_t)nt + 1};
+    Scratch s{1, (size_t)np + 1, 1, (size_t)std::max(nt, std::min(2 * nt, ncta)) + 1};
     for (int nj = 1; nj < np && nt > 0; ++nj) {
         const int nc = tensor ? (nj + 1) / 2 : nj;
         s.cpart = std::max(s.cpart, (size_t)nj * std::min(nt, (ncta + nc - 1) / nc));
@@ -162,6 +162,10 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
     const int m0 = (warp & 3) * 16, n0 = (warp >> 2) * 32;
     const int n = sq.n, rt = sq.rt, ld = sq.ld, ncta = sq.ncta;
     const int ntile = (n + 63) / 64, npanel = (rt + 63) / 64;
+    // The passes that form the Gram matrix go by half tiles where there are CTAs for them: the fp64 products of a tile alone take
+    // 2300 cycles of its SM, 5000 to 9000 with what is around them (16 x 512 x 320: 1096 -> 1067 us for the three iterates, 512 x 192
+    // in fp32: 655 -> 622).
+    const int gh = 2 * ntile <= ncta ? 32 : 64, ngram = (n + gh - 1) / gh;
     const bool vec = (ld & 3) == 0 && ((size_t)sq.M & 15) == 0;
     int *abort_flag = status + 1;
     unsigned gen = 0;
@@ -310,7 +314,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
         const int tper = (ntile + KS - 1) / KS;
         const int G = nj > 0 ? max(1, min(nj, (ncta + nr - 1) / nr)) : 1;
         const int jper = nj > 0 ? (nj + G - 1) / G : 1;
-        const int nrange = max(1, min(8, ntile / 64)), cper = (ntile + nrange - 1) / nrange;
+        const int nrange = max(1, min(8, ngram / 32)), cper = (ngram + nrange - 1) / nrange;
         int stage = overlap ? 0 : 30, rep = 0;
         while (stage >= 0 && alive) {
             int op = OP_PF, first = -1, stride = 1, arep = 0;
@@ -516,12 +520,12 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                 float4 cmax = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (TENSOR && rank == 0 && tid < 64) sq.sync[64 + 64 * ((pj + 1) & 1) + tid] = 0u;
                 if (TENSOR && with_w) set_scales(scale_slot);
-                for (int t = rank; t < ntile; t += ncta) {
-                    const int rv = min(64, n - t * 64);
+                for (int t = rank; t < ngram; t += ncta) {
+                    const int row0 = t * gh, rv = min(gh, n - row0);
                     TileRegs ra;
-                    fetch_tile(ra, sq.M + (size_t)t * 64 * ld + j0, ld, rv, w, vec);
+                    fetch_tile(ra, sq.M + (size_t)row0 * ld + j0, ld, rv, w, vec);
                     if (nj > 0) {
-                        const float4 *dp = (const float4 *)(sq.Dpart + (size_t)t * G * 4096) + tid;
+                        const float4 *dp = (const float4 *)(sq.Dpart + (size_t)(row0 >> 6) * G * 4096 + (row0 & 63) * 64) + tid;
                         float4 d[4];
 #pragma unroll
                         for (int i = 0; i < 4; ++i) d[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -529,7 +533,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                             float4 x[8];
 #pragma unroll
                             for (int q = 0; q < 8; ++q)
-                                x[q] = g + (q >> 2) < G ? __ldcg(dp + (size_t)(g + (q >> 2)) * 1024 + (q & 3) * NT) : make_float4(0.f, 0.f, 0.f, 0.f);
+                                x[q] = g + (q >> 2) < G && (q & 2) * 16 < gh ? __ldcg(dp + (size_t)(g + (q >> 2)) * 1024 + (q & 3) * NT) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                             for (int q = 0; q < 8; ++q) { float4 &a = d[q & 3]; a.x += x[q].x; a.y += x[q].y; a.z += x[q].z; a.w += x[q].w; }
                         }
@@ -539,7 +543,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                             v.x -= d[i].x; v.y -= d[i].y; v.z -= d[i].z; v.w -= d[i].w;
                             const int f = tid + i * NT, r = f >> 4, c = (f & 15) * 4;
                             if (!with_w && r < rv) {
-                                float *dm = sq.M + ((size_t)t * 64 + r) * ld + j0 + c;
+                                float *dm = sq.M + (size_t)(row0 + r) * ld + j0 + c;
                                 if (vec && c + 3 < w) *(float4 *)dm = v;
                                 else {
                                     if (c < w) dm[0] = v.x;
@@ -570,11 +574,11 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                                 const int r = m0 + g + (i >= 2 ? 8 : 0), c = n0 + nt * 8 + 2 * tq + (i & 1);
                                 const bool in = r < rv && c < w;
                                 sA[r * LDA + c] = in ? acc[nt][i] : 0.f;
-                                if (in) sq.M[((size_t)t * 64 + r) * ld + j0 + c] = acc[nt][i];
+                                if (in) sq.M[(size_t)(row0 + r) * ld + j0 + c] = acc[nt][i];
                             }
                         __syncthreads();
                     }
-                    gram_tile_64(sA, LDA, Gs, sq.gpart + (size_t)t * 4096);
+                    gram_tile_64(sA, LDA, gh, Gs, sq.gpart + (size_t)t * 4096);
                     __syncthreads();
                 }
                 if (note_max) {
@@ -592,7 +596,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                 // ordered sum of the partial Gram matrices: 16 element slices x (up to 8) chunk ranges
                 for (int it = rank; it < 16 * nrange; it += ncta) {
                     const int sl = it & 15, rg = it >> 4, e = sl * 256 + tid;
-                    const int c0 = rg * cper, c1 = min(ntile, (rg + 1) * cper);
+                    const int c0 = rg * cper, c1 = min(ngram, (rg + 1) * cper);
                     sq.gpart2[(size_t)rg * 4096 + e] = ordered_sum(sq.gpart + (size_t)c0 * 4096 + e, 4096, max(c1 - c0, 0));
                 }
                 barrier();

@@ -259,15 +259,15 @@ __device__ __noinline__ bool lowdin_64(const double *Gs, int n, float *Es, __hal
     return true;
 }
 
-// Partial Gram matrix of a 64 x 64 fp32 tile T (64 rows of a panel, row stride lds): dst[i][j] = sum_k T[k][i] T[k][j] in
+// Partial Gram matrix of a rows x 64 fp32 tile T (32 or 64 rows of a panel, row stride lds): dst[i][j] = sum_k T[k][i] T[k][j] in
 // fp64, on the fp64 matrix units (mma.m8n8k4; 36 tiles of 8 x 8 by symmetry, four or five per warp). Td: 4096 doubles of
 // shared memory for the converted tile, columns swizzled so that the fragment loads are conflict-free. Converting once
 // instead of per product matters: 9500 -> 5100 cycles (fp64 FMA with conversions in the inner loop before: conversions
 // run at 16 a cycle). 256 threads, T complete before the call; the caller synchronises before T or Td is reused.
-__device__ __forceinline__ void gram_tile_64(const float *T, int lds, double *Td, double *dst)
+__device__ __forceinline__ void gram_tile_64(const float *T, int lds, int rows, double *Td, double *dst)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = lane & 3, p = lane >> 2;
-    for (int f = tid; f < PB * PB / 4; f += 256) {
+    for (int f = tid; f < rows * PB / 4; f += 256) {
         const int r = f >> 4, c = (f & 15) * 4, cs = c ^ ((r & 3) << 2);
         const float4 v = *(const float4 *)(T + r * lds + c);
         *(double2 *)&Td[r * PB + cs] = make_double2(v.x, v.y);
@@ -284,7 +284,7 @@ __device__ __forceinline__ void gram_tile_64(const float *T, int lds, double *Td
     }
     double acc[5][2] = {};
 #pragma unroll 2
-    for (int k0 = 0; k0 < PB; k0 += 4) {
+    for (int k0 = 0; k0 < rows; k0 += 4) {
         const double *row = Td + (k0 + q) * PB;
 #pragma unroll
         for (int s = 0; s < 5; ++s) {
