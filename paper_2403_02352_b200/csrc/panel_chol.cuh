@@ -60,7 +60,7 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, flo
 {
     __shared__ double rs[PB];          // 1 / sqrt(diagonal of the Gram matrix)
     __shared__ int dep[PB];
-    __shared__ double2 xcol[2][32];    // the column in work of a diagonal block and its neighbour, by step parity
+    __shared__ __align__(16) double xcol[2][16], xdiag[2][16];     // the column in work of a diagonal block and the diagonal entries, by step parity
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     double *X = work;
     if (tid < PB) {
@@ -81,24 +81,26 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, flo
         if (warp == 0) {
             // the diagonal block: 16 dependent pivots. The unscaled column is exchanged through shared memory before its
             // pivot is known, and the next pivot comes from the current one and two entries that every lane already has
-            // (d - e^2 / piv), so the chain per column is one reciprocal and two multiply-adds. The entries move one place
-            // down per step, so the column in work is e[0] and a loop body serves several steps. Unrolled by 8: 415 us for the
-            // orthonormalisation of 16 x 512 x 320; by 16: 426, by 4: 416, rolled: 452, and 523 with the exchange by shuffles.
+            // (d - e^2 / piv), so the chain per column is one reciprocal and two multiply-adds (11 cycles each). Instructions count
+            // more than that chain: the code runs once per panel, and all 15 entries in every step of a loop over 16 columns
+            // (unrolled by 8) took 410 cycles a column, twice that chain. Straight code updates the entries right of the column only.
+            // 16 x 512 x 320: 1067 -> 1008 us for the three iterates, 512 x 192 in fp32: 622 -> 566; same values.
             double e[16];
 #pragma unroll
             for (int k = 0; k < 16; ++k) e[k] = lane < 16 ? Gs[(b + lane) * LDC + b + k] : (lane - 16 == k ? 1.0 : 0.0);
-            xcol[0][lane] = lane < 16 ? make_double2(e[0], e[1]) : make_double2(0.0, 0.0);      // (entries beyond the block: zero)
-            xcol[1][lane] = make_double2(0.0, 0.0);
+            if (lane < 16) { xcol[0][lane] = e[0]; xdiag[0][lane] = e[1]; }
             __syncwarp();
-            double piv = xcol[0][0].x;
+            double piv = xcol[0][0];
             bool bad = false;
-#pragma unroll 8
-            for (int c = 0; c < 16; ++c) {
-                const double2 *col = xcol[c & 1] + c;
-                double ck[16];
 #pragma unroll
-                for (int k = 1; k < 16; ++k) ck[k] = col[k].x;
-                const double dn = col[1].y;
+            for (int c = 0; c < 16; ++c) {
+                double ck[16], dn = 0.0;
+#pragma unroll
+                for (int k = (c + 1) & ~1; k < 16; k += 2) {
+                    const double2 v = *(const double2 *)&xcol[c & 1][k];
+                    ck[k] = v.x; ck[k + 1] = v.y;
+                }
+                if (c < 15) dn = xdiag[c & 1][c + 1];
                 const bool dep_c = !(piv > 1e-10);
                 // 1/sqrt from the hardware's 20-bit approximation and one step of third order, ~2^-58 relative: an error of the
                 // step goes into the entries that are left, which may be 1e-10 of those it comes from
@@ -107,13 +109,16 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, flo
                 const double h = fma(-piv * y, y, 1.0);
                 y = fma(y * h, fma(0.375, h, 0.5), y);
                 // a dependent column: unit pivot, zeros below; its row of the inverse keeps its scale
-                const double ic = dep_c ? 0.0 : y * y, f = e[0] * ic;
-                piv = fma(-ck[1] * ck[1], ic, dn);
+                const double ic = dep_c ? 0.0 : y * y, f = e[c] * ic;
+                if (c < 15) piv = fma(-ck[c + 1 < 16 ? c + 1 : 15] * ck[c + 1 < 16 ? c + 1 : 15], ic, dn);
                 bad |= dep_c && c == lane;
-                if (lane >= 16) X[(b + c) * LDC + b + lane - 16] = c >= lane - 16 ? (dep_c ? e[0] : e[0] * y) : 0.0;
+                if (lane >= 16) X[(b + c) * LDC + b + lane - 16] = c >= lane - 16 ? (dep_c ? e[c] : e[c] * y) : 0.0;
 #pragma unroll
-                for (int k = 1; k < 16; ++k) e[k - 1] = fma(-f, ck[k], e[k]);
-                if (lane < 16 && c < 15) xcol[(c + 1) & 1][lane] = make_double2(e[0], e[1]);
+                for (int k = c + 1; k < 16; ++k) e[k] = fma(-f, ck[k], e[k]);
+                if (lane < 16 && c < 15) {
+                    xcol[(c + 1) & 1][lane] = e[c + 1 < 16 ? c + 1 : 15];
+                    if (c < 14) xdiag[(c + 1) & 1][lane] = e[c + 2 < 16 ? c + 2 : 15];
+                }
                 __syncwarp();
             }
             if (lane < 16 && b + lane < n && bad) dep[b + lane] = 1;
