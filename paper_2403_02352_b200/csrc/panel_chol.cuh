@@ -69,11 +69,20 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, flo
         dep[tid] = 0;
     }
     __syncthreads();
-    // D^-1 G D^-1 in place: unit diagonal (0 for a zero column); X = 0
-    for (int e = tid; e < PB * PB; e += 256) {
-        const int r = e >> 6, c = e & 63;
-        Gs[r * LDC + c] = r == c ? (rs[r] > 0.0 ? 1.0 : 0.0) : Gs[r * LDC + c] * rs[r] * rs[c];
-        X[r * LDC + c] = 0.0;
+    // D^-1 G D^-1 in place: unit diagonal (0 for a zero column); the ten 16 x 16 blocks of the lower triangle, which are all
+    // that is read of the matrix
+    {
+        const int r = tid >> 4, c = tid & 15;
+        double rr[4], rc[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { rr[k] = rs[16 * k + r]; rc[k] = rs[16 * k + c]; }
+#pragma unroll
+        for (int bi = 0; bi < 4; ++bi)
+#pragma unroll
+            for (int bj = 0; bj <= bi; ++bj) {
+                double *g = Gs + (16 * bi + r) * LDC + 16 * bj + c;
+                *g = bi == bj && r == c ? (rr[bi] > 0.0 ? 1.0 : 0.0) : *g * rr[bi] * rc[bj];
+            }
     }
     __syncthreads();
     for (int p = 0; p < 4; ++p) {
@@ -172,14 +181,16 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, flo
         else if (strip == 0) asm volatile("bar.sync 2, 96;" ::: "memory");
     }
     __syncthreads();
-    // W[k][c] = (L^-1)[c][k] / D_k
+    // W[k][c] = (L^-1)[c][k] / D_k; the blocks of L^-1 above the diagonal have not been written
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int f = tid + 256 * i, k = f & 63, c = (f >> 6) * 4;
         const double rk = rs[k];
-        float4 w;
-        w.x = (float)(rk * X[c * LDC + k]); w.y = (float)(rk * X[(c + 1) * LDC + k]);
-        w.z = (float)(rk * X[(c + 2) * LDC + k]); w.w = (float)(rk * X[(c + 3) * LDC + k]);
+        float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k >> 4 <= c >> 4) {
+            w.x = (float)(rk * X[c * LDC + k]); w.y = (float)(rk * X[(c + 1) * LDC + k]);
+            w.z = (float)(rk * X[(c + 2) * LDC + k]); w.w = (float)(rk * X[(c + 3) * LDC + k]);
+        }
         *(float4 *)(rinv + k * PB + c) = w;
     }
     // (the diagonal of L^-1 holds the reciprocal square roots of the pivots)
