@@ -371,7 +371,11 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                     }
                     __syncthreads();
                     // a nearly orthonormal panel gets its factor from a short series instead of the factorisation
-                    if (!(series_ok && lowdin_64(Gs, w, sA, (__half *)sB, sq.W, sq.flags))) chol_invert_64(Gs, (double *)osm, w, sq.W, sq.flags);
+                    if (!(series_ok && lowdin_64(Gs, w, sA, (__half *)sB, sq.W, sq.flags))) {
+                        // from the second projection of unit columns on, a column of which nothing is left is given up
+                        const bool tried = stage == 24 ? rep >= 1 : stage == 33 && rep >= 2;
+                        chol_invert_64(Gs, (double *)osm, w, tried ? LOST2 : 0.0, sq.W, sq.flags);
+                    }
                     __syncthreads();
                 } else if (first >= 0) {
                     set_scales(scale_slot);
