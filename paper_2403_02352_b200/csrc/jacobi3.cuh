@@ -35,6 +35,11 @@ constexpr int LDA = 68;           // shared-memory row stride (floats) of A-oper
 constexpr int LDB = 72;           // shared-memory row stride of B-operand style tiles
 constexpr int MAXSEQ = 32;        // sequences per launch
 constexpr int SYNC_WORDS = 64;    // words of Seq::sync before the list of SMs (which the first sequence of a launch holds)
+// Rows of G whose diagonal entry is at most NEGLIGIBLE times the largest one (rows of B below 2^-37 of the longest) are what a
+// rank-deficient input leaves: rounding, with a Gram matrix that is not even positive, so that rotations among such rows do not
+// end. No pass waits for their entries, they are not rotated against each other, and one whose diagonal entry is not positive is
+// not rotated at all. (A token that is that small stays in use: rotations against longer rows go on as long as a pass does.)
+constexpr float NEGLIGIBLE = 0x1p-74f;
 constexpr int VSTRIDE = 2 * BLK * BLK + 2 * BLK + 2 * JB * JB;   // floats of a published transform (see below)
 
 struct Seq {
@@ -42,8 +47,8 @@ struct Seq {
     int *vflag;                   // 2 x npairs: the pair rotated in this step
     unsigned *sync;               // 64 words. [0]: arrivals at the group barrier (monotonic); largest scaled off-diagonal
                                   // entry, slot sweep % 4: [1..4] met in a sweep, [8..11] in the whole matrix after it;
-                                  // [5]: sweeps used; by step parity: [16..17] work tickets of the update, [20..21] pivot
-                                  // blocks fetched; [32]: arrivals of the whole launch
+                                  // [5]: sweeps used; [6]: largest diagonal entry at the start; by step parity: [16..17] work
+                                  // tickets of the update, [20..21] pivot blocks fetched; [32]: arrivals of the whole launch
     int n, np, nb;                // size, padded size (multiple of 64), number of 32-row blocks (even)
     int ncta, npu;                // CTAs that own this sequence; those of them that solve pivot blocks
     int pivot0, worker0;          // numbers of the first of its pivot CTAs and of the first of the others (see seat_of)
@@ -185,12 +190,13 @@ __device__ __forceinline__ void rotate_block(float2 ra, float2 rb, float &ee, fl
 template <int W> struct Band {
     static constexpr int D0 = W == 0 ? 0 : 5 * W - 2, ND = W == 0 ? 3 : (W == 3 ? 4 : 5);
     float ee[ND], eo[ND], oe[ND], oo[ND];
-    // loads the offsets from As, returns the largest scaled off-diagonal entry among them
-    __device__ __forceinline__ float load(const float *As)
+    // loads the offsets from As, without the entries that are not rotated (see NEGLIGIBLE; rows with a diagonal entry of at most
+    // `least`), and returns the largest scaled off-diagonal entry among those that a pass waits for
+    __device__ __forceinline__ float load(const float *As, float least)
     {
         const int k = threadIdx.x & 31;
         const float de = As[k * (LDP + 1)], dd = As[(32 + k) * (LDP + 1)];
-        const float re = de > 0.f ? rsqrtf(de) : 0.f, ro = dd > 0.f ? rsqrtf(dd) : 0.f;
+        const float re = de > least ? rsqrtf(de) : 0.f, ro = dd > least ? rsqrtf(dd) : 0.f;
         float me = 0.f, mo = 0.f;                                // in the even rows and in the odd ones, without re and ro
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
@@ -202,6 +208,17 @@ template <int W> struct Band {
             me = fmaxf(me, fabsf(eo[i]) * lo); mo = fmaxf(mo, fabsf(oe[i]) * le);
         }
         mo = fmaxf(me * re, mo * ro);
+        // (zero: padding, or a row of zeros)
+        if (__any_sync(0xffffffffu, (de <= least && de != 0.f) || (dd <= least && dd != 0.f))) {
+            auto keep = [&](float &g, float a, float b) { if (fminf(a, b) <= 0.f || fmaxf(a, b) <= least) g = 0.f; };
+#pragma unroll
+            for (int i = 0; i < ND; ++i) {
+                const int l = (k + D0 + i) & 31;
+                const float fe = __shfl_sync(0xffffffffu, de, l), fo = __shfl_sync(0xffffffffu, dd, l);
+                keep(eo[i], de, fo); keep(oe[i], dd, fe);
+                if (D0 + i > 0) { keep(ee[i], de, fe); keep(oo[i], dd, fo); }
+            }
+        }
         return mo;
     }
     // the 32 rounds; the diagonal quadrants (both blocks after the cross rotations) go back to As
@@ -399,11 +416,11 @@ __device__ void pivot_load(float *sm, const float *G, int np, int I, int J)
 // vout. cross_only: the 32 rounds that pair the two blocks' rows; otherwise all 63 rounds. Returns the largest
 // scaled off-diagonal entry found in the block before rotating (block-uniform); when it is <= tol_rot nothing is
 // rotated or published.
-template <int W> __device__ __forceinline__ float pivot_warp(float *As, PivotShared &sh, bool cross_only, float tol_rot, float *quad)
+template <int W> __device__ __forceinline__ float pivot_warp(float *As, PivotShared &sh, bool cross_only, float tol_rot, float least, float *quad)
 {
     const float tol2 = tol_rot * tol_rot;
     Band<W> band;
-    float mo = band.load(As);
+    float mo = band.load(As, least);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mo = fmaxf(mo, __shfl_xor_sync(0xffffffffu, mo, o));
     if ((threadIdx.x & 31) == 0) sh.red[W] = mo;
@@ -446,7 +463,7 @@ constexpr int LDV = 66;           // row stride of the transform in shared memor
 __device__ __forceinline__ float inv_pow2(float x) { return __uint_as_float(0x7f000000u - __float_as_uint(x)); }
 
 template <bool TENSOR>
-__device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *vout, bool &rotated)
+__device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float least, float *vout, bool &rotated)
 {
     __shared__ __align__(16) PivotShared sh;
     const int tid = threadIdx.x, warp = tid >> 5, l = tid & 31;
@@ -462,10 +479,10 @@ __device__ float pivot_rotate(float *sm, bool cross_only, float tol_rot, float *
         vout[V_D + tid] = d;
         vout[V_S + tid] = d;                                     // (overwritten below where rows are rotated)
     }
-    if (warp == 0) mo = pivot_warp<0>(As, sh, cross_only, tol_rot, vout + V_Q);
-    else if (warp == 1) mo = pivot_warp<1>(As, sh, cross_only, tol_rot, vout + V_Q);
-    else if (warp == 2) mo = pivot_warp<2>(As, sh, cross_only, tol_rot, vout + V_Q);
-    else if (warp == 3) mo = pivot_warp<3>(As, sh, cross_only, tol_rot, vout + V_Q);
+    if (warp == 0) mo = pivot_warp<0>(As, sh, cross_only, tol_rot, least, vout + V_Q);
+    else if (warp == 1) mo = pivot_warp<1>(As, sh, cross_only, tol_rot, least, vout + V_Q);
+    else if (warp == 2) mo = pivot_warp<2>(As, sh, cross_only, tol_rot, least, vout + V_Q);
+    else if (warp == 3) mo = pivot_warp<3>(As, sh, cross_only, tol_rot, least, vout + V_Q);
     else {
         const int h = warp - 4;
         __syncthreads();
@@ -1190,15 +1207,16 @@ __device__ int seat_of(const Batch &batch, int *abort_flag)
     return seat;
 }
 
-// This CTA's share (rows rank, rank + ncta, ...) of the largest |g_ij| / sqrt(g_ii g_jj), i < j. rs: np floats of shared memory.
-__device__ float matrix_max(float *rs, const Seq &sq, int rank)
+// This CTA's share (rows rank, rank + ncta, ...) of the largest |g_ij| / sqrt(g_ii g_jj), i < j, negligible rows left out.
+// rs: np floats of shared memory.
+__device__ float matrix_max(float *rs, const Seq &sq, int rank, float least)
 {
     __shared__ float part[NT / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = sq.n, np = sq.np;
 #pragma unroll 4
     for (int i = tid; i < np; i += NT) {
         const float d = i < n ? __ldcg(sq.G + (size_t)i * np + i) : 0.f;
-        rs[i] = d > 0.f ? rsqrtf(d) : 0.f;
+        rs[i] = d > least ? rsqrtf(d) : 0.f;
     }
     __syncthreads();
     float mo = 0.f;
@@ -1249,11 +1267,12 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
     int *abort_flag = status + 1;
     unsigned gen = 0, gstep = 0;
     bool converged = false, alive = true;
+    const float least = __uint_as_float(__ldcg(sq.sync + 6)) * NEGLIGIBLE;
 
     // rotates the block held in shared memory for pair pr of (sweep, step); publishes to parity par
     auto pivot_finish = [&](int sweep, int step, int pr, int par) {
         bool rotated;
-        const float mo = pivot_rotate<TENSOR>(j3sm, step > 0, tol_rot, sq.Vbuf + ((size_t)par * npairs + pr) * VSTRIDE, rotated);
+        const float mo = pivot_rotate<TENSOR>(j3sm, step > 0, tol_rot, least, sq.Vbuf + ((size_t)par * npairs + pr) * VSTRIDE, rotated);
         if (tid == 0) {
             sq.vflag[par * npairs + pr] = rotated ? 1 : 0;
             atomicMax(sq.sync + 1 + sweep % 4, __float_as_uint(mo));
@@ -1332,7 +1351,7 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
         if (mo <= tol_conv) { converged = true; ++sweep; break; }
         // The largest scaled off-diagonal entry of the matrix as the sweep has left it: a few microseconds, against a whole
         // sweep (65 steps at n = 2112) to find the same by visiting every pair again.
-        const float left = matrix_max(j3sm, sq, rank);
+        const float left = matrix_max(j3sm, sq, rank, least);
         if (tid == 0) atomicMax(sq.sync + 8 + sweep % 4, __float_as_uint(left));
         alive = group_barrier(sq.sync, ++gen, (unsigned)sq.ncta, abort_flag);
         if (!alive) break;
@@ -1344,7 +1363,7 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
     }
 }
 
-// Wt = identity, padding of G = 0, synchronisation words = 0; a non-finite entry of G (an input with Inf / NaN,
+// Wt = identity, padding of G = 0, synchronisation words = 0 but for the largest diagonal entry; a non-finite entry of G (an input with Inf / NaN,
 // or one whose squares overflow fp32) raises ATP_ERR_RANGE. grid (x, count).
 __global__ void init_kernel(const __grid_constant__ Batch batch, int *status)
 {
@@ -1358,7 +1377,16 @@ __global__ void init_kernel(const __grid_constant__ Batch batch, int *status)
         else if (!isfinite(sq.G[e])) bad = true;
     }
     if (__syncthreads_or(bad) && threadIdx.x == 0) raise_status(status, ATP_ERR_RANGE);
-    if (blockIdx.x == 0 && threadIdx.x < SYNC_WORDS) sq.sync[threadIdx.x] = 0u;
+    if (blockIdx.x == 0) {
+        __shared__ unsigned top;
+        if (threadIdx.x == 0) top = 0u;
+        __syncthreads();
+        float m = 0.f;
+        for (int i = threadIdx.x; i < sq.n; i += blockDim.x) m = fmaxf(m, sq.G[(size_t)i * (sq.np + 1)]);
+        atomicMax(&top, __float_as_uint(m));
+        __syncthreads();
+        if (threadIdx.x < SYNC_WORDS) sq.sync[threadIdx.x] = threadIdx.x == 6 ? top : 0u;
+    }
 }
 
 // Host side: hands every sequence a group of CTAs in proportion to the size of its update (at most one
