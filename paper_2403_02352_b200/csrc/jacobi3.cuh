@@ -758,7 +758,8 @@ __device__ void pivot_form_half(float *sm, const Seq &sq, const float *Gsrc, con
 }
 
 // The same where the current step did the 32 cross rounds only: the diagonal blocks of N are then those of the rotated pivot
-// blocks, published with the transforms (or still in G, where the pair was not rotated), and W1 X12 W2^T is all that is left
+// blocks, published with the transforms (or still in G, where the pair was not rotated; store_diagonal writes them to G, so that
+// there is one version of them), and W1 X12 W2^T is all that is left
 // to form: one block of G to fetch instead of three, a quarter of the arithmetic (10000 -> 6500 cycles of a step at r~ = 1088 in
 // bf16, 15500 -> 9000 at r~ = 192 in fp32; jacobi_persistent of one 32768 x 1088 iterate 4730 -> 3740 us).
 template <bool TENSOR>
@@ -931,6 +932,19 @@ __device__ bool wait_fetched(Fetched &f)
     return f.ok;
 }
 
+// The two 32 x 32 diagonal blocks of a rotated pair go to G as its pivot solve left them (published behind the transform, in the
+// steps of 32 rounds), not as the products of the item (p, p) give them. The next pivot block is formed from them, so G has to
+// hold the same values: computed twice, the two versions of a diagonal block part with every step of a sweep, and where a row's
+// diagonal entry is rounding noise (rank-deficient inputs) one may be negative and the other not, which clips good entries of G
+// (put4_clamped).
+__device__ __forceinline__ void store_diagonal(float *G, int np, int I, int J, const float *P)
+{
+    const int i = threadIdx.x >> 3, c = (threadIdx.x & 7) * 4;
+    const float4 a = __ldcg((const float4 *)(P + V_Q + i * JB + c)), b = __ldcg((const float4 *)(P + V_Q + JB * JB + i * JB + c));
+    *(float4 *)(G + (size_t)(I * JB + i) * np + I * JB + c) = a;
+    *(float4 *)(G + (size_t)(J * JB + i) * np + J * JB + c) = b;
+}
+
 // One block (p, q) of G on the fp32 units: Vt_p G_pq Vt_q^T.
 __device__ bool g_block(float *sm, const Seq &sq, float *G, const float *Vbuf, const int *vflag, int step, int p, int q, Fetched &fetched)
 {
@@ -963,7 +977,10 @@ __device__ bool g_block(float *sm, const Seq &sq, float *G, const float *Vbuf, c
     }
     if (fq) product64_fma<true>(Tm, Vq, LDA, m0, n0, acc);       // out = T * Vt_q^T
     if (!wait_fetched(fetched)) return false;
+    const bool carried = p == q && step > 0;                     // the diagonal blocks come from the pivot solve
+    if (carried) store_diagonal(G, np, Ip, Jp, Vbuf + (size_t)p * VSTRIDE);
     const int gr0 = glob_of_loc(Ip, Jp, m0 + g), gr1 = glob_of_loc(Ip, Jp, m0 + g + 8);
+    if (!carried || ((m0 ^ n0) & JB))
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
         const int gc = glob_of_loc(Iq, Jq, n0 + nt * 8 + 2 * t);         // gc, gc + 1 are contiguous
@@ -1069,8 +1086,11 @@ __device__ bool g_block_half(float *sm, const Seq &sq, float *G, const float *Vb
         hs::product64<false, true>(Bk, Vq, m0, n0, acc);
     }
     if (!wait_fetched(fetched)) return false;
+    const bool carried = p == q && step > 0;                     // the diagonal blocks come from the pivot solve
+    if (carried) store_diagonal(G, np, Ip, Jp, Pp);
     const int gr0 = glob_of_loc(Ip, Jp, m0 + g), gr1 = glob_of_loc(Ip, Jp, m0 + g + 8);
     const float s0 = sp[m0 + g] * k, s1 = sp[m0 + g + 8] * k;
+    if (!carried || ((m0 ^ n0) & JB))
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
         const int lc = n0 + nt * 8 + 2 * t, gc = glob_of_loc(Iq, Jq, lc);        // gc, gc + 1 are contiguous
@@ -1363,8 +1383,8 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
     }
 }
 
-// Wt = identity, padding of G = 0, synchronisation words = 0 but for the largest diagonal entry; a non-finite entry of G (an input with Inf / NaN,
-// or one whose squares overflow fp32) raises ATP_ERR_RANGE. grid (x, count).
+// Wt = identity, padding of G = 0, synchronisation words = 0 but for the largest diagonal entry; a non-finite entry of G (an
+// input with Inf / NaN, or one whose squares overflow fp32) raises ATP_ERR_RANGE. grid (x, count).
 __global__ void init_kernel(const __grid_constant__ Batch batch, int *status)
 {
     bool bad = false;
