@@ -33,7 +33,13 @@ namespace orth {
 using j3::BLK; using j3::NT; using j3::LDA; using j3::LDB;
 constexpr int MAXSEQ = 32;
 constexpr int SYNC_WORDS = 256;   // words of Seq::sync before the SM list
-constexpr int EXTRA = 3;          // repetitions of a panel beyond those asked for
+constexpr int EXTRA = 6;          // repetitions of a panel beyond those asked for
+// Length outside the finished columns and those before it in the panel at which a unit column that has been projected and factored
+// `tries` times is given up: 1e-5, like a column whose pivot says so, then more, because what is new keeps its length once it has
+// been projected. Where a panel has no other direction to offer (rows of zeros, rows repeated: all columns lie in the same few
+// dimensions) every projection leaves the rounding of the one before, and normalising that gave U^T U - I of up to the number of
+// panels.
+constexpr float lost_length(int tries) { return tries <= 0 ? 0.f : tries == 1 ? 1e-5f : tries == 2 ? 1e-3f : 0.1f; }
 constexpr int NRED = 8;           // second-level partial Gram sums (chunk ranges)
 
 struct Seq {
@@ -372,9 +378,15 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                     __syncthreads();
                     // a nearly orthonormal panel gets its factor from a short series instead of the factorisation
                     if (!(series_ok && lowdin_64(Gs, w, sA, (__half *)sB, sq.W, sq.flags))) {
-                        // from the second projection of unit columns on, a column of which nothing is left is given up
-                        const bool tried = stage == 24 ? rep >= 1 : stage == 33 && rep >= 2;
-                        chol_invert_64(Gs, (double *)osm, w, tried ? LOST2 : 0.0, sq.W, sq.flags);
+                        // given up (see lost_length): columns of which nothing is left, but not the replacements of the last factor
+                        const float lost = lost_length(stage == 24 ? rep : stage == 33 ? rep - 1 : 0);
+                        const bool old = lost > 0.f && tid < w && !(__ldcg(sq.flags + tid) & 1);
+                        chol_invert_64(Gs, (double *)osm, w, sq.W, sq.flags);
+                        if (lost > 0.f) {
+                            __syncthreads();
+                            // the diagonal of the factor: 1 / length outside the columns before
+                            if (old && __ldcg(sq.W + tid * 65) * lost >= 1.f) sq.flags[tid] |= 1;
+                        }
                     }
                     __syncthreads();
                 } else if (first >= 0) {

@@ -6,7 +6,7 @@
 // columns is below 1e-5 of its norm) is flagged as dependent: bit 0 of its word in flags[0..63]. Bit 1: the column is shorter
 // than SHRUNK; where it had unit length before the projection, what rounding left of the finished columns in it is no longer
 // small against it. Bit 2: its scaled pivot is below ILL_PIVOT^2, so W enlarges a rounding error of the panel more than
-// 1 / ILL_PIVOT times. A column of which the square of what the pivot leaves is at most `lost` counts as dependent as well.
+// 1 / ILL_PIVOT times.
 // Four panels of 16 columns. What bounds it is the chain of 64 pivots, so a panel's diagonal block is factored inside one
 // warp, without a barrier: lane i < 16 holds row i of the block, lane 16 + j column j of its inverse (which starts as the
 // identity); with m = (entry of column c) / L_cc in every lane, the right-looking step
@@ -23,11 +23,6 @@
 
 constexpr int PB = 64;            // orthonormalisation panel width
 constexpr double ILL_PIVOT = 0x1p-5, SHRUNK = 0.25;
-// A unit column that has been projected and factored before is given up when less than 1e-5 of its length lies outside the
-// finished columns and those before it in the panel (squared here), like a column whose pivot says so. Where a panel has no other
-// direction to offer (rows of zeros, rows repeated: all columns lie in the same few dimensions) every projection leaves the
-// rounding of the one before, and normalising that gave U^T U - I of up to the number of panels.
-constexpr double LOST2 = 1e-10;
 
 constexpr int LDC = 68;           // row stride (doubles) in shared memory: the fragments below are free of bank conflicts
 
@@ -60,9 +55,8 @@ __device__ __forceinline__ void dmma_store(double *c, const double (&acc)[2][2])
 #pragma unroll
     for (int t = 0; t < 2; ++t) { c[g * LDC + 8 * t + 2 * q] = acc[t][0]; c[g * LDC + 8 * t + 2 * q + 1] = acc[t][1]; }
 }
-// lost: LOST2, or 0 where no column is to be given up for its length. Gs is overwritten. work: 64 x LDC doubles of shared memory
-// (ends as L^-1, lower triangle). 256 threads.
-__device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, double lost, float *rinv, int *flags)
+// Gs is overwritten. work: 64 x LDC doubles of shared memory (ends as L^-1, lower triangle). 256 threads.
+__device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, float *rinv, int *flags)
 {
     __shared__ double rs[PB];          // 1 / sqrt(diagonal of the Gram matrix)
     __shared__ int dep[PB];
@@ -200,11 +194,8 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, dou
         *(float4 *)(rinv + k * PB + c) = w;
     }
     // (the diagonal of L^-1 holds the reciprocal square roots of the pivots)
-    if (tid < PB) {
-        const double x = X[tid * (LDC + 1)], left = x * rs[tid];                 // 1 / length of what is left of the column
-        const bool none = dep[tid] || !(rs[tid] > 0.0) || left * left * lost >= 1.0;
-        flags[tid] = tid >= n ? 0 : (none ? 1 : 0) | (rs[tid] > 1.0 / SHRUNK ? 2 : 0) | (x > 1.0 / ILL_PIVOT ? 4 : 0);
-    }
+    if (tid < PB)
+        flags[tid] = tid >= n ? 0 : (dep[tid] || !(rs[tid] > 0.0) ? 1 : 0) | (rs[tid] > 1.0 / SHRUNK ? 2 : 0) | (X[tid * (LDC + 1)] > 1.0 / ILL_PIVOT ? 4 : 0);
 }
 
 

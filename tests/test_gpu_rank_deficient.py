@@ -84,6 +84,28 @@ def test_tokens_that_fall_below_rounding(octaves):
         c.close()
 
 
+# nearly as many components as tokens, which fall by more octaves than the iterates hold: with columns given up at 1e-5 only and
+# three more repetitions, a few columns stayed in the span of the others (U^T U - I of 0.4 to 0.8, a leading singular value off by
+# 10 %)
+@pytest.mark.parametrize("L,r,octaves,seed", [(600, 560, 60, 1), (600, 560, 100, 1), (600, 560, 100, 2), (300, 300, 60, 1), (130, 130, 100, 1)])
+def test_falling_tokens_nearly_square(L, r, octaves, seed):
+    import paper_2403_02352_b200 as atp
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    X = torch.randn((L, 1024), generator=gen, device="cuda") * torch.exp2(-torch.arange(L, device="cuda") * (octaves / L))[:, None]
+    X = X[torch.randperm(L, generator=gen, device="cuda")].bfloat16()
+    c = atp.Context(0)
+    try:
+        U, _, sigma = atp.atp_principal_basis(c, X, [L], [r])
+        c.poll()
+        u = U[:, :r].double()
+        assert (u.T @ u - torch.eye(r, device="cuda")).abs().max() <= 2e-2
+        exact = torch.linalg.svdvals(X.double())[:r]
+        lead = exact > 1e-4 * exact[0]
+        assert ((sigma.double() - exact) / exact)[lead].abs().max() <= 1e-3
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("k,dtype", [(-30, torch.float32), (-36, torch.float32), (-40, torch.float32), (-46, torch.float32),
                                      (-30, torch.bfloat16)])
 def test_one_tiny_token(k, dtype):
