@@ -3,15 +3,17 @@
 // orthonormal range basis into singular vectors, X' = [sigma_i v_i]).
 //
 // One cooperative launch diagonalises every sequence of a batch. Each sequence owns a fixed group of
-// CTAs that loops over sweeps and steps on its own and leaves when its matrix has converged; the
+// CTAs (pivot CTAs, one a pair as a rule, and workers; see launch and seat_of) that loops over sweeps and steps on its own and leaves when its matrix has converged; the
 // CTAs of a group meet at a counter in global memory (bounded spin) instead of at kernel boundaries.
 // Blocks of 32 rows; a step handles n/64 disjoint block pairs (round-robin order) in two phases:
 //   pivot : per pair, the 64 x 64 pivot block is rotated on chip by cyclic Jacobi (first step of a sweep: all
 //           2016 pairs of its 64 rows once, in 63 rounds; other steps: the 1024 pairs across its two blocks, in
 //           32 rounds). The block lives in registers (see "pivot phase" below); a round is a rotation per row
 //           pair, one block barrier and a shift of the pairing. The accumulated row transform Vt (64 x 64)
-//           is published. The pivot block of the NEXT step is formed on chip from the matrix before this step's
-//           update (pivot_form), so the chain of pivot solves runs beside the update and never waits for it.
+//           is published, and of a step of 32 rounds the two diagonal blocks of the rotated pivot block. The pivot
+//           block of the NEXT step is formed on chip from those and one block of the matrix before this step's update
+//           (pivot_form_cross; after a sweep's first step from three blocks, pivot_form), so the chain of pivot solves
+//           runs beside the update and never waits for it.
 //   apply : every 64 x 64 block (p, q) of G becomes Vt_p G_pq Vt_q^T (upper triangle computed, mirror
 //           stored), rows of Wt become Vt_p Wt, both in place. The pivot CTAs of the step read blocks of G as they
 //           were before the update; a counter of fetched pivot blocks holds the first store of every updating
@@ -34,7 +36,7 @@ constexpr int NT = 256;           // threads per CTA
 constexpr int LDA = 68;           // shared-memory row stride (floats) of A-operand style tiles
 constexpr int LDB = 72;           // shared-memory row stride of B-operand style tiles
 constexpr int MAXSEQ = 32;        // sequences per launch
-constexpr int SYNC_WORDS = 64;    // words of Seq::sync before the list of SMs (which the first sequence of a launch holds)
+constexpr int SYNC_WORDS = 64;
 // Rows of G whose diagonal entry is at most NEGLIGIBLE times the largest one (rows of B below 2^-37 of the longest) are what a
 // rank-deficient input leaves: rounding, with a Gram matrix that is not even positive, so that rotations among such rows do not
 // end. No pass waits for their entries, they are not rotated against each other, and one whose diagonal entry is not positive is
@@ -45,7 +47,8 @@ constexpr int VSTRIDE = 2 * BLK * BLK + 2 * BLK + 2 * JB * JB;   // floats of a 
 struct Seq {
     float *G, *Wt, *Vbuf;         // G, Wt: np x np (ld = np); Vbuf: 2 x npairs x VSTRIDE (by step parity)
     int *vflag;                   // 2 x npairs: the pair rotated in this step
-    unsigned *sync;               // 64 words. [0]: arrivals at the group barrier (monotonic); largest scaled off-diagonal
+    unsigned *sync;               // SYNC_WORDS words (in the first sequence of a launch the list of SMs, 2 words an SM, lies behind
+                                  // them). [0]: arrivals at the group barrier (monotonic); largest scaled off-diagonal
                                   // entry, slot sweep % 4: [1..4] met in a sweep, [8..11] in the whole matrix after it;
                                   // [5]: sweeps used; [6]: largest diagonal entry at the start; by step parity: [16..17] work
                                   // tickets of the update, [20..21] pivot blocks fetched; [32]: arrivals of the whole launch
@@ -72,8 +75,8 @@ __device__ __forceinline__ void rr_pair(int nb, int step, int t, int &I, int &J)
     else { I = step + t; J = step - t; I -= I >= m ? m : 0; J += J < 0 ? m : 0; }
     if (I > J) { const int x = I; I = J; J = x; }
 }
-// The pair t that block b is in at a step, its two blocks and which of them b is.
-__device__ __forceinline__ void rr_locate(int nb, int step, int b, int &t, int &h, int &I, int &J)
+// The pair t that block b is in at a step, and whether b is the second of its two blocks.
+__device__ __forceinline__ void rr_locate(int nb, int step, int b, int &t, int &h)
 {
     const int m = nb - 1;
     int x = b - step, other;
@@ -82,7 +85,7 @@ __device__ __forceinline__ void rr_locate(int nb, int step, int b, int &t, int &
     else if (x == 0) { t = 0; other = m; }
     else if (x < nb / 2) { t = x; other = step - t; other += other < 0 ? m : 0; }
     else { t = m - x; other = step + t; other -= other >= m ? m : 0; }
-    I = min(b, other); J = max(b, other); h = b == J;
+    h = b > other;
 }
 
 using ::group_barrier;
@@ -761,16 +764,16 @@ __device__ void pivot_form_half(float *sm, const Seq &sq, const float *Gsrc, con
 // blocks, published with the transforms (or still in G, where the pair was not rotated; store_diagonal writes them to G, so that
 // there is one version of them), and W1 X12 W2^T is all that is left
 // to form: one block of G to fetch instead of three, a quarter of the arithmetic (10000 -> 6500 cycles of a step at r~ = 1088 in
-// bf16, 15500 -> 9000 at r~ = 192 in fp32; jacobi_persistent of one 32768 x 1088 iterate 4730 -> 3740 us).
+// bf16, 15500 -> 9000 at r~ = 192 in fp32; jacobi_persistent of one 32768 x 1088 iterate 4730 -> 3740 us). Not for the step after
+// a sweep's first one: the 31 rounds inside the blocks give a transform, no blocks, so those are formed from G.
 template <bool TENSOR>
-__device__ void pivot_form_cross(float *sm, const Seq &sq, const float *Vcur, int step, int b1, int b2, const int *flags, unsigned *fetched)
+__device__ void pivot_form_cross(float *sm, const Seq &sq, const float *Vcur, int step, int b1, int p1, int h1, int f1, int b2, int p2, int h2, int f2, unsigned *fetched)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, np = sq.np;
     __shared__ float srow[BLK];
-    int p1, h1, I1, J1, p2, h2, I2, J2;
-    rr_locate(sq.nb, step, b1, p1, h1, I1, J1);
-    rr_locate(sq.nb, step, b2, p2, h2, I2, J2);
-    const int f1 = flags[p1], f2 = flags[p2];
+    int I1, J1, I2, J2;
+    rr_pair(sq.nb, step, p1, I1, J1);
+    rr_pair(sq.nb, step, p2, I2, J2);
     const float *P1 = Vcur + (size_t)p1 * VSTRIDE, *P2 = Vcur + (size_t)p2 * VSTRIDE;
     float *As = sm;                                              // slot 0; the operands live in the others
     const int c = (tid & 15) * 4;
@@ -1168,8 +1171,8 @@ __device__ bool apply_item(float *sm, const Seq &sq, const float *Vbuf, const in
 
 // ---- the kernel --------------------------------------------------------------------------------
 // Schedule of a group. The pivot block of a pair of step s+1 is a function of the matrix before the update of
-// step s and of two transforms of step s (pivot_form), all of which are complete at the barrier that ends step
-// s-1. Every step therefore runs, side by side,
+// step s and of two pivot solves of step s (pivot_form, pivot_form_cross), all of which are complete at the barrier
+// that ends step s-1. Every step therefore runs, side by side,
 //   1. the pivot solves of the NEXT step (a few CTAs; this chain of rotation rounds is the critical path), and
 //   2. the update of this step, its blocks handed out by a ticket counter so that the pivot CTAs join in when
 //      they are through,
@@ -1178,7 +1181,6 @@ __device__ bool apply_item(float *sm, const Seq &sq, const float *Vbuf, const in
 // blocks it forms its pivot block from. Vt and the rotated-flags are double buffered by step parity, because
 // the pivots of step s+1 publish while the update of step s still reads.
 // status[0]: sticky device status word of the context; status[1]: abort flag of bounded waits.
-constexpr int MATE_ITEMS = 2;
 constexpr int MAXPAIRS = 72;                  // np <= 4608
 
 // Number of this CTA in the order in which roles are given out: pivot solves go to CTAs on SMs of their own (two of them on one
@@ -1330,16 +1332,16 @@ jacobi_persistent_kernel(const __grid_constant__ Batch batch, float tol_conv, fl
             // 1. pivots of the next step
             if (has_next && rank < npairs) {
                 for (int pr = rank; pr < npairs; pr += sq.ncta) {
-                    int b1, b2, p1, h1, p2, h2, I, J;
+                    int b1, b2, p1, h1, p2, h2;
                     rr_pair(sq.nb, nstep, pr, b1, b2);
-                    rr_locate(sq.nb, step, b1, p1, h1, I, J);
-                    rr_locate(sq.nb, step, b2, p2, h2, I, J);
+                    rr_locate(sq.nb, step, b1, p1, h1);
+                    rr_locate(sq.nb, step, b2, p2, h2);
                     const int f1 = flag_s[p1], f2 = flag_s[p2];
                     if (!f1 && !f2) {
                         pivot_load(j3sm, sq.G, sq.np, b1, b2);
                         __syncthreads();
                         if (tid == 0) atomicAdd(sq.sync + 20 + par, 1u);
-                    } else if (step > 0) pivot_form_cross<TENSOR>(j3sm, sq, Vcur, step, b1, b2, flag_s, sq.sync + 20 + par);
+                    } else if (step > 0) pivot_form_cross<TENSOR>(j3sm, sq, Vcur, step, b1, p1, h1, f1, b2, p2, h2, f2, sq.sync + 20 + par);
                     else if (TENSOR) pivot_form_half(j3sm, sq, sq.G, Vcur, step, p1, h1, f1, p2, h2, f2, sq.sync + 20 + par);
                     else pivot_form(j3sm, sq, sq.G, Vcur, step, p1, h1, f1, p2, h2, f2, sq.sync + 20 + par);
                     pivot_finish(nsweep, nstep, pr, par ^ 1);
@@ -1409,9 +1411,15 @@ __global__ void init_kernel(const __grid_constant__ Batch batch, int *status)
     }
 }
 
-// Host side: hands every sequence a group of CTAs in proportion to the size of its update (at most one
-// CTA per block of the update, at least one) and launches the kernel cooperatively, so that all
-// groups are resident together and the group barriers cannot starve.
+// Host side: gives every sequence its group of CTAs and launches the kernel cooperatively, so that all groups are resident
+// together and the group barriers cannot starve. Up to as many pairs of blocks as SMs a sequence gets a CTA for each of its pairs
+// and shares the rest with the others in proportion to the items of their updates (at most one an item); beyond, all CTAs are
+// shared by size, at least one to a sequence. An empty sequence gets none.
+// The CTAs beside the pivots stay away (seat_of) as long as the others have at most MATE_ITEMS items each. The rotation of one
+// iterate with r~ = 768: 1886 us, 2358 without seats; 1088: 3250, 3810; 1408, the largest below the line: 4694, 5311; 1472, the
+// first above: 5585 without, 5678 with; 1792: 8692, 9368. Three iterates of 576: 1575, 1884; 8 of 320: 916, 1008; 16 of 320, above:
+// 1130, 1260. (12 of 320, above as well, would be 3 % faster with seats.) Up to as many CTAs as SMs there is nothing to seat.
+constexpr int MATE_ITEMS = 2;
 template <bool TENSOR>
 static inline atp_status launch(atp_ctx *ctx, Batch &jb, float tol_conv, float tol_left, float tol_rot, int max_sweeps, bool raise_not_converged)
 {
@@ -1441,8 +1449,6 @@ static inline atp_status launch(atp_ctx *ctx, Batch &jb, float tol_conv, float t
         all_items += items[i];
     }
     if (wsum <= 0) return ATP_OK;
-    // Every pair a CTA of its own and the rest of the CTAs in proportion to the items of the update, if all pairs find an SM
-    // each; the CTAs beside them stay away as long as the others have at most MATE_ITEMS items each.
     const bool own = pairs <= ctx->sm_count;
     auto share = [&](int workers, int i) { return (int)std::min<double>(items[i], (double)workers * items[i] / all_items); };
     bool apart = own && per_sm == 2;

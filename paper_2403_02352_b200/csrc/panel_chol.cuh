@@ -15,7 +15,10 @@
 // warps finish the trailing update of the panel before meanwhile (the block that is factored next goes first), then all
 // warps form the rows of L below the panel (A_21 X_11^T) and the blocks of the inverse left of it (-X_pp L_p,: X), in
 // strips of 8 x 16 on the fp64 matrix units (with scalar multiply-adds these were bound by shared-memory reads).
-// Cycles: 40300 (first form: 4 x 4 blocks per thread, 16-way bank conflicts) -> 34600 -> 16800.
+// Cycles from block barrier to block barrier, in the kernel: 27000 -> 19600 (16 x 512 x 320 in bf16, 1024 x 764 the same), 38100 ->
+// 23700 in fp32 (1024 x 764), since the diagonal blocks are straight code that updates what lies right of its column. The fp32
+// kernel keeps more in registers around it and spills 72 bytes here, the bf16 kernel none. (The first form, 4 x 4 blocks per
+// thread with 16-way bank conflicts, took 40300 in either.)
 #pragma once
 #include "common.cuh"
 #include "jacobi3.cuh"
@@ -91,8 +94,8 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, flo
             // the diagonal block: 16 dependent pivots. The unscaled column is exchanged through shared memory before its
             // pivot is known, and the next pivot comes from the current one and two entries that every lane already has
             // (d - e^2 / piv), so the chain per column is one reciprocal and two multiply-adds (11 cycles each). Instructions count
-            // more than that chain: the code runs once per panel, and all 15 entries in every step of a loop over 16 columns
-            // (unrolled by 8) took 410 cycles a column, twice that chain. Straight code updates the entries right of the column only.
+            // more than that chain: all 15 entries in every step of a loop over 16 columns (unrolled by 8) took 410 cycles a column
+            // with what is around it, twice that chain. Straight code updates the entries right of the column only.
             // 16 x 512 x 320: 1067 -> 1008 us for the three iterates, 512 x 192 in fp32: 622 -> 566; same values.
             double e[16];
 #pragma unroll
@@ -119,14 +122,14 @@ __device__ __noinline__ void chol_invert_64(double *Gs, double *work, int n, flo
                 y = fma(y * h, fma(0.375, h, 0.5), y);
                 // a dependent column: unit pivot, zeros below; its row of the inverse keeps its scale
                 const double ic = dep_c ? 0.0 : y * y, f = e[c] * ic;
-                if (c < 15) piv = fma(-ck[c + 1 < 16 ? c + 1 : 15] * ck[c + 1 < 16 ? c + 1 : 15], ic, dn);
+                if (c < 15) piv = fma(-ck[c + 1] * ck[c + 1], ic, dn);
                 bad |= dep_c && c == lane;
                 if (lane >= 16) X[(b + c) * LDC + b + lane - 16] = c >= lane - 16 ? (dep_c ? e[c] : e[c] * y) : 0.0;
 #pragma unroll
                 for (int k = c + 1; k < 16; ++k) e[k] = fma(-f, ck[k], e[k]);
                 if (lane < 16 && c < 15) {
-                    xcol[(c + 1) & 1][lane] = e[c + 1 < 16 ? c + 1 : 15];
-                    if (c < 14) xdiag[(c + 1) & 1][lane] = e[c + 2 < 16 ? c + 2 : 15];
+                    xcol[(c + 1) & 1][lane] = e[c + 1];
+                    if (c < 14) xdiag[(c + 1) & 1][lane] = e[c + 2];
                 }
                 __syncwarp();
             }
