@@ -98,7 +98,7 @@ ALT_INNER = 2        # rounds per component of Algorithm 1, as the paper runs it
 # DRAM bytes (read + write) of one launch of the dominant kernel, from ncu captures of extractions of the same sizes
 # (mean of the two passes of a rotation); other workloads / kernels: no capture, null.
 NCU_DRAM_BYTES_PER_LAUNCH = {("bert_large_bf16", 256, "jacobi_persistent"): 11.9e6,
-                             ("llama7b_bf16", 2048, "jacobi_persistent"): 30.4e6}
+                             ("llama7b_bf16", 2048, "jacobi_persistent"): 32.5e6}
 
 
 def alt_start_vectors(w, seed):

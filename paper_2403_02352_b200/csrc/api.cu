@@ -182,8 +182,9 @@ const char *atp_status_string(atp_status s)
 // 16 bytes, so X and the residual are read once, in 16-byte loads that are all in flight together, and the statistics
 // (fp32; LayerNorm's second moment about the mean) are taken from registers. HBM-bound: 2 or 3 times rows * cols * size.
 // 4096 x 4096 bf16 with residual: 73 -> 22.5 us (the row-in-memory kernel below read two bytes a lane, and everything two or
-// three times) -> 21.0 with a programmatic launch (4800 GB/s): the CTAs come up while the launch before is still draining.
-// Streaming stores and loads past L1 change nothing (20.2 and 20.5 against 20.3 us, each timed alone).
+// three times) -> 20.9 back to back with a programmatic launch (4800 GB/s): the CTAs come up while the launch before, which
+// triggers at its own start, is draining. After a kernel that does not trigger nothing changes (behind a memset of 256 MB, events
+// included: 26.6 us with and without; 2000 x 5000 22.5). Streaming stores and loads past L1 change nothing (within 0.2 us).
 // ----------------------------------------------------------------------------------------------
 template <typename T> struct Vec16 { static constexpr int N = 16 / sizeof(T); };
 template <typename T, int NV>
