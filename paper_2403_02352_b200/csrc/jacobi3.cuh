@@ -274,6 +274,7 @@ template <int W> struct Band {
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
             const int l = (k + D0 + i) & 31;
+            if (D0 + i == 16 && k >= 16) continue;               // (two lanes have these entries, equal but for rounding)
             const float e = ee[i] * de * sh.sd[0][l], o = oo[i] * dd * sh.sd[0][32 + l];
             As[k * LDP + l] = e; As[l * LDP + k] = e;
             As[(32 + k) * LDP + 32 + l] = o; As[(32 + l) * LDP + 32 + k] = o;
@@ -948,6 +949,29 @@ __device__ __forceinline__ void store_diagonal(float *G, int np, int I, int J, c
     *(float4 *)(G + (size_t)(J * JB + i) * np + J * JB + c) = b;
 }
 
+// A fragment of an updated block of G (rows gr0, gr1; columns gc, gc + 1) goes out with its mirror. Of a block (p, p) only what
+// lies on and above the diagonal does: computed both ways, the two triangles differ by rounding, and a rotation, which reads one
+// of them, never takes away the difference.
+__device__ __forceinline__ void store_mirrored(float *G, int np, int gr0, int gr1, int gc, float v0, float v1, float v2, float v3)
+{
+    *(float2 *)(G + (size_t)gr0 * np + gc) = make_float2(v0, v1);
+    *(float2 *)(G + (size_t)gr1 * np + gc) = make_float2(v2, v3);
+    G[(size_t)gc * np + gr0] = v0; G[(size_t)(gc + 1) * np + gr0] = v1;
+    G[(size_t)gc * np + gr1] = v2; G[(size_t)(gc + 1) * np + gr1] = v3;
+}
+__device__ __forceinline__ void store_upper(float *G, int np, int gr0, int gr1, int gc, float v0, float v1, float v2, float v3)
+{
+    auto put = [&](int r, int c, float v) { if (r <= c) { G[(size_t)r * np + c] = v; G[(size_t)c * np + r] = v; } };
+    put(gr0, gc, v0); put(gr0, gc + 1, v1); put(gr1, gc, v2); put(gr1, gc + 1, v3);
+}
+// 0: this warp (rows m0 .., columns n0 .. of the block) stores nothing, 1: the triangle on and above the diagonal, 2: all, mirrored.
+__device__ __forceinline__ int part_stored(bool diagonal, bool carried, int m0, int n0)
+{
+    const bool same_half = !((m0 ^ n0) & JB);
+    if (!diagonal) return 2;
+    return same_half ? (carried ? 0 : 1) : m0 < n0 ? 2 : 0;
+}
+
 // One block (p, q) of G on the fp32 units: Vt_p G_pq Vt_q^T.
 __device__ bool g_block(float *sm, const Seq &sq, float *G, const float *Vbuf, const int *vflag, int step, int p, int q, Fetched &fetched)
 {
@@ -983,17 +1007,14 @@ __device__ bool g_block(float *sm, const Seq &sq, float *G, const float *Vbuf, c
     const bool carried = p == q && step > 0;                     // the diagonal blocks come from the pivot solve
     if (carried) store_diagonal(G, np, Ip, Jp, Vbuf + (size_t)p * VSTRIDE);
     const int gr0 = glob_of_loc(Ip, Jp, m0 + g), gr1 = glob_of_loc(Ip, Jp, m0 + g + 8);
-    if (!carried || ((m0 ^ n0) & JB))
+    const int part = part_stored(p == q, carried, m0, n0);
+    if (part)
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const int gc = glob_of_loc(Iq, Jq, n0 + nt * 8 + 2 * t);         // gc, gc + 1 are contiguous
-        *(float2 *)(G + (size_t)gr0 * np + gc) = make_float2(acc[nt][0], acc[nt][1]);
-        *(float2 *)(G + (size_t)gr1 * np + gc) = make_float2(acc[nt][2], acc[nt][3]);
-        if (q != p) {                                            // mirror block
-            G[(size_t)gc * np + gr0] = acc[nt][0]; G[(size_t)(gc + 1) * np + gr0] = acc[nt][1];
-            G[(size_t)gc * np + gr1] = acc[nt][2]; G[(size_t)(gc + 1) * np + gr1] = acc[nt][3];
+        for (int nt = 0; nt < 4; ++nt) {
+            const int gc = glob_of_loc(Iq, Jq, n0 + nt * 8 + 2 * t);     // gc, gc + 1 are contiguous
+            if (part == 2) store_mirrored(G, np, gr0, gr1, gc, acc[nt][0], acc[nt][1], acc[nt][2], acc[nt][3]);
+            else store_upper(G, np, gr0, gr1, gc, acc[nt][0], acc[nt][1], acc[nt][2], acc[nt][3]);
         }
-    }
     __syncthreads();                                             // tiles are reused by the next block
     return true;
 }
@@ -1093,19 +1114,16 @@ __device__ bool g_block_half(float *sm, const Seq &sq, float *G, const float *Vb
     if (carried) store_diagonal(G, np, Ip, Jp, Pp);
     const int gr0 = glob_of_loc(Ip, Jp, m0 + g), gr1 = glob_of_loc(Ip, Jp, m0 + g + 8);
     const float s0 = sp[m0 + g] * k, s1 = sp[m0 + g + 8] * k;
-    if (!carried || ((m0 ^ n0) & JB))
+    const int part = part_stored(p == q, carried, m0, n0);
+    if (part)
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const int lc = n0 + nt * 8 + 2 * t, gc = glob_of_loc(Iq, Jq, lc);        // gc, gc + 1 are contiguous
-        const float q0 = sqv[lc], q1 = sqv[lc + 1];
-        const float v0 = acc[nt][0] * s0 * q0, v1 = acc[nt][1] * s0 * q1, v2 = acc[nt][2] * s1 * q0, v3 = acc[nt][3] * s1 * q1;
-        *(float2 *)(G + (size_t)gr0 * np + gc) = make_float2(v0, v1);
-        *(float2 *)(G + (size_t)gr1 * np + gc) = make_float2(v2, v3);
-        if (q != p) {                                            // mirror block
-            G[(size_t)gc * np + gr0] = v0; G[(size_t)(gc + 1) * np + gr0] = v1;
-            G[(size_t)gc * np + gr1] = v2; G[(size_t)(gc + 1) * np + gr1] = v3;
+        for (int nt = 0; nt < 4; ++nt) {
+            const int lc = n0 + nt * 8 + 2 * t, gc = glob_of_loc(Iq, Jq, lc);    // gc, gc + 1 are contiguous
+            const float q0 = sqv[lc], q1 = sqv[lc + 1];
+            const float v0 = acc[nt][0] * s0 * q0, v1 = acc[nt][1] * s0 * q1, v2 = acc[nt][2] * s1 * q0, v3 = acc[nt][3] * s1 * q1;
+            if (part == 2) store_mirrored(G, np, gr0, gr1, gc, v0, v1, v2, v3);
+            else store_upper(G, np, gr0, gr1, gc, v0, v1, v2, v3);
         }
-    }
     __syncthreads();                                             // tiles are reused by the next block
     return true;
 }

@@ -65,3 +65,19 @@ def test_what_the_second_pass_leaves_in_bf16():
         finally:
             c.close()
     assert worst <= 4.5e-5
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("L,r", [(300, 60), (64, 40), (300, 150), (700, 400)])
+def test_rotated_matrix_is_symmetric(L, r, dtype):
+    # to the last bit, in matrices of one pair of blocks, of two and of many: what the two triangles differ by is never rotated away
+    import paper_2403_02352_b200 as atp
+    c = atp.Context(0)
+    try:
+        noise = torch.randn((L, 1024), device="cuda", generator=torch.Generator(device="cuda").manual_seed(L + r))
+        _, _, sig = atp.atp_principal_basis(c, (planted(1, L, 1024, 16, 1) + 0.02 * noise).to(dtype), [L], [r])
+        c.poll()
+        g = rotated_gram(c, sig.double(), min(L, r + 64))
+        assert bool((g == g.T).all())
+    finally:
+        c.close()
