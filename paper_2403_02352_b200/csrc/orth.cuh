@@ -378,14 +378,22 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                     __syncthreads();
                     // a nearly orthonormal panel gets its factor from a short series instead of the factorisation
                     if (!(series_ok && lowdin_64(Gs, w, sA, (__half *)sB, sq.W, sq.flags))) {
-                        // given up (see lost_length): columns of which nothing is left, but not the replacements of the last factor
+                        // given up (see lost_length): columns of which nothing is left, but not the replacements of the last factor.
+                        // Where the factor is that of unit columns, one that has lost half of its length asks for another repetition:
+                        // the factor enlarges what the finished columns' own errors have left in it, by up to 128 within the limits
+                        // of a benign factor, and the next panel starts from that (581 x 952 tokens that fall by 60 octaves, six
+                        // panels: U^T U - I of 0.2).
+                        const bool unit = stage == 24 || (stage == 33 && rep > 0);
                         const float lost = lost_length(stage == 24 ? rep : stage == 33 ? rep - 1 : 0);
-                        const bool old = lost > 0.f && tid < w && !(__ldcg(sq.flags + tid) & 1);
+                        const bool old = unit && tid < w && !(__ldcg(sq.flags + tid) & 1);
                         chol_invert_64(Gs, (double *)osm, w, sq.W, sq.flags);
-                        if (lost > 0.f) {
+                        if (unit) {
                             __syncthreads();
                             // the diagonal of the factor: 1 / length outside the columns before
-                            if (old && __ldcg(sq.W + tid * 65) * lost >= 1.f) sq.flags[tid] |= 1;
+                            if (old) {
+                                const float inv = __ldcg(sq.W + tid * 65);
+                                sq.flags[tid] |= (inv * lost >= 1.f ? 1 : 0) | (inv > 2.f ? 4 : 0);
+                            }
                         }
                     }
                     __syncthreads();

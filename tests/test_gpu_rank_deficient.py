@@ -106,6 +106,24 @@ def test_falling_tokens_nearly_square(L, r, octaves, seed):
         c.close()
 
 
+# six panels of components down to 1e-10 of the first: each panel enlarged what the errors of the finished ones had left in it, up to a
+# hundredfold, as long as a unit column that had lost less than three quarters of its length counted as done (U^T U - I of 0.2)
+def test_errors_of_finished_panels_do_not_grow():
+    import paper_2403_02352_b200 as atp
+    L, d, r = 581, 952, 290
+    gen = torch.Generator(device="cuda").manual_seed(255)
+    X = torch.randn((L, d), generator=gen, device="cuda") * torch.exp2(-60 * torch.arange(L, device="cuda") / L)[:, None]
+    X = X[torch.randperm(L, generator=gen, device="cuda")].bfloat16()
+    c = atp.Context(0)
+    try:
+        U, _, _ = atp.atp_principal_basis(c, X, [L], [r])
+        c.poll()
+        u = U[:, :r].double()
+        assert (u.T @ u - torch.eye(r, device="cuda")).abs().max() <= 2e-2
+    finally:
+        c.close()
+
+
 # with the two triangles of G computed each for itself the first of these (33 of 40 seeds of a like case) ran into the sweep limit
 @pytest.mark.parametrize("seed,L,d,dtype", [(33, 64, 64, torch.float32), (34, 64, 64, torch.float32), (22, 33, 40, torch.float32),
                                             (15, 64, 64, torch.bfloat16), (3, 33, 40, torch.bfloat16), (1, 200, 304, torch.float32)])
