@@ -382,7 +382,7 @@ orth_persistent_kernel(const __grid_constant__ Batch batch, int reps, uint64_t s
                         // Where the factor is that of unit columns, one that has lost half of its length asks for another repetition:
                         // the factor enlarges what the finished columns' own errors have left in it, by up to 128 within the limits
                         // of a benign factor, and the next panel starts from that (581 x 952 tokens that fall by 60 octaves, six
-                        // panels: U^T U - I of 0.2).
+                        // panels: U^T U - I of 0.2, 5e-3 with it).
                         const bool unit = stage == 24 || (stage == 33 && rep > 0);
                         const float lost = lost_length(stage == 24 ? rep : stage == 33 ? rep - 1 : 0);
                         const bool old = unit && tid < w && !(__ldcg(sq.flags + tid) & 1);
